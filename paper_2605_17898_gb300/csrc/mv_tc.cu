@@ -537,13 +537,14 @@ cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int
         a.log2s2 = fmt == kFmtF16 ? 15.0f : kp.log2_s2;
         a.col_scale = fmt == kFmtF16 ? col_scale : nullptr;
         // the drain's blocks go to out by TMA reduce when out's rows are 16-byte aligned
+        // (box: one drain warp's slab of 32 rows x t / 2 columns, swizzled by its row length)
         CUtensorMap mo;
         memset(&mo, 0, sizeof mo);
         const bool aligned = (uintptr_t)out % 16 == 0 && ldo % 4 == 0;
         a.add_mode = aligned ? tcs::kAddTma : tcs::kAddScalar;
-        if (aligned && !make_map_strided(&mo, out, (uint64_t)t, (uint64_t)N, (uint64_t)ldo * 4, (uint32_t)t,
-                                         (uint32_t)tcs::kTile,
-                                         t == 32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B))
+        if (aligned &&
+            !make_map_strided(&mo, out, (uint64_t)t, (uint64_t)N, (uint64_t)ldo * 4, (uint32_t)(t / 2), 32u,
+                              t == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B))
             a.add_mode = tcs::kAddVec4;
         a.budget = wait_budget;
         a.gate = nullptr;

@@ -152,6 +152,64 @@ static __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, 
     }
 }
 
+// mbar_wait by a whole converged warp: true only if every lane's wait succeeded, so that the warp leaves
+// its loop together.
+static __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, long long budget,
+                                                   volatile int *abort_flag, int *err, int code, int sleep_ns = 0) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, budget, abort_flag, err, code, sleep_ns));
+}
+
+// Non-blocking test of the phase with the given parity.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// Bounded wait of a whole converged warp until N phases have completed. Each poll tests all of them before
+// it looks at any answer: a test takes ~140 cycles to answer under the product's load (measured), so waiting
+// for one barrier after the other costs that much for each even when all are already complete.
+template <int N>
+static __device__ __forceinline__ bool mbar_wait_all_warp(const uint32_t (&bar)[N], const uint32_t (&parity)[N],
+                                                       long long budget, volatile int *abort_flag, int *err, int code) {
+    auto poll = [&]() {
+        bool ok = true;
+#pragma unroll
+        for (int k = 0; k < N; ++k) ok &= mbar_test(bar[k], parity[k]);
+        return __all_sync(0xffffffffu, ok);
+    };
+    if (poll()) return true;
+    const long long t0 = clock64();
+    while (true) {
+        if (poll()) return true;
+        const bool late = clock64() - t0 > budget;
+        if (__any_sync(0xffffffffu, late || *abort_flag)) {
+            if (late) {
+                *abort_flag = 1;
+                atomicOr(err, code);
+            }
+            return false;
+        }
+    }
+}
+
+// True in one lane of a converged warp, the same lane at every call.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int c0, int c1, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
@@ -237,6 +295,15 @@ __device__ __forceinline__ void tmem_ld<32>(uint32_t taddr, uint32_t (&r)[32]) {
 }
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// The wait for loads in flight into r, with r as its operands so that no use of them moves above it.
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+                 :
+                 : "memory");
+}
 
 // Round two floats to a packed pair (first in the low half) and read the pair back as floats.
 template <int FMT>
@@ -344,7 +411,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + L::kBar + 192);
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + L::kBar + 200);
 
-    const int warp = threadIdx.x >> 5;
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);  // warp-uniform for the compiler
     const int lane = threadIdx.x & 31;
     const int64_t row0 = (int64_t)blockIdx.x * kBM;
     const int c_begin = blockIdx.y * a.chunks_per_split;
@@ -413,7 +480,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
     } else if (warp == kMmaWarp) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        // The whole warp runs the loop and elects a lane for each pair of MMAs, so that descriptors stay in uniform
+        // registers (from a divergent one-lane branch the microbenchmarked issue took twice as long): N = 20000,
+        // D = 8, t = 32 446 -> 436 us, D = 4, t = 16 278 -> 260 us; unchanged at N = 4099 (latency).
+        {
             const uint32_t idesc2 = instr_desc<2 * T, FMT>();  // K_hi x [V_hi V_lo]
             const uint32_t idesc1 = instr_desc<T, FMT>();      // K_lo x V_hi
             bool issued = false;
@@ -425,9 +495,9 @@ __global__ void __launch_bounds__(kThreads, 1)
                 const bool group_end = (it % kGroup) == kGroup - 1 || it == n_it - 1;
                 // the drain warps must have read this buffer's previous group (g - 2)
                 if (group_start && g >= 2 &&
-                    !mbar_wait(bar_acc_empty(buf), ((g >> 1) - 1) & 1, a.budget, abort_flag, a.err, kErrWaitAcc, 32))
+                    !mbar_wait_warp(bar_acc_empty(buf), ((g >> 1) - 1) & 1, a.budget, abort_flag, a.err, kErrWaitAcc, 32))
                     break;
-                if (!mbar_wait(bar_ready(s), (it / kStages) & 1, a.budget, abort_flag, a.err, kErrWaitReady, 32)) break;
+                if (!mbar_wait_warp(bar_ready(s), (it / kStages) & 1, a.budget, abort_flag, a.err, kErrWaitReady, 32)) break;
                 tc_fence_after();
                 const uint32_t acc = tmem_acc + (uint32_t)(buf * kAccCols);
                 const uint32_t st = smem_u32(smem + s * L::kStage);
@@ -445,22 +515,28 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const uint32_t first = (group_start && ks == 0) ? 0u : 1u;
                     if constexpr (ATMEM) {
                         const uint32_t ah = a_col + 8 * ks, al = a_col + 32 + 8 * ks;
-                        mma_ts(acc, ah, dbv, idesc2, first);
-                        mma_ts(acc_lo, al, dbv, idesc1, first);
+                        if (elect_one()) {
+                            mma_ts(acc, ah, dbv, idesc2, first);
+                            mma_ts(acc_lo, al, dbv, idesc1, first);
+                        }
                     } else {
                         const uint64_t dah = smem_desc(st + ks * 4096, 2048, 128);
                         const uint64_t dal = smem_desc(st + L::kA + ks * 4096, 2048, 128);
-                        mma_ss(acc, dah, dbv, idesc2, first);
-                        mma_ss(acc_lo, dal, dbv, idesc1, first);
+                        if (elect_one()) {
+                            mma_ss(acc, dah, dbv, idesc2, first);
+                            mma_ss(acc_lo, dal, dbv, idesc1, first);
+                        }
                     }
                 }
-                mma_commit(bar_empty(s));
-                if (group_end) mma_commit(bar_acc_full(buf));
+                if (elect_one()) {
+                    mma_commit(bar_empty(s));
+                    if (group_end) mma_commit(bar_acc_full(buf));
+                }
                 issued = true;
             }
             if (issued) {
                 // every MMA this thread issued has completed before the CTA frees tensor memory
-                mma_commit(bar_fin);
+                if (elect_one()) mma_commit(bar_fin);
                 volatile int no_abort = 0;
                 mbar_wait(bar_fin, 0, kDrainBudget, &no_abort, a.err, 0);
             }

@@ -12,7 +12,7 @@ cudaError_t launch_tcs_inst(dim3 grid, const CUtensorMap &mx, const CUtensorMap 
                             const TcsArgs &a,
                             cudaStream_t st) {
     constexpr int DP = D <= 4 ? 4 : 8;
-    constexpr int bytes = DOT ? TcdLayout<T, DP>::kBytes : TcsLayout<T, DP>::kBytes;
+    constexpr int bytes = TcsLayout<T, DP, DOT>::kBytes;
     static bool configured = false;
     if (!configured) {
         cudaError_t e = cudaFuncSetAttribute(mv_tcs_kernel<KIND, D, T, FMT, DOT, BANDED>,
@@ -20,7 +20,7 @@ cudaError_t launch_tcs_inst(dim3 grid, const CUtensorMap &mx, const CUtensorMap 
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    mv_tcs_kernel<KIND, D, T, FMT, DOT, BANDED><<<grid, DOT ? kDotThreads : kThreads, bytes, st>>>(mx, mv, mo, a);
+    mv_tcs_kernel<KIND, D, T, FMT, DOT, BANDED><<<grid, kTcsThreads, bytes, st>>>(mx, mv, mo, a);
     return cudaGetLastError();
 }
 
