@@ -398,8 +398,10 @@ bool kernel_timing_on(const lgp_ctx *ctx, cudaStream_t st) {
     return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
 }
 
+// v_ready, tail: see launch_mv_tc (v_ready for the tensor-core products only).
 lgp_status matvec_prepared(lgp_ctx *ctx, const Prepared &pp, const float *V, int64_t ldv, float *out, int64_t ldo,
-                           int t, int prec, const int *skip, cudaStream_t st, int dist_form = -1) {
+                           int t, int prec, const int *skip, cudaStream_t st, int dist_form = -1, bool v_ready = false,
+                           ProductTail *tail = nullptr) {
     if (is_tc(prec)) {
         lgp_status s = ensure(ctx, ctx->vsplit, (size_t)tc_vsplit_bytes(pp.Np, t));
         if (s != LGP_OK) return s;
@@ -413,7 +415,7 @@ lgp_status matvec_prepared(lgp_ctx *ctx, const Prepared &pp, const float *V, int
                               (float *)ctx->mv_partial.p,
                               (int64_t)(ctx->mv_partial.bytes / sizeof(float)), skip, (int *)ctx->flags.p + 1,
                               ctx->wait_budget, ctx->num_sms, st, forced, tc_operands_valid(ctx, pp, t, prec),
-                              dist_form, timed ? ctx->kev[0] : nullptr, timed ? ctx->kev[1] : nullptr));
+                              dist_form, timed ? ctx->kev[0] : nullptr, timed ? ctx->kev[1] : nullptr, v_ready, tail));
         if (timed) ctx->kev_set = true;
         if (forced == kTcSymmetric) {
             ctx->sym_kind = pp.kp.kind;
@@ -440,6 +442,7 @@ lgp_status matvec_prepared(lgp_ctx *ctx, const Prepared &pp, const float *V, int
     m.partial_cap = (int64_t)(ctx->mv_partial.bytes / sizeof(float));
     m.skip = skip;
     m.num_sms = ctx->num_sms;
+    m.tail = tail;
     const bool timed = kernel_timing_on(ctx, st);
     if (timed) cudaEventRecord(ctx->kev[0], st);
     LGP_CUDA(launch_mv_simt(m, st));
@@ -583,18 +586,19 @@ lgp_status build_precond(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X, con
     return LGP_OK;
 }
 
+// Kernel launches of one CG iteration: the product kernel (both distance instances where the host does not know the
+// form), the split of p where it is not part of the step, and the step.
+int cg_iteration_launches(const lgp_ctx *ctx, const Prepared &pp, int t, int prec, bool precond, int dist_form = -1) {
+    int n = 1 + 3;
+    if (is_tc(prec)) {
+        if (needs_dot(ctx, pp, t, prec) && dist_form < 0) ++n;
+        if (precond) n += tc_fmt(prec) == 1 ? 2 : 1;
+        // the row kernel's split reduction is part of the step, also when preconditioned
+    }
+    return n + (precond ? 4 : 0);
+}
+
 // Run CG on the internal stream: init, then replay a captured chunk of iterations until done.
-int matvec_launches(const lgp_ctx *ctx, const Prepared &pp, int t, int prec, int dist_form = -1) {
-    return is_tc(prec) ? mv_tc_launches(pp.Np, t, ctx->num_sms, tc_fmt(prec), tc_splits_for(ctx, pp, t, prec), pp.kp.kind,
-                                        pp.kp.D, tc_operands_valid(ctx, pp, t, prec), dist_form)
-                       : mv_simt_launches(pp.N, pp.Np, t, ctx->num_sms);
-}
-
-// Kernel launches of one CG iteration (the product plus the five vector/scalar kernels).
-int cg_iteration_launches(const lgp_ctx *ctx, const Prepared &pp, int t, int prec, int dist_form = -1) {
-    return matvec_launches(ctx, pp, t, prec, dist_form) + 5;
-}
-
 lgp_status run_cg(lgp_ctx *ctx, const Prepared &pp, const float *B, int64_t ldb, int t, const lgp_options *opt,
                   int hist_len, int prec, CgBuffers *bout, int *chunks_run = nullptr, const Precond *pc = nullptr,
                   const float *X0 = nullptr) {
@@ -641,17 +645,33 @@ lgp_status run_cg(lgp_ctx *ctx, const Prepared &pp, const float *B, int64_t ldb,
     launch_cg_init(B, ldb, pp.N, pp.Np, t, b, opt->tol, opt->max_iter, hist_len, st, X0, t);
     LGP_CUDA(cudaGetLastError());
 
+    // plain CG on the tensor cores: p is split by the pass that updates it, the first p here
+    const bool fused_split = is_tc(prec) && !pc;
+    CgSplit split = {};
+    if (fused_split) {
+        const bool symmetric = tc_splits_for(ctx, pp, t, prec) == kTcSymmetric;
+        split = tc_cg_split(pp.kp, pp.Np, t, tc_fmt(prec), ctx->vsplit.p, symmetric ? b.Kp : nullptr);
+        LGP_CUDA(launch_v_split(pp.kp, pp.N, pp.Np, b.p, t, t, tc_fmt(prec), ctx->vsplit.p, split.out_init, t, nullptr,
+                                ctx->num_sms, st));
+        if (tc_fmt(prec) == 1)
+            LGP_CUDA(cudaMemcpyAsync(b.state->pmax, split.vmax, t * sizeof(unsigned int), cudaMemcpyDeviceToDevice, st));
+    }
+    auto iteration = [&]() -> lgp_status {
+        ProductTail tail;
+        const lgp_status r =
+            matvec_prepared(ctx, pp, b.p, t, b.Kp, t, t, prec, &b.state->done, st, dist_form, fused_split, &tail);
+        if (r == LGP_OK) launch_cg_after_matvec(pp.N, t, b, tail, fused_split ? &split : nullptr, st);
+        return r;
+    };
+
     const char *graph_env = std::getenv("LGP_CG_GRAPH");
     if (graph_env && graph_env[0] == '0') {
         // Host-driven loop: the same kernels launched one by one, the done flag read back after
         // every chunk (a profiler then sees each launch on its own).
         int launched = 0;
         while (true) {
-            for (int k = 0; k < kChunk; ++k) {
-                if ((s = matvec_prepared(ctx, pp, b.p, t, b.Kp, t, t, prec, &b.state->done, st, dist_form)) != LGP_OK)
-                    return s;
-                launch_cg_after_matvec(pp.N, pp.Np, t, b, st);
-            }
+            for (int k = 0; k < kChunk; ++k)
+                if ((s = iteration()) != LGP_OK) return s;
             launch_cg_chunk_tally(b.state, st);
             ++launched;
             LGP_CUDA(cudaMemcpyAsync(ctx->h_state, b.state, sizeof(CgState), cudaMemcpyDeviceToHost, st));
@@ -719,10 +739,7 @@ lgp_status run_cg(lgp_ctx *ctx, const Prepared &pp, const float *B, int64_t ldb,
             return fail(ctx, LGP_ERR_CUDA, "capture to graph: %s", cudaGetErrorString(ce));
         }
         lgp_status cs = LGP_OK;
-        for (int k = 0; k < kChunk && cs == LGP_OK; ++k) {
-            cs = matvec_prepared(ctx, pp, b.p, t, b.Kp, t, t, prec, &b.state->done, st, dist_form);
-            if (cs == LGP_OK) launch_cg_after_matvec(pp.N, pp.Np, t, b, st);
-        }
+        for (int k = 0; k < kChunk && cs == LGP_OK; ++k) cs = iteration();
         if (cs == LGP_OK) launch_cg_loop_condition(h, b.state, st);
         cudaGraph_t captured = nullptr;
         ce = cudaStreamEndCapture(st, &captured);
@@ -1640,20 +1657,20 @@ lgp_status lgp_lml_and_grad(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X, 
         info->logdet_precond = k > 0 ? pc.logdet : 0.0;
         (void)chunks;
         // prep_x, y copy, probes, CG init (2), the loop's chunks, column dots (2), SLQ (2), adjoint (3)
-        // preconditioned: 3 more launches per iteration and in the CG init; the build (init, 2 per rank step, Gram,
+        // preconditioned: 3 more launches in the CG init; the build (init, 2 per rank step, Gram,
         // float32 copy), the P-distributed probes, and P^{-1} of the probe block with the y copy
-        const int pc_iter = k > 0 ? 3 : 0;
         const int pc_once = k > 0 ? (2 * k + 3) + 3 + 1 + 4 : 0;
         // the products' X-only operands, built once before the loop (transpose; box and operands of the dot form)
         const int opnd_once = is_tc(prec) && tc_operands_valid(ctx, pp, t, prec) ? (ctx->opnd_dot ? 3 : 1) : 0;
         if (!single) {
-            info->launches = 3 + 2 +
-                             ran * (kChunk * (cg_iteration_launches(ctx, pp, t, prec, ctx->cg_dist_form) + pc_iter) + 1) +
-                             2 + 2 + (grad ? 3 : 0) + pc_once + opnd_once;
+            const int split_once = is_tc(prec) && k == 0 ? (tc_fmt(prec) == 1 ? 2 : 1) : 0;
+            info->launches = 3 + 2 + split_once +
+                             ran * (kChunk * cg_iteration_launches(ctx, pp, t, prec, k > 0, ctx->cg_dist_form) + 1) + 2 + 2 +
+                             (grad ? 3 : 0) + pc_once + opnd_once;
         } else {
             // per column: CG init (2), copy and gather (2); the chunks of all columns; per column in the
             // gradient: two column copies and one adjoint pass
-            info->launches = 3 + 4 * t + ran * (kChunk * (mv_simt_launches(pp.N, pp.Np, 1, ctx->num_sms) + 5) + 1) +
+            info->launches = 3 + 4 * t + ran * (kChunk * cg_iteration_launches(ctx, pp, 1, LGP_PREC_FP32, false) + 1) +
                              2 + 2 + (grad ? 2 + 3 * t : 0);
         }
     }

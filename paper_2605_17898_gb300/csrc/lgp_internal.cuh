@@ -164,6 +164,10 @@ struct CgState {
     double w0[kMaxT];  // b^T P^{-1} b: the Lanczos quadrature weight of each column
     double alpha[kMaxT];
     double beta[kMaxT];
+    double thresh[kMaxT];       // a column stops once r^T r <= thresh = (tol ||b||)^2
+    unsigned int rmax[kMaxT];   // float bits of max |r| after the last update (solves whose p is split here)
+    unsigned int pmax[kMaxT];   // float bits of max |p|
+    unsigned int ticket;        // blocks of the current kernel that have written their partial sums
 };
 
 // ---------------------------------------------------------------- launchers (defined in the .cu files)
@@ -183,6 +187,15 @@ void launch_var_from_dots(const double *dots, int c0, int t, float s2, float *va
 void launch_var_from_probes(const float *Z, int64_t ldz, const float *Q, int64_t ldq, int64_t M, int m, float s2,
                             float *var, cudaStream_t st);
 
+// What a product left for its caller to finish when asked to (the CG step, which reads the same rows anyway):
+// S > 1 column-split partial sums, out = sum_k part[k * stride + e] + noise V. S = 1: out is complete.
+struct ProductTail {
+    const float *part = nullptr;
+    int S = 1;
+    int64_t stride = 0;
+    float noise = 0.0f;
+};
+
 // mv_simt.cu
 struct MvLaunch {
     const KernelParams *kp;
@@ -197,13 +210,14 @@ struct MvLaunch {
     int64_t partial_cap;  // floats available in partial
     const int *skip;      // device flag: skip all work when *skip != 0 (may be nullptr)
     int num_sms;
+    // With tail set, column-split partial sums are left to the caller (see ProductTail).
+    struct ProductTail *tail = nullptr;
     // Cross product out = K(Xr, Xs) V (no noise term): prescaled row points [Npr, dpad] and their
     // count; Xr == nullptr gives the square product K_y V.
     const float *Xr = nullptr;
     int64_t Nr = 0, Npr = 0;
 };
 cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st);
-int mv_simt_launches(int64_t N, int64_t Np, int t, int num_sms);
 int64_t mv_simt_partial_floats(int64_t N, int64_t Np, int t, int num_sms);
 // Split partial floats of the cross product with Nr output rows (Npr padded) and N columns.
 int64_t mv_simt_cross_partial_floats(int64_t Nr, int64_t Npr, int64_t N, int t, int num_sms);
@@ -231,13 +245,32 @@ constexpr int kTcSymmetric = -1;
 // dist_form (symmetric product with the dot form allowed): -1 = not known on the host, so both distance
 // instances launch and the device gate word lets one of them work; 0 / 1 = only the difference / dot
 // instance launches (the caller read the gate word, which must then give the same answer).
+// v_ready: V is already split in the workspace, and out of a symmetric product already holds sigma^2 V
+// (launch_v_split, launch_p_split). tail (optional): see ProductTail.
 // ev_begin / ev_end (optional): recorded on st immediately before and after the product kernel's
 // launch(es), after the V split and operand kernels (the kernel timing of lgp_last_kernel_ms).
 cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, const float *V, int64_t ldv,
                          float *out, int64_t ldo, int t, int fmt, void *vsplit, float *partial, int64_t partial_cap,
                          const int *skip, int *err_flag, long long wait_budget, int num_sms, cudaStream_t st,
                          int forced_splits = 0, bool operands_ready = false, int dist_form = -1,
-                         cudaEvent_t ev_begin = nullptr, cudaEvent_t ev_end = nullptr);
+                         cudaEvent_t ev_begin = nullptr, cudaEvent_t ev_end = nullptr, bool v_ready = false,
+                         ProductTail *tail = nullptr);
+// A CG solve's vector p as the split operand of its products (p row stride t, the workspace of one vsplit).
+struct CgSplit {
+    int fmt;
+    uint16_t *vs;         // stacked [V_hi; V_lo]
+    unsigned int *vmax;   // f16: per-column bound on |p| (float bits) that sets the scaling exponents
+    float *col_scale;
+    float s2;
+    float *out_init;      // [N, t] set to noise * p (symmetric product), or nullptr
+    float noise;
+};
+CgSplit tc_cg_split(const KernelParams &kp, int64_t Np, int t, int fmt, void *vsplit, float *out_init);
+// The split operands of V (column maxima for f16, halves, scaling factors), and out_init = noise V if given.
+cudaError_t launch_v_split(const KernelParams &kp, int64_t N, int64_t Np, const float *V, int64_t ldv, int t, int fmt,
+                           void *vsplit, float *out_init, int64_t ldo, const int *skip, int num_sms, cudaStream_t st);
+// p = r + beta p for the active columns and p's split operands, in one pass (the CG step's last launch).
+void launch_p_split(const CgSplit &sp, float *p, const float *r, int64_t N, int t, CgState *state, cudaStream_t st);
 // The operands of the tensor-core products that depend on X alone, into the t-column V-split workspace:
 // the transposed prescaled X, and with dot = true the dot-form distance data of the symmetric product
 // (box, centred split operands, squared norms, the gate word).
@@ -245,9 +278,6 @@ cudaError_t launch_tc_operands(const KernelParams &kp, const float *Xs, int64_t 
                                bool dot, cudaStream_t st);
 int64_t mv_tc_partial_floats(int64_t Np, int t, int num_sms);
 int64_t mv_tc_partial_floats(int64_t Np, int t, int num_sms, int forced_splits);
-// Kernels one split tensor-core product launches (arguments as launch_mv_tc).
-int mv_tc_launches(int64_t Np, int t, int num_sms, int fmt, int forced_splits = 0, int kind = -1, int D = 0,
-                   bool operands_ready = false, int dist_form = -1);
 // Up to four kernel choices worth timing: kTcSymmetric (when tc_symmetric_ok) and the three most
 // wave-efficient split counts.
 void tc_split_candidates(int64_t Np, int num_sms, int *cand, int *n);
@@ -301,7 +331,9 @@ struct CgBuffers {
 // X0 (may be null): warm start x0 [N, ldx0], with K_y x0 already in b.Kp.
 void launch_cg_init(const float *B, int64_t ldb, int64_t N, int64_t Np, int t, const CgBuffers &b, double tol,
                     int max_iter, int hist_len, cudaStream_t st, const float *X0 = nullptr, int64_t ldx0 = 0);
-void launch_cg_after_matvec(int64_t N, int64_t Np, int t, const CgBuffers &b, cudaStream_t st);
+// One CG iteration after its product (b.Kp, or its partial sums in tail); split: p's halves for the next product.
+void launch_cg_after_matvec(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,
+                            cudaStream_t st);
 void launch_cg_copy_out(const CgBuffers &b, int64_t N, int t, float *Xsol, int64_t ldx, cudaStream_t st);
 // Column 0 of the single-column run b1 (state, first hist_len Lanczos coefficients) into column c of a
 // t-column state and history; dst->loop_chunks accumulates.

@@ -92,10 +92,6 @@ int64_t mv_simt_cross_partial_floats(int64_t Nr, int64_t Npr, int64_t N, int t, 
     return S > 1 ? S * Npr * t : 0;
 }
 
-int mv_simt_launches(int64_t N, int64_t Np, int t, int num_sms) {
-    return mv_simt_partial_floats(N, Np, t, num_sms) > 0 ? 2 : 1;
-}
-
 cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st) {
     const bool cross = m.Xr != nullptr;
     const int64_t Nr = cross ? m.Nr : m.N, Npr = cross ? m.Npr : m.Np;
@@ -136,7 +132,15 @@ cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st) {
         case LGP_MATERN32: e = mv_simt_dispatch_m32(m.kp->D, sh.TT, sh.R, grid, a, st); break;
         default: e = cudaErrorInvalidValue;
     }
+    if (m.tail) *m.tail = ProductTail();
     if (e != cudaSuccess || S == 1) return e;
+    if (m.tail) {
+        m.tail->part = m.partial;
+        m.tail->S = (int)S;
+        m.tail->stride = Npr * m.t;
+        m.tail->noise = m.kp->noise;
+        return cudaSuccess;
+    }
     reduce_split_kernel<<<grid_for(Nr * m.t), 256, 0, st>>>(m.partial, (int)S, Npr, Nr, m.t, m.V, m.ldv, m.out,
                                                             m.ldo, m.kp->noise, a.cross, m.skip);
     return cudaGetLastError();

@@ -42,6 +42,41 @@ __device__ __forceinline__ int col_exponent(unsigned int maxbits) {
     return min(60, max(-60, 15 - ex));
 }
 
+// The halves of column c of rows 8g .. 8g + 7 (values v, scaled by 2^ec for f16) in the order below.
+template <int T, int FMT>
+__device__ __forceinline__ void store_split(uint16_t *__restrict__ vs, int64_t g, int c, const float (&vals)[8], int ec) {
+    uint32_t hw[4], lw[4];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        uint16_t h, l;
+        if (FMT == kFmtBF16) {
+            const float v = vals[k];
+            const __nv_bfloat16 hb = __float2bfloat16_rn(v);
+            const __nv_bfloat16 lb = __float2bfloat16_rn(v - __bfloat162float(hb));
+            h = *reinterpret_cast<const uint16_t *>(&hb);
+            l = *reinterpret_cast<const uint16_t *>(&lb);
+        } else {
+            const float v = ldexpf(vals[k], ec);
+            const __half hh = __float2half_rn(v);
+            const __half lh = __float2half_rn(v - __half2float(hh));
+            h = *reinterpret_cast<const uint16_t *>(&hh);
+            l = *reinterpret_cast<const uint16_t *>(&lh);
+        }
+        if (k & 1) {
+            hw[k >> 1] |= (uint32_t)h << 16;
+            lw[k >> 1] |= (uint32_t)l << 16;
+        } else {
+            hw[k >> 1] = h;
+            lw[k >> 1] = l;
+        }
+    }
+    const int64_t q = (8 * g) / kBK;
+    const int jj = (int)(8 * g - q * kBK);  // multiple of 8
+    const int64_t chunk = q * kBK * 2 * T + (int64_t)(jj >> 3) * (2 * T / 8) * 64 + (c & 7) * 8;
+    *reinterpret_cast<uint4 *>(vs + chunk + (int64_t)(c >> 3) * 64) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+    *reinterpret_cast<uint4 *>(vs + chunk + (int64_t)((T + c) >> 3) * 64) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+}
+
 // V -> stacked [V_hi; V_lo] in the tile order the MMA reads: B row c' = c (hi) or t + c (lo);
 // element (j, c') of chunk q = j / 64 sits at q*64*2t + ((j%64)/8 * 2t/8 + c'/8) * 64 + (c'%8) * 8 + j%8;
 // rows j >= N are zero. One thread per (8-row group, column): its 8 hi and 8 lo values are contiguous
@@ -64,38 +99,69 @@ __global__ void split_v_kernel(const float *__restrict__ V, int64_t ldv, int64_t
             ec = col_exponent(vmax[c]);
             if (g == 0) col_scale[c] = ldexpf(s2, -15 - ec);
         }
-        uint32_t hw[4], lw[4];
+        float v[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
             const int64_t j = 8 * g + k;
-            float v = j < N ? V[j * ldv + c] : 0.0f;
-            if (out_init && j < N) out_init[j * ldo + c] = noise * v;
-            uint16_t h, l;
-            if (FMT == kFmtBF16) {
-                const __nv_bfloat16 hb = __float2bfloat16_rn(v);
-                const __nv_bfloat16 lb = __float2bfloat16_rn(v - __bfloat162float(hb));
-                h = *reinterpret_cast<const uint16_t *>(&hb);
-                l = *reinterpret_cast<const uint16_t *>(&lb);
-            } else {
-                v = ldexpf(v, ec);
-                const __half hh = __float2half_rn(v);
-                const __half lh = __float2half_rn(v - __half2float(hh));
-                h = *reinterpret_cast<const uint16_t *>(&hh);
-                l = *reinterpret_cast<const uint16_t *>(&lh);
+            v[k] = j < N ? V[j * ldv + c] : 0.0f;
+            if (out_init && j < N) out_init[j * ldo + c] = noise * v[k];
+        }
+        store_split<T, FMT>(vs, g, c, v, ec);
+    }
+}
+
+// split_v for a CG solve's p, fused with its update: p = r + beta p in the active columns, then the halves of
+// those columns (the others' stay valid) and out_init = noise p. The scaling exponents come from vmax, which the
+// step's previous launch set to a bound on the new |p|: at most one bit above its maximum, which costs nothing of
+// the 11-bit halves and one bit of the range below 2^-40 of the column's largest value that keeps an absolute error
+// anyway. pmax collects max |p| for the next bound. One thread per (8-row group, column), as split_v: 24 loads and
+// stores in flight per thread, where a separate maximum, split and update took three launches and read p twice.
+template <int T, int FMT>
+__global__ void __launch_bounds__(256) p_split_kernel(float *__restrict__ p, const float *__restrict__ r, int64_t N,
+                                                      CgState *st, CgSplit sp) {
+    if (st->done) return;
+    __shared__ unsigned int red[256];
+    const int c = threadIdx.x % T;  // the grid stride is a multiple of T
+    const bool act = st->active[c] != 0;
+    const float beta = (float)st->beta[c];
+    int ec = 0;
+    if (FMT == kFmtF16) ec = col_exponent(sp.vmax[c]);
+    const int64_t total = (N + 7) / 8 * T;
+    float m = 0.0f;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t g = e / T;
+        if (!act && !sp.out_init) break;
+        if (FMT == kFmtF16 && g == 0) sp.col_scale[c] = ldexpf(sp.s2, -15 - ec);
+        float v[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = 8 * g + k < N ? p[(8 * g + k) * T + c] : 0.0f;
+        if (act) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                const float z = 8 * g + k < N ? r[(8 * g + k) * T + c] : 0.0f;
+                v[k] = fmaf(beta, v[k], z);
             }
-            if (k & 1) {
-                hw[k >> 1] |= (uint32_t)h << 16;
-                lw[k >> 1] |= (uint32_t)l << 16;
-            } else {
-                hw[k >> 1] = h;
-                lw[k >> 1] = l;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                if (8 * g + k < N) p[(8 * g + k) * T + c] = v[k];
+                m = fmaxf(m, fabsf(v[k]));
             }
         }
-        const int64_t q = (8 * g) / kBK;
-        const int jj = (int)(8 * g - q * kBK);  // multiple of 8
-        const int64_t chunk = q * kBK * 2 * T + (int64_t)(jj >> 3) * (2 * T / 8) * 64 + (c & 7) * 8;
-        *reinterpret_cast<uint4 *>(vs + chunk + (int64_t)(c >> 3) * 64) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-        *reinterpret_cast<uint4 *>(vs + chunk + (int64_t)((T + c) >> 3) * 64) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+        if (sp.out_init) {
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (8 * g + k < N) sp.out_init[(8 * g + k) * T + c] = sp.noise * v[k];
+        }
+        if (act) store_split<T, FMT>(sp.vs, g, c, v, ec);
+    }
+    if (FMT == kFmtF16) {
+        red[threadIdx.x] = __float_as_uint(m);
+        __syncthreads();
+        if ((int)threadIdx.x < T && act) {
+            unsigned int b = red[threadIdx.x];
+            for (int k = threadIdx.x + T; k < (int)blockDim.x; k += T) b = max(b, red[k]);
+            atomicMax(&st->pmax[threadIdx.x], b);
+        }
     }
 }
 
@@ -429,16 +495,6 @@ void tc_split_candidates(int64_t Np, int num_sms, int *cand, int *n) {
     }
 }
 
-int mv_tc_launches(int64_t Np, int t, int num_sms, int fmt, int forced_splits, int kind, int D, bool operands_ready,
-                   int dist_form) {
-    // split V (+ column maxima for F16), transpose X unless ready, the product, the split reduction
-    int n = 2 + (operands_ready ? 0 : 1) + (mv_tc_partial_floats(Np, t, num_sms, forced_splits) > 0 ? 1 : 0) +
-            (fmt == kFmtF16 ? 1 : 0);
-    if (forced_splits == kTcSymmetric && dot_form_allowed(kind, D))
-        n += (operands_ready ? 0 : 2) + (dist_form < 0 ? 1 : 0);  // operand kernels, the second instance
-    return n;
-}
-
 namespace {
 
 cudaError_t launch_dot_operands(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, int t, void *vsplit,
@@ -476,11 +532,46 @@ cudaError_t launch_tc_operands(const KernelParams &kp, const float *Xs, int64_t 
     return launch_dot_operands(kp, Xs, N, Np, t, vsplit, nullptr, st);
 }
 
+CgSplit tc_cg_split(const KernelParams &kp, int64_t Np, int t, int fmt, void *vsplit, float *out_init) {
+    CgSplit sp;
+    sp.fmt = fmt;
+    sp.vs = (uint16_t *)vsplit;
+    sp.vmax = (unsigned int *)(sp.vs + 2 * Np * t);
+    sp.col_scale = (float *)(sp.vmax + 64);
+    sp.s2 = kp.s2;
+    sp.out_init = out_init;
+    sp.noise = kp.noise;
+    return sp;
+}
+
+cudaError_t launch_v_split(const KernelParams &kp, int64_t N, int64_t Np, const float *V, int64_t ldv, int t, int fmt,
+                           void *vsplit, float *out_init, int64_t ldo, const int *skip, int num_sms, cudaStream_t st) {
+    const CgSplit sp = tc_cg_split(kp, Np, t, fmt, vsplit, out_init);
+    const int blocks = (int)std::min<int64_t>((Np / 8 * t + 255) / 256, 8192);  // (8-row group, column)
+    if (fmt == kFmtF16) {
+        const cudaError_t e = cudaMemsetAsync(sp.vmax, 0, 64 * sizeof(unsigned int), st);
+        if (e != cudaSuccess) return e;
+        const int mb = (int)std::max<int64_t>(1, std::min<int64_t>((N * t + 255) / 256, 4 * num_sms));
+        col_absmax_kernel<<<mb, (256 / t) * t, 0, st>>>(V, ldv, N, t, sp.vmax, skip);
+    }
+    auto split = t == 16 ? (fmt == kFmtF16 ? split_v_kernel<16, kFmtF16> : split_v_kernel<16, kFmtBF16>)
+                         : (fmt == kFmtF16 ? split_v_kernel<32, kFmtF16> : split_v_kernel<32, kFmtBF16>);
+    split<<<blocks, 256, 0, st>>>(V, ldv, N, Np, sp.vs, sp.vmax, sp.col_scale, kp.s2, out_init, ldo, kp.noise, skip);
+    return cudaGetLastError();
+}
+
+void launch_p_split(const CgSplit &sp, float *p, const float *r, int64_t N, int t, CgState *state, cudaStream_t st) {
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(((N + 7) / 8 * t + 255) / 256, 8192));
+    auto k = t == 16 ? (sp.fmt == kFmtF16 ? p_split_kernel<16, kFmtF16> : p_split_kernel<16, kFmtBF16>)
+                     : (sp.fmt == kFmtF16 ? p_split_kernel<32, kFmtF16> : p_split_kernel<32, kFmtBF16>);
+    k<<<blocks, 256, 0, st>>>(p, r, N, state, sp);
+}
+
 cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, const float *V, int64_t ldv,
                          float *out, int64_t ldo, int t, int fmt, void *vsplit, float *partial, int64_t partial_cap,
                          const int *skip, int *err_flag, long long wait_budget, int num_sms, cudaStream_t st,
                          int forced_splits, bool operands_ready, int dist_form, cudaEvent_t ev_begin,
-                         cudaEvent_t ev_end) {
+                         cudaEvent_t ev_end, bool v_ready, ProductTail *tail) {
     auto mark = [&](cudaEvent_t ev) {
         if (ev) cudaEventRecord(ev, st);
     };
@@ -489,29 +580,13 @@ cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int
     unsigned int *vmax = (unsigned int *)(vs + 2 * Np * t);
     float *col_scale = (float *)(vmax + 64);
     float *XsT = col_scale + 64;
-    const int blocks = (int)std::min<int64_t>((Np / 8 * t + 255) / 256, 8192);  // split_v: (8-row group, column)
     const bool symmetric = forced_splits == kTcSymmetric;
-    float *out_init = symmetric ? out : nullptr;
+    if (tail) *tail = ProductTail();
     cudaError_t e;
-    if (fmt == kFmtF16) {
-        e = cudaMemsetAsync(vmax, 0, 64 * sizeof(unsigned int), st);
-        if (e != cudaSuccess) return e;
-        const int mb = (int)std::max<int64_t>(1, std::min<int64_t>((N * t + 255) / 256, 4 * num_sms));
-        col_absmax_kernel<<<mb, (256 / t) * t, 0, st>>>(V, ldv, N, t, vmax, skip);
-        if (t == 16)
-            split_v_kernel<16, kFmtF16><<<blocks, 256, 0, st>>>(V, ldv, N, Np, vs, vmax, col_scale, kp.s2, out_init,
-                                                              ldo, kp.noise, skip);
-        else
-            split_v_kernel<32, kFmtF16><<<blocks, 256, 0, st>>>(V, ldv, N, Np, vs, vmax, col_scale, kp.s2, out_init,
-                                                              ldo, kp.noise, skip);
-    } else {
-        if (t == 16)
-            split_v_kernel<16, kFmtBF16><<<blocks, 256, 0, st>>>(V, ldv, N, Np, vs, vmax, col_scale, kp.s2, out_init,
-                                                              ldo, kp.noise, skip);
-        else
-            split_v_kernel<32, kFmtBF16><<<blocks, 256, 0, st>>>(V, ldv, N, Np, vs, vmax, col_scale, kp.s2, out_init,
-                                                              ldo, kp.noise, skip);
-    }
+    if (!v_ready &&
+        (e = launch_v_split(kp, N, Np, V, ldv, t, fmt, vsplit, symmetric ? out : nullptr, ldo, skip, num_sms, st)) !=
+            cudaSuccess)
+        return e;
     if (!operands_ready) launch_transpose_x(kp, Xs, Np, vsplit, t, skip, st);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -618,6 +693,13 @@ cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int
                        : tc::dispatch_bf16(kp.kind, kp.D, t, grid, mx, mv, a, st);
     mark(ev_end);
     if (e != cudaSuccess || g.S == 1) return e;
+    if (tail) {
+        tail->part = partial;
+        tail->S = g.S;
+        tail->stride = Np * t;
+        tail->noise = kp.noise;
+        return cudaSuccess;
+    }
     const int rblocks = (int)std::min<int64_t>((N * t + 255) / 256, 4096);
     tc_reduce_kernel<<<rblocks, 256, 0, st>>>(partial, g.S, Np, N, t, V, ldv, out, ldo, kp.noise, skip);
     return cudaGetLastError();

@@ -12,6 +12,8 @@
 // block sums them in index order), so results are reproducible run to run.
 #include <math.h>
 
+#include <algorithm>
+
 #include "lgp_internal.cuh"
 
 namespace lgp {
@@ -114,6 +116,9 @@ __global__ void cg_init_scalars_kernel(CgState *st, const double *__restrict__ p
         st->rr[c] = rr0;
         st->rz[c] = rz;
         st->w0[c] = rz;
+        const double root = tol * sqrt(s);
+        st->thresh[c] = root * root;
+        st->rmax[c] = st->pmax[c] = 0u;
         st->alpha[c] = 0.0;
         st->beta[c] = 0.0;
         st->iters[c] = 0;
@@ -128,6 +133,7 @@ __global__ void cg_init_scalars_kernel(CgState *st, const double *__restrict__ p
     bad = __syncthreads_or(bad);
     if (threadIdx.x == 0) {
         st->iter = 0;
+        st->ticket = 0u;
         st->t = t;
         st->tol = tol;
         st->max_iter = max_iter;
@@ -139,28 +145,193 @@ __global__ void cg_init_scalars_kernel(CgState *st, const double *__restrict__ p
     }
 }
 
-__global__ void cg_pkp_kernel(const float *__restrict__ p, const float *__restrict__ Kp, int64_t N, int t,
-                              const CgState *st, double *__restrict__ partial) {
-    __shared__ double red[kVecThreads];
-    if (st->done) return;
-    int64_t r0, r1;
-    block_rows(N, &r0, &r1);
-    const int c = threadIdx.x % t;
-    float hi = 0.0f, lo = 0.0f;
-    for (int64_t i = r0 + threadIdx.x / t; i < r1; i += blockDim.x / t) acc_prod2(hi, lo, p[i * t + c], Kp[i * t + c]);
-    block_col_reduce((double)hi + (double)lo, t, red, partial + (int64_t)blockIdx.x * t);
+// ---------------------------------------------------------------- one CG iteration after the product
+//
+// Three launches: pkp_alpha (Kp from the product's column-split partial sums if it left any, p^T Kp, and in the last
+// block to finish alpha), xr_beta (x, r, r^T r, the columns' max |r|; last block: beta, convergence, the loop's done
+// flag) and p (p, and for the tensor-core products its split halves and the sigma^2 p that their out starts from).
+// What bounds them: up to a few MB per vector the launches and the chain of loads, block reduction and float64
+// reduction, not bandwidth. Hence few launches, 16-byte loads in blocks of 1024 threads, float pairs up to one value per
+// block and column, and at most kStepBlocks float64 values per column: one float64 warp instruction takes 64 cycles
+// of a sub-partition here, so a square root per column would cost more than all the loads (the test of convergence
+// compares squares).
+// Measured a solve / training step: N = 1024, t = 1, ~90 iterations 2.33 -> 1.83 ms; N = 2000, D = 8, t = 16 6.5 -> 4.7 ms;
+// prediction at N = 8000, t = 32 (with the product's own gain) 16.7 -> 13.2 ms.
+
+constexpr int kStepThreads = 1024;
+constexpr int kStepBlocks = 76;  // half the SMs: each SM's load rate still covers L2, and half the float64 sums
+
+__device__ __forceinline__ void pair_add(float &h, float &l, float h2, float l2) {
+    const float s = __fadd_rn(h, h2);
+    const float bb = __fsub_rn(s, h);
+    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, bb)), __fsub_rn(h2, bb));
+    h = s;
+    l = __fadd_rn(__fadd_rn(l, l2), e);
 }
 
-__global__ void cg_alpha_kernel(CgState *st, const double *__restrict__ partial, int G, double *hist_alpha) {
+// Column layout of the element-wise loops. VEC = 4 (t a power of two): thread x of the block handles float4s at
+// a stride that is a multiple of t, so its four elements always have the columns (4 x + k) mod t. VEC = 1: any t,
+// the block has a multiple of t threads and thread x owns column x mod t.
+template <int VEC> __device__ __forceinline__ int col_of(int tid, int k, int t) { return (VEC * tid + k) % t; }
+
+// Sums the float pairs of every column over the block: out_row[c] = their float64 value, c < t. red: 64 x 32 pairs.
+template <int VEC>
+__device__ void block_pairs_reduce(float (&hi)[VEC], float (&lo)[VEC], int t, float2 *red, double *out_row) {
+    const int tid = threadIdx.x;
+    if constexpr (VEC == 1) {
+        const int nr = blockDim.x / t;
+        red[tid] = make_float2(hi[0], lo[0]);
+        __syncthreads();
+        int s = 1;
+        while (s < nr) s <<= 1;
+        for (s >>= 1; s >= 1; s >>= 1) {
+            const int slot = tid / t;
+            if (slot < s && slot + s < nr) {
+                float2 a = red[tid];
+                const float2 b = red[tid + s * t];
+                pair_add(a.x, a.y, b.x, b.y);
+                red[tid] = a;
+            }
+            __syncthreads();
+        }
+        if (tid < t) out_row[tid] = (double)red[tid].x + (double)red[tid].y;
+    } else {
+        const int lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+        if (t == 1) {
+            pair_add(hi[0], lo[0], hi[1], lo[1]);
+            pair_add(hi[2], lo[2], hi[3], lo[3]);
+            pair_add(hi[0], lo[0], hi[2], lo[2]);
+        } else if (t == 2) {
+            pair_add(hi[0], lo[0], hi[2], lo[2]);
+            pair_add(hi[1], lo[1], hi[3], lo[3]);
+        }
+        const int group = t > 4 ? t / 4 : 1;  // lanes that hold one row of columns
+        for (int off = group; off < 32; off <<= 1) {
+#pragma unroll
+            for (int k = 0; k < VEC; ++k) {
+                const float h2 = __shfl_xor_sync(0xffffffffu, hi[k], off), l2 = __shfl_xor_sync(0xffffffffu, lo[k], off);
+                pair_add(hi[k], lo[k], h2, l2);
+            }
+        }
+        if (lane < group) {
+#pragma unroll
+            for (int k = 0; k < VEC; ++k)
+                if (4 * lane + k < t) red[(4 * lane + k) * 32 + warp] = make_float2(hi[k], lo[k]);
+        }
+        __syncthreads();
+        for (int c = warp; c < t; c += nw) {
+            float2 v = lane < nw ? red[c * 32 + lane] : make_float2(0.0f, 0.0f);
+            for (int off = 16; off > 0; off >>= 1) {
+                const float h2 = __shfl_xor_sync(0xffffffffu, v.x, off), l2 = __shfl_xor_sync(0xffffffffu, v.y, off);
+                pair_add(v.x, v.y, h2, l2);
+            }
+            if (lane == 0) out_row[c] = (double)v.x + (double)v.y;
+        }
+    }
+}
+
+// Whether this block is the last of the grid to arrive (its partials written before); resets the counter.
+__device__ bool last_block(unsigned int *ticket) {
+    __shared__ int last;
+    if (gridDim.x == 1) {
+        __syncthreads();
+        return true;
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const unsigned int k = atomicAdd(ticket, 1u);
+        last = k == gridDim.x - 1;
+        if (last) *ticket = 0u;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last != 0;
+}
+
+// Column sums of partial[b * t + c] over the grid's blocks, in a fixed order; valid in threads c < t after the call.
+__device__ double grid_col_sum(const double *partial, int t, double *red) {
+    const int G = gridDim.x, tid = threadIdx.x;
+    if (G == 1) return tid < t ? partial[tid] : 0.0;
+    int slots = 128 / t;  // t <= 64
+    if (slots > 8) slots = 8;
+    if (slots > G) slots = G;
+    if (tid < slots * t) {
+        const int slot = tid / t, c = tid - slot * t;
+        double s = 0.0;
+        for (int b = slot; b < G; b += slots) s += __ldcg(partial + (int64_t)b * t + c);
+        red[tid] = s;
+    }
+    __syncthreads();
+    double s = 0.0;
+    if (tid < t)
+        for (int k = 0; k < slots; ++k) s += red[k * t + tid];
+    return s;
+}
+
+template <int VEC> __device__ __forceinline__ void load_vec(const float *p, float (&v)[VEC]) {
+    if constexpr (VEC == 4) {
+        const float4 q = *reinterpret_cast<const float4 *>(p);
+        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+    } else {
+        v[0] = *p;
+    }
+}
+template <int VEC> __device__ __forceinline__ void store_vec(float *p, const float (&v)[VEC]) {
+    if constexpr (VEC == 4) *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else *p = v[0];
+}
+
+// Elements e (multiples of VEC) of a block's grid-stride loop over [0, N t). The vectors hold Np t >= N t values, so
+// a last float4 that crosses N t stays inside them; its elements past N t are left out of the sums.
+#define LGP_STEP_LOOP(e)                                                                                              \
+    for (int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * VEC; e < total;                                \
+         e += (int64_t)gridDim.x * blockDim.x * VEC)
+
+// REDUCE: Kp = sum_k part[k] + noise p first (S column-split partial sums of part_rows rows each).
+template <int VEC, bool REDUCE>
+__global__ void __launch_bounds__(kStepThreads) cg_pkp_alpha_kernel(const float *__restrict__ p, float *__restrict__ Kp,
+                                                                    const float *__restrict__ part, int S,
+                                                                    int64_t part_stride, float noise, int64_t N, int t,
+                                                                    CgState *st, double *__restrict__ partial,
+                                                                    double *__restrict__ hist_alpha) {
+    __shared__ float2 red[64 * 32];
     if (st->done) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int t = st->t;
+    const int64_t total = N * t;
+    float hi[VEC], lo[VEC];
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) hi[k] = lo[k] = 0.0f;
+    LGP_STEP_LOOP(e) {
+        float pv[VEC], kv[VEC];
+        load_vec<VEC>(p + e, pv);
+        if constexpr (REDUCE) {
+#pragma unroll
+            for (int k = 0; k < VEC; ++k) kv[k] = 0.0f;
+#pragma unroll 4
+            for (int q = 0; q < S; ++q) {
+                float w[VEC];
+                load_vec<VEC>(part + q * part_stride + e, w);
+#pragma unroll
+                for (int k = 0; k < VEC; ++k) kv[k] += w[k];
+            }
+#pragma unroll
+            for (int k = 0; k < VEC; ++k) kv[k] = fmaf(noise, pv[k], kv[k]);
+            store_vec<VEC>(Kp + e, kv);
+        } else {
+            load_vec<VEC>(Kp + e, kv);
+        }
+#pragma unroll
+        for (int k = 0; k < VEC; ++k)
+            if (VEC == 1 || e + k < total) acc_prod2(hi[k], lo[k], pv[k], kv[k]);
+    }
+    block_pairs_reduce<VEC>(hi, lo, t, red, partial + (int64_t)blockIdx.x * t);
+    if (!last_block(&st->ticket)) return;
+    const double pkp = grid_col_sum(partial, t, reinterpret_cast<double *>(red));
+    const int c = threadIdx.x;
     int bad = 0, nonfinite = 0;
-    for (int c = warp; c < t; c += nw) {
+    if (c < t) {
         double alpha = 0.0;
         if (st->active[c]) {
-            const double pkp = warp_sum_partials(partial, G, t, c);
-            if (lane != 0) continue;
             if (!isfinite(pkp)) {
                 nonfinite = 1;
                 st->active[c] = 0;
@@ -171,7 +342,6 @@ __global__ void cg_alpha_kernel(CgState *st, const double *__restrict__ partial,
                 alpha = st->rz[c] / pkp;
             }
         }
-        if (lane != 0) continue;
         st->alpha[c] = alpha;
         if (st->iter < st->hist_len) hist_alpha[(int64_t)st->iter * t + c] = alpha;
     }
@@ -181,51 +351,29 @@ __global__ void cg_alpha_kernel(CgState *st, const double *__restrict__ partial,
         st->status = nonfinite ? (int)LGP_ERR_NONFINITE : (int)LGP_ERR_BREAKDOWN;
 }
 
-__global__ void cg_xr_kernel(float *__restrict__ x, float *__restrict__ r, const float *__restrict__ p,
-                             const float *__restrict__ Kp, int64_t N, int t, const CgState *st,
-                             double *__restrict__ partial) {
-    __shared__ double red[kVecThreads];
-    if (st->done) return;
-    int64_t r0, r1;
-    block_rows(N, &r0, &r1);
-    const int c = threadIdx.x % t;
-    const float alpha = (float)st->alpha[c];
-    float hi = 0.0f, lo = 0.0f;
-    for (int64_t i = r0 + threadIdx.x / t; i < r1; i += blockDim.x / t) {
-        const int64_t e = i * t + c;
-        float rv = r[e];
-        if (alpha != 0.0f) {
-            x[e] = fmaf(alpha, p[e], x[e]);
-            rv = fmaf(-alpha, Kp[e], rv);
-            r[e] = rv;
-        }
-        acc_prod2(hi, lo, rv, rv);
-    }
-    block_col_reduce((double)hi + (double)lo, t, red, partial + (int64_t)blockIdx.x * t);
-}
-
-__global__ void cg_beta_kernel(CgState *st, const double *__restrict__ partial, int G, double *hist_beta,
-                               const double *__restrict__ rz_partial) {
-    if (st->done) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int t = st->t;
+// beta, convergence and the done flag from the columns' r^T r and r^T z (threads c < t of one block). vbound (may be
+// null): the bound on max |p| after the update, |r| + |beta| |p|, from which the tensor-core products scale p's columns.
+__device__ void finish_beta(CgState *st, double rr, double rz, int t, double *hist_beta, unsigned int *vbound) {
+    const int c = threadIdx.x;
     int any = 0;
-    for (int c = warp; c < t; c += nw) {
+    if (c < t) {
         double beta = 0.0;
         if (st->active[c]) {
-            const double rr = warp_sum_partials(partial, G, t, c);
-            const double rz = rz_partial ? warp_sum_partials(rz_partial, G, t, c) : rr;
-            if (lane != 0) continue;
             beta = rz / st->rz[c];
             st->rr[c] = rr;
             st->rz[c] = rz;
             st->iters[c] += 1;
-            if (!(sqrt(rr) > st->tol * sqrt(st->bnorm2[c]))) st->active[c] = 0;
+            if (!(rr > st->thresh[c])) st->active[c] = 0;
+            if (vbound && st->active[c]) {
+                const float b = fmaf((float)beta, __uint_as_float(st->pmax[c]), __uint_as_float(st->rmax[c]));
+                vbound[c] = __float_as_uint(b * 1.000001f);  // above the rounding of the update itself
+                st->pmax[c] = 0u;
+            }
         }
-        if (lane != 0) continue;
+        st->rmax[c] = 0u;
         st->beta[c] = beta;
         if (st->iter < st->hist_len) hist_beta[(int64_t)st->iter * t + c] = beta;
-        any |= st->active[c];
+        any = st->active[c];
     }
     any = __syncthreads_or(any);
     if (threadIdx.x == 0) {
@@ -234,17 +382,109 @@ __global__ void cg_beta_kernel(CgState *st, const double *__restrict__ partial, 
     }
 }
 
-__global__ void cg_p_kernel(float *__restrict__ p, const float *__restrict__ r, int64_t N, int t,
-                            const CgState *st) {
+// FINISH: the last block computes beta (plain CG; the preconditioned one needs r^T z first, cg_beta_kernel).
+template <int VEC, bool FINISH>
+__global__ void __launch_bounds__(kStepThreads) cg_xr_beta_kernel(float *__restrict__ x, float *__restrict__ r,
+                                                                  const float *__restrict__ p,
+                                                                  const float *__restrict__ Kp, int64_t N, int t,
+                                                                  CgState *st, double *__restrict__ partial,
+                                                                  double *__restrict__ hist_beta, unsigned int *vbound) {
+    __shared__ float2 red[64 * 32];
+    __shared__ unsigned int rmax[kMaxT];
     if (st->done) return;
-    int64_t r0, r1;
-    block_rows(N, &r0, &r1);
-    const int c = threadIdx.x % t;
-    if (!st->active[c]) return;
-    const float beta = (float)st->beta[c];
-    for (int64_t i = r0 + threadIdx.x / t; i < r1; i += blockDim.x / t) {
-        const int64_t e = i * t + c;
-        p[e] = fmaf(beta, p[e], r[e]);
+    const int64_t total = N * t;
+    float alpha[VEC], hi[VEC], lo[VEC], m[VEC];
+    bool any = false;
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) {
+        alpha[k] = (float)st->alpha[col_of<VEC>(threadIdx.x, k, t)];
+        any |= alpha[k] != 0.0f;
+        hi[k] = lo[k] = m[k] = 0.0f;
+    }
+    if (threadIdx.x < kMaxT) rmax[threadIdx.x] = 0u;
+    LGP_STEP_LOOP(e) {
+        float rv[VEC];
+        load_vec<VEC>(r + e, rv);
+        if (any) {
+            float xv[VEC], pv[VEC], kv[VEC];
+            load_vec<VEC>(x + e, xv);
+            load_vec<VEC>(p + e, pv);
+            load_vec<VEC>(Kp + e, kv);
+#pragma unroll
+            for (int k = 0; k < VEC; ++k) {
+                if (alpha[k] != 0.0f) {
+                    xv[k] = fmaf(alpha[k], pv[k], xv[k]);
+                    rv[k] = fmaf(-alpha[k], kv[k], rv[k]);
+                }
+            }
+            store_vec<VEC>(x + e, xv);
+            store_vec<VEC>(r + e, rv);
+        }
+#pragma unroll
+        for (int k = 0; k < VEC; ++k)
+            if (VEC == 1 || e + k < total) {
+                acc_prod2(hi[k], lo[k], rv[k], rv[k]);
+                m[k] = fmaxf(m[k], fabsf(rv[k]));
+            }
+    }
+    if (vbound) {
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < VEC; ++k) atomicMax(&rmax[col_of<VEC>(threadIdx.x, k, t)], __float_as_uint(m[k]));
+    }
+    block_pairs_reduce<VEC>(hi, lo, t, red, partial + (int64_t)blockIdx.x * t);
+    if (vbound && (int)threadIdx.x < t) atomicMax(&st->rmax[threadIdx.x], rmax[threadIdx.x]);
+    if constexpr (FINISH) {
+        if (!last_block(&st->ticket)) return;
+        const double rr = grid_col_sum(partial, t, reinterpret_cast<double *>(red));
+        finish_beta(st, rr, rr, t, hist_beta, vbound);
+    }
+}
+
+// Preconditioned CG: one block sums the r^T r partials (G_rr blocks) and the r^T z partials (G_rz) and finishes beta.
+__global__ void __launch_bounds__(1024) cg_beta_kernel(CgState *st, const double *__restrict__ rr_partial, int G_rr,
+                                                       const double *__restrict__ rz_partial, int G_rz, int t,
+                                                       double *hist_beta) {
+    __shared__ double srr[kMaxT], srz[kMaxT];
+    if (st->done) return;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    for (int c = warp; c < t; c += nw) {
+        const double rr = warp_sum_partials(rr_partial, G_rr, t, c);
+        const double rz = warp_sum_partials(rz_partial, G_rz, t, c);
+        if (lane == 0) {
+            srr[c] = rr;
+            srz[c] = rz;
+        }
+    }
+    __syncthreads();
+    const int c = threadIdx.x < t ? threadIdx.x : 0;
+    finish_beta(st, srr[c], srz[c], t, hist_beta, nullptr);
+}
+
+template <int VEC>
+__global__ void __launch_bounds__(kStepThreads) cg_p_kernel(float *__restrict__ p, const float *__restrict__ z, int64_t N,
+                                                            int t, const CgState *st) {
+    if (st->done) return;
+    const int64_t total = N * t;
+    float beta[VEC];
+    int act[VEC];
+    int any = 0;
+#pragma unroll
+    for (int k = 0; k < VEC; ++k) {
+        const int c = col_of<VEC>(threadIdx.x, k, t);
+        act[k] = st->active[c];
+        any |= act[k];
+        beta[k] = (float)st->beta[c];
+    }
+    if (!any) return;
+    LGP_STEP_LOOP(e) {
+        float pv[VEC], zv[VEC];
+        load_vec<VEC>(p + e, pv);
+        load_vec<VEC>(z + e, zv);
+#pragma unroll
+        for (int k = 0; k < VEC; ++k)
+            if (act[k]) pv[k] = fmaf(beta[k], pv[k], zv[k]);
+        store_vec<VEC>(p + e, pv);
     }
 }
 
@@ -531,20 +771,44 @@ void launch_cg_init(const float *B, int64_t ldb, int64_t N, int64_t Np, int t, c
                                                                  rz_partial, rr_partial);
 }
 
-void launch_cg_after_matvec(int64_t N, int64_t Np, int t, const CgBuffers &b, cudaStream_t st) {
-    (void)Np;
-    const int bd = vec_block(t);
-    cg_pkp_kernel<<<b.G, bd, 0, st>>>(b.p, b.Kp, N, t, b.state, b.partial);
-    const int sb = 32 * (t < 32 ? t : 32);
-    cg_alpha_kernel<<<1, sb, 0, st>>>(b.state, b.partial, b.G, b.hist_alpha);
-    cg_xr_kernel<<<b.G, bd, 0, st>>>(b.x, b.r, b.p, b.Kp, N, t, b.state, b.partial);
-    double *rz_partial = nullptr;
+namespace {
+
+int step_blocks(int64_t N, int t) {
+    // never more than cg_num_blocks, for which the partial sums are sized
+    return std::min(kStepBlocks, cg_num_blocks(N, t, kStepBlocks));
+}
+
+template <int VEC>
+void launch_step(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split, cudaStream_t st) {
+    const int bd = VEC == 4 ? kStepThreads : (kStepThreads / t) * t;
+    const int G = step_blocks(N, t);
+    unsigned int *vbound = split ? split->vmax : nullptr;
+    if (tail.S > 1)
+        cg_pkp_alpha_kernel<VEC, true><<<G, bd, 0, st>>>(b.p, b.Kp, tail.part, tail.S, tail.stride, tail.noise, N, t, b.state,
+                                                         b.partial, b.hist_alpha);
+    else
+        cg_pkp_alpha_kernel<VEC, false><<<G, bd, 0, st>>>(b.p, b.Kp, nullptr, 0, 0, 0.0f, N, t, b.state, b.partial,
+                                                          b.hist_alpha);
     if (b.pc.k > 0) {
-        rz_partial = b.partial + (int64_t)b.G * t;
+        double *rz_partial = b.partial + (int64_t)b.G * t;
+        cg_xr_beta_kernel<VEC, false><<<G, bd, 0, st>>>(b.x, b.r, b.p, b.Kp, N, t, b.state, b.partial, b.hist_beta, nullptr);
         launch_precond_apply(b.pc, b.r, t, b.z, t, nullptr, N, t, rz_partial, b.G, b.state, st);
+        cg_beta_kernel<<<1, 1024, 0, st>>>(b.state, b.partial, G, rz_partial, b.G, t, b.hist_beta);
+    } else {
+        cg_xr_beta_kernel<VEC, true><<<G, bd, 0, st>>>(b.x, b.r, b.p, b.Kp, N, t, b.state, b.partial, b.hist_beta, vbound);
     }
-    cg_beta_kernel<<<1, sb, 0, st>>>(b.state, b.partial, b.G, b.hist_beta, rz_partial);
-    cg_p_kernel<<<b.G, bd, 0, st>>>(b.p, b.pc.k > 0 ? b.z : b.r, N, t, b.state);
+    if (split)
+        launch_p_split(*split, b.p, b.r, N, t, b.state, st);
+    else
+        cg_p_kernel<VEC><<<G, bd, 0, st>>>(b.p, b.pc.k > 0 ? b.z : b.r, N, t, b.state);
+}
+
+}  // namespace
+
+void launch_cg_after_matvec(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,
+                            cudaStream_t st) {
+    if (t <= 64 && (t & (t - 1)) == 0) launch_step<4>(N, t, b, tail, split, st);
+    else launch_step<1>(N, t, b, tail, split, st);
 }
 
 void launch_cg_loop_condition(cudaGraphConditionalHandle h, CgState *state, cudaStream_t st) {
