@@ -473,7 +473,7 @@ lgp_status cg_buffers(lgp_ctx *ctx, int64_t N, int64_t Np, int t, int hist_len, 
     lgp_status s;
     if ((s = ensure(ctx, ctx->cg_vec, (size_t)5 * Np * t * sizeof(float))) != LGP_OK) return s;
     b->G = cg_num_blocks(N, t, ctx->num_sms);
-    if ((s = ensure(ctx, ctx->cg_partial, (size_t)b->G * 3 * t * sizeof(double))) != LGP_OK) return s;
+    if ((s = ensure(ctx, ctx->cg_partial, (size_t)cg_partial_doubles(b->G, t) * sizeof(double))) != LGP_OK) return s;
     if ((s = ensure(ctx, ctx->cg_state, sizeof(CgState))) != LGP_OK) return s;
     if ((s = ensure(ctx, ctx->cg_hist, (size_t)2 * std::max(hist_len, 1) * t * sizeof(double))) != LGP_OK) return s;
     float *v = (float *)ctx->cg_vec.p;
@@ -778,7 +778,7 @@ lgp_status run_cg_columns(lgp_ctx *ctx, const Prepared &pp, const float *B, int 
     const int Gt = cg_num_blocks(pp.N, t, ctx->num_sms);
     lgp_status s;
     // every t-column buffer exists before the first solve, so nothing moves between the column runs
-    if ((s = ensure(ctx, ctx->cg_partial, (size_t)Gt * 3 * t * sizeof(double))) != LGP_OK ||
+    if ((s = ensure(ctx, ctx->cg_partial, (size_t)cg_partial_doubles(Gt, t) * sizeof(double))) != LGP_OK ||
         (s = ensure(ctx, ctx->sr_x, (size_t)pp.Np * t * sizeof(float))) != LGP_OK ||
         (s = ensure(ctx, ctx->sr_state, sizeof(CgState))) != LGP_OK ||
         (s = ensure(ctx, ctx->sr_hist, (size_t)2 * std::max(hist_len, 1) * t * sizeof(double))) != LGP_OK)

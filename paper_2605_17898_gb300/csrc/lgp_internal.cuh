@@ -188,10 +188,10 @@ void launch_var_from_probes(const float *Z, int64_t ldz, const float *Q, int64_t
                             float *var, cudaStream_t st);
 
 // What a product left for its caller to finish when asked to (the CG step, which reads the same rows anyway):
-// S > 1 column-split partial sums, out = sum_k part[k * stride + e] + noise V. S = 1: out is complete.
+// S partial sums, out = sum_k part[k * stride + e] + noise V. part = nullptr: out is complete.
 struct ProductTail {
     const float *part = nullptr;
-    int S = 1;
+    int S = 0;
     int64_t stride = 0;
     float noise = 0.0f;
 };
@@ -321,7 +321,7 @@ void launch_precond_probes(const double *L64, int64_t Np, int k, const float *E,
 struct CgBuffers {
     float *x, *r, *p, *Kp;   // [Np, t]
     float *z;                // [Np, t] P^{-1} r (preconditioned solves only)
-    double *partial;         // [G, 3t] block partial dots
+    double *partial;         // block partial dots, cg_partial_doubles(G, t)
     int G;                   // blocks of the vector kernels
     CgState *state;
     double *hist_alpha;      // [hist_len, t]
@@ -344,6 +344,7 @@ void launch_cg_loop_condition(cudaGraphConditionalHandle h, CgState *state, cuda
 // Host-driven loop (LGP_CG_GRAPH=0): counts one chunk in state->loop_chunks.
 void launch_cg_chunk_tally(CgState *state, cudaStream_t st);
 int cg_num_blocks(int64_t N, int t, int num_sms);
+int64_t cg_partial_doubles(int G, int t);
 
 // Column dot products sum_i A[i,c] B[i,c] and sum_i A[i,c]^2 (float64), c < t: out[2t].
 void launch_col_dots(const float *A, const float *B, int64_t N, int t, double *partial, int G, double *out,

@@ -2,6 +2,7 @@
 #include <algorithm>
 
 #include "mv_simt.cuh"
+#include "mv_sym.cuh"
 
 namespace lgp {
 
@@ -32,6 +33,39 @@ int64_t choose_split(int64_t N, int64_t row_blocks, int64_t col_groups, int num_
     return (N + *cols_per_split - 1) / *cols_per_split;
 }
 
+// Symmetric product (mv_sym.cuh): block edge E, blocks G and padded column count TT for a square product of N rows
+// and t columns, or E = 0 where the row-by-row kernel runs (t > 4; or N so large that the partial sums, G per row,
+// would take more than 256 MiB even with the largest blocks).
+struct SymGrid {
+    int E = 0, G = 0, TT = 0;
+};
+
+constexpr int64_t kSymMaxPartial = 256ll << 20;
+
+SymGrid sym_grid(int64_t N, int64_t Np, int t, int num_sms) {
+    SymGrid g;
+    if (t > 4) return g;
+    // The largest blocks that still give every SM enough tiles to even out the last ones (a tile's set-up and its
+    // sums are paid per tile, and each block is one more partial sum per row: N = 50000, D = 4, t = 1 with
+    // E = 256 535 us, 512 476); larger ones only to keep the partial sums in bounds.
+    auto tiles_per_sm = [&](int64_t E) {
+        const int64_t G = (N + E - 1) / E;
+        return G * (G + 1) / 2 / num_sms;
+    };
+    const int TT = t <= 2 ? t : 4;
+    int64_t E = 64;
+    if (tiles_per_sm(512) >= 16) E = 512;
+    else if (tiles_per_sm(256) >= 8) E = 256;
+    else if (tiles_per_sm(128) >= 5) E = 128;
+    auto bytes = [&](int64_t e) { return (N + e - 1) / e * Np * t * (int64_t)sizeof(float); };
+    if (E == 512 && bytes(E) > kSymMaxPartial) E = 1024;
+    if (bytes(E) > kSymMaxPartial) return g;
+    g.E = (int)E;
+    g.G = (int)((N + E - 1) / E);
+    g.TT = TT;
+    return g;
+}
+
 // Rows are the output's (N, padded Np); cross = 1 drops the noise term (V has other rows).
 __global__ void reduce_split_kernel(const float *__restrict__ partial, int S, int64_t Np, int64_t N, int t,
                                     const float *__restrict__ V, int64_t ldv, float *__restrict__ out, int64_t ldo,
@@ -44,6 +78,43 @@ __global__ void reduce_split_kernel(const float *__restrict__ partial, int S, in
         float s = 0.0f;
         for (int k = 0; k < S; ++k) s += partial[((int64_t)k * Np + i) * t + c];
         out[i * ldo + c] = cross ? s : fmaf(noise, V[i * ldv + c], s);
+    }
+}
+
+// The same for many splits (S >= 8): 8 lanes share 4 consecutive elements, lane q taking splits q, q + 8, ... as 16-byte
+// loads, so that the loads of one element's splits overlap (product at t = 1: N = 5000, 40 splits 22 -> 19 us; N = 50000, 98
+// splits 476 -> 472 us).
+__global__ void __launch_bounds__(256) reduce_many_kernel(const float *__restrict__ partial, int S, int64_t Np, int64_t N,
+                                                          int t, const float *__restrict__ V, int64_t ldv,
+                                                          float *__restrict__ out, int64_t ldo, float noise, int cross,
+                                                          const int *skip) {
+    if (skip && *skip) return;
+    const int lane = threadIdx.x & 31, q = lane >> 2;
+    const int64_t total = N * t;
+    const int64_t e = 4 * (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32 * 4 + (lane & 3));
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (e < total) {
+#pragma unroll 4
+        for (int k = q; k < S; k += 8) {
+            const float4 v = *reinterpret_cast<const float4 *>(partial + (int64_t)k * Np * t + e);
+            s.x += v.x;
+            s.y += v.y;
+            s.z += v.z;
+            s.w += v.w;
+        }
+    }
+#pragma unroll
+    for (int off = 4; off < 32; off <<= 1) {
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, off);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, off);
+        s.z += __shfl_xor_sync(0xffffffffu, s.z, off);
+        s.w += __shfl_xor_sync(0xffffffffu, s.w, off);
+    }
+    if (q < 4 && e + q < total) {
+        const float v = q == 0 ? s.x : q == 1 ? s.y : q == 2 ? s.z : s.w;
+        const int64_t i = (e + q) / t;
+        const int c = (int)(e + q - i * t);
+        out[i * ldo + c] = cross ? v : fmaf(noise, V[i * ldv + c], v);
     }
 }
 
@@ -73,6 +144,8 @@ inline int grid_for(int64_t n) {
 }  // namespace
 
 int64_t mv_simt_partial_floats(int64_t N, int64_t Np, int t, int num_sms) {
+    const SymGrid sg = sym_grid(N, Np, t, num_sms);
+    if (sg.E) return (int64_t)sg.G * Np * t;
     const SimtShape sh = simt_shape(t);
     const int64_t BM = (int64_t)kSimtThreads * sh.R;
     const int64_t rb = (N + BM - 1) / BM;
@@ -92,9 +165,52 @@ int64_t mv_simt_cross_partial_floats(int64_t Nr, int64_t Npr, int64_t N, int t, 
     return S > 1 ? S * Npr * t : 0;
 }
 
+// The sum of S partial results and the noise term, or, with m.tail, what the caller needs to take it over.
+static cudaError_t finish_splits(const MvLaunch &m, int S, int64_t Nr, int64_t Npr, int cross, cudaStream_t st) {
+    if (m.tail) {
+        m.tail->part = m.partial;
+        m.tail->S = S;
+        m.tail->stride = Npr * m.t;
+        m.tail->noise = m.kp->noise;
+        return cudaSuccess;
+    }
+    if (S >= 8)
+        reduce_many_kernel<<<(unsigned)((Nr * m.t + 127) / 128), 256, 0, st>>>(m.partial, S, Npr, Nr, m.t, m.V, m.ldv, m.out,
+                                                                               m.ldo, m.kp->noise, cross, m.skip);
+    else
+        reduce_split_kernel<<<grid_for(Nr * m.t), 256, 0, st>>>(m.partial, S, Npr, Nr, m.t, m.V, m.ldv, m.out, m.ldo,
+                                                                m.kp->noise, cross, m.skip);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st) {
     const bool cross = m.Xr != nullptr;
     const int64_t Nr = cross ? m.Nr : m.N, Npr = cross ? m.Npr : m.Np;
+    if (m.tail) *m.tail = ProductTail();
+    const SymGrid sg = cross ? SymGrid() : sym_grid(m.N, m.Np, m.t, m.num_sms);
+    if (sg.E && m.partial != nullptr && (int64_t)sg.G * m.Np * m.t <= m.partial_cap) {
+        SymArgs a;
+        a.Xs = m.Xs;
+        a.V = m.V;
+        a.part = m.partial;
+        a.skip = m.skip;
+        a.N = m.N;
+        a.Np = m.Np;
+        a.ldv = m.ldv;
+        a.E = sg.E;
+        a.G = sg.G;
+        a.t = m.t;
+        a.log2s2 = m.kp->log2_s2;
+        cudaError_t e;
+        switch (m.kp->kind) {
+            case LGP_RBF: e = mv_sym_dispatch_rbf(m.kp->D, sg.TT, a, st); break;
+            case LGP_MATERN52: e = mv_sym_dispatch_m52(m.kp->D, sg.TT, a, st); break;
+            case LGP_MATERN12: e = mv_sym_dispatch_m12(m.kp->D, sg.TT, a, st); break;
+            case LGP_MATERN32: e = mv_sym_dispatch_m32(m.kp->D, sg.TT, a, st); break;
+            default: e = cudaErrorInvalidValue;
+        }
+        return e != cudaSuccess ? e : finish_splits(m, sg.G, m.N, m.Np, 0, st);
+    }
     const SimtShape sh = simt_shape(m.t);
     const int64_t BM = (int64_t)kSimtThreads * sh.R;
     const int64_t rb = (Nr + BM - 1) / BM;
@@ -132,18 +248,8 @@ cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st) {
         case LGP_MATERN32: e = mv_simt_dispatch_m32(m.kp->D, sh.TT, sh.R, grid, a, st); break;
         default: e = cudaErrorInvalidValue;
     }
-    if (m.tail) *m.tail = ProductTail();
     if (e != cudaSuccess || S == 1) return e;
-    if (m.tail) {
-        m.tail->part = m.partial;
-        m.tail->S = (int)S;
-        m.tail->stride = Npr * m.t;
-        m.tail->noise = m.kp->noise;
-        return cudaSuccess;
-    }
-    reduce_split_kernel<<<grid_for(Nr * m.t), 256, 0, st>>>(m.partial, (int)S, Npr, Nr, m.t, m.V, m.ldv, m.out,
-                                                            m.ldo, m.kp->noise, a.cross, m.skip);
-    return cudaGetLastError();
+    return finish_splits(m, (int)S, Nr, Npr, a.cross, st);
 }
 
 int64_t mv_grad_partial_floats(int64_t N, int64_t Np, int t, int D, int num_sms) {

@@ -288,8 +288,9 @@ template <int VEC> __device__ __forceinline__ void store_vec(float *p, const flo
     for (int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * VEC; e < total;                                \
          e += (int64_t)gridDim.x * blockDim.x * VEC)
 
-// REDUCE: Kp = sum_k part[k] + noise p first (S column-split partial sums of part_rows rows each).
-template <int VEC, bool REDUCE>
+// LANES > 0: Kp = sum_k part[k] + noise p first (S partial sums, part_stride apart), LANES lanes of a warp sharing the
+// partial sums of each VEC elements (8 where there are many, so that their loads overlap).
+template <int VEC, int LANES>
 __global__ void __launch_bounds__(kStepThreads) cg_pkp_alpha_kernel(const float *__restrict__ p, float *__restrict__ Kp,
                                                                     const float *__restrict__ part, int S,
                                                                     int64_t part_stride, float noise, int64_t N, int t,
@@ -298,31 +299,65 @@ __global__ void __launch_bounds__(kStepThreads) cg_pkp_alpha_kernel(const float 
     __shared__ float2 red[64 * 32];
     if (st->done) return;
     const int64_t total = N * t;
+    // LANES = 8: element thread u of the block's blockDim / 8 is lanes with (lane & 3) = u mod 4 of warp u / 4
+    constexpr int L = LANES > 1 ? LANES : 1;
+    const int sub = L > 1 ? (threadIdx.x & 31) / (32 / L) : 0;
+    const int u = L > 1 ? (int)(threadIdx.x >> 5) * (32 / L) + (int)(threadIdx.x & (32 / L - 1)) : (int)threadIdx.x;
+    const int nu = blockDim.x / L;
     float hi[VEC], lo[VEC];
 #pragma unroll
     for (int k = 0; k < VEC; ++k) hi[k] = lo[k] = 0.0f;
-    LGP_STEP_LOOP(e) {
+    // (with L > 1 every lane of a warp runs the same rounds: the bound is its first element thread's)
+    for (int64_t e0 = ((int64_t)blockIdx.x * nu + (L > 1 ? u - (u & (32 / L - 1)) : u)) * VEC; e0 < total;
+         e0 += (int64_t)gridDim.x * nu * VEC) {
+        const int64_t e = e0 + (L > 1 ? (u & (32 / L - 1)) * VEC : 0);
+        const bool in = L == 1 || e < total;
         float pv[VEC], kv[VEC];
-        load_vec<VEC>(p + e, pv);
-        if constexpr (REDUCE) {
 #pragma unroll
-            for (int k = 0; k < VEC; ++k) kv[k] = 0.0f;
+        for (int k = 0; k < VEC; ++k) pv[k] = kv[k] = 0.0f;
+        if (in) load_vec<VEC>(p + e, pv);
+        if constexpr (LANES > 0) {
+            if (in) {
 #pragma unroll 4
-            for (int q = 0; q < S; ++q) {
-                float w[VEC];
-                load_vec<VEC>(part + q * part_stride + e, w);
+                for (int q = sub; q < S; q += L) {
+                    float w[VEC];
+                    load_vec<VEC>(part + q * part_stride + e, w);
 #pragma unroll
-                for (int k = 0; k < VEC; ++k) kv[k] += w[k];
+                    for (int k = 0; k < VEC; ++k) kv[k] += w[k];
+                }
+            }
+            if constexpr (L > 1) {
+#pragma unroll
+                for (int off = 32 / L; off < 32; off <<= 1)
+#pragma unroll
+                    for (int k = 0; k < VEC; ++k) kv[k] += __shfl_xor_sync(0xffffffffu, kv[k], off);
             }
 #pragma unroll
             for (int k = 0; k < VEC; ++k) kv[k] = fmaf(noise, pv[k], kv[k]);
-            store_vec<VEC>(Kp + e, kv);
+            if (in && sub == 0) store_vec<VEC>(Kp + e, kv);
         } else {
             load_vec<VEC>(Kp + e, kv);
         }
+        if (sub == 0) {
 #pragma unroll
-        for (int k = 0; k < VEC; ++k)
-            if (VEC == 1 || e + k < total) acc_prod2(hi[k], lo[k], pv[k], kv[k]);
+            for (int k = 0; k < VEC; ++k)
+                if (VEC == 1 || e + k < total) acc_prod2(hi[k], lo[k], pv[k], kv[k]);
+        }
+    }
+    if constexpr (L > 1) {
+        // element thread u's sums to thread u, whose columns they have
+        if (sub == 0) {
+#pragma unroll
+            for (int k = 0; k < VEC; ++k) red[u * VEC + k] = make_float2(hi[k], lo[k]);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < VEC; ++k) {
+            const float2 v = (int)threadIdx.x < nu ? red[threadIdx.x * VEC + k] : make_float2(0.0f, 0.0f);
+            hi[k] = v.x;
+            lo[k] = v.y;
+        }
+        __syncthreads();
     }
     block_pairs_reduce<VEC>(hi, lo, t, red, partial + (int64_t)blockIdx.x * t);
     if (!last_block(&st->ticket)) return;
@@ -749,6 +784,8 @@ int cg_num_blocks(int64_t N, int t, int num_sms) {
     return (int)g;
 }
 
+int64_t cg_partial_doubles(int G, int t) { return (int64_t)std::max(3 * G, kStepBlocks) * t; }
+
 void launch_cg_init(const float *B, int64_t ldb, int64_t N, int64_t Np, int t, const CgBuffers &b, double tol,
                     int max_iter, int hist_len, cudaStream_t st, const float *X0, int64_t ldx0) {
     (void)Np;
@@ -783,12 +820,18 @@ void launch_step(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, 
     const int bd = VEC == 4 ? kStepThreads : (kStepThreads / t) * t;
     const int G = step_blocks(N, t);
     unsigned int *vbound = split ? split->vmax : nullptr;
-    if (tail.S > 1)
-        cg_pkp_alpha_kernel<VEC, true><<<G, bd, 0, st>>>(b.p, b.Kp, tail.part, tail.S, tail.stride, tail.noise, N, t, b.state,
-                                                         b.partial, b.hist_alpha);
-    else
-        cg_pkp_alpha_kernel<VEC, false><<<G, bd, 0, st>>>(b.p, b.Kp, nullptr, 0, 0, 0.0f, N, t, b.state, b.partial,
-                                                          b.hist_alpha);
+    if (tail.part && tail.S >= 16 && VEC == 4) {
+        const int64_t per = kStepThreads / 8 * VEC;  // elements of a block's round
+        const int G8 = (int)std::min<int64_t>(kStepBlocks, (N * t + per - 1) / per);
+        cg_pkp_alpha_kernel<VEC, VEC == 4 ? 8 : 1><<<G8, bd, 0, st>>>(
+            b.p, b.Kp, tail.part, tail.S, tail.stride, tail.noise, N, t, b.state, b.partial, b.hist_alpha);
+    } else if (tail.part) {
+        cg_pkp_alpha_kernel<VEC, 1><<<G, bd, 0, st>>>(b.p, b.Kp, tail.part, tail.S, tail.stride, tail.noise, N, t, b.state,
+                                                      b.partial, b.hist_alpha);
+    } else {
+        cg_pkp_alpha_kernel<VEC, 0><<<G, bd, 0, st>>>(b.p, b.Kp, nullptr, 0, 0, 0.0f, N, t, b.state, b.partial,
+                                                      b.hist_alpha);
+    }
     if (b.pc.k > 0) {
         double *rz_partial = b.partial + (int64_t)b.G * t;
         cg_xr_beta_kernel<VEC, false><<<G, bd, 0, st>>>(b.x, b.r, b.p, b.Kp, N, t, b.state, b.partial, b.hist_beta, nullptr);
