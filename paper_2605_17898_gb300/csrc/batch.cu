@@ -15,119 +15,60 @@ namespace lgp {
 
 namespace {
 
-constexpr int kBatchThreads = 128;
-constexpr int kBatchR = 2;
-constexpr int kBatchBM = kBatchThreads * kBatchR;
+constexpr int kBatchBM = 256;  // rows of a work item
+template <int TT> using BatchTile = RowTile<TT, 2, 128>;
 
-// One 256-row block of one problem: K_y p for those rows over all of the problem's columns. The
+// One 256-row block of one problem: K_y p for those rows over all of the problem's columns (or one split of them). The
 // distance runs over the problem's own D coordinates (the rows are stored padded to DP).
 template <int KIND, int D, int TT>
-__device__ void batch_item(const BatchGp &g, int64_t row0, int split, const float *__restrict__ Xs_all,
-                           const float *__restrict__ p_all, float *__restrict__ kp_all, float *__restrict__ part,
-                           int t, float *xs, float *vs) {
-    constexpr int DP = D <= 4 ? 4 : 8;
-    const int tid = threadIdx.x;
-    const float *Xs = Xs_all + g.xs_off;
-    const float *V = p_all + g.vec_off * t;
-    float *out = kp_all + g.vec_off * t;
-    float xi[kBatchR][D];
-    float tot[kBatchR][TT];
-#pragma unroll
-    for (int r = 0; r < kBatchR; ++r) {
-        const int64_t i = row0 + r * kBatchThreads + tid;
-#pragma unroll
-        for (int d = 0; d < D; ++d) xi[r][d] = (i < g.Np) ? Xs[i * DP + d] : 0.0f;
-#pragma unroll
-        for (int c = 0; c < TT; ++c) tot[r][c] = 0.0f;
-    }
+__device__ void batch_item(const BatchGp &g, int64_t row0, int split, const BatchArgs &a, float *xs, float *vs, float *tot) {
+    using S = BatchTile<TT>;
+    static_assert(S::kRows == kBatchBM, "an item is one block of rows");
+    const int t = a.t;
+    const float *Xs = a.Xs + g.xs_off;
+    const float *V = a.p + g.vec_off * t;
+    float *out = a.kp + g.vec_off * t;
     const int64_t jb = (int64_t)split * g.cols_per_split;
     const int64_t je = min(g.N, jb + g.cols_per_split);
-    for (int64_t j0 = jb; j0 < je; j0 += kSimtBN) {
-        __syncthreads();
-        for (int e = tid; e < kSimtBN * DP / 4; e += kBatchThreads) {
-            const int64_t j = j0 + (e * 4) / DP;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (j < g.Np) v = *reinterpret_cast<const float4 *>(Xs + j0 * DP + e * 4);
-            *reinterpret_cast<float4 *>(xs + e * 4) = v;
-        }
-        for (int e = tid; e < kSimtBN * TT; e += kBatchThreads) {
-            const int jj = e / TT;
-            const int c = e - jj * TT;
-            const int64_t j = j0 + jj;
-            vs[e] = (j < je && c < t) ? V[j * t + c] : 0.0f;
-        }
-        __syncthreads();
-        float acc[kBatchR][TT];
+    float sum[S::R][TT];
+    simt_rows<KIND, D, S>(Xs, row0, g.Np, Xs, g.Np, V, t, 0, t, jb, je, g.log2s2, xs, vs, tot, sum);
 #pragma unroll
-        for (int r = 0; r < kBatchR; ++r)
-#pragma unroll
-            for (int c = 0; c < TT; ++c) acc[r][c] = 0.0f;
-#pragma unroll 2
-        for (int jj = 0; jj < kSimtBN; ++jj) {
-            float xj[D];
-            load_x_smem<D>(xs + jj * DP, xj);
-            float v[TT];
-            if (TT % 4 == 0) {
-#pragma unroll
-                for (int c = 0; c < TT; c += 4) {
-                    const float4 q = *reinterpret_cast<const float4 *>(vs + jj * TT + c);
-                    v[c] = q.x;
-                    v[(c + 1) % TT] = q.y;
-                    v[(c + 2) % TT] = q.z;
-                    v[(c + 3) % TT] = q.w;
-                }
-            } else {
-#pragma unroll
-                for (int c = 0; c < TT; ++c) v[c] = vs[jj * TT + c];
-            }
-#pragma unroll
-            for (int r = 0; r < kBatchR; ++r) {
-                const float k = Entry<KIND>::k(sqdist<D>(xi[r], xj), g.log2s2);
-#pragma unroll
-                for (int c = 0; c < TT; ++c) acc[r][c] = fmaf(k, v[c], acc[r][c]);
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < kBatchR; ++r)
-#pragma unroll
-            for (int c = 0; c < TT; ++c) tot[r][c] += acc[r][c];
-    }
-#pragma unroll
-    for (int r = 0; r < kBatchR; ++r) {
-        const int64_t i = row0 + r * kBatchThreads + tid;
+    for (int r = 0; r < S::R; ++r) {
+        const int64_t i = row0 + r * S::kThreads + threadIdx.x;
         if (i >= g.N) continue;
         if (g.splits > 1) {
-            float *dst = part + g.part_off + ((int64_t)split * g.Np + i) * t;
+            float *dst = a.part + g.part_off + ((int64_t)split * g.Np + i) * t;
 #pragma unroll
             for (int c = 0; c < TT; ++c)
-                if (c < t) dst[c] = tot[r][c];
+                if (c < t) dst[c] = sum[r][c];
         } else {
 #pragma unroll
             for (int c = 0; c < TT; ++c)
-                if (c < t) out[i * t + c] = fmaf(g.noise, V[i * t + c], tot[r][c]);
+                if (c < t) out[i * t + c] = fmaf(g.noise, V[i * t + c], sum[r][c]);
         }
     }
 }
 
 template <int KIND, int TT>
 __device__ __forceinline__ void batch_item_d(const BatchGp &g, int64_t row0, int split, const BatchArgs &a, float *xs,
-                                             float *vs) {
+                                             float *vs, float *tot) {
     switch (g.D) {
-        case 1: batch_item<KIND, 1, TT>(g, row0, split, a.Xs, a.p, a.kp, a.part, a.t, xs, vs); break;
-        case 2: batch_item<KIND, 2, TT>(g, row0, split, a.Xs, a.p, a.kp, a.part, a.t, xs, vs); break;
-        case 3: batch_item<KIND, 3, TT>(g, row0, split, a.Xs, a.p, a.kp, a.part, a.t, xs, vs); break;
-        case 4: batch_item<KIND, 4, TT>(g, row0, split, a.Xs, a.p, a.kp, a.part, a.t, xs, vs); break;
-        case 5: batch_item<KIND, 5, TT>(g, row0, split, a.Xs, a.p, a.kp, a.part, a.t, xs, vs); break;
-        case 6: batch_item<KIND, 6, TT>(g, row0, split, a.Xs, a.p, a.kp, a.part, a.t, xs, vs); break;
-        case 7: batch_item<KIND, 7, TT>(g, row0, split, a.Xs, a.p, a.kp, a.part, a.t, xs, vs); break;
-        default: batch_item<KIND, 8, TT>(g, row0, split, a.Xs, a.p, a.kp, a.part, a.t, xs, vs);
+        case 1: batch_item<KIND, 1, TT>(g, row0, split, a, xs, vs, tot); break;
+        case 2: batch_item<KIND, 2, TT>(g, row0, split, a, xs, vs, tot); break;
+        case 3: batch_item<KIND, 3, TT>(g, row0, split, a, xs, vs, tot); break;
+        case 4: batch_item<KIND, 4, TT>(g, row0, split, a, xs, vs, tot); break;
+        case 5: batch_item<KIND, 5, TT>(g, row0, split, a, xs, vs, tot); break;
+        case 6: batch_item<KIND, 6, TT>(g, row0, split, a, xs, vs, tot); break;
+        case 7: batch_item<KIND, 7, TT>(g, row0, split, a, xs, vs, tot); break;
+        default: batch_item<KIND, 8, TT>(g, row0, split, a, xs, vs, tot);
     }
 }
 
 template <int TT>
-__global__ void __launch_bounds__(kBatchThreads) batch_mv_kernel(BatchArgs a) {
+__global__ void __launch_bounds__(BatchTile<TT>::kThreads) batch_mv_kernel(BatchArgs a) {
     __shared__ __align__(16) float xs[kSimtBN * 8];
     __shared__ __align__(16) float vs[kSimtBN * TT];
+    __shared__ float tot[BatchTile<TT>::kTotFloats];
     __shared__ int item_s;
     if (a.done && *a.done) return;
     while (true) {
@@ -141,10 +82,10 @@ __global__ void __launch_bounds__(kBatchThreads) batch_mv_kernel(BatchArgs a) {
         const BatchGp g = a.gps[it.gp];
         const int64_t row0 = (int64_t)it.row_block * kBatchBM;
         switch (g.kind) {
-            case LGP_RBF: batch_item_d<LGP_RBF, TT>(g, row0, it.split, a, xs, vs); break;
-            case LGP_MATERN52: batch_item_d<LGP_MATERN52, TT>(g, row0, it.split, a, xs, vs); break;
-            case LGP_MATERN12: batch_item_d<LGP_MATERN12, TT>(g, row0, it.split, a, xs, vs); break;
-            default: batch_item_d<LGP_MATERN32, TT>(g, row0, it.split, a, xs, vs);
+            case LGP_RBF: batch_item_d<LGP_RBF, TT>(g, row0, it.split, a, xs, vs, tot); break;
+            case LGP_MATERN52: batch_item_d<LGP_MATERN52, TT>(g, row0, it.split, a, xs, vs, tot); break;
+            case LGP_MATERN12: batch_item_d<LGP_MATERN12, TT>(g, row0, it.split, a, xs, vs, tot); break;
+            default: batch_item_d<LGP_MATERN32, TT>(g, row0, it.split, a, xs, vs, tot);
         }
     }
 }
@@ -373,11 +314,11 @@ cudaError_t launch_batch_product(const BatchArgs &a, int num_sms, cudaStream_t s
     if (e != cudaSuccess) return e;
     const int grid = std::max(1, std::min(a.n_items, num_sms * 6));
     switch (a.tt) {
-        case 1: batch_mv_kernel<1><<<grid, kBatchThreads, 0, st>>>(a); break;
-        case 2: batch_mv_kernel<2><<<grid, kBatchThreads, 0, st>>>(a); break;
-        case 4: batch_mv_kernel<4><<<grid, kBatchThreads, 0, st>>>(a); break;
-        case 8: batch_mv_kernel<8><<<grid, kBatchThreads, 0, st>>>(a); break;
-        case 16: batch_mv_kernel<16><<<grid, kBatchThreads, 0, st>>>(a); break;
+        case 1: batch_mv_kernel<1><<<grid, BatchTile<1>::kThreads, 0, st>>>(a); break;
+        case 2: batch_mv_kernel<2><<<grid, BatchTile<2>::kThreads, 0, st>>>(a); break;
+        case 4: batch_mv_kernel<4><<<grid, BatchTile<4>::kThreads, 0, st>>>(a); break;
+        case 8: batch_mv_kernel<8><<<grid, BatchTile<8>::kThreads, 0, st>>>(a); break;
+        case 16: batch_mv_kernel<16><<<grid, BatchTile<16>::kThreads, 0, st>>>(a); break;
         default: return cudaErrorInvalidValue;
     }
     bsplit_reduce_kernel<<<a.n_vblocks, vec_threads(a.t), 0, st>>>(a);

@@ -126,6 +126,39 @@ template <> struct Entry<LGP_MATERN32> {
     }
 };
 
+// Two entries at once from squared distances accumulated on packed float32x2 operations. The accumulation starts at
+// acc0: RBF folds the outputscale exponent into it (acc = rh2 - log2 s^2, k = 2^-acc), Matern-5/2 uses k = e + e (rh +
+// rh2 / 3). A packed operation on three different register pairs runs at half rate (mv_sym.cuh), so the
+// multiply-adds by constants are scalar.
+template <int KIND> struct PackedEntry;
+template <> struct PackedEntry<LGP_RBF> {
+    static __device__ __forceinline__ float2 acc0(float ls2) { return make_float2(-ls2, -ls2); }
+    static __device__ __forceinline__ float2 k(float2 acc, float) { return make_float2(ex2_approx(-acc.x), ex2_approx(-acc.y)); }
+};
+template <> struct PackedEntry<LGP_MATERN52> {
+    static __device__ __forceinline__ float2 acc0(float) { return make_float2(0.0f, 0.0f); }
+    static __device__ __forceinline__ float2 k(float2 r2, float ls2) {
+        const float2 r = make_float2(sqrt_approx(r2.x), sqrt_approx(r2.y));
+        const float2 e = make_float2(ex2_approx(fmaf(r.x, -kLog2e, ls2)), ex2_approx(fmaf(r.y, -kLog2e, ls2)));
+        const float2 q = make_float2(fmaf(r2.x, 1.0f / 3.0f, r.x), fmaf(r2.y, 1.0f / 3.0f, r.y));
+        return __ffma2_rn(e, q, e);
+    }
+};
+template <> struct PackedEntry<LGP_MATERN12> {
+    static __device__ __forceinline__ float2 acc0(float) { return make_float2(0.0f, 0.0f); }
+    static __device__ __forceinline__ float2 k(float2 r2, float ls2) {
+        return make_float2(ex2_approx(ls2 - sqrt_approx(r2.x)), ex2_approx(ls2 - sqrt_approx(r2.y)));
+    }
+};
+template <> struct PackedEntry<LGP_MATERN32> {
+    static __device__ __forceinline__ float2 acc0(float) { return make_float2(0.0f, 0.0f); }
+    static __device__ __forceinline__ float2 k(float2 r2, float ls2) {
+        const float2 r = make_float2(sqrt_approx(r2.x), sqrt_approx(r2.y));
+        const float2 e = make_float2(ex2_approx(fmaf(r.x, -kLog2e, ls2)), ex2_approx(fmaf(r.y, -kLog2e, ls2)));
+        return __ffma2_rn(e, r, e);
+    }
+};
+
 // Host: the kind is one the library implements.
 inline bool kind_supported(int kind) {
     return kind == LGP_RBF || kind == LGP_MATERN52 || kind == LGP_MATERN12 || kind == LGP_MATERN32;

@@ -8,26 +8,36 @@ namespace lgp {
 
 namespace {
 
+// CTAs per SM that the row kernel's splits aim at (64 threads each), down to one column tile per split: at small N the
+// tiles of a split are a serial chain of loads and barriers. Against at least 4 tiles per split: N = 1200, D = 6, t = 8
+// 35 -> 15 us, N = 4099, D = 5, t = 5 39 -> 25 us; 16 -> 32 CTAs: N = 20000, D = 8, t = 8 410 -> 388 us. (The partial
+// sums stay at kRowCtas x SMs x rows of a CTA x t floats.)
+constexpr int kRowCtas = 32;
+
+// Padded columns of a launch and its CTA's rows.
 struct SimtShape {
-    int TT, R;
+    int TT, BM;
 };
 
+template <int TT> constexpr SimtShape shape_of() { return {TT, RowShape<TT>::kRows}; }
+
 SimtShape simt_shape(int t) {
-    if (t == 1) return {1, 4};
-    if (t == 2) return {2, 4};
-    if (t <= 4) return {4, 4};
-    if (t <= 8) return {8, 2};
-    if (t <= 16) return {16, 1};
-    return {32, 1};
+    if (t == 1) return shape_of<1>();
+    if (t == 2) return shape_of<2>();
+    if (t <= 4) return shape_of<4>();
+    if (t <= 8) return shape_of<8>();
+    if (t <= 16) return shape_of<16>();
+    return shape_of<32>();
 }
 
 // Column splits so that row blocks x splits x column groups fill the GPU a few
 // times over; each split covers a whole number of BN tiles.
-int64_t choose_split(int64_t N, int64_t row_blocks, int64_t col_groups, int num_sms, int64_t *cols_per_split) {
+int64_t choose_split(int64_t N, int64_t row_blocks, int64_t col_groups, int num_sms, int64_t *cols_per_split,
+                     int ctas_per_sm = 8, int64_t tiles_per_split = 4) {
     const int64_t col_tiles = (N + kSimtBN - 1) / kSimtBN;
-    const int64_t want = (int64_t)num_sms * 8;
+    const int64_t want = (int64_t)num_sms * ctas_per_sm;
     int64_t s = (want + row_blocks * col_groups - 1) / (row_blocks * col_groups);
-    s = std::max<int64_t>(1, std::min<int64_t>(s, std::max<int64_t>(1, col_tiles / 4)));
+    s = std::max<int64_t>(1, std::min<int64_t>(s, std::max<int64_t>(1, col_tiles / tiles_per_split)));
     const int64_t tiles_per = (col_tiles + s - 1) / s;
     *cols_per_split = tiles_per * kSimtBN;
     return (N + *cols_per_split - 1) / *cols_per_split;
@@ -147,21 +157,21 @@ int64_t mv_simt_partial_floats(int64_t N, int64_t Np, int t, int num_sms) {
     const SymGrid sg = sym_grid(N, Np, t, num_sms);
     if (sg.E) return (int64_t)sg.G * Np * t;
     const SimtShape sh = simt_shape(t);
-    const int64_t BM = (int64_t)kSimtThreads * sh.R;
+    const int64_t BM = sh.BM;
     const int64_t rb = (N + BM - 1) / BM;
     const int64_t cg = (t + sh.TT - 1) / sh.TT;
     int64_t cps;
-    const int64_t S = choose_split(N, rb, cg, num_sms, &cps);
+    const int64_t S = choose_split(N, rb, cg, num_sms, &cps, kRowCtas, 1);
     return S > 1 ? S * Np * t : 0;
 }
 
 int64_t mv_simt_cross_partial_floats(int64_t Nr, int64_t Npr, int64_t N, int t, int num_sms) {
     const SimtShape sh = simt_shape(t);
-    const int64_t BM = (int64_t)kSimtThreads * sh.R;
+    const int64_t BM = sh.BM;
     const int64_t rb = (Nr + BM - 1) / BM;
     const int64_t cg = (t + sh.TT - 1) / sh.TT;
     int64_t cps;
-    const int64_t S = choose_split(N, rb, cg, num_sms, &cps);
+    const int64_t S = choose_split(N, rb, cg, num_sms, &cps, kRowCtas, 1);
     return S > 1 ? S * Npr * t : 0;
 }
 
@@ -212,11 +222,11 @@ cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st) {
         return e != cudaSuccess ? e : finish_splits(m, sg.G, m.N, m.Np, 0, st);
     }
     const SimtShape sh = simt_shape(m.t);
-    const int64_t BM = (int64_t)kSimtThreads * sh.R;
+    const int64_t BM = sh.BM;
     const int64_t rb = (Nr + BM - 1) / BM;
     const int64_t cg = (m.t + sh.TT - 1) / sh.TT;
     int64_t cps;
-    int64_t S = choose_split(m.N, rb, cg, m.num_sms, &cps);
+    int64_t S = choose_split(m.N, rb, cg, m.num_sms, &cps, kRowCtas, 1);
     if (S > 1 && (m.partial == nullptr || S * Npr * m.t > m.partial_cap)) {
         S = 1;
         cps = m.N;
@@ -242,10 +252,10 @@ cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st) {
     const dim3 grid((unsigned)rb, (unsigned)S, (unsigned)cg);
     cudaError_t e;
     switch (m.kp->kind) {
-        case LGP_RBF: e = mv_simt_dispatch_rbf(m.kp->D, sh.TT, sh.R, grid, a, st); break;
-        case LGP_MATERN52: e = mv_simt_dispatch_m52(m.kp->D, sh.TT, sh.R, grid, a, st); break;
-        case LGP_MATERN12: e = mv_simt_dispatch_m12(m.kp->D, sh.TT, sh.R, grid, a, st); break;
-        case LGP_MATERN32: e = mv_simt_dispatch_m32(m.kp->D, sh.TT, sh.R, grid, a, st); break;
+        case LGP_RBF: e = mv_simt_dispatch_rbf(m.kp->D, sh.TT, grid, a, st); break;
+        case LGP_MATERN52: e = mv_simt_dispatch_m52(m.kp->D, sh.TT, grid, a, st); break;
+        case LGP_MATERN12: e = mv_simt_dispatch_m12(m.kp->D, sh.TT, grid, a, st); break;
+        case LGP_MATERN32: e = mv_simt_dispatch_m32(m.kp->D, sh.TT, grid, a, st); break;
         default: e = cudaErrorInvalidValue;
     }
     if (e != cudaSuccess || S == 1) return e;

@@ -1,8 +1,7 @@
 // FP32 SIMT kernels of the matrix-free product family (templates; instantiated per kernel kind).
 //
-// All three kernels share one structure: a CTA of 128 threads owns a block of
-// 128*R rows of the output; each thread keeps R prescaled rows xh_i in
-// registers. The CTA sweeps a range of columns j in tiles of BN=64 staged in
+// All three kernels share one structure: a CTA owns a block of rows of the
+// output; each thread keeps R prescaled rows xh_i in registers. The CTA sweeps a range of columns j in tiles of BN=64 staged in
 // shared memory (prescaled x_j plus the matching right-hand-side rows), and
 // every thread generates its R x BN kernel entries in registers, uses them and
 // drops them: no entry is ever written to global memory (Sec. 3 "GPU
@@ -82,92 +81,152 @@ __device__ __forceinline__ void stage_x(float *xs, const float *__restrict__ Xs,
     }
 }
 
-// ------------------------------------------------------------------ product K_y V (columns c0..c0+TT-1)
+// ------------------------------------------------------------------ product rows (columns c0..c0+TT-1)
 
-template <int KIND, int D, int TT, int R>
-__global__ void __launch_bounds__(kSimtThreads) mv_simt_kernel(SimtArgs a) {
-    constexpr int DP = DPad<D>::value;
-    constexpr int BM = kSimtThreads * R;
-    __shared__ __align__(16) float xs[kSimtBN * DP];
-    __shared__ __align__(16) float vs[kSimtBN * TT];
-    if (a.skip && *a.skip) return;
+// Columns, rows per thread and threads of a CTA. A shared-memory load costs the floats it delivers to the registers
+// (128 bytes per SM and clock, broadcast or not), D + TT of them per column and R rows, so the large products take R = 4
+// (one row per thread at TT = 16, 32 and two at TT = 8 were bound by these loads); the batched product, whose problems
+// are small, takes R = 2 for more warps in flight.
+// Product call, before -> now: N = 20000, D = 8: t = 8 443 -> 390 us, t = 12 771 -> 548, t = 32 1129 -> 958; N = 4099, D = 5, t = 5
+// 39 -> 29. Batched solve of 48 GPs, t = 8: R = 4 in 64 threads 11.87 ms, R = 2 in 128 threads 11.16.
+template <int TT_, int R_, int THREADS> struct RowTile {
+    static constexpr int TT = TT_, R = R_, kThreads = THREADS;
+    static constexpr int kRows = R * kThreads;
+    // running totals in shared memory where the registers hold only one tile's sums
+    static constexpr bool kTotShared = TT >= 8;
+    static constexpr int kTotFloats = kTotShared ? R * TT * kThreads : 1;
+};
+template <int TT> using RowShape = RowTile<TT, TT == 32 ? 2 : 4, 64>;
 
+// sum_j k(x_i, x_j) V[j, c0..c0+TT) over jb <= j < je for this thread's rows i = row0 + r kThreads + tid, added up per
+// tile of kSimtBN columns. Distances run on packed operations over pairs of columns (x_j - x_i as x_j + (-x_i), the
+// row's coordinates kept twice), the V multiply-adds are scalar (three different register pairs would run at half
+// rate). xs [D][kSimtBN], vs [kSimtBN][TT], tot [kTotFloats]: shared memory.
+template <int KIND, int D, class S>
+__device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t row0, int64_t Npr,
+                                          const float *__restrict__ Xs, int64_t Np, const float *__restrict__ V, int64_t ldv,
+                                          int c0, int t, int64_t jb, int64_t je, float log2s2, float *xs, float *vs, float *tot,
+                                          float (&sum)[S::R][S::TT]) {
+    constexpr int DP = DPad<D>::value, TT = S::TT, R = S::R, NT = S::kThreads;
     const int tid = threadIdx.x;
-    const int64_t row0 = (int64_t)blockIdx.x * BM;
-    const int c0 = blockIdx.z * TT;
-    const int64_t jb = (int64_t)blockIdx.y * a.cols_per_split;
-    const int64_t je = min(a.N, jb + a.cols_per_split);
-
-    float xi[R][D];
-    float tot[R][TT];
+    float2 xi[R][D];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-        const int64_t i = row0 + r * kSimtThreads + tid;
+        const int64_t i = row0 + r * NT + tid;
 #pragma unroll
-        for (int d = 0; d < D; ++d) xi[r][d] = (i < a.Npr) ? a.Xr[i * DP + d] : 0.0f;
+        for (int d = 0; d < D; ++d) {
+            const float x = i < Npr ? -Xr[i * DP + d] : 0.0f;
+            xi[r][d] = make_float2(x, x);
+        }
 #pragma unroll
-        for (int c = 0; c < TT; ++c) tot[r][c] = 0.0f;
+        for (int c = 0; c < TT; ++c) {
+            sum[r][c] = 0.0f;
+            if constexpr (S::kTotShared) tot[(r * TT + c) * NT + tid] = 0.0f;
+        }
     }
-
+    const float2 acc0 = PackedEntry<KIND>::acc0(log2s2);
     for (int64_t j0 = jb; j0 < je; j0 += kSimtBN) {
         __syncthreads();
-        stage_x<D>(xs, a.Xs, j0, a.Np);
-        for (int e = tid; e < kSimtBN * TT; e += kSimtThreads) {
-            const int jj = e / TT;
-            const int c = e - jj * TT;
-            const int64_t j = j0 + jj;
-            vs[e] = (j < je && c0 + c < a.t) ? a.V[j * a.ldv + c0 + c] : 0.0f;
+        for (int e = tid; e < kSimtBN * (DP / 4); e += NT) {
+            const int jj = e % kSimtBN, q = e / kSimtBN;
+            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (j0 + jj < Np) v = *reinterpret_cast<const float4 *>(Xs + (j0 + jj) * DP + 4 * q);
+            const float f[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (4 * q + k < D) xs[(4 * q + k) * kSimtBN + jj] = f[k];
+        }
+        for (int e = tid; e < kSimtBN * TT; e += NT) {
+            const int jj = e / TT, c = e - jj * TT;
+            vs[e] = (j0 + jj < je && c0 + c < t) ? V[(j0 + jj) * ldv + c0 + c] : 0.0f;
         }
         __syncthreads();
-
         float acc[R][TT];
 #pragma unroll
         for (int r = 0; r < R; ++r)
 #pragma unroll
             for (int c = 0; c < TT; ++c) acc[r][c] = 0.0f;
-
-#pragma unroll 2
-        for (int jj = 0; jj < kSimtBN; ++jj) {
-            float xj[D];
-            load_x_smem<D>(xs + jj * DP, xj);
-            float v[TT];
-            if (TT % 4 == 0) {
+#pragma unroll 4
+        for (int jj = 0; jj < kSimtBN; jj += 2) {
+            float2 xj[D], k[R];
 #pragma unroll
-                for (int c = 0; c < TT; c += 4) {
-                    const float4 q = *reinterpret_cast<const float4 *>(vs + jj * TT + c);
-                    v[c] = q.x; v[(c + 1) % TT] = q.y; v[(c + 2) % TT] = q.z; v[(c + 3) % TT] = q.w;
-                }
-            } else {
-#pragma unroll
-                for (int c = 0; c < TT; ++c) v[c] = vs[jj * TT + c];
-            }
+            for (int d = 0; d < D; ++d) xj[d] = *reinterpret_cast<const float2 *>(xs + d * kSimtBN + jj);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const float k = Entry<KIND>::k(sqdist<D>(xi[r], xj), a.log2s2);
+                float2 dd = __fadd2_rn(xj[0], xi[r][0]);
+                float2 r2 = __ffma2_rn(dd, dd, acc0);
 #pragma unroll
-                for (int c = 0; c < TT; ++c) acc[r][c] = fmaf(k, v[c], acc[r][c]);
+                for (int d = 1; d < D; ++d) {
+                    dd = __fadd2_rn(xj[d], xi[r][d]);
+                    r2 = __ffma2_rn(dd, dd, r2);
+                }
+                k[r] = PackedEntry<KIND>::k(r2, log2s2);
+            }
+            constexpr int CV = TT < 4 ? TT : 4;  // V columns per load
+#pragma unroll
+            for (int c = 0; c < TT; c += CV) {
+                float v0[CV], v1[CV];
+                if constexpr (CV == 4) {
+                    const float4 a = *reinterpret_cast<const float4 *>(vs + jj * TT + c);
+                    const float4 b = *reinterpret_cast<const float4 *>(vs + (jj + 1) * TT + c);
+                    v0[0] = a.x; v0[1] = a.y; v0[2] = a.z; v0[3] = a.w;
+                    v1[0] = b.x; v1[1] = b.y; v1[2] = b.z; v1[3] = b.w;
+                } else {
+#pragma unroll
+                    for (int q = 0; q < CV; ++q) {
+                        v0[q] = vs[jj * TT + q];
+                        v1[q] = vs[(jj + 1) * TT + q];
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int q = 0; q < CV; ++q) acc[r][c + q] = fmaf(k[r].y, v1[q], fmaf(k[r].x, v0[q], acc[r][c + q]));
             }
         }
 #pragma unroll
         for (int r = 0; r < R; ++r)
 #pragma unroll
-            for (int c = 0; c < TT; ++c) tot[r][c] += acc[r][c];
+            for (int c = 0; c < TT; ++c) {
+                if constexpr (S::kTotShared) tot[(r * TT + c) * NT + tid] += acc[r][c];
+                else sum[r][c] += acc[r][c];
+            }
     }
-
+    if constexpr (S::kTotShared) {
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int64_t i = row0 + r * kSimtThreads + tid;
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < TT; ++c) sum[r][c] = tot[(r * TT + c) * NT + tid];
+    }
+}
+
+template <int KIND, int D, int TT>
+__global__ void __launch_bounds__(RowShape<TT>::kThreads) mv_simt_kernel(SimtArgs a) {
+    using S = RowShape<TT>;
+    __shared__ __align__(16) float xs[kSimtBN * D];
+    __shared__ __align__(16) float vs[kSimtBN * TT];
+    __shared__ float tot[S::kTotFloats];
+    if (a.skip && *a.skip) return;
+    const int64_t row0 = (int64_t)blockIdx.x * S::kRows;
+    const int c0 = blockIdx.z * TT;
+    const int64_t jb = (int64_t)blockIdx.y * a.cols_per_split;
+    const int64_t je = min(a.N, jb + a.cols_per_split);
+    float sum[S::R][TT];
+    simt_rows<KIND, D, S>(a.Xr, row0, a.Npr, a.Xs, a.Np, a.V, a.ldv, c0, a.t, jb, je, a.log2s2, xs, vs, tot, sum);
+#pragma unroll
+    for (int r = 0; r < S::R; ++r) {
+        const int64_t i = row0 + r * S::kThreads + threadIdx.x;
         if (i >= a.Nr) continue;
         if (a.partial) {
             float *dst = a.partial + ((int64_t)blockIdx.y * a.Npr + i) * a.t + c0;
 #pragma unroll
             for (int c = 0; c < TT; ++c)
-                if (c0 + c < a.t) dst[c] = tot[r][c];
+                if (c0 + c < a.t) dst[c] = sum[r][c];
         } else {
 #pragma unroll
             for (int c = 0; c < TT; ++c)
                 if (c0 + c < a.t)
-                    a.out[i * a.ldo + c0 + c] = a.cross ? tot[r][c] : fmaf(a.noise, a.V[i * a.ldv + c0 + c], tot[r][c]);
+                    a.out[i * a.ldo + c0 + c] = a.cross ? sum[r][c] : fmaf(a.noise, a.V[i * a.ldv + c0 + c], sum[r][c]);
         }
     }
 }
@@ -379,16 +438,16 @@ __global__ void __launch_bounds__(kSimtThreads) adjoint_bilinear_kernel(AdjArgs 
 }
 
 // Kind-specific dispatchers (one translation unit per kernel kind).
-cudaError_t mv_simt_dispatch_rbf(int D, int TT, int R, dim3 grid, const SimtArgs &a, cudaStream_t st);
-cudaError_t mv_simt_dispatch_m52(int D, int TT, int R, dim3 grid, const SimtArgs &a, cudaStream_t st);
+cudaError_t mv_simt_dispatch_rbf(int D, int TT, dim3 grid, const SimtArgs &a, cudaStream_t st);
+cudaError_t mv_simt_dispatch_m52(int D, int TT, dim3 grid, const SimtArgs &a, cudaStream_t st);
 cudaError_t mv_grad_dispatch_rbf(int D, int TT, dim3 grid, const GradArgs &a, cudaStream_t st);
 cudaError_t mv_grad_dispatch_m52(int D, int TT, dim3 grid, const GradArgs &a, cudaStream_t st);
 cudaError_t adjoint_dispatch_rbf(int D, int TT, dim3 grid, const AdjArgs &a, cudaStream_t st);
 cudaError_t adjoint_dispatch_m52(int D, int TT, dim3 grid, const AdjArgs &a, cudaStream_t st);
-cudaError_t mv_simt_dispatch_m12(int D, int TT, int R, dim3 grid, const SimtArgs &a, cudaStream_t st);
+cudaError_t mv_simt_dispatch_m12(int D, int TT, dim3 grid, const SimtArgs &a, cudaStream_t st);
 cudaError_t mv_grad_dispatch_m12(int D, int TT, dim3 grid, const GradArgs &a, cudaStream_t st);
 cudaError_t adjoint_dispatch_m12(int D, int TT, dim3 grid, const AdjArgs &a, cudaStream_t st);
-cudaError_t mv_simt_dispatch_m32(int D, int TT, int R, dim3 grid, const SimtArgs &a, cudaStream_t st);
+cudaError_t mv_simt_dispatch_m32(int D, int TT, dim3 grid, const SimtArgs &a, cudaStream_t st);
 cudaError_t mv_grad_dispatch_m32(int D, int TT, dim3 grid, const GradArgs &a, cudaStream_t st);
 cudaError_t adjoint_dispatch_m32(int D, int TT, dim3 grid, const AdjArgs &a, cudaStream_t st);
 
@@ -398,26 +457,26 @@ cudaError_t adjoint_dispatch_m32(int D, int TT, dim3 grid, const AdjArgs &a, cud
 #define LGP_DEFINE_SIMT_DISPATCH(KIND, SUFFIX)                                                                   \
     namespace lgp {                                                                                            \
     template <int D>                                                                                           \
-    static cudaError_t mv_simt_d_##SUFFIX(int TT, int R, dim3 grid, const SimtArgs &a, cudaStream_t st) {      \
-        if (TT == 1 && R == 4) mv_simt_kernel<KIND, D, 1, 4><<<grid, kSimtThreads, 0, st>>>(a);                \
-        else if (TT == 2 && R == 4) mv_simt_kernel<KIND, D, 2, 4><<<grid, kSimtThreads, 0, st>>>(a);           \
-        else if (TT == 4 && R == 4) mv_simt_kernel<KIND, D, 4, 4><<<grid, kSimtThreads, 0, st>>>(a);           \
-        else if (TT == 8 && R == 2) mv_simt_kernel<KIND, D, 8, 2><<<grid, kSimtThreads, 0, st>>>(a);           \
-        else if (TT == 16 && R == 1) mv_simt_kernel<KIND, D, 16, 1><<<grid, kSimtThreads, 0, st>>>(a);         \
-        else if (TT == 32 && R == 1) mv_simt_kernel<KIND, D, 32, 1><<<grid, kSimtThreads, 0, st>>>(a);         \
+    static cudaError_t mv_simt_d_##SUFFIX(int TT, dim3 grid, const SimtArgs &a, cudaStream_t st) {             \
+        if (TT == 1) mv_simt_kernel<KIND, D, 1><<<grid, RowShape<1>::kThreads, 0, st>>>(a);                     \
+        else if (TT == 2) mv_simt_kernel<KIND, D, 2><<<grid, RowShape<2>::kThreads, 0, st>>>(a);                \
+        else if (TT == 4) mv_simt_kernel<KIND, D, 4><<<grid, RowShape<4>::kThreads, 0, st>>>(a);                \
+        else if (TT == 8) mv_simt_kernel<KIND, D, 8><<<grid, RowShape<8>::kThreads, 0, st>>>(a);                \
+        else if (TT == 16) mv_simt_kernel<KIND, D, 16><<<grid, RowShape<16>::kThreads, 0, st>>>(a);             \
+        else if (TT == 32) mv_simt_kernel<KIND, D, 32><<<grid, RowShape<32>::kThreads, 0, st>>>(a);             \
         else return cudaErrorInvalidValue;                                                                     \
         return cudaGetLastError();                                                                             \
     }                                                                                                          \
-    cudaError_t mv_simt_dispatch_##SUFFIX(int D, int TT, int R, dim3 grid, const SimtArgs &a, cudaStream_t st) { \
+    cudaError_t mv_simt_dispatch_##SUFFIX(int D, int TT, dim3 grid, const SimtArgs &a, cudaStream_t st) {      \
         switch (D) {                                                                                           \
-            case 1: return mv_simt_d_##SUFFIX<1>(TT, R, grid, a, st);                                          \
-            case 2: return mv_simt_d_##SUFFIX<2>(TT, R, grid, a, st);                                          \
-            case 3: return mv_simt_d_##SUFFIX<3>(TT, R, grid, a, st);                                          \
-            case 4: return mv_simt_d_##SUFFIX<4>(TT, R, grid, a, st);                                          \
-            case 5: return mv_simt_d_##SUFFIX<5>(TT, R, grid, a, st);                                          \
-            case 6: return mv_simt_d_##SUFFIX<6>(TT, R, grid, a, st);                                          \
-            case 7: return mv_simt_d_##SUFFIX<7>(TT, R, grid, a, st);                                          \
-            case 8: return mv_simt_d_##SUFFIX<8>(TT, R, grid, a, st);                                          \
+            case 1: return mv_simt_d_##SUFFIX<1>(TT, grid, a, st);                                             \
+            case 2: return mv_simt_d_##SUFFIX<2>(TT, grid, a, st);                                             \
+            case 3: return mv_simt_d_##SUFFIX<3>(TT, grid, a, st);                                             \
+            case 4: return mv_simt_d_##SUFFIX<4>(TT, grid, a, st);                                             \
+            case 5: return mv_simt_d_##SUFFIX<5>(TT, grid, a, st);                                             \
+            case 6: return mv_simt_d_##SUFFIX<6>(TT, grid, a, st);                                             \
+            case 7: return mv_simt_d_##SUFFIX<7>(TT, grid, a, st);                                             \
+            case 8: return mv_simt_d_##SUFFIX<8>(TT, grid, a, st);                                             \
         }                                                                                                      \
         return cudaErrorInvalidValue;                                                                          \
     }                                                                                                          \

@@ -29,7 +29,7 @@
 // t = 8 the folds and V's loads outweigh the saved distances (N = 20000, D = 3 269 -> 285 us): the row kernel keeps t > 4.
 #pragma once
 
-#include "mv_tc.cuh"
+#include "lgp_internal.cuh"
 
 namespace lgp {
 
@@ -50,33 +50,6 @@ template <int D, int TT> struct SymShape {
     static constexpr int R = D <= 4 && TT <= 2 ? 8 : 4;
     static constexpr int C = 4;
     static constexpr int RB = 8 * R;  // rows of one sweep
-};
-
-// Two entries from the accumulated squared distances (which start at acc0): tc::Entry2 with the multiply-adds by
-// constants as scalar operations.
-template <int KIND> struct SymEntry;
-template <> struct SymEntry<LGP_RBF> {
-    static __device__ __forceinline__ float2 k(float2 acc, float) { return make_float2(ex2_approx(-acc.x), ex2_approx(-acc.y)); }
-};
-template <> struct SymEntry<LGP_MATERN52> {
-    static __device__ __forceinline__ float2 k(float2 r2, float ls2) {
-        const float2 r = make_float2(sqrt_approx(r2.x), sqrt_approx(r2.y));
-        const float2 e = make_float2(ex2_approx(fmaf(r.x, -kLog2e, ls2)), ex2_approx(fmaf(r.y, -kLog2e, ls2)));
-        const float2 q = make_float2(fmaf(r2.x, 1.0f / 3.0f, r.x), fmaf(r2.y, 1.0f / 3.0f, r.y));
-        return __ffma2_rn(e, q, e);
-    }
-};
-template <> struct SymEntry<LGP_MATERN12> {
-    static __device__ __forceinline__ float2 k(float2 r2, float ls2) {
-        return make_float2(ex2_approx(ls2 - sqrt_approx(r2.x)), ex2_approx(ls2 - sqrt_approx(r2.y)));
-    }
-};
-template <> struct SymEntry<LGP_MATERN32> {
-    static __device__ __forceinline__ float2 k(float2 r2, float ls2) {
-        const float2 r = make_float2(sqrt_approx(r2.x), sqrt_approx(r2.y));
-        const float2 e = make_float2(ex2_approx(fmaf(r.x, -kLog2e, ls2)), ex2_approx(fmaf(r.y, -kLog2e, ls2)));
-        return __ffma2_rn(e, r, e);
-    }
 };
 
 // Row sets of the 4 warps (the others share a sweep's columns).
@@ -162,7 +135,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
     __syncthreads();
 
     const float ls2 = a.log2s2;
-    const float2 acc_init = tc::Entry2<KIND>::acc0(make_float2(ls2, ls2));
+    const float2 acc_init = PackedEntry<KIND>::acc0(ls2);
     const int wr = warp / WC, wc = warp % WC;
     const int cw = E / WC, c_lo = wc * cw;  // columns of this warp
     float *mycol = col + wr * E * TT + sym_fold_index<NV>(lane);
@@ -229,7 +202,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
                         dd = __fadd2_rn(xj[h][d], xi[r][d]);
                         r2 = __ffma2_rn(dd, dd, r2);
                     }
-                    const float2 k = SymEntry<KIND>::k(r2, ls2);
+                    const float2 k = PackedEntry<KIND>::k(r2, ls2);
 #pragma unroll
                     for (int q = 0; q < TT; ++q) {
                         acc[r][q] = fmaf(k.y, vj[c1 + q], fmaf(k.x, vj[c0 + q], acc[r][q]));
