@@ -588,12 +588,12 @@ lgp_status build_precond(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X, con
 
 // Kernel launches of one CG iteration: the product kernel (both distance instances where the host does not know the
 // form), the split of p where it is not part of the step, and the step.
-int cg_iteration_launches(const lgp_ctx *ctx, const Prepared &pp, int t, int prec, bool precond, int dist_form = -1) {
-    int n = 1 + 3;
+int cg_iteration_launches(const lgp_ctx *ctx, const Prepared &pp, int t, int prec, const CgBuffers &b, int dist_form = -1) {
+    const bool precond = b.pc.k > 0;
+    int n = 1 + (cg_cluster_ok(pp.N, t, b) ? 1 : 3);
     if (is_tc(prec)) {
         if (needs_dot(ctx, pp, t, prec) && dist_form < 0) ++n;
         if (precond) n += tc_fmt(prec) == 1 ? 2 : 1;
-        // the row kernel's split reduction is part of the step, also when preconditioned
     }
     return n + (precond ? 4 : 0);
 }
@@ -1665,12 +1665,12 @@ lgp_status lgp_lml_and_grad(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X, 
         if (!single) {
             const int split_once = is_tc(prec) && k == 0 ? (tc_fmt(prec) == 1 ? 2 : 1) : 0;
             info->launches = 3 + 2 + split_once +
-                             ran * (kChunk * cg_iteration_launches(ctx, pp, t, prec, k > 0, ctx->cg_dist_form) + 1) + 2 + 2 +
+                             ran * (kChunk * cg_iteration_launches(ctx, pp, t, prec, b, ctx->cg_dist_form) + 1) + 2 + 2 +
                              (grad ? 3 : 0) + pc_once + opnd_once;
         } else {
             // per column: CG init (2), copy and gather (2); the chunks of all columns; per column in the
             // gradient: two column copies and one adjoint pass
-            info->launches = 3 + 4 * t + ran * (kChunk * cg_iteration_launches(ctx, pp, 1, LGP_PREC_FP32, false) + 1) +
+            info->launches = 3 + 4 * t + ran * (kChunk * cg_iteration_launches(ctx, pp, 1, LGP_PREC_FP32, b) + 1) +
                              2 + 2 + (grad ? 2 + 3 * t : 0);
         }
     }
