@@ -1,14 +1,16 @@
 // Many independent GP solves of uneven size advanced together.
 //
 // Per CG iteration, one persistent launch computes K_y(g) p(g) for every problem g:
-// its CTAs pull work items (problem, block of 256 rows) from a list sorted by cost
+// its CTAs pull work items (problem, block of 256 rows, column split) from a list sorted by cost
 // (longest first) through an atomic counter, so large and small problems share the
 // GPU without one launch per problem. Problems whose columns have all converged are
-// skipped. The vector updates and the float64 scalar recurrences then run as segmented
-// versions of the single-problem CG kernels: every vector block belongs to one problem,
-// and each (problem, column) scalar is reduced from that problem's block partials in a
-// fixed order, so the results do not depend on which CTA took which item.
+// skipped. One more launch is the rest of the iteration: a thread-block cluster (or one CTA) per problem
+// adds the product's partial sums and runs the problem's whole CG step, its column sums exchanged
+// through distributed shared memory in a fixed order, so the results do not depend on which CTA took which item.
+#include <cooperative_groups.h>
+
 #include "batch.cuh"
+#include "cg_reduce.cuh"
 #include "mv_simt.cuh"
 
 namespace lgp {
@@ -70,7 +72,7 @@ __global__ void __launch_bounds__(BatchTile<TT>::kThreads) batch_mv_kernel(Batch
     __shared__ __align__(16) float vs[kSimtBN * TT];
     __shared__ float tot[BatchTile<TT>::kTotFloats];
     __shared__ int item_s;
-    if (a.done && *a.done) return;
+    if (*a.done || *a.n_done >= a.n_gp) return;
     while (true) {
         __syncthreads();
         if (threadIdx.x == 0) item_s = atomicAdd(a.item_counter, 1);
@@ -93,6 +95,7 @@ __global__ void __launch_bounds__(BatchTile<TT>::kThreads) batch_mv_kernel(Batch
 // ---------------------------------------------------------------- segmented CG kernels
 
 constexpr int kVec = 256;
+constexpr int kMaxBatchT = 16;
 
 __device__ void seg_col_reduce(double v, int t, double *red, double *out_row) {
     const int tid = threadIdx.x;
@@ -144,139 +147,205 @@ __global__ void bscal_init_kernel(BatchArgs a, double tol, int max_iter) {
     for (int b = g.blk0; b < g.blk1; ++b) s += a.partial[(int64_t)b * a.t + c];
     a.bnorm2[k] = s;
     a.rr[k] = s;
-    a.alpha[k] = 0.0;
-    a.beta[k] = 0.0;
     a.iters[k] = 0;
     const bool bad = !isfinite(s);
     a.active[k] = (s > 0.0) && !bad;
     if (bad) atomicOr(&a.st->status, 1);
 }
 
-__global__ void bdone_kernel(BatchArgs a, int first) {
-    __shared__ int any_s;
-    if (threadIdx.x == 0) any_s = 0;
+// Problems without an active column are done from the start; a non-finite right-hand side ends the whole call.
+__global__ void bdone_kernel(BatchArgs a) {
+    __shared__ int n_s;
+    if (threadIdx.x == 0) n_s = 0;
     __syncthreads();
-    if (!first && *a.done) return;
-    int any = 0;
+    int n = 0;
     for (int gi = threadIdx.x; gi < a.n_gp; gi += blockDim.x) {
         int act = 0;
         for (int c = 0; c < a.t; ++c) act |= a.active[gi * a.t + c];
         a.gp_done[gi] = !act;
-        any |= act;
+        n += !act;
     }
-    if (any) atomicOr(&any_s, 1);
+    atomicAdd(&n_s, n);
     __syncthreads();
     if (threadIdx.x == 0) {
-        if (!first) a.st->iter += 1;
-        *a.done = (!any_s || a.st->iter >= a.st->max_iter || (first && a.st->status)) ? 1 : 0;
+        *a.n_done = n_s;
+        *a.item_counter = 0;
+        *a.done = a.st->status ? 1 : 0;
     }
 }
 
-// K_y p for problems whose product was split over columns: the partial sums in split order plus
-// sigma^2 p (one vector block per CTA).
-__global__ void bsplit_reduce_kernel(BatchArgs a) {
-    if (*a.done) return;
-    const BatchVecBlock vb = a.vblocks[blockIdx.x];
-    const BatchGp g = a.gps[vb.gp];
-    if (g.splits <= 1 || a.gp_done[vb.gp]) return;
-    const int t = a.t;
-    const int c = threadIdx.x % t;
-    for (int64_t i = vb.r0 + threadIdx.x / t; i < vb.r1; i += blockDim.x / t) {
-        float sum = 0.0f;
-        for (int k = 0; k < g.splits; ++k) sum += a.part[g.part_off + ((int64_t)k * g.Np + i) * t + c];
-        const int64_t e = (g.vec_off + i) * t + c;
-        a.kp[e] = fmaf(g.noise, a.p[e], sum);
-    }
-}
+// ---------------------------------------------------------------- the CG step
 
-__global__ void bpkp_kernel(BatchArgs a) {
-    __shared__ double red[kVec];
-    if (*a.done) return;
-    const BatchVecBlock vb = a.vblocks[blockIdx.x];
-    const BatchGp g = a.gps[vb.gp];
-    const int t = a.t;
-    const int c = threadIdx.x % t;
-    float hi = 0.0f, lo = 0.0f;
-    if (!a.gp_done[vb.gp]) {
-        for (int64_t i = vb.r0 + threadIdx.x / t; i < vb.r1; i += blockDim.x / t) {
-            const int64_t e = (g.vec_off + i) * t + c;
-            acc_prod2(hi, lo, a.p[e], a.kp[e]);
+// One problem's CG step after the product: Kp = sum_k part[k] + noise p (or as the product left it), alpha, x, r, beta,
+// p and the problem's state, by one cluster of CL CTAs whose three passes over the problem's vectors meet at the
+// cluster barrier. As segmented kernels the step took seven launches an iteration (with the product's memset nine),
+// each a few microseconds for vectors that fit L2 many times over.
+template <int CL> __device__ double batch_cluster_sum(double *mine, int t) {
+    double s = 0.0;
+    if constexpr (CL == 1) {
+        __syncthreads();
+        if ((int)threadIdx.x < t) s = mine[threadIdx.x];
+    } else {
+        cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+        cl.sync();
+        if ((int)threadIdx.x < t) {
+#pragma unroll
+            for (int q = 0; q < CL; ++q) s += cl.map_shared_rank(mine, q)[threadIdx.x];
         }
     }
-    seg_col_reduce((double)hi + (double)lo, t, red, a.partial + (int64_t)blockIdx.x * t);
+    return s;
 }
 
-__global__ void balpha_kernel(BatchArgs a) {
-    if (*a.done) return;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= a.n_gp * a.t) return;
-    const int gi = k / a.t, c = k % a.t;
-    double alpha = 0.0;
-    if (a.active[k]) {
-        const BatchGp g = a.gps[gi];
-        double pkp = 0.0;
-        for (int b = g.blk0; b < g.blk1; ++b) pkp += a.partial[(int64_t)b * a.t + c];
-        if (!isfinite(pkp) || !(pkp > 0.0)) {
-            a.active[k] = 0;
-            atomicOr(&a.st->status, isfinite(pkp) ? 2 : 1);
+template <int VEC> __device__ __forceinline__ void load_vec(const float *p, float (&v)[VEC]) {
+    if constexpr (VEC == 4) {
+        const float4 q = *reinterpret_cast<const float4 *>(p);
+        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+    } else {
+        v[0] = *p;
+    }
+}
+template <int VEC> __device__ __forceinline__ void store_vec(float *p, const float (&v)[VEC]) {
+    if constexpr (VEC == 4) *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else *p = v[0];
+}
+
+// Block of VEC = 4 (t a power of two): kVec threads; VEC = 1: a multiple of t. (A problem's vectors hold Np t >= N t
+// values from a multiple of 16 bytes, so a last float4 that crosses N t stays inside them.)
+template <int VEC, int CL>
+__global__ void __launch_bounds__(kVec) batch_step_kernel(BatchArgs a) {
+    __shared__ float2 red[kMaxBatchT * 32 > kVec ? kMaxBatchT * 32 : kVec];
+    __shared__ double sum1[kMaxBatchT], sum2[kMaxBatchT];
+    __shared__ float s_alpha[kMaxBatchT], s_beta[kMaxBatchT];
+    __shared__ int s_act[kMaxBatchT];
+    const int gi = blockIdx.x / CL, rank = blockIdx.x % CL;
+    if (blockIdx.x == 0 && threadIdx.x == 0) *a.item_counter = 0;
+    if (*a.done || a.gp_done[gi]) return;  // the same for the whole cluster: its rank 0 sets gp_done after the last barrier
+    const BatchGp g = a.gps[gi];
+    const int tid = threadIdx.x, t = a.t, k = gi * t + (tid < t ? tid : 0);
+    const int active = a.active[k], iters = a.iters[k];
+    const double rr0 = a.rr[k];
+    const int64_t total = g.N * t, base = g.vec_off * t;
+    float *x = a.x + base, *r = a.r + base, *p = a.p + base, *kp = a.kp + base;
+    const float *part = a.part + g.part_off;
+    const int64_t stride = g.Np * t;
+    const int64_t e0 = ((int64_t)rank * blockDim.x + tid) * VEC, step = (int64_t)CL * blockDim.x * VEC;
+
+    float hi[VEC], lo[VEC];
+    auto clear = [&]() {
+#pragma unroll
+        for (int q = 0; q < VEC; ++q) hi[q] = lo[q] = 0.0f;
+    };
+    clear();
+    for (int64_t e = e0; e < total; e += step) {
+        float pv[VEC], kv[VEC];
+        load_vec<VEC>(p + e, pv);
+        if (g.splits > 1) {
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) kv[q] = 0.0f;
+#pragma unroll 8
+            for (int s = 0; s < g.splits; ++s) {
+                float w[VEC];
+                load_vec<VEC>(part + s * stride + e, w);
+#pragma unroll
+                for (int q = 0; q < VEC; ++q) kv[q] += w[q];
+            }
+#pragma unroll
+            for (int q = 0; q < VEC; ++q) kv[q] = fmaf(g.noise, pv[q], kv[q]);
+            store_vec<VEC>(kp + e, kv);
         } else {
-            alpha = a.rr[k] / pkp;
+            load_vec<VEC>(kp + e, kv);
         }
+#pragma unroll
+        for (int q = 0; q < VEC; ++q)
+            if (VEC == 1 || e + q < total) acc_prod2(hi[q], lo[q], pv[q], kv[q]);
     }
-    a.alpha[k] = alpha;
-}
-
-__global__ void bxr_kernel(BatchArgs a) {
-    __shared__ double red[kVec];
-    if (*a.done) return;
-    const BatchVecBlock vb = a.vblocks[blockIdx.x];
-    const BatchGp g = a.gps[vb.gp];
-    const int t = a.t;
-    const int c = threadIdx.x % t;
-    const float alpha = (float)a.alpha[vb.gp * t + c];
-    float hi = 0.0f, lo = 0.0f;
-    for (int64_t i = vb.r0 + threadIdx.x / t; i < vb.r1; i += blockDim.x / t) {
-        const int64_t e = (g.vec_off + i) * t + c;
-        float rv = a.r[e];
-        if (alpha != 0.0f) {
-            a.x[e] = fmaf(alpha, a.p[e], a.x[e]);
-            rv = fmaf(-alpha, a.kp[e], rv);
-            a.r[e] = rv;
+    block_pairs_reduce<VEC>(hi, lo, t, red, sum1);
+    const double pkp = batch_cluster_sum<CL>(sum1, t);
+    int failed = 0;
+    if (tid < t) {
+        double alpha = 0.0;
+        if (active) {
+            if (!isfinite(pkp)) failed = 1;
+            else if (!(pkp > 0.0)) failed = 2;
+            else alpha = rr0 / pkp;
         }
-        acc_prod2(hi, lo, rv, rv);
+        s_alpha[tid] = (float)alpha;
     }
-    seg_col_reduce((double)hi + (double)lo, t, red, a.partial + (int64_t)blockIdx.x * t);
-}
+    __syncthreads();
 
-__global__ void bbeta_kernel(BatchArgs a) {
-    if (*a.done) return;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= a.n_gp * a.t) return;
-    const int gi = k / a.t, c = k % a.t;
-    double beta = 0.0;
-    if (a.active[k]) {
-        const BatchGp g = a.gps[gi];
-        double rr = 0.0;
-        for (int b = g.blk0; b < g.blk1; ++b) rr += a.partial[(int64_t)b * a.t + c];
-        beta = rr / a.rr[k];
-        a.rr[k] = rr;
-        a.iters[k] += 1;
-        if (!(sqrt(rr) > a.st->tol * sqrt(a.bnorm2[k]))) a.active[k] = 0;
+    float al[VEC];
+    clear();
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) al[q] = s_alpha[col_of<VEC>(tid, q, t)];
+    for (int64_t e = e0; e < total; e += step) {
+        float xv[VEC], rv[VEC], pv[VEC], kv[VEC];
+        load_vec<VEC>(x + e, xv);
+        load_vec<VEC>(r + e, rv);
+        load_vec<VEC>(p + e, pv);
+        load_vec<VEC>(kp + e, kv);
+#pragma unroll
+        for (int q = 0; q < VEC; ++q) {
+            if (al[q] != 0.0f) {
+                xv[q] = fmaf(al[q], pv[q], xv[q]);
+                rv[q] = fmaf(-al[q], kv[q], rv[q]);
+            }
+            if (VEC == 1 || e + q < total) acc_prod2(hi[q], lo[q], rv[q], rv[q]);
+        }
+        store_vec<VEC>(x + e, xv);
+        store_vec<VEC>(r + e, rv);
     }
-    a.beta[k] = beta;
-}
+    block_pairs_reduce<VEC>(hi, lo, t, red, sum2);
+    const double rr = batch_cluster_sum<CL>(sum2, t);
+    int act = 0;
+    if (tid < t) {
+        double beta = 0.0;
+        if (active && !failed) {
+            beta = rr / rr0;
+            const double root = a.st->tol * sqrt(a.bnorm2[k]);
+            act = rr > root * root;
+        }
+        s_beta[tid] = (float)beta;
+        s_act[tid] = act;
+    }
+    __syncthreads();
 
-__global__ void bp_kernel(BatchArgs a) {
-    if (*a.done) return;
-    const BatchVecBlock vb = a.vblocks[blockIdx.x];
-    const BatchGp g = a.gps[vb.gp];
-    const int t = a.t;
-    const int c = threadIdx.x % t;
-    if (!a.active[vb.gp * t + c]) return;
-    const float beta = (float)a.beta[vb.gp * t + c];
-    for (int64_t i = vb.r0 + threadIdx.x / t; i < vb.r1; i += blockDim.x / t) {
-        const int64_t e = (g.vec_off + i) * t + c;
-        a.p[e] = fmaf(beta, a.p[e], a.r[e]);
+    float be[VEC];
+    int ac[VEC];
+#pragma unroll
+    for (int q = 0; q < VEC; ++q) {
+        be[q] = s_beta[col_of<VEC>(tid, q, t)];
+        ac[q] = s_act[col_of<VEC>(tid, q, t)];
+    }
+    for (int64_t e = e0; e < total; e += step) {
+        float pv[VEC], rv[VEC];
+        load_vec<VEC>(p + e, pv);
+        load_vec<VEC>(r + e, rv);
+#pragma unroll
+        for (int q = 0; q < VEC; ++q)
+            if (ac[q]) pv[q] = fmaf(be[q], pv[q], rv[q]);
+        store_vec<VEC>(p + e, pv);
+    }
+    // the state, by rank 0 once every CTA has read the old one and nobody reads this CTA's sums any more
+    if constexpr (CL == 1) __syncthreads();
+    else cooperative_groups::this_cluster().sync();
+    if (rank == 0) {
+        int stop = 0;
+        if (tid < t && active) {
+            if (failed) {
+                atomicOr(&a.st->status, failed);
+            } else {
+                a.rr[k] = rr;
+                a.iters[k] = iters + 1;
+            }
+            a.active[k] = act;
+            stop = iters + 1 >= a.st->max_iter;
+        }
+        stop = __syncthreads_or(stop);
+        const int any = __syncthreads_or(act);
+        if (tid == 0 && (stop || !any)) {
+            a.gp_done[gi] = 1;
+            atomicAdd(a.n_done, 1);
+        }
     }
 }
 
@@ -291,7 +360,7 @@ __global__ void bcopy_out_kernel(BatchArgs a) {
 
 __global__ void batch_loop_condition_kernel(cudaGraphConditionalHandle h, BatchArgs a) {
     a.st->loop_chunks += 1;
-    const bool more = !*a.done && a.st->loop_chunks < a.st->max_chunks;
+    const bool more = !*a.done && *a.n_done < a.n_gp && a.st->loop_chunks < a.st->max_chunks;
     cudaGraphSetConditional(h, more ? 1u : 0u);
 }
 
@@ -305,13 +374,30 @@ cudaError_t launch_batch_init(const BatchArgs &a, double tol, int max_iter, cuda
     binit_kernel<<<a.n_vblocks, vec_threads(a.t), 0, st>>>(a);
     const int n = a.n_gp * a.t;
     bscal_init_kernel<<<(n + 255) / 256, 256, 0, st>>>(a, tol, max_iter);
-    bdone_kernel<<<1, 256, 0, st>>>(a, 1);
+    bdone_kernel<<<1, 256, 0, st>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_batch_product(const BatchArgs &a, int num_sms, cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(a.item_counter, 0, sizeof(int), st);
-    if (e != cudaSuccess) return e;
+namespace {
+
+template <int VEC, int CL> cudaError_t launch_step(const BatchArgs &a, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(a.n_gp * CL), 1, 1);
+    cfg.blockDim = dim3(VEC == 4 ? kVec : vec_threads(a.t), 1, 1);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CL;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = CL > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, batch_step_kernel<VEC, CL>, a);
+}
+
+}  // namespace
+
+cudaError_t launch_batch_iteration(const BatchArgs &a, int num_sms, cudaStream_t st) {
     const int grid = std::max(1, std::min(a.n_items, num_sms * 6));
     switch (a.tt) {
         case 1: batch_mv_kernel<1><<<grid, BatchTile<1>::kThreads, 0, st>>>(a); break;
@@ -321,23 +407,15 @@ cudaError_t launch_batch_product(const BatchArgs &a, int num_sms, cudaStream_t s
         case 16: batch_mv_kernel<16><<<grid, BatchTile<16>::kThreads, 0, st>>>(a); break;
         default: return cudaErrorInvalidValue;
     }
-    bsplit_reduce_kernel<<<a.n_vblocks, vec_threads(a.t), 0, st>>>(a);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_batch_iteration(const BatchArgs &a, int num_sms, cudaStream_t st) {
-    cudaError_t e = launch_batch_product(a, num_sms, st);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int n = a.n_gp * a.t;
-    const int sb = (n + 255) / 256;
-    const int vt = vec_threads(a.t);
-    bpkp_kernel<<<a.n_vblocks, vt, 0, st>>>(a);
-    balpha_kernel<<<sb, 256, 0, st>>>(a);
-    bxr_kernel<<<a.n_vblocks, vt, 0, st>>>(a);
-    bbeta_kernel<<<sb, 256, 0, st>>>(a);
-    bdone_kernel<<<1, 256, 0, st>>>(a, 0);
-    bp_kernel<<<a.n_vblocks, vt, 0, st>>>(a);
-    return cudaGetLastError();
+    // One CTA per problem where its vectors are at most two loads per thread, or up to four when there is a problem for
+    // every SM anyway; else a cluster of 8. Solve of 64 problems with N = 200, t = 8: one CTA 2237 us, cluster 2418;
+    // 200 with N = 500, t = 8: 7239 and 8621; one with N = 1000, t = 8: 3277 and 2467.
+    const bool pow2 = (a.t & (a.t - 1)) == 0;
+    if (a.max_elems <= 8 * kVec || (a.max_elems <= 16 * kVec && a.n_gp >= num_sms))
+        return pow2 ? launch_step<4, 1>(a, st) : launch_step<1, 1>(a, st);
+    return pow2 ? launch_step<4, 8>(a, st) : launch_step<1, 8>(a, st);
 }
 
 cudaError_t launch_batch_loop_condition(cudaGraphConditionalHandle h, const BatchArgs &a, cudaStream_t st) {

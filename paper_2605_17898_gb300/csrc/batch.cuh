@@ -47,19 +47,19 @@ struct BatchArgs {
     float *x, *r, *p, *kp;
     float *part;                         // column-split partial sums of the product
     double *partial;                     // [n_vblocks, t]
-    double *rr, *bnorm2, *alpha, *beta;  // [n_gp * t]
+    double *rr, *bnorm2;                 // [n_gp * t]
     int *active, *iters;                 // [n_gp * t]
     int *gp_done;                        // [n_gp]
-    int *done;
+    int *done;    // 1: the call ends (non-finite right-hand side)
+    int *n_done;  // problems with gp_done set
+    int64_t max_elems;  // largest N t of the problems
     int *item_counter;
     BatchState *st;
 };
 
 int batch_item_rows();
 cudaError_t launch_batch_init(const BatchArgs &a, double tol, int max_iter, cudaStream_t st);
-// The product alone (K_y p of every active problem, column-split partial sums reduced): the part of an
-// iteration that the split choice changes, timed by the split tuner.
-cudaError_t launch_batch_product(const BatchArgs &a, int num_sms, cudaStream_t st);
+// One CG iteration of every problem that is not done: the product and the step.
 cudaError_t launch_batch_iteration(const BatchArgs &a, int num_sms, cudaStream_t st);
 cudaError_t launch_batch_copy_out(const BatchArgs &a, cudaStream_t st);
 // Body tail of the device-side batch loop: condition = not done and under the chunk cap.

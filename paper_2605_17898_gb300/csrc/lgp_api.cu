@@ -1069,7 +1069,7 @@ lgp_status upload_batch_plan(lgp_ctx *ctx, BatchPlan &P, int t, cudaStream_t st,
     const size_t o_gps = off; off = al(off + P.gps.size() * sizeof(BatchGp));
     const size_t o_items = off; off = al(off + P.items.size() * sizeof(BatchItem));
     const size_t o_vb = off; off = al(off + P.vblocks.size() * sizeof(BatchVecBlock));
-    const size_t o_rr = off; off = al(off + 4 * (size_t)ng_t * sizeof(double));
+    const size_t o_rr = off; off = al(off + 2 * (size_t)ng_t * sizeof(double));
     const size_t o_act = off; off = al(off + 2 * (size_t)ng_t * sizeof(int));
     const size_t o_gpd = off; off = al(off + (size_t)n_b * sizeof(int));
     const size_t o_misc = off; off = al(off + 256);
@@ -1102,14 +1102,15 @@ lgp_status upload_batch_plan(lgp_ctx *ctx, BatchPlan &P, int t, cudaStream_t st,
     double *dd = (double *)(meta + o_rr);
     A.rr = dd;
     A.bnorm2 = dd + ng_t;
-    A.alpha = dd + 2 * ng_t;
-    A.beta = dd + 3 * ng_t;
     int *ii = (int *)(meta + o_act);
     A.active = ii;
     A.iters = ii + ng_t;
     A.gp_done = (int *)(meta + o_gpd);
     A.done = (int *)(meta + o_misc);
     A.item_counter = (int *)(meta + o_misc + 4);
+    A.n_done = (int *)(meta + o_misc + 8);
+    A.max_elems = 0;
+    for (const BatchGp &G : P.gps) A.max_elems = std::max(A.max_elems, G.N * t);
     A.st = (BatchState *)(meta + o_misc + 64);
     LGP_CUDA(cudaMemcpyAsync(meta + o_gps, P.gps.data(), P.gps.size() * sizeof(BatchGp), cudaMemcpyHostToDevice, st));
     LGP_CUDA(cudaMemcpyAsync(meta + o_items, P.items.data(), P.items.size() * sizeof(BatchItem),
@@ -1128,8 +1129,8 @@ lgp_status upload_batch_plan(lgp_ctx *ctx, BatchPlan &P, int t, cudaStream_t st,
 // caller's own X and right-hand sides: the problem alone in the work list (the case its split count
 // decides: its last iterations, with no other problem left) with the fixed rule's count and with a
 // quarter, half, double and four times that many (at least one, at most one 64-column tile per split).
-// Each candidate: one untimed and three timed products (the persistent launch and its split
-// reduction, CUDA events). Cached in the context and, with LGP_AUTOTUNE_CACHE, in the product-choice
+// Each candidate: one untimed and three timed iterations (the persistent launch and the step, which reads the
+// split sums; CUDA events). Cached in the context and, with LGP_AUTOTUNE_CACHE, in the product-choice
 // file (key suffix |split); LGP_AUTOTUNE=0 keeps the rule.
 lgp_status batch_split_choice(lgp_ctx *ctx, const KernelParams &kp, const lgp_hyper *h, const float *X,
                               const float *B, int64_t N, int t, int64_t *S_out) {
@@ -1172,14 +1173,14 @@ lgp_status batch_split_choice(lgp_ctx *ctx, const KernelParams &kp, const lgp_hy
         plan_add_problem(P, N, kp, X, B, nullptr, t, cands[k]);
         BatchArgs A;
         if ((s = upload_batch_plan(ctx, P, t, st, &A)) != LGP_OK) break;
-        if (launch_batch_init(A, 0.0, 1, st) != cudaSuccess) {
+        if (launch_batch_init(A, 0.0, 1 << 30, st) != cudaSuccess) {  // tol 0: no repetition finds the problem done
             s = fail(ctx, LGP_ERR_CUDA, "batch split tuning: init failed");
             break;
         }
         float ms = 0.0f;
         for (int rep = 0; rep < 4 && s == LGP_OK; ++rep) {
             cudaEventRecord(e0, st);
-            const cudaError_t ce = launch_batch_product(A, ctx->num_sms, st);
+            const cudaError_t ce = launch_batch_iteration(A, ctx->num_sms, st);
             cudaEventRecord(e1, st);
             float m = 0.0f;
             if (ce != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
