@@ -72,6 +72,8 @@ __global__ void __launch_bounds__(BatchTile<TT>::kThreads) batch_mv_kernel(Batch
     __shared__ __align__(16) float vs[kSimtBN * TT];
     __shared__ float tot[BatchTile<TT>::kTotFloats];
     __shared__ int item_s;
+    chain_wait();
+    chain_next();
     if (*a.done || *a.n_done >= a.n_gp) return;
     while (true) {
         __syncthreads();
@@ -217,6 +219,8 @@ __global__ void __launch_bounds__(kVec) batch_step_kernel(BatchArgs a) {
     __shared__ double sum1[kMaxBatchT], sum2[kMaxBatchT];
     __shared__ float s_alpha[kMaxBatchT], s_beta[kMaxBatchT];
     __shared__ int s_act[kMaxBatchT];
+    chain_wait();
+    chain_next();
     const int gi = blockIdx.x / CL, rank = blockIdx.x % CL;
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.item_counter = 0;
     if (*a.done || a.gp_done[gi]) return;  // the same for the whole cluster: its rank 0 sets gp_done after the last barrier
@@ -385,13 +389,15 @@ template <int VEC, int CL> cudaError_t launch_step(const BatchArgs &a, cudaStrea
     cfg.gridDim = dim3((unsigned)(a.n_gp * CL), 1, 1);
     cfg.blockDim = dim3(VEC == 4 ? kVec : vec_threads(a.t), 1, 1);
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CL;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = CL;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = CL > 1 ? 1 : 0;
+    cfg.numAttrs = CL > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, batch_step_kernel<VEC, CL>, a);
 }
 
@@ -399,15 +405,15 @@ template <int VEC, int CL> cudaError_t launch_step(const BatchArgs &a, cudaStrea
 
 cudaError_t launch_batch_iteration(const BatchArgs &a, int num_sms, cudaStream_t st) {
     const int grid = std::max(1, std::min(a.n_items, num_sms * 6));
+    cudaError_t e;
     switch (a.tt) {
-        case 1: batch_mv_kernel<1><<<grid, BatchTile<1>::kThreads, 0, st>>>(a); break;
-        case 2: batch_mv_kernel<2><<<grid, BatchTile<2>::kThreads, 0, st>>>(a); break;
-        case 4: batch_mv_kernel<4><<<grid, BatchTile<4>::kThreads, 0, st>>>(a); break;
-        case 8: batch_mv_kernel<8><<<grid, BatchTile<8>::kThreads, 0, st>>>(a); break;
-        case 16: batch_mv_kernel<16><<<grid, BatchTile<16>::kThreads, 0, st>>>(a); break;
+        case 1: e = launch_chained(batch_mv_kernel<1>, grid, BatchTile<1>::kThreads, 0, st, a); break;
+        case 2: e = launch_chained(batch_mv_kernel<2>, grid, BatchTile<2>::kThreads, 0, st, a); break;
+        case 4: e = launch_chained(batch_mv_kernel<4>, grid, BatchTile<4>::kThreads, 0, st, a); break;
+        case 8: e = launch_chained(batch_mv_kernel<8>, grid, BatchTile<8>::kThreads, 0, st, a); break;
+        case 16: e = launch_chained(batch_mv_kernel<16>, grid, BatchTile<16>::kThreads, 0, st, a); break;
         default: return cudaErrorInvalidValue;
     }
-    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     // One CTA per problem where its vectors are at most two loads per thread, or up to four when there is a problem for
     // every SM anyway; else a cluster of 8. Solve of 64 problems with N = 200, t = 8: one CTA 2237 us, cluster 2418;

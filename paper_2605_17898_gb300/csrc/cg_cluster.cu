@@ -80,6 +80,8 @@ __global__ void __launch_bounds__(kClThreads, 1) cg_cluster_kernel(const Cluster
     __shared__ int s_exp[kMaxT], s_act[kMaxT];
     __shared__ __align__(16) float tile[4 * kClThreads];
     CgState *st = a.st;
+    chain_wait();
+    chain_next();
     if (st->done) return;
     const int tid = threadIdx.x, t = a.t;
     const int rank = CL == 1 ? 0 : (int)cg::this_cluster().block_rank();
@@ -309,13 +311,15 @@ cudaError_t launch_cluster(const ClusterArgs &a, cudaStream_t st) {
     cfg.gridDim = dim3(CL, 1, 1);
     cfg.blockDim = dim3(kClThreads, 1, 1);
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CL;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = CL;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = CL > 1 ? 1 : 0;
+    cfg.numAttrs = CL > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, cg_cluster_kernel<CL>, a);
 }
 

@@ -176,6 +176,32 @@ inline double prescale_of(int kind) {
     return 0.0;
 }
 
+// ---------------------------------------------------------------- chained launches
+
+// A kernel whose first statement is chain_wait() may be launched with launch_chained: its CTAs are then placed while the
+// previous kernel of the stream still runs its last ones, and wait here until that kernel has finished and its writes are
+// visible. chain_wait comes before any access to memory and before any return (a kernel that ended without it could
+// finish before its predecessor); its chain_next, from which on the successor may be placed, comes with it.
+// Product call with its eight small kernels, N = 20000, D = 8, t = 16: 168 -> 154 us; solve of N = 1024, t = 1 (two kernels an
+// iteration): 945 -> 866 us.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... Params, class... Args>
+cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
 // ---------------------------------------------------------------- CG state on the device
 
 // Per-column CG scalars (float64) and flags, plus the Lanczos history.

@@ -80,6 +80,8 @@ SymGrid sym_grid(int64_t N, int64_t Np, int t, int num_sms) {
 __global__ void reduce_split_kernel(const float *__restrict__ partial, int S, int64_t Np, int64_t N, int t,
                                     const float *__restrict__ V, int64_t ldv, float *__restrict__ out, int64_t ldo,
                                     float noise, int cross, const int *skip) {
+    chain_wait();
+    chain_next();
     if (skip && *skip) return;
     const int64_t total = N * t;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
@@ -98,6 +100,8 @@ __global__ void __launch_bounds__(256) reduce_many_kernel(const float *__restric
                                                           int t, const float *__restrict__ V, int64_t ldv,
                                                           float *__restrict__ out, int64_t ldo, float noise, int cross,
                                                           const int *skip) {
+    chain_wait();
+    chain_next();
     if (skip && *skip) return;
     const int lane = threadIdx.x & 31, q = lane >> 2;
     const int64_t total = N * t;
@@ -185,12 +189,10 @@ static cudaError_t finish_splits(const MvLaunch &m, int S, int64_t Nr, int64_t N
         return cudaSuccess;
     }
     if (S >= 8)
-        reduce_many_kernel<<<(unsigned)((Nr * m.t + 127) / 128), 256, 0, st>>>(m.partial, S, Npr, Nr, m.t, m.V, m.ldv, m.out,
-                                                                               m.ldo, m.kp->noise, cross, m.skip);
-    else
-        reduce_split_kernel<<<grid_for(Nr * m.t), 256, 0, st>>>(m.partial, S, Npr, Nr, m.t, m.V, m.ldv, m.out, m.ldo,
-                                                                m.kp->noise, cross, m.skip);
-    return cudaGetLastError();
+        return launch_chained(reduce_many_kernel, (unsigned)((Nr * m.t + 127) / 128), 256, 0, st, m.partial, S, Npr, Nr, m.t,
+                              m.V, m.ldv, m.out, m.ldo, m.kp->noise, cross, m.skip);
+    return launch_chained(reduce_split_kernel, grid_for(Nr * m.t), 256, 0, st, m.partial, S, Npr, Nr, m.t, m.V, m.ldv, m.out,
+                          m.ldo, m.kp->noise, cross, m.skip);
 }
 
 cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st) {

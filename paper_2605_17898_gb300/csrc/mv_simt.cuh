@@ -206,6 +206,8 @@ __global__ void __launch_bounds__(RowShape<TT>::kThreads) mv_simt_kernel(SimtArg
     __shared__ __align__(16) float xs[kSimtBN * D];
     __shared__ __align__(16) float vs[kSimtBN * TT];
     __shared__ float tot[S::kTotFloats];
+    chain_wait();
+    chain_next();
     if (a.skip && *a.skip) return;
     const int64_t row0 = (int64_t)blockIdx.x * S::kRows;
     const int c0 = blockIdx.z * TT;
@@ -458,14 +460,13 @@ cudaError_t adjoint_dispatch_m32(int D, int TT, dim3 grid, const AdjArgs &a, cud
     namespace lgp {                                                                                            \
     template <int D>                                                                                           \
     static cudaError_t mv_simt_d_##SUFFIX(int TT, dim3 grid, const SimtArgs &a, cudaStream_t st) {             \
-        if (TT == 1) mv_simt_kernel<KIND, D, 1><<<grid, RowShape<1>::kThreads, 0, st>>>(a);                     \
-        else if (TT == 2) mv_simt_kernel<KIND, D, 2><<<grid, RowShape<2>::kThreads, 0, st>>>(a);                \
-        else if (TT == 4) mv_simt_kernel<KIND, D, 4><<<grid, RowShape<4>::kThreads, 0, st>>>(a);                \
-        else if (TT == 8) mv_simt_kernel<KIND, D, 8><<<grid, RowShape<8>::kThreads, 0, st>>>(a);                \
-        else if (TT == 16) mv_simt_kernel<KIND, D, 16><<<grid, RowShape<16>::kThreads, 0, st>>>(a);             \
-        else if (TT == 32) mv_simt_kernel<KIND, D, 32><<<grid, RowShape<32>::kThreads, 0, st>>>(a);             \
-        else return cudaErrorInvalidValue;                                                                     \
-        return cudaGetLastError();                                                                             \
+        if (TT == 1) return launch_chained(mv_simt_kernel<KIND, D, 1>, grid, RowShape<1>::kThreads, 0, st, a); \
+        if (TT == 2) return launch_chained(mv_simt_kernel<KIND, D, 2>, grid, RowShape<2>::kThreads, 0, st, a); \
+        if (TT == 4) return launch_chained(mv_simt_kernel<KIND, D, 4>, grid, RowShape<4>::kThreads, 0, st, a); \
+        if (TT == 8) return launch_chained(mv_simt_kernel<KIND, D, 8>, grid, RowShape<8>::kThreads, 0, st, a); \
+        if (TT == 16) return launch_chained(mv_simt_kernel<KIND, D, 16>, grid, RowShape<16>::kThreads, 0, st, a);\
+        if (TT == 32) return launch_chained(mv_simt_kernel<KIND, D, 32>, grid, RowShape<32>::kThreads, 0, st, a);\
+        return cudaErrorInvalidValue;                                                                          \
     }                                                                                                          \
     cudaError_t mv_simt_dispatch_##SUFFIX(int D, int TT, dim3 grid, const SimtArgs &a, cudaStream_t st) {      \
         switch (D) {                                                                                           \

@@ -94,7 +94,6 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
     using S = SymShape<D, TT>;
     constexpr int R = S::R, C = S::C, RB = S::RB, NV = C * TT;
     extern __shared__ float4 sym_smem[];
-    if (a.skip && *a.skip) return;
     const int E = a.E;
     float *xs = reinterpret_cast<float *>(sym_smem);        // [D][E]
     float *vs = xs + D * E;                                 // [E][TT]
@@ -117,6 +116,9 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rl = lane & 7, cl = lane >> 3;
 
+    chain_wait();
+    chain_next();
+    if (a.skip && *a.skip) return;
     // column side: -x_j and V_j; column sums zero
     for (int e = tid; e < E * (DP / 4); e += kSymThreads) {
         const int j = e / (DP / 4), q = e - j * (DP / 4);
@@ -275,8 +277,7 @@ cudaError_t launch_mv_sym_inst(const SymArgs &a, cudaStream_t st) {
             configured = true;
         }
     }
-    mv_sym_kernel<KIND, D, TT><<<a.G * (a.G + 1) / 2, kSymThreads, bytes, st>>>(a);
-    return cudaGetLastError();
+    return launch_chained(mv_sym_kernel<KIND, D, TT>, dim3((unsigned)(a.G * (a.G + 1) / 2)), kSymThreads, bytes, st, a);
 }
 
 template <int KIND, int TT>

@@ -19,6 +19,8 @@ using tc::kBM;
 // reduces its columns in shared memory and adds one atomicMax per column.
 __global__ void __launch_bounds__(256) col_absmax_kernel(const float *__restrict__ V, int64_t ldv, int64_t N, int T,
                                                          unsigned int *__restrict__ vmax, const int *skip) {
+    chain_wait();
+    chain_next();
     if (skip && *skip) return;
     __shared__ unsigned int red[256];
     const int c = threadIdx.x % T;
@@ -46,6 +48,8 @@ __global__ void split_v_kernel(const float *__restrict__ V, int64_t ldv, int64_t
                                uint16_t *__restrict__ vs,
                                const unsigned int *__restrict__ vmax, float *__restrict__ col_scale, float s2,
                                float *__restrict__ out_init, int64_t ldo, float noise, const int *skip) {
+    chain_wait();
+    chain_next();
     if (skip && *skip) return;
     const int64_t total = (Np / 8) * T;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
@@ -76,6 +80,8 @@ __global__ void split_v_kernel(const float *__restrict__ V, int64_t ldv, int64_t
 template <int T, int FMT>
 __global__ void __launch_bounds__(256) p_split_kernel(float *__restrict__ p, const float *__restrict__ r, int64_t N,
                                                       CgState *st, CgSplit sp) {
+    chain_wait();
+    chain_next();
     if (st->done) return;
     __shared__ unsigned int red[256];
     const int c = threadIdx.x % T;  // the grid stride is a multiple of T
@@ -125,6 +131,8 @@ __global__ void __launch_bounds__(256) p_split_kernel(float *__restrict__ p, con
 // XsT[d, j] = Xs[j, d]: the transposed prescaled X the tensor-core product stages by TMA.
 __global__ void transpose_x_kernel(const float *__restrict__ Xs, int64_t Np, int dpad, float *__restrict__ XsT,
                                    const int *skip) {
+    chain_wait();
+    chain_next();
     if (skip && *skip) return;
     const int64_t total = Np * dpad;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
@@ -147,6 +155,8 @@ __device__ __forceinline__ float float_of_ord(unsigned int o) {
 // words[8 + d] = ord(max -x_d); the words start at zero (below every ordered float).
 __global__ void dot_bbox_kernel(const float *__restrict__ Xs, int64_t N, int dpad, unsigned int *__restrict__ words,
                                 const int *skip) {
+    chain_wait();
+    chain_next();
     if (skip && *skip) return;
     unsigned int hi[8], lo[8];
 #pragma unroll
@@ -193,6 +203,8 @@ template <int DP>
 __global__ void dot_operands_kernel(const float *__restrict__ Xs, int64_t N, int64_t Np,
                                     unsigned int *__restrict__ words, float *__restrict__ arow,
                                     uint4 *__restrict__ ua, uint4 *__restrict__ ub, const int *skip) {
+    chain_wait();
+    chain_next();
     if (skip && *skip) return;
     constexpr int KG = 32;
     static_assert(3 * DP + 6 <= KG, "Gram operand row too short");
@@ -258,6 +270,8 @@ __global__ void dot_operands_kernel(const float *__restrict__ Xs, int64_t N, int
 __global__ void tc_reduce_kernel(const float *__restrict__ partial, int S, int64_t Np, int64_t N, int t,
                                  const float *__restrict__ V, int64_t ldv, float *__restrict__ out, int64_t ldo,
                                  float noise, const int *skip) {
+    chain_wait();
+    chain_next();
     if (skip && *skip) return;
     const int64_t total = N * t;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
@@ -463,20 +477,18 @@ cudaError_t launch_dot_operands(const KernelParams &kp, const float *Xs, int64_t
     cudaError_t e = cudaMemsetAsync(words, 0, 32 * sizeof(unsigned int), st);
     if (e != cudaSuccess) return e;
     const int bb = (int)std::min<int64_t>((N + 255) / 256, 1024);
-    dot_bbox_kernel<<<bb, 256, 0, st>>>(Xs, N, kp.dpad, words, skip);
+    launch_chained(dot_bbox_kernel, bb, 256, 0, st, Xs, N, kp.dpad, words, skip);
     const int ob = (int)std::min<int64_t>((Np + 255) / 256, 4096);
-    if (kp.dpad <= 4)
-        dot_operands_kernel<4><<<ob, 256, 0, st>>>(Xs, N, Np, words, arow, (uint4 *)ua, (uint4 *)ub, skip);
-    else
-        dot_operands_kernel<8><<<ob, 256, 0, st>>>(Xs, N, Np, words, arow, (uint4 *)ua, (uint4 *)ub, skip);
+    launch_chained(kp.dpad <= 4 ? dot_operands_kernel<4> : dot_operands_kernel<8>, ob, 256, 0, st, Xs, N, Np, words, arow,
+                   (uint4 *)ua, (uint4 *)ub, skip);
     return cudaGetLastError();
 }
 
 void launch_transpose_x(const KernelParams &kp, const float *Xs, int64_t Np, void *vsplit, int t, const int *skip,
                         cudaStream_t st) {
     float *XsT = (float *)((uint8_t *)vsplit + 2 * Np * t * 2 + 2 * 64 * 4);
-    transpose_x_kernel<<<(int)std::min<int64_t>((Np * kp.dpad + 255) / 256, 4096), 256, 0, st>>>(Xs, Np, kp.dpad,
-                                                                                              XsT, skip);
+    launch_chained(transpose_x_kernel, (int)std::min<int64_t>((Np * kp.dpad + 255) / 256, 4096), 256, 0, st, Xs, Np, kp.dpad,
+                   XsT, skip);
 }
 
 }  // namespace
@@ -509,11 +521,12 @@ cudaError_t launch_v_split(const KernelParams &kp, int64_t N, int64_t Np, const 
         const cudaError_t e = cudaMemsetAsync(sp.vmax, 0, 64 * sizeof(unsigned int), st);
         if (e != cudaSuccess) return e;
         const int mb = (int)std::max<int64_t>(1, std::min<int64_t>((N * t + 255) / 256, 4 * num_sms));
-        col_absmax_kernel<<<mb, (256 / t) * t, 0, st>>>(V, ldv, N, t, sp.vmax, skip);
+        launch_chained(col_absmax_kernel, mb, (256 / t) * t, 0, st, V, ldv, N, t, sp.vmax, skip);
     }
     auto split = t == 16 ? (fmt == kFmtF16 ? split_v_kernel<16, kFmtF16> : split_v_kernel<16, kFmtBF16>)
                          : (fmt == kFmtF16 ? split_v_kernel<32, kFmtF16> : split_v_kernel<32, kFmtBF16>);
-    split<<<blocks, 256, 0, st>>>(V, ldv, N, Np, sp.vs, sp.vmax, sp.col_scale, kp.s2, out_init, ldo, kp.noise, skip);
+    launch_chained(split, blocks, 256, 0, st, V, ldv, N, Np, sp.vs, sp.vmax, sp.col_scale, kp.s2, out_init, ldo, kp.noise,
+                   skip);
     return cudaGetLastError();
 }
 
@@ -521,7 +534,7 @@ void launch_p_split(const CgSplit &sp, float *p, const float *r, int64_t N, int 
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(((N + 7) / 8 * t + 255) / 256, 8192));
     auto k = t == 16 ? (sp.fmt == kFmtF16 ? p_split_kernel<16, kFmtF16> : p_split_kernel<16, kFmtBF16>)
                      : (sp.fmt == kFmtF16 ? p_split_kernel<32, kFmtF16> : p_split_kernel<32, kFmtBF16>);
-    k<<<blocks, 256, 0, st>>>(p, r, N, state, sp);
+    launch_chained(k, blocks, 256, 0, st, p, r, N, state, sp);
 }
 
 cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, const float *V, int64_t ldv,
@@ -658,7 +671,7 @@ cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int
         return cudaSuccess;
     }
     const int rblocks = (int)std::min<int64_t>((N * t + 255) / 256, 4096);
-    tc_reduce_kernel<<<rblocks, 256, 0, st>>>(partial, g.S, Np, N, t, V, ldv, out, ldo, kp.noise, skip);
+    launch_chained(tc_reduce_kernel, rblocks, 256, 0, st, partial, g.S, Np, N, t, V, ldv, out, ldo, kp.noise, skip);
     return cudaGetLastError();
 }
 

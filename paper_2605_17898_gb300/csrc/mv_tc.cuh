@@ -199,6 +199,11 @@ static __device__ __forceinline__ bool mbar_wait_all_warp(const uint32_t (&bar)[
     }
 }
 
+// Gives back the tensor memory of the allocating warp (converged).
+template <int COLS> __device__ __forceinline__ void tmem_free(uint32_t tmem) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(COLS) : "memory");
+}
+
 // True in one lane of a converged warp, the same lane at every call.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;
@@ -403,8 +408,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     constexpr int kStages = L::kStages;
     constexpr int kTmemCols = TmemCols<ATMEM>::value;
     extern __shared__ uint8_t smem_raw[];
-    if (a.skip && *a.skip) return;
-
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L::kBar);
     // bars: full[4], ready[4], empty[4], acc_full[2], acc_empty[2], fin
@@ -451,6 +454,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_acc = *tmem_slot;
+    // barriers and tensor memory are ready; from here on the inputs are needed
+    chain_wait();
+    chain_next();
+    if (a.skip && *a.skip) {
+        if (warp == kMmaWarp) tmem_free<kTmemCols>(tmem_acc);
+        return;
+    }
 
     if (warp == kProducerWarp) {
         // ------------------------------------------------------------ producer (TMA)
@@ -727,8 +737,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     if (warp == kMmaWarp) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_acc), "n"(kTmemCols)
-                     : "memory");
+        tmem_free<kTmemCols>(tmem_acc);
     }
 }
 

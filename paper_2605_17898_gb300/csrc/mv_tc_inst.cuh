@@ -18,8 +18,7 @@ cudaError_t launch_tc_inst(dim3 grid, const CUtensorMap &mx, const CUtensorMap &
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    mv_tc_kernel<KIND, D, T, FMT><<<grid, kThreads, bytes, st>>>(mx, mv, a);
-    return cudaGetLastError();
+    return launch_chained(mv_tc_kernel<KIND, D, T, FMT>, grid, kThreads, bytes, st, mx, mv, a);
 }
 
 template <int KIND, int T, int FMT>

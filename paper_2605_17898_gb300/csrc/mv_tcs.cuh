@@ -69,6 +69,7 @@ namespace lgp {
 namespace tcs {
 
 using tc::elect_one;
+using tc::tmem_free;
 using tc::fence_async_smem;
 using tc::kDrainBudget;
 using tc::kErrWaitAcc;
@@ -289,9 +290,6 @@ __global__ void __launch_bounds__(kTcsThreads, 1)
     constexpr int DP = D <= 4 ? 4 : 8;
     using L = TcsLayout<T, DP, DOT>;
     extern __shared__ uint8_t smem_raw[];
-    if (a.skip && *a.skip) return;
-    if (a.gate && (__uint_as_float(*a.gate) <= a.gate_lim) != DOT) return;
-
     uint8_t *smem = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + L::kBar);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + L::kBar + 384);
@@ -347,19 +345,27 @@ __global__ void __launch_bounds__(kTcsThreads, 1)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
     }
-    // the per-column epilogue factors (float16 halves), read by the drain from shared memory
-    float *col_scale = reinterpret_cast<float *>(smem + L::kBar + 512);
-    if (a.col_scale && threadIdx.x < T) col_scale[threadIdx.x] = a.col_scale[threadIdx.x];
     if (warp == kMmaWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
                      "n"(L::kTmemCols)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    // barriers and tensor memory are being set up; from here on the inputs are needed
+    chain_wait();
+    chain_next();
+    const bool idle = (a.skip && *a.skip) || (a.gate && (__uint_as_float(*a.gate) <= a.gate_lim) != DOT);
+    // the per-column epilogue factors (float16 halves), read by the drain from shared memory
+    float *col_scale = reinterpret_cast<float *>(smem + L::kBar + 512);
+    if (a.col_scale && threadIdx.x < T) col_scale[threadIdx.x] = a.col_scale[threadIdx.x];
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_acc = *tmem_slot;
+    if (idle) {
+        if (warp == kMmaWarp) tmem_free<L::kTmemCols>(tmem_acc);
+        return;
+    }
 
     Walk w;
     w.init(ord);
@@ -845,8 +851,7 @@ __global__ void __launch_bounds__(kTcsThreads, 1)
     __syncthreads();
     if (warp == kMmaWarp) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_acc), "n"(L::kTmemCols)
-                     : "memory");
+        tmem_free<L::kTmemCols>(tmem_acc);
     }
 }
 

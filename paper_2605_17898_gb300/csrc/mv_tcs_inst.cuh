@@ -20,8 +20,7 @@ cudaError_t launch_tcs_inst(dim3 grid, const CUtensorMap &mx, const CUtensorMap 
         if (e != cudaSuccess) return e;
         configured = true;
     }
-    mv_tcs_kernel<KIND, D, T, FMT, DOT, BANDED><<<grid, kTcsThreads, bytes, st>>>(mx, mv, mo, a);
-    return cudaGetLastError();
+    return launch_chained(mv_tcs_kernel<KIND, D, T, FMT, DOT, BANDED>, grid, kTcsThreads, bytes, st, mx, mv, mo, a);
 }
 
 // The dot-form instance: the banded tile order when the band is narrower than the triangle

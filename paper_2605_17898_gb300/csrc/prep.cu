@@ -12,6 +12,8 @@ struct ScaleArg {
 // Xs[i, d] = X[i, d] * scale[d] for i < N, d < D; zero in the padded rows and columns.
 __global__ void prep_x_kernel(const float *__restrict__ X, int64_t N, int D, int dpad, ScaleArg sc,
                               float *__restrict__ Xs, int64_t Np, int *err_flag) {
+    chain_wait();
+    chain_next();
     const int64_t total = Np * dpad;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = e / dpad;
@@ -75,7 +77,7 @@ void launch_prep_x(const float *X, int64_t N, int D, int dpad, const float *scal
                    int *err_flag, cudaStream_t st) {
     ScaleArg sc;
     for (int d = 0; d < kMaxD; ++d) sc.s[d] = d < D ? scale_host[d] : 0.0f;
-    prep_x_kernel<<<grid_for(Np * dpad, 256), 256, 0, st>>>(X, N, D, dpad, sc, Xs, Np, err_flag);
+    launch_chained(prep_x_kernel, grid_for(Np * dpad, 256), 256, 0, st, X, N, D, dpad, sc, Xs, Np, err_flag);
 }
 
 void launch_rademacher(uint64_t seed, int64_t N, int m, float *Z, int64_t ldz, int col0, cudaStream_t st) {

@@ -228,6 +228,8 @@ __global__ void __launch_bounds__(kStepThreads) cg_pkp_alpha_kernel(const float 
                                                                     CgState *st, double *__restrict__ partial,
                                                                     double *__restrict__ hist_alpha) {
     __shared__ float2 red[64 * 32];
+    chain_wait();
+    chain_next();
     if (st->done) return;
     const int64_t total = N * t;
     // LANES = 8: element thread u of the block's blockDim / 8 is lanes with (lane & 3) = u mod 4 of warp u / 4
@@ -357,6 +359,8 @@ __global__ void __launch_bounds__(kStepThreads) cg_xr_beta_kernel(float *__restr
                                                                   double *__restrict__ hist_beta, unsigned int *vbound) {
     __shared__ float2 red[64 * 32];
     __shared__ unsigned int rmax[kMaxT];
+    chain_wait();
+    chain_next();
     if (st->done) return;
     const int64_t total = N * t;
     float alpha[VEC], hi[VEC], lo[VEC], m[VEC];
@@ -412,6 +416,8 @@ __global__ void __launch_bounds__(1024) cg_beta_kernel(CgState *st, const double
                                                        const double *__restrict__ rz_partial, int G_rz, int t,
                                                        double *hist_beta) {
     __shared__ double srr[kMaxT], srz[kMaxT];
+    chain_wait();
+    chain_next();
     if (st->done) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     for (int c = warp; c < t; c += nw) {
@@ -430,6 +436,8 @@ __global__ void __launch_bounds__(1024) cg_beta_kernel(CgState *st, const double
 template <int VEC>
 __global__ void __launch_bounds__(kStepThreads) cg_p_kernel(float *__restrict__ p, const float *__restrict__ z, int64_t N,
                                                             int t, const CgState *st) {
+    chain_wait();
+    chain_next();
     if (st->done) return;
     const int64_t total = N * t;
     float beta[VEC];
@@ -754,27 +762,29 @@ void launch_step(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, 
     if (tail.part && tail.S >= 16 && VEC == 4) {
         const int64_t per = kStepThreads / 8 * VEC;  // elements of a block's round
         const int G8 = (int)std::min<int64_t>(kStepBlocks, (N * t + per - 1) / per);
-        cg_pkp_alpha_kernel<VEC, VEC == 4 ? 8 : 1><<<G8, bd, 0, st>>>(
-            b.p, b.Kp, tail.part, tail.S, tail.stride, tail.noise, N, t, b.state, b.partial, b.hist_alpha);
+        launch_chained(cg_pkp_alpha_kernel<VEC, VEC == 4 ? 8 : 1>, G8, bd, 0, st, b.p, b.Kp, tail.part, tail.S, tail.stride,
+                       tail.noise, N, t, b.state, b.partial, b.hist_alpha);
     } else if (tail.part) {
-        cg_pkp_alpha_kernel<VEC, 1><<<G, bd, 0, st>>>(b.p, b.Kp, tail.part, tail.S, tail.stride, tail.noise, N, t, b.state,
-                                                      b.partial, b.hist_alpha);
+        launch_chained(cg_pkp_alpha_kernel<VEC, 1>, G, bd, 0, st, b.p, b.Kp, tail.part, tail.S, tail.stride, tail.noise, N, t,
+                       b.state, b.partial, b.hist_alpha);
     } else {
-        cg_pkp_alpha_kernel<VEC, 0><<<G, bd, 0, st>>>(b.p, b.Kp, nullptr, 0, 0, 0.0f, N, t, b.state, b.partial,
-                                                      b.hist_alpha);
+        launch_chained(cg_pkp_alpha_kernel<VEC, 0>, G, bd, 0, st, b.p, b.Kp, nullptr, 0, 0, 0.0f, N, t, b.state, b.partial,
+                       b.hist_alpha);
     }
     if (b.pc.k > 0) {
         double *rz_partial = b.partial + (int64_t)b.G * t;
-        cg_xr_beta_kernel<VEC, false><<<G, bd, 0, st>>>(b.x, b.r, b.p, b.Kp, N, t, b.state, b.partial, b.hist_beta, nullptr);
+        launch_chained(cg_xr_beta_kernel<VEC, false>, G, bd, 0, st, b.x, b.r, b.p, b.Kp, N, t, b.state, b.partial, b.hist_beta,
+                       nullptr);
         launch_precond_apply(b.pc, b.r, t, b.z, t, nullptr, N, t, rz_partial, b.G, b.state, st);
-        cg_beta_kernel<<<1, 1024, 0, st>>>(b.state, b.partial, G, rz_partial, b.G, t, b.hist_beta);
+        launch_chained(cg_beta_kernel, 1, 1024, 0, st, b.state, b.partial, G, rz_partial, b.G, t, b.hist_beta);
     } else {
-        cg_xr_beta_kernel<VEC, true><<<G, bd, 0, st>>>(b.x, b.r, b.p, b.Kp, N, t, b.state, b.partial, b.hist_beta, vbound);
+        launch_chained(cg_xr_beta_kernel<VEC, true>, G, bd, 0, st, b.x, b.r, b.p, b.Kp, N, t, b.state, b.partial, b.hist_beta,
+                       vbound);
     }
     if (split)
         launch_p_split(*split, b.p, b.r, N, t, b.state, st);
     else
-        cg_p_kernel<VEC><<<G, bd, 0, st>>>(b.p, b.pc.k > 0 ? b.z : b.r, N, t, b.state);
+        launch_chained(cg_p_kernel<VEC>, G, bd, 0, st, b.p, b.pc.k > 0 ? b.z : b.r, N, t, b.state);
 }
 
 }  // namespace
