@@ -64,6 +64,7 @@ struct lgp_ctx {
     // the last symmetric-tile product: its kind, padded rows and columns (for the distance-form query)
     int sym_kind = -1, sym_D = 0, sym_t = 0;
     int64_t sym_Np = 0;
+    bool sym_dot = false;  // whether it considered the dot form
     // prepare_x calls so far; the X-only operands of the tensor-core products in vsplit (transposed X,
     // with opnd_dot also the dot-form distance operands) belong to prepared X number opnd_version (built for
     // opnd_t columns at workspace address opnd_buf), 0 = none
@@ -222,7 +223,9 @@ struct Prepared {
     uint64_t version;  // distinguishes successive preparations of the context's xs buffer
 };
 
-lgp_status prepare_x(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X, int64_t N, cudaStream_t st, Prepared *pp) {
+// tc_t > 0: a tensor-core product of that many columns follows, whose maxima words are cleared on the way.
+lgp_status prepare_x(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X, int64_t N, cudaStream_t st, Prepared *pp,
+                     int tc_t = 0) {
     NvtxRange nvtx_range("lgp.prepare_x");
     lgp_status s = make_params(ctx, hyp, &pp->kp);
     if (s != LGP_OK) return s;
@@ -234,7 +237,12 @@ lgp_status prepare_x(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X, int64_t
     if (s != LGP_OK) return s;
     pp->xs = (float *)ctx->xs.p;
     pp->version = ++ctx->prep_version;
-    launch_prep_x(X, N, pp->kp.D, pp->kp.dpad, pp->kp.scale, pp->xs, pp->Np, (int *)ctx->flags.p, st);
+    unsigned int *vmax = nullptr, *words = nullptr;
+    if (tc_t > 0) {
+        if ((s = ensure(ctx, ctx->vsplit, (size_t)tc_vsplit_bytes(pp->Np, tc_t))) != LGP_OK) return s;
+        tc_max_words(pp->Np, tc_t, ctx->vsplit.p, &vmax, &words);
+    }
+    launch_prep_x(X, N, pp->kp.D, pp->kp.dpad, pp->kp.scale, pp->xs, pp->Np, (int *)ctx->flags.p, st, vmax, words);
     LGP_CUDA(cudaGetLastError());
     return LGP_OK;
 }
@@ -298,12 +306,12 @@ lgp_status autotune_tc(lgp_ctx *ctx, const Prepared &pp, const float *V, int64_t
     const char *env = std::getenv("LGP_AUTOTUNE");
     const char *sym = std::getenv("LGP_TC_SYMMETRIC");
     int cand[4], n = 0;
-    tc_split_candidates(pp.Np, ctx->num_sms, cand, &n);
+    tc_split_candidates(pp.Np, pp.kp.kind, pp.kp.D, ctx->num_sms, cand, &n);
     if (sym && sym[0] == '1' && tc_symmetric_ok(pp.Np)) {
         ctx->tc_splits[key] = kTcSymmetric;
         return LGP_OK;
     }
-    if (sym && sym[0] == '0' && n > 0 && cand[0] == kTcSymmetric) {
+    if (sym && sym[0] == '0' && n > 0 && cand[0] < 0) {
         for (int k = 1; k < n; ++k) cand[k - 1] = cand[k];
         --n;
     }
@@ -372,6 +380,14 @@ bool tc_operands_valid(const lgp_ctx *ctx, const Prepared &pp, int t, int prec) 
            ctx->opnd_buf_bytes == ctx->vsplit.bytes && (ctx->opnd_dot || !needs_dot(ctx, pp, t, prec));
 }
 
+void mark_tc_operands(lgp_ctx *ctx, const Prepared &pp, int t, int prec) {
+    ctx->opnd_version = pp.version;
+    ctx->opnd_t = t;
+    ctx->opnd_dot = needs_dot(ctx, pp, t, prec);
+    ctx->opnd_buf = ctx->vsplit.p;
+    ctx->opnd_buf_bytes = ctx->vsplit.bytes;
+}
+
 // Builds the X-only operands of the tensor-core products of prepared X once (not inside the products of a
 // solve, where X does not change): the transposed X and, for a symmetric product that may take the dot
 // form, its distance operands.
@@ -379,13 +395,9 @@ lgp_status ensure_tc_operands(lgp_ctx *ctx, const Prepared &pp, int t, int prec,
     if (!is_tc(prec) || tc_operands_valid(ctx, pp, t, prec)) return LGP_OK;
     lgp_status s = ensure(ctx, ctx->vsplit, (size_t)tc_vsplit_bytes(pp.Np, t));
     if (s != LGP_OK) return s;
-    const bool dot = needs_dot(ctx, pp, t, prec);
-    LGP_CUDA(launch_tc_operands(pp.kp, pp.xs, pp.N, pp.Np, t, ctx->vsplit.p, dot, st));
-    ctx->opnd_version = pp.version;
-    ctx->opnd_t = t;
-    ctx->opnd_dot = dot;
-    ctx->opnd_buf = ctx->vsplit.p;
-    ctx->opnd_buf_bytes = ctx->vsplit.bytes;
+    LGP_CUDA(launch_tc_operands(pp.kp, pp.xs, pp.N, pp.Np, t, ctx->vsplit.p, needs_dot(ctx, pp, t, prec),
+                                ctx->num_sms, st));
+    mark_tc_operands(ctx, pp, t, prec);
     return LGP_OK;
 }
 
@@ -401,7 +413,7 @@ bool kernel_timing_on(const lgp_ctx *ctx, cudaStream_t st) {
 // v_ready, tail: see launch_mv_tc (v_ready for the tensor-core products only).
 lgp_status matvec_prepared(lgp_ctx *ctx, const Prepared &pp, const float *V, int64_t ldv, float *out, int64_t ldo,
                            int t, int prec, const int *skip, cudaStream_t st, int dist_form = -1, bool v_ready = false,
-                           ProductTail *tail = nullptr) {
+                           ProductTail *tail = nullptr, bool zeroed = false) {
     if (is_tc(prec)) {
         lgp_status s = ensure(ctx, ctx->vsplit, (size_t)tc_vsplit_bytes(pp.Np, t));
         if (s != LGP_OK) return s;
@@ -409,15 +421,19 @@ lgp_status matvec_prepared(lgp_ctx *ctx, const Prepared &pp, const float *V, int
         const int64_t pf = mv_tc_partial_floats(pp.Np, t, ctx->num_sms, forced);
         s = ensure(ctx, ctx->mv_partial, (size_t)std::max<int64_t>(pf, 1) * sizeof(float));
         if (s != LGP_OK) return s;
-        if ((s = ensure_tc_operands(ctx, pp, t, prec, st)) != LGP_OK) return s;
+        // operands that this X still lacks are built with the split of V, unless that may be skipped or is done
+        if ((skip || v_ready) && (s = ensure_tc_operands(ctx, pp, t, prec, st)) != LGP_OK) return s;
         const bool timed = kernel_timing_on(ctx, st);
         LGP_CUDA(launch_mv_tc(pp.kp, pp.xs, pp.N, pp.Np, V, ldv, out, ldo, t, tc_fmt(prec), ctx->vsplit.p,
                               (float *)ctx->mv_partial.p,
                               (int64_t)(ctx->mv_partial.bytes / sizeof(float)), skip, (int *)ctx->flags.p + 1,
                               ctx->wait_budget, ctx->num_sms, st, forced, tc_operands_valid(ctx, pp, t, prec),
-                              dist_form, timed ? ctx->kev[0] : nullptr, timed ? ctx->kev[1] : nullptr, v_ready, tail));
+                              dist_form, timed ? ctx->kev[0] : nullptr, timed ? ctx->kev[1] : nullptr, v_ready, tail,
+                              zeroed));
+        mark_tc_operands(ctx, pp, t, prec);
         if (timed) ctx->kev_set = true;
-        if (forced == kTcSymmetric) {
+        if (forced < 0) {
+            ctx->sym_dot = forced == kTcSymmetric;
             ctx->sym_kind = pp.kp.kind;
             ctx->sym_D = pp.kp.D;
             ctx->sym_t = t;
@@ -649,7 +665,7 @@ lgp_status run_cg(lgp_ctx *ctx, const Prepared &pp, const float *B, int64_t ldb,
     const bool fused_split = is_tc(prec) && !pc;
     CgSplit split = {};
     if (fused_split) {
-        const bool symmetric = tc_splits_for(ctx, pp, t, prec) == kTcSymmetric;
+        const bool symmetric = tc_splits_for(ctx, pp, t, prec) < 0;
         split = tc_cg_split(pp.kp, pp.Np, t, tc_fmt(prec), ctx->vsplit.p, symmetric ? b.Kp : nullptr);
         LGP_CUDA(launch_v_split(pp.kp, pp.N, pp.Np, b.p, t, t, tc_fmt(prec), ctx->vsplit.p, split.out_init, t, nullptr,
                                 ctx->num_sms, st));
@@ -1312,7 +1328,7 @@ int32_t lgp_tc_kernel_choice(const lgp_ctx *ctx, int64_t N, int32_t D, int32_t k
     const std::vector<int64_t> key = {pad_rows(N), (int64_t)t, (int64_t)tc_fmt(p), (int64_t)D, (int64_t)kind};
     auto it = ctx->tc_splits.find(key);
     if (it == ctx->tc_splits.end()) return LGP_TC_UNTUNED;
-    return it->second == kTcSymmetric ? LGP_TC_SYMMETRIC : LGP_TC_ROW;
+    return it->second < 0 ? LGP_TC_SYMMETRIC : LGP_TC_ROW;
 }
 
 int32_t lgp_batch_route_choice(const lgp_ctx *ctx, int64_t N, int32_t D, int32_t kind, int32_t t) {
@@ -1363,7 +1379,7 @@ lgp_status lgp_tc_distance_form(lgp_ctx *ctx, lgp_stream stream, int32_t *form, 
         *form = LGP_DIST_NONE;
         return LGP_OK;
     }
-    if (!dot_form_allowed(ctx->sym_kind, ctx->sym_D)) {
+    if (!ctx->sym_dot || !dot_form_allowed(ctx->sym_kind, ctx->sym_D)) {
         *form = LGP_DIST_DIFF;
         return LGP_OK;
     }
@@ -1412,7 +1428,7 @@ lgp_status lgp_kernel_matvec(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X,
     if (p < 0) return fail(ctx, (lgp_status)p, "precision %d unsupported for t=%d", prec, t);
     cudaStream_t st = (cudaStream_t)stream;
     Prepared pp;
-    if ((s = prepare_x(ctx, hyp, X, N, st, &pp)) != LGP_OK) return s;
+    if ((s = prepare_x(ctx, hyp, X, N, st, &pp, is_tc(p) ? tp : 0)) != LGP_OK) return s;
     // an explicit split precision at other t: the product runs on tp zero-padded columns
     const float *Vu = V;
     float *Ou = out;
@@ -1433,7 +1449,7 @@ lgp_status lgp_kernel_matvec(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X,
         if (cap == cudaStreamCaptureStatusNone && (s = autotune_tc(ctx, pp, Vu, tp, Ou, tp, tp, p, st)) != LGP_OK)
             return s;
     }
-    if ((s = matvec_prepared(ctx, pp, Vu, tp, Ou, tp, tp, p, nullptr, st)) != LGP_OK) return s;
+    if ((s = matvec_prepared(ctx, pp, Vu, tp, Ou, tp, tp, p, nullptr, st, -1, false, nullptr, true)) != LGP_OK) return s;
     if (tp != t) {
         launch_copy_cols(Ou, tp, out, t, N, t, 0, st);
         LGP_CUDA(cudaGetLastError());
@@ -1661,8 +1677,8 @@ lgp_status lgp_lml_and_grad(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X, 
         // preconditioned: 3 more launches in the CG init; the build (init, 2 per rank step, Gram,
         // float32 copy), the P-distributed probes, and P^{-1} of the probe block with the y copy
         const int pc_once = k > 0 ? (2 * k + 3) + 3 + 1 + 4 : 0;
-        // the products' X-only operands, built once before the loop (transpose; box and operands of the dot form)
-        const int opnd_once = is_tc(prec) && tc_operands_valid(ctx, pp, t, prec) ? (ctx->opnd_dot ? 3 : 1) : 0;
+        // the products' X-only operands, built once before the loop (transpose with box; operands of the dot form)
+        const int opnd_once = is_tc(prec) && tc_operands_valid(ctx, pp, t, prec) ? (ctx->opnd_dot ? 2 : 1) : 0;
         if (!single) {
             const int split_once = is_tc(prec) && k == 0 ? (tc_fmt(prec) == 1 ? 2 : 1) : 0;
             info->launches = 3 + 2 + split_once +

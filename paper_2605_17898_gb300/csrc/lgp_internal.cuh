@@ -233,7 +233,7 @@ struct CgState {
 
 // prep.cu
 void launch_prep_x(const float *X, int64_t N, int D, int dpad, const float *scale_host, float *Xs, int64_t Np,
-                   int *err_flag, cudaStream_t st);
+                   int *err_flag, cudaStream_t st, unsigned int *zero64 = nullptr, unsigned int *zero32 = nullptr);
 void launch_rademacher(uint64_t seed, int64_t N, int m, float *Z, int64_t ldz, int col0, cudaStream_t st);
 void launch_scan_finite(const float *A, int64_t n, int *err_flag, cudaStream_t st);
 void launch_copy_cols(const float *src, int64_t lds, float *dst, int64_t ldd, int64_t rows, int cols, int dst_col0,
@@ -297,7 +297,9 @@ int64_t tc_vsplit_bytes(int64_t Np, int t);
 // fmt: 0 = bfloat16 halves, 1 = scaled float16 halves
 // forced_splits > 0 overrides the column-split count (the autotuner's choice); 0 = wave-efficiency heuristic;
 // kTcSymmetric = the symmetric-tile kernel (mv_tcs.cuh), which adds onto out instead of writing partials.
+// kTcSymmetricDiff = the same, always in the difference form.
 constexpr int kTcSymmetric = -1;
+constexpr int kTcSymmetricDiff = -2;
 // operands_ready: the operands that depend on X alone are already in vsplit (launch_tc_operands, once
 // per prepared X): the transposed X and, where the symmetric product may take the dot form, its
 // distance operands; otherwise the product builds them first.
@@ -305,7 +307,8 @@ constexpr int kTcSymmetric = -1;
 // instances launch and the device gate word lets one of them work; 0 / 1 = only the difference / dot
 // instance launches (the caller read the gate word, which must then give the same answer).
 // v_ready: V is already split in the workspace, and out of a symmetric product already holds sigma^2 V
-// (launch_v_split, launch_p_split). tail (optional): see ProductTail.
+// (launch_v_split, launch_p_split). tail (optional): see ProductTail. zeroed: nothing has been collected in the words of
+// tc_max_words since launch_prep_x cleared them, but for this X and V.
 // ev_begin / ev_end (optional): recorded on st immediately before and after the product kernel's
 // launch(es), after the V split and operand kernels (the kernel timing of lgp_last_kernel_ms).
 cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, const float *V, int64_t ldv,
@@ -313,7 +316,7 @@ cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int
                          const int *skip, int *err_flag, long long wait_budget, int num_sms, cudaStream_t st,
                          int forced_splits = 0, bool operands_ready = false, int dist_form = -1,
                          cudaEvent_t ev_begin = nullptr, cudaEvent_t ev_end = nullptr, bool v_ready = false,
-                         ProductTail *tail = nullptr);
+                         ProductTail *tail = nullptr, bool zeroed = false);
 // A CG solve's vector p as the split operand of its products (p row stride t, the workspace of one vsplit).
 struct CgSplit {
     int fmt;
@@ -333,13 +336,15 @@ void launch_p_split(const CgSplit &sp, float *p, const float *r, int64_t N, int 
 // The operands of the tensor-core products that depend on X alone, into the t-column V-split workspace:
 // the transposed prescaled X, and with dot = true the dot-form distance data of the symmetric product
 // (box, centred split operands, squared norms, the gate word).
-cudaError_t launch_tc_operands(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, int t, void *vsplit,
-                               bool dot, cudaStream_t st);
+cudaError_t launch_tc_operands(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, int t, void *vsplit, bool dot,
+                               int num_sms, cudaStream_t st);
+// The words in which the passes over V (64 words) and X (32 words) collect maxima
+void tc_max_words(int64_t Np, int t, void *vsplit, unsigned int **vmax, unsigned int **words);
 int64_t mv_tc_partial_floats(int64_t Np, int t, int num_sms);
 int64_t mv_tc_partial_floats(int64_t Np, int t, int num_sms, int forced_splits);
-// Up to four kernel choices worth timing: kTcSymmetric (when tc_symmetric_ok) and the three most
+// Up to four kernel choices worth timing: kTcSymmetric or kTcSymmetricDiff (when tc_symmetric_ok) and the three most
 // wave-efficient split counts.
-void tc_split_candidates(int64_t Np, int num_sms, int *cand, int *n);
+void tc_split_candidates(int64_t Np, int kind, int D, int num_sms, int *cand, int *n);
 bool tc_symmetric_ok(int64_t Np);
 // Dot-form distance of the symmetric product: whether it is considered for (kind, D), its limit on
 // max |u|^2, and the byte offset of the word holding the measured max in the V-split workspace.

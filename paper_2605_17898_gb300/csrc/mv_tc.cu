@@ -14,45 +14,19 @@ namespace {
 using tc::kBK;
 using tc::kBM;
 
-// Per-column largest |V| as float bits (non-negative floats order like their bit patterns). Thread
-// (row r, column c) of a block of 256 (T divides 256) scans rows r, r + rows-per-grid, ...; the block
-// reduces its columns in shared memory and adds one atomicMax per column.
-__global__ void __launch_bounds__(256) col_absmax_kernel(const float *__restrict__ V, int64_t ldv, int64_t N, int T,
-                                                         unsigned int *__restrict__ vmax, const int *skip) {
-    chain_wait();
-    chain_next();
-    if (skip && *skip) return;
-    __shared__ unsigned int red[256];
-    const int c = threadIdx.x % T;
-    unsigned int m = 0;
-    for (int64_t j = (int64_t)blockIdx.x * (blockDim.x / T) + threadIdx.x / T; j < N;
-         j += (int64_t)gridDim.x * (blockDim.x / T))
-        m = max(m, __float_as_uint(fabsf(V[j * ldv + c])));
-    red[threadIdx.x] = m;
-    __syncthreads();
-    if ((int)threadIdx.x < T) {
-        for (int k = threadIdx.x + T; k < (int)blockDim.x; k += T) m = max(m, red[k]);
-        atomicMax(vmax + c, m);
-    }
-}
-
 // V -> stacked [V_hi; V_lo] in the tile order the MMA reads: B row c' = c (hi) or t + c (lo);
 // element (j, c') of chunk q = j / 64 sits at q*64*2t + ((j%64)/8 * 2t/8 + c'/8) * 64 + (c'%8) * 8 + j%8;
 // rows j >= N are zero. One thread per (8-row group, column): its 8 hi and 8 lo values are contiguous
 // in that order and go out as one 16-byte store each; the warp's loads of a row are contiguous.
 // FMT f16: V is first scaled per column by 2^e_c and col_scale[c] = s^2 2^-15 2^-e_c is written.
 // With out_init set, also out_init[j, c] = noise * V[j, c] for j < N (the symmetric product adds
-// onto it).
+// onto it). Blocks b of nb.
 template <int T, int FMT>
-__global__ void split_v_kernel(const float *__restrict__ V, int64_t ldv, int64_t N, int64_t Np,
-                               uint16_t *__restrict__ vs,
-                               const unsigned int *__restrict__ vmax, float *__restrict__ col_scale, float s2,
-                               float *__restrict__ out_init, int64_t ldo, float noise, const int *skip) {
-    chain_wait();
-    chain_next();
-    if (skip && *skip) return;
+__device__ void split_v(const float *__restrict__ V, int64_t ldv, int64_t N, int64_t Np, uint16_t *__restrict__ vs,
+                        const unsigned int *__restrict__ vmax, float *__restrict__ col_scale, float s2,
+                        float *__restrict__ out_init, int64_t ldo, float noise, int b, int nb) {
     const int64_t total = (Np / 8) * T;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t e = b * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)nb * blockDim.x) {
         const int64_t g = e / T;  // rows 8g .. 8g + 7
         const int c = (int)(e - g * T);
         int ec = 0;
@@ -128,20 +102,6 @@ __global__ void __launch_bounds__(256) p_split_kernel(float *__restrict__ p, con
     }
 }
 
-// XsT[d, j] = Xs[j, d]: the transposed prescaled X the tensor-core product stages by TMA.
-__global__ void transpose_x_kernel(const float *__restrict__ Xs, int64_t Np, int dpad, float *__restrict__ XsT,
-                                   const int *skip) {
-    chain_wait();
-    chain_next();
-    if (skip && *skip) return;
-    const int64_t total = Np * dpad;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int d = (int)(e / Np);
-        const int64_t j = e - (int64_t)d * Np;
-        XsT[e] = Xs[j * dpad + d];
-    }
-}
-
 // Monotone map of a float onto unsigned integers (and back), so that atomicMax orders floats.
 __device__ __forceinline__ unsigned int ord_of(float f) {
     const unsigned int u = __float_as_uint(f);
@@ -151,44 +111,75 @@ __device__ __forceinline__ float float_of_ord(unsigned int o) {
     return __uint_as_float((o & 0x80000000u) ? (o & 0x7FFFFFFFu) : ~o);
 }
 
-// Dot-form distance, step 1: bounding box of the prescaled rows i < N. words[d] = ord(max x_d),
-// words[8 + d] = ord(max -x_d); the words start at zero (below every ordered float).
-__global__ void dot_bbox_kernel(const float *__restrict__ Xs, int64_t N, int dpad, unsigned int *__restrict__ words,
-                                const int *skip) {
+// First pass over a product's inputs. Blocks below x_blocks: XsT[d, j] = Xs[j, d], the transposed prescaled X that the
+// product stages by TMA, and with words set the bounding box of the rows i < N for the dot form: words[d] = ord(max x_d),
+// words[8 + d] = ord(max -x_d). The other blocks: the per-column largest |V| as float bits (non-negative floats order like
+// their bit patterns); thread (row r, column c) of a block's 256 (T divides 256). words and vmax start at zero (below every
+// ordered float).
+__global__ void __launch_bounds__(256) tc_scan_kernel(const float *__restrict__ Xs, int64_t N, int64_t Np, int dpad,
+                                                      float *__restrict__ XsT, unsigned int *__restrict__ words, int x_blocks,
+                                                      const float *__restrict__ V, int64_t ldv, int T,
+                                                      unsigned int *__restrict__ vmax, const int *skip) {
     chain_wait();
     chain_next();
     if (skip && *skip) return;
+    __shared__ unsigned int red[256];
+    if ((int)blockIdx.x >= x_blocks) {
+        const int b = blockIdx.x - x_blocks, nb = gridDim.x - x_blocks;
+        const int c = threadIdx.x % T;
+        const int64_t step = (int64_t)nb * (256 / T);
+        unsigned int m = 0;
+#pragma unroll 4
+        for (int64_t j = (int64_t)b * (256 / T) + threadIdx.x / T; j < N; j += step)
+            m = max(m, __float_as_uint(fabsf(V[j * ldv + c])));
+        red[threadIdx.x] = m;
+        __syncthreads();
+        if ((int)threadIdx.x < T) {
+            for (int k = threadIdx.x + T; k < 256; k += T) m = max(m, red[k]);
+            atomicMax(vmax + c, m);
+        }
+        return;
+    }
     unsigned int hi[8], lo[8];
 #pragma unroll
     for (int d = 0; d < 8; ++d) hi[d] = lo[d] = 0u;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t i = blockIdx.x * 256ll + threadIdx.x; i < Np; i += x_blocks * 256ll) {
+        float x[8] = {};
+        const float4 q0 = *reinterpret_cast<const float4 *>(Xs + i * dpad);
+        x[0] = q0.x; x[1] = q0.y; x[2] = q0.z; x[3] = q0.w;
+        if (dpad == 8) {
+            const float4 q1 = *reinterpret_cast<const float4 *>(Xs + i * dpad + 4);
+            x[4] = q1.x; x[5] = q1.y; x[6] = q1.z; x[7] = q1.w;
+        }
 #pragma unroll
         for (int d = 0; d < 8; ++d) {
             if (d < dpad) {
-                const float x = Xs[i * dpad + d];
-                hi[d] = max(hi[d], ord_of(x));
-                lo[d] = max(lo[d], ord_of(-x));
+                XsT[d * Np + i] = x[d];
+                if (i < N) {
+                    hi[d] = max(hi[d], ord_of(x[d]));
+                    lo[d] = max(lo[d], ord_of(-x[d]));
+                }
             }
         }
     }
+    if (!words) return;
     // warp, then block, then one global atomic per word and block
-    __shared__ unsigned int blk[16];
-    if (threadIdx.x < 16) blk[threadIdx.x] = 0u;
+    if (threadIdx.x < 16) red[threadIdx.x] = 0u;
     __syncthreads();
 #pragma unroll
     for (int d = 0; d < 8; ++d) {
         const unsigned int h = __reduce_max_sync(0xffffffffu, hi[d]);
         const unsigned int l = __reduce_max_sync(0xffffffffu, lo[d]);
         if ((threadIdx.x & 31) == 0 && d < dpad) {
-            atomicMax(blk + d, h);
-            atomicMax(blk + 8 + d, l);
+            atomicMax(red + d, h);
+            atomicMax(red + 8 + d, l);
         }
     }
     __syncthreads();
-    if (threadIdx.x < 16 && (threadIdx.x & 7) < dpad) atomicMax(words + threadIdx.x, blk[threadIdx.x]);
+    if (threadIdx.x < 16 && (int)(threadIdx.x & 7) < dpad) atomicMax(words + threadIdx.x, red[threadIdx.x]);
 }
 
-// Dot-form distance, step 2: per row j, the centred coordinates u = x - c (c the box centre)
+// Dot-form distance: per row j, the centred coordinates u = x - c (c the box centre)
 // split as u = h + m (h = f16(u), m = f16(u - h)), the squared norm a_j = sum_d (h^2 + 2 h m)
 // (what the Gram products below give for <u_j, u_j> without the m m term) in float32 and in three
 // float16 parts, and the two Gram operand rows, K-major, in the tile layout the MMA reads
@@ -198,14 +189,12 @@ __global__ void dot_bbox_kernel(const float *__restrict__ Xs, int64_t N, int dpa
 //   B role:  [2h | 2h | 2m | -a_h -a_m -a_l | 1 1 1 | 0 ...]
 // so that A_i . B_j = 2 (h_i h_j + m_i h_j + h_i m_j) - a_j - a_i = -|u_i - u_j|^2 to about 22 bits: the
 // tensor core hands the generation the negated squared distance itself.
-// words[16] collects max a_j over rows j < N (float bits, a_j >= 0).
+// words[16] collects max a_j over rows j < N (float bits, a_j >= 0). Every product of halves is exact in float32 and the
+// sum carries its rounding errors along, so that a_j is the exact sum rounded once (float64 runs at a 64th of the rate).
+// Blocks b of nb.
 template <int DP>
-__global__ void dot_operands_kernel(const float *__restrict__ Xs, int64_t N, int64_t Np,
-                                    unsigned int *__restrict__ words, float *__restrict__ arow,
-                                    uint4 *__restrict__ ua, uint4 *__restrict__ ub, const int *skip) {
-    chain_wait();
-    chain_next();
-    if (skip && *skip) return;
+__device__ void dot_operands(const float *__restrict__ Xs, int64_t N, int64_t Np, unsigned int *words,
+                             float *__restrict__ arow, uint4 *__restrict__ ua, uint4 *__restrict__ ub, int b, int nb) {
     constexpr int KG = 32;
     static_assert(3 * DP + 6 <= KG, "Gram operand row too short");
     constexpr int kTileBytes = 128 * KG * 2;
@@ -213,19 +202,24 @@ __global__ void dot_operands_kernel(const float *__restrict__ Xs, int64_t N, int
 #pragma unroll
     for (int d = 0; d < DP; ++d) c[d] = 0.5f * (float_of_ord(words[d]) - float_of_ord(words[8 + d]));
     unsigned int amax = 0u;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < Np; j += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t j = b * (int64_t)blockDim.x + threadIdx.x; j < Np; j += (int64_t)nb * blockDim.x) {
         __half h[DP], m[DP];
-        double a = 0.0;
+        float a = 0.0f, rest = 0.0f;
+        auto add = [&](float x) {  // a + rest += x without rounding (two-sum)
+            const float s = __fadd_rn(a, x), v = __fsub_rn(s, a);
+            rest = __fadd_rn(rest, __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(x, v)));
+            a = s;
+        };
 #pragma unroll
         for (int d = 0; d < DP; ++d) {
             const float u = Xs[j * DP + d] - c[d];
             h[d] = __float2half_rn(u);
             const float hf = __half2float(h[d]);
             m[d] = __float2half_rn(u - hf);
-            const double hd = hf, md = __half2float(m[d]);
-            a += hd * hd + 2.0 * hd * md;
+            add(__fmul_rn(hf, hf));
+            add(__fmul_rn(2.0f * hf, __half2float(m[d])));
         }
-        const float a32 = (float)a;
+        const float a32 = __fadd_rn(a, rest);
         const __half ah = __float2half_rn(a32);
         const float r1 = a32 - __half2float(ah);
         const __half am = __float2half_rn(r1);
@@ -265,6 +259,26 @@ __global__ void dot_operands_kernel(const float *__restrict__ Xs, int64_t N, int
     }
     amax = __reduce_max_sync(0xffffffffu, amax);
     if ((threadIdx.x & 31) == 0) atomicMax(words + 16, amax);
+}
+
+// Second pass: blocks below op_blocks the dot form's operands, the others the split of V (either may be absent).
+template <int T, int FMT, int DP>
+__global__ void __launch_bounds__(256) tc_operands_kernel(const float *__restrict__ Xs, int64_t N, int64_t Np,
+                                                          unsigned int *words, float *__restrict__ arow,
+                                                          uint4 *__restrict__ ua, uint4 *__restrict__ ub, int op_blocks,
+                                                          const float *__restrict__ V, int64_t ldv,
+                                                          uint16_t *__restrict__ vs, const unsigned int *__restrict__ vmax,
+                                                          float *__restrict__ col_scale, float s2,
+                                                          float *__restrict__ out_init, int64_t ldo, float noise,
+                                                          const int *skip) {
+    chain_wait();
+    chain_next();
+    if (skip && *skip) return;
+    if ((int)blockIdx.x < op_blocks)
+        dot_operands<DP>(Xs, N, Np, words, arow, ua, ub, blockIdx.x, op_blocks);
+    else
+        split_v<T, FMT>(V, ldv, N, Np, vs, vmax, col_scale, s2, out_init, ldo, noise, blockIdx.x - op_blocks,
+                        gridDim.x - op_blocks);
 }
 
 __global__ void tc_reduce_kernel(const float *__restrict__ partial, int S, int64_t Np, int64_t N, int t,
@@ -433,7 +447,7 @@ bool dot_form_allowed(int kind, int D) {
 }
 
 int64_t mv_tc_partial_floats(int64_t Np, int t, int num_sms, int forced_splits) {
-    if (forced_splits == kTcSymmetric) return 0;
+    if (forced_splits < 0) return 0;
     const TcGrid g = tc_grid(Np, num_sms, forced_splits);
     return g.S > 1 ? (int64_t)g.S * Np * t : 0;
 }
@@ -442,10 +456,19 @@ int64_t mv_tc_partial_floats(int64_t Np, int t, int num_sms) { return mv_tc_part
 
 bool tc_symmetric_ok(int64_t Np) { return Np / tcs::kTile >= 8; }
 
-void tc_split_candidates(int64_t Np, int num_sms, int *cand, int *n) {
+// The symmetric kernel is timed against the row kernel from kSymMinRows rows on (from eight tiles on where the difference form
+// is its only one), at first in the difference form alone. Below, the row kernel gives the same bits at every run; its
+// distances and the difference form's are float32, those of the dot form are not (error of a training step at N = 2000:
+// 5.6e-6 in the dot form, 7e-7 in the two others). From dot_min_rows on the dot form is the faster one. Product call with the
+// row kernel -> in the difference form: N = 6000, D = 3, t = 16 52 -> 26 us; N = 7500, D = 2, t = 16 60 -> 27.
+static constexpr int64_t kSymMinRows = 4608;
+static int64_t dot_min_rows(int D) { return D > 4 ? 6144 : 8192; }
+
+void tc_split_candidates(int64_t Np, int kind, int D, int num_sms, int *cand, int *n) {
     const int rb = (int)(Np / kBM), total = (int)(Np / kBK);
     *n = 0;
-    if (tc_symmetric_ok(Np)) cand[(*n)++] = kTcSymmetric;
+    if (tc_symmetric_ok(Np) && (Np >= kSymMinRows || !dot_form_allowed(kind, D)))
+        cand[(*n)++] = Np < dot_min_rows(D) ? kTcSymmetricDiff : kTcSymmetric;
     // the three most wave-efficient split counts, best first
     for (int k = 0; k < 3; ++k) {
         int best_s = 0;
@@ -466,41 +489,6 @@ void tc_split_candidates(int64_t Np, int num_sms, int *cand, int *n) {
     }
 }
 
-namespace {
-
-cudaError_t launch_dot_operands(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, int t, void *vsplit,
-                                const int *skip, cudaStream_t st) {
-    unsigned int *words = (unsigned int *)((uint8_t *)vsplit + tc_dot_gate_offset(Np, t) - 16 * 4);
-    float *arow = (float *)(words + 32);
-    uint8_t *ua = (uint8_t *)(arow + Np);
-    uint8_t *ub = ua + Np * 64;
-    cudaError_t e = cudaMemsetAsync(words, 0, 32 * sizeof(unsigned int), st);
-    if (e != cudaSuccess) return e;
-    const int bb = (int)std::min<int64_t>((N + 255) / 256, 1024);
-    launch_chained(dot_bbox_kernel, bb, 256, 0, st, Xs, N, kp.dpad, words, skip);
-    const int ob = (int)std::min<int64_t>((Np + 255) / 256, 4096);
-    launch_chained(kp.dpad <= 4 ? dot_operands_kernel<4> : dot_operands_kernel<8>, ob, 256, 0, st, Xs, N, Np, words, arow,
-                   (uint4 *)ua, (uint4 *)ub, skip);
-    return cudaGetLastError();
-}
-
-void launch_transpose_x(const KernelParams &kp, const float *Xs, int64_t Np, void *vsplit, int t, const int *skip,
-                        cudaStream_t st) {
-    float *XsT = (float *)((uint8_t *)vsplit + 2 * Np * t * 2 + 2 * 64 * 4);
-    launch_chained(transpose_x_kernel, (int)std::min<int64_t>((Np * kp.dpad + 255) / 256, 4096), 256, 0, st, Xs, Np, kp.dpad,
-                   XsT, skip);
-}
-
-}  // namespace
-
-cudaError_t launch_tc_operands(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, int t, void *vsplit,
-                               bool dot, cudaStream_t st) {
-    launch_transpose_x(kp, Xs, Np, vsplit, t, nullptr, st);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || !dot) return e;
-    return launch_dot_operands(kp, Xs, N, Np, t, vsplit, nullptr, st);
-}
-
 CgSplit tc_cg_split(const KernelParams &kp, int64_t Np, int t, int fmt, void *vsplit, float *out_init) {
     CgSplit sp;
     sp.fmt = fmt;
@@ -513,21 +501,58 @@ CgSplit tc_cg_split(const KernelParams &kp, int64_t Np, int t, int fmt, void *vs
     return sp;
 }
 
+namespace {
+
+// The passes over a product's inputs that its kernel needs done: with x the transposed X (and with dot the distance
+// operands), with V the split of V. zeroed: the words they collect maxima in are zero already (launch_prep_x).
+cudaError_t launch_tc_inputs(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, bool x, bool dot, const float *V,
+                             int64_t ldv, int t, int fmt, void *vsplit, float *out_init, int64_t ldo, bool zeroed,
+                             const int *skip, int num_sms, cudaStream_t st) {
+    const CgSplit sp = tc_cg_split(kp, Np, t, fmt, vsplit, out_init);
+    float *XsT = sp.col_scale + 64;
+    unsigned int *words = (unsigned int *)(XsT + 8 * Np);
+    float *arow = (float *)(words + 32);
+    uint8_t *ua = (uint8_t *)(arow + Np);
+    uint8_t *ub = ua + Np * 64;
+    const bool absmax = V && fmt == kFmtF16;
+    cudaError_t e;
+    if (!zeroed) {
+        if (absmax && (e = cudaMemsetAsync(sp.vmax, 0, 64 * sizeof(unsigned int), st)) != cudaSuccess) return e;
+        if (dot && (e = cudaMemsetAsync(words, 0, 32 * sizeof(unsigned int), st)) != cudaSuccess) return e;
+    }
+    const int xb = x ? (int)std::min<int64_t>((Np + 255) / 256, 2 * num_sms) : 0;
+    const int mb = absmax ? (int)std::max<int64_t>(1, std::min<int64_t>((N * t + 255) / 256, 4 * num_sms)) : 0;
+    if (xb + mb > 0 && (e = launch_chained(tc_scan_kernel, xb + mb, 256, 0, st, Xs, N, Np, kp.dpad, XsT,
+                                           dot ? words : nullptr, xb, V, ldv, t, sp.vmax, skip)) != cudaSuccess)
+        return e;
+    const int ob = dot ? (int)std::min<int64_t>((Np + 255) / 256, 4096) : 0;
+    const int vb = V ? (int)std::min<int64_t>((Np / 8 * t + 255) / 256, 8192) : 0;  // (8-row group, column)
+    if (ob + vb == 0) return cudaSuccess;
+    auto pick = [&](auto dp) {
+        constexpr int DP = decltype(dp)::value;
+        return t == 16 ? (fmt == kFmtF16 ? tc_operands_kernel<16, kFmtF16, DP> : tc_operands_kernel<16, kFmtBF16, DP>)
+                       : (fmt == kFmtF16 ? tc_operands_kernel<32, kFmtF16, DP> : tc_operands_kernel<32, kFmtBF16, DP>);
+    };
+    auto k = kp.dpad <= 4 ? pick(std::integral_constant<int, 4>()) : pick(std::integral_constant<int, 8>());
+    return launch_chained(k, ob + vb, 256, 0, st, Xs, N, Np, words, arow, (uint4 *)ua, (uint4 *)ub, ob, V, ldv, sp.vs, sp.vmax,
+                          sp.col_scale, kp.s2, out_init, ldo, kp.noise, skip);
+}
+
+}  // namespace
+
+cudaError_t launch_tc_operands(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, int t, void *vsplit, bool dot,
+                               int num_sms, cudaStream_t st) {
+    return launch_tc_inputs(kp, Xs, N, Np, true, dot, nullptr, 0, t, kFmtF16, vsplit, nullptr, 0, false, nullptr, num_sms, st);
+}
+
 cudaError_t launch_v_split(const KernelParams &kp, int64_t N, int64_t Np, const float *V, int64_t ldv, int t, int fmt,
                            void *vsplit, float *out_init, int64_t ldo, const int *skip, int num_sms, cudaStream_t st) {
-    const CgSplit sp = tc_cg_split(kp, Np, t, fmt, vsplit, out_init);
-    const int blocks = (int)std::min<int64_t>((Np / 8 * t + 255) / 256, 8192);  // (8-row group, column)
-    if (fmt == kFmtF16) {
-        const cudaError_t e = cudaMemsetAsync(sp.vmax, 0, 64 * sizeof(unsigned int), st);
-        if (e != cudaSuccess) return e;
-        const int mb = (int)std::max<int64_t>(1, std::min<int64_t>((N * t + 255) / 256, 4 * num_sms));
-        launch_chained(col_absmax_kernel, mb, (256 / t) * t, 0, st, V, ldv, N, t, sp.vmax, skip);
-    }
-    auto split = t == 16 ? (fmt == kFmtF16 ? split_v_kernel<16, kFmtF16> : split_v_kernel<16, kFmtBF16>)
-                         : (fmt == kFmtF16 ? split_v_kernel<32, kFmtF16> : split_v_kernel<32, kFmtBF16>);
-    launch_chained(split, blocks, 256, 0, st, V, ldv, N, Np, sp.vs, sp.vmax, sp.col_scale, kp.s2, out_init, ldo, kp.noise,
-                   skip);
-    return cudaGetLastError();
+    return launch_tc_inputs(kp, nullptr, N, Np, false, false, V, ldv, t, fmt, vsplit, out_init, ldo, false, skip, num_sms, st);
+}
+
+void tc_max_words(int64_t Np, int t, void *vsplit, unsigned int **vmax, unsigned int **words) {
+    *vmax = (unsigned int *)((uint16_t *)vsplit + 2 * Np * t);
+    *words = *vmax + 128 + 8 * Np;
 }
 
 void launch_p_split(const CgSplit &sp, float *p, const float *r, int64_t N, int t, CgState *state, cudaStream_t st) {
@@ -541,7 +566,7 @@ cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int
                          float *out, int64_t ldo, int t, int fmt, void *vsplit, float *partial, int64_t partial_cap,
                          const int *skip, int *err_flag, long long wait_budget, int num_sms, cudaStream_t st,
                          int forced_splits, bool operands_ready, int dist_form, cudaEvent_t ev_begin,
-                         cudaEvent_t ev_end, bool v_ready, ProductTail *tail) {
+                         cudaEvent_t ev_end, bool v_ready, ProductTail *tail, bool zeroed) {
     auto mark = [&](cudaEvent_t ev) {
         if (ev) cudaEventRecord(ev, st);
     };
@@ -550,16 +575,13 @@ cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int
     unsigned int *vmax = (unsigned int *)(vs + 2 * Np * t);
     float *col_scale = (float *)(vmax + 64);
     float *XsT = col_scale + 64;
-    const bool symmetric = forced_splits == kTcSymmetric;
+    const bool symmetric = forced_splits < 0;
     if (tail) *tail = ProductTail();
     cudaError_t e;
-    if (!v_ready &&
-        (e = launch_v_split(kp, N, Np, V, ldv, t, fmt, vsplit, symmetric ? out : nullptr, ldo, skip, num_sms, st)) !=
-            cudaSuccess)
+    const bool dot_allowed = forced_splits == kTcSymmetric && dot_form_allowed(kp.kind, kp.D);
+    if ((e = launch_tc_inputs(kp, Xs, N, Np, !operands_ready, !operands_ready && dot_allowed, v_ready ? nullptr : V, ldv, t, fmt,
+                              vsplit, symmetric ? out : nullptr, ldo, zeroed, skip, num_sms, st)) != cudaSuccess)
         return e;
-    if (!operands_ready) launch_transpose_x(kp, Xs, Np, vsplit, t, skip, st);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
 
     const CUtensorMapDataType vt = fmt == kFmtF16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
     if (symmetric) {
@@ -602,16 +624,14 @@ cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int
             return fmt == kFmtF16 ? tcs::dispatch_f16(kp.kind, kp.D, t, grid, mx, mv, mo, a, st)
                                   : tcs::dispatch_bf16(kp.kind, kp.D, t, grid, mx, mv, mo, a, st);
         };
-        if (!dot_form_allowed(kp.kind, kp.D)) {
+        if (!dot_allowed) {
             mark(ev_begin);
             e = launch();
             mark(ev_end);
             return e;
         }
-        // dot form: operands (unless the caller built them for this X), then the instance of the known
-        // distance form, or both instances, of which the gate word lets exactly one work
-        if (!operands_ready && (e = launch_dot_operands(kp, Xs, N, Np, t, vsplit, skip, st)) != cudaSuccess)
-            return e;
+        // dot form: the instance of the known distance form, or both instances, of which the gate word lets exactly
+        // one work
         unsigned int *words = (unsigned int *)(XsT + 8 * Np);
         float *arow = (float *)(words + 32);
         uint8_t *ua = (uint8_t *)(arow + Np);

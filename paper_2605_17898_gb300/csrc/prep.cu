@@ -9,11 +9,17 @@ struct ScaleArg {
     float s[kMaxD];
 };
 
-// Xs[i, d] = X[i, d] * scale[d] for i < N, d < D; zero in the padded rows and columns.
+// Xs[i, d] = X[i, d] * scale[d] for i < N, d < D; zero in the padded rows and columns. Clears 64 and 32 words for the
+// kernels that follow (a memset node would end the chain of launches).
 __global__ void prep_x_kernel(const float *__restrict__ X, int64_t N, int D, int dpad, ScaleArg sc,
-                              float *__restrict__ Xs, int64_t Np, int *err_flag) {
+                              float *__restrict__ Xs, int64_t Np, int *err_flag, unsigned int *zero64,
+                              unsigned int *zero32) {
     chain_wait();
     chain_next();
+    if (blockIdx.x == 0 && zero64 && threadIdx.x < 64) {
+        zero64[threadIdx.x] = 0u;
+        if (threadIdx.x < 32) zero32[threadIdx.x] = 0u;
+    }
     const int64_t total = Np * dpad;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = e / dpad;
@@ -74,10 +80,11 @@ inline int grid_for(int64_t n, int threads) {
 }  // namespace
 
 void launch_prep_x(const float *X, int64_t N, int D, int dpad, const float *scale_host, float *Xs, int64_t Np,
-                   int *err_flag, cudaStream_t st) {
+                   int *err_flag, cudaStream_t st, unsigned int *zero64, unsigned int *zero32) {
     ScaleArg sc;
     for (int d = 0; d < kMaxD; ++d) sc.s[d] = d < D ? scale_host[d] : 0.0f;
-    launch_chained(prep_x_kernel, grid_for(Np * dpad, 256), 256, 0, st, X, N, D, dpad, sc, Xs, Np, err_flag);
+    launch_chained(prep_x_kernel, grid_for(Np * dpad, 256), 256, 0, st, X, N, D, dpad, sc, Xs, Np, err_flag, zero64,
+                   zero32);
 }
 
 void launch_rademacher(uint64_t seed, int64_t N, int m, float *Z, int64_t ldz, int col0, cudaStream_t st) {
