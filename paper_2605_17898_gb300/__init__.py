@@ -172,14 +172,36 @@ class Hyper:
         return h, ls  # keep ls alive while h is used
 
 
-def _stream_ptr(stream=None):
+_float_arrays: dict[int, type] = {}
+
+
+def _c_hyper(p) -> lgp_hyper:
+    """The lgp_hyper of a Hyper, or of any object with its fields, with its own lengthscales."""
+    ls = np.asarray(p.log_lengthscale, dtype=np.float32)
+    if ls.ndim != 1:
+        h, h._keep = Hyper.of(p).to_c()
+        return h
+    n = ls.shape[0]
+    arr = _float_arrays.get(n)
+    if arr is None:
+        arr = _float_arrays[n] = ctypes.c_float * n
+    return lgp_hyper(int(p.kind), n, arr(*ls.tolist()), float(p.log_outputscale), float(p.log_noise))
+
+
+# Small products are bound by the host (N = 1024, t = 1: 6.6 us on the GPU, 30 us a call, of which the library takes 6.5): the
+# stream's handle comes straight from torch (3.1 us through torch.cuda.current_stream), the hyperparameters are packed
+# without numpy's pointer objects (2.9 us) and pointers go in as integers.
+def _stream_ptr(stream=None) -> int:
+    if stream is not None:
+        return stream.cuda_stream
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    if torch.cuda.is_initialized():
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return torch.cuda.current_stream().cuda_stream
 
 
-def _ptr(t) -> ctypes.c_void_p:
-    return ctypes.c_void_p(t.data_ptr())
+def _ptr(t) -> int:
+    return t.data_ptr()
 
 
 def _f32_dev(a, device):
@@ -288,12 +310,11 @@ def lgp_kernel_matvec(X, hyp, V, prec: int = LGP_PREC_AUTO, out=None, ctx: Conte
     N, t = V2.shape
     if out is None:
         out = torch.empty((N, t), device=V.device, dtype=torch.float32)
-    h, keep = Hyper.of(hyp).to_c()
+    h = _c_hyper(hyp)
     s = ctx.lib.lgp_kernel_matvec(ctx.h, ctypes.byref(h), _ptr(X), _ptr(V2), _ptr(out), int(N), int(t), int(prec),
                                   _stream_ptr(stream))
     if check:
         ctx._check(s)
-    del keep
     return out.reshape(-1) if squeeze else out
 
 
@@ -307,10 +328,9 @@ def lgp_kernel_matvec_noalloc(X, hyp, V, out, prec: int = LGP_PREC_AUTO, stream=
     overlapping calls on different streams race.
     """
     N, t = V.shape
-    h, keep = Hyper.of(hyp).to_c()
+    h = _c_hyper(hyp)
     s = load().lgp_kernel_matvec_noalloc(ctypes.byref(h), _ptr(X), _ptr(V), _ptr(out), int(N), int(t), int(prec),
                                          _stream_ptr(stream))
-    del keep
     return int(s)
 
 
@@ -340,10 +360,9 @@ def lgp_kernel_matvec_grad(X, hyp, W, ctx: Context | None = None, stream=None):
     N, t = W2.shape
     D = X.shape[1]
     G = torch.empty((D + 2, N, t), device=W.device, dtype=torch.float32)
-    h, keep = Hyper.of(hyp).to_c()
+    h = _c_hyper(hyp)
     ctx._check(ctx.lib.lgp_kernel_matvec_grad(ctx.h, ctypes.byref(h), _ptr(X), _ptr(W2), _ptr(G), int(N), int(t),
                                               _stream_ptr(stream)))
-    del keep
     return G
 
 
@@ -373,13 +392,12 @@ def lgp_cg_solve(X, hyp, B, tol: float = 1e-6, max_iter: int = 1000, prec: int =
         out.copy_(x0.reshape(N, t))
     iters = np.zeros(t, dtype=np.int32)
     rel = np.zeros(t, dtype=np.float64)
-    h, keep = Hyper.of(hyp).to_c()
+    h = _c_hyper(hyp)
     o = _options(tol, max_iter, prec=prec, precond_rank=precond_rank,
                  flags=LGP_OPT_WARM_START if x0 is not None else 0)
     s = ctx._check(ctx.lib.lgp_cg_solve(ctx.h, ctypes.byref(h), _ptr(X), _ptr(B2), _ptr(out), int(N), int(t),
                                         ctypes.byref(o), iters.ctypes.data_as(ctypes.c_void_p),
                                         rel.ctypes.data_as(ctypes.c_void_p), _stream_ptr(stream)))
-    del keep
     return (out.reshape(-1) if squeeze else out), iters, rel, s
 
 
@@ -399,13 +417,12 @@ def lgp_lml_and_grad(X, y, hyp, n_probes: int = 15, lanczos_steps: int = LGP_MAX
     lml = ctypes.c_double(0.0)
     grad = np.zeros(D + 2, dtype=np.float64)
     info = lgp_lml_info()
-    h, keep = Hyper.of(hyp).to_c()
+    h = _c_hyper(hyp)
     o = _options(tol, max_iter, lanczos_steps, n_probes, prec, seed, precond_rank,
                  flags=LGP_OPT_SINGLE_RHS if single_rhs else 0)
     s = ctx._check(ctx.lib.lgp_lml_and_grad(ctx.h, ctypes.byref(h), _ptr(X), _ptr(y), N, ctypes.byref(o),
                                             ctypes.byref(lml), grad.ctypes.data_as(ctypes.c_void_p) if want_grad
                                             else None, ctypes.byref(info), _stream_ptr(stream)))
-    del keep
     d = {k: getattr(info, k) for k, _ in lgp_lml_info._fields_}
     d["status"] = s
     return lml.value, (grad if want_grad else None), d
@@ -425,12 +442,11 @@ def lgp_predict(X, y, hyp, Xs, n_probes: int = 0, seed: int = 0, tol: float = 1e
     mean = torch.empty(M, device=X.device, dtype=torch.float32)
     var = torch.empty(M, device=X.device, dtype=torch.float32) if want_var else None
     info = lgp_predict_info()
-    h, keep = Hyper.of(hyp).to_c()
+    h = _c_hyper(hyp)
     o = _options(tol, max_iter, 0, n_probes, prec, seed, precond_rank)
     s = ctx._check(ctx.lib.lgp_predict(ctx.h, ctypes.byref(h), _ptr(X), _ptr(y), N, _ptr(Xs), M, ctypes.byref(o),
                                        _ptr(mean), _ptr(var) if var is not None else None, ctypes.byref(info),
                                        _stream_ptr(stream)), allow_warn=True)
-    del keep
     return mean, var, {k: getattr(info, k) for k, _ in info._fields_}, s
 
 
@@ -455,9 +471,9 @@ def lgp_batch_cg_solve(Xs, hyps, Bs, tol: float = 1e-6, max_iter: int = 1000, pr
     hs = (lgp_hyper * n)()
     keep = []
     for g, hp in enumerate(hyps):
-        h, k = Hyper.of(hp).to_c()
+        h = _c_hyper(hp)
         hs[g] = h
-        keep.append(k)
+        keep.append(h)
     Xp = (ctypes.c_void_p * n)(*[X.data_ptr() for X in Xs])
     Bp = (ctypes.c_void_p * n)(*[B.data_ptr() for B in Bs])
     Sp = (ctypes.c_void_p * n)(*[S.data_ptr() for S in sols])
@@ -470,7 +486,6 @@ def lgp_batch_cg_solve(Xs, hyps, Bs, tol: float = 1e-6, max_iter: int = 1000, pr
                                               Ns.ctypes.data_as(ctypes.c_void_p), t, ctypes.byref(o),
                                               iters.ctypes.data_as(ctypes.c_void_p),
                                               rel.ctypes.data_as(ctypes.c_void_p), _stream_ptr(stream)))
-    del keep
     return sols, iters, rel, s
 
 
