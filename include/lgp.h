@@ -76,7 +76,7 @@ typedef enum { LGP_RBF = 0, LGP_MATERN52 = 1, LGP_MATERN12 = 2, LGP_MATERN32 = 3
  * The split kernels take t in {16, 32}. lgp_kernel_matvec and lgp_cg_solve also accept an explicit split
  * precision for any other t <= 32: they run it on the columns zero-padded to 16 (t < 16) or 32, and return
  * the caller's t. Single right-hand sides at large N gain most: at N = 100000, D = 8, the padded split
- * product takes about 2.9 ms against 7.5 ms for the float32 one. lgp_lml_and_grad and lgp_predict keep
+ * product takes about 2.8 ms against 3.7 ms for the float32 one. lgp_lml_and_grad and lgp_predict keep
  * t in {16, 32} for the split modes.
  * AUTO picks SPLIT_F16 for t in {16, 32} and FP32 otherwise. */
 typedef enum {
@@ -173,8 +173,8 @@ const char *lgp_status_string(int32_t status);
  *   LGP_TC_BANDS=1      let the symmetric-tile kernel's dot form visit its tiles in column bands
  *                       whose operands stay in L2 (N above about 157000 at t = 32, 262000 at
  *                       t = 16): at N = 500000, t = 32 about 1 GB of DRAM traffic per product
- *                       instead of 115 GB, for a product about 4% slower (measured 68.2 against
- *                       65.6 ms); for GPUs whose memory bandwidth other work needs meanwhile. */
+ *                       instead of 115 GB, for a product about 7% slower (measured 75.4 against
+ *                       70.5 ms at D = 8); for GPUs whose memory bandwidth other work needs meanwhile. */
 
 /* Create a context bound to CUDA device `device` (its workspace starts empty).
  * Returns LGP_ERR_INVALID_ARG for a NULL ctx or a device that does not exist,

@@ -1,15 +1,16 @@
-// One CG step after the product as a single launch, for vectors of at most 65536 elements (plain CG, t a power of two):
+// One CG step after the product as a single launch, for vectors of at most 262144 elements (plain CG, t a power of two):
 // the step's three grid-wide stages (p^T Kp, r^T r, the update of p) are stages of one thread-block cluster, which
 // exchanges its column sums through distributed shared memory and meets at the hardware's cluster barrier.
 //
 // What bounds it: latency. The three launches of solver.cu cost about 2 us each beyond their work, and between them
-// every vector goes to L2 and back; here x, r, p and Kp are read once into registers and each grid-wide sum costs a
-// cluster barrier. One CTA (no barrier) where a single SM can take the product's partial sums in about a microsecond, 8
-// CTAs (the portable cluster size) otherwise.
+// every vector goes to L2 and back; here up to 65536 elements of x, r, p and Kp are read once into the registers of 8
+// CTAs (the portable cluster size; one CTA, without a barrier, where a single SM can take the product's partial sums in
+// about a microsecond). Up to 262144 elements 16 CTAs keep p and r and read x and Kp once more; that holds while their SMs
+// can also take the product's partial sums in a few microseconds.
 //
 // Measured against the three launches: solve of N = 1024, t = 1, ~90 iterations 1.62 -> 0.95 ms; training step of N = 2000,
-// D = 8, t = 16 4.65 -> 3.73 ms. Larger vectors than the cluster's registers hold keep the three launches, whose blocks
-// spread over more SMs.
+// D = 8, t = 16 4.65 -> 3.73 ms; with 16 CTAs, solves at t = 32 of N = 3000 4.54 -> 4.18 ms, N = 8000 8.02 -> 7.53; at
+// N = 4099, t = 16 6.66 -> 5.89. Larger vectors keep the three launches, whose blocks spread over more SMs.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -24,7 +25,9 @@ namespace {
 namespace cg = cooperative_groups;
 
 constexpr int kClThreads = 512;
-constexpr int kClVecs = 4;  // float4s per thread and vector
+constexpr int kClVecs = 4;  // float4s per thread and vector that are all held in registers
+constexpr int kClWide = 16, kClWideVecs = 8;  // larger vectors
+constexpr int64_t kClWideParts = 1 << 21;     // partial sums that a cluster of 16 takes (about 4 us of its SMs' loads)
 constexpr int64_t kClusterOneFloats = 1 << 15;  // partial sums that one CTA takes alone (about 1.3 us of its SM's loads)
 
 struct ClusterArgs {
@@ -71,7 +74,8 @@ __device__ void split_tile(const ClusterArgs &a, const float *tile, int row0, in
     }
 }
 
-template <int CL>
+// VECS float4s per thread and vector; above kClVecs only p and r stay in registers, Kp and x come from the L2 cache again.
+template <int CL, int VECS>
 __global__ void __launch_bounds__(kClThreads, 1) cg_cluster_kernel(const ClusterArgs a) {
     __shared__ float2 red[64 * 32];
     __shared__ double sum1[kMaxT], sum2[kMaxT];
@@ -95,39 +99,12 @@ __global__ void __launch_bounds__(kClThreads, 1) cg_cluster_kernel(const Cluster
     if (tid < kMaxT) rmax[tid] = pmax[tid] = 0u;
 
     // ---- p, Kp (with the product's partial sums), r, x into registers; p^T Kp
-    float4 pv[kClVecs], kv[kClVecs], rv[kClVecs], xv[kClVecs];
+    constexpr bool kHold = VECS <= kClVecs;
+    constexpr int kHeld = kHold ? VECS : 1;
+    float4 pv[VECS], rv[VECS], kv[kHeld], xv[kHeld];
     float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
     auto index = [&](int m) { return ((m * CL + rank) * kClThreads + tid) * 4; };
-#pragma unroll
-    for (int m = 0; m < kClVecs; ++m) {
-        const int e = index(m);
-        pv[m] = kv[m] = rv[m] = xv[m] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (e < a.total) {
-            pv[m] = *reinterpret_cast<const float4 *>(a.p + e);
-            rv[m] = *reinterpret_cast<const float4 *>(a.r + e);
-            xv[m] = *reinterpret_cast<const float4 *>(a.x + e);
-            if (!a.part) kv[m] = *reinterpret_cast<const float4 *>(a.Kp + e);
-        }
-    }
-    if (a.part) {
-#pragma unroll
-        for (int m = 0; m < kClVecs; ++m) {
-            const int e = index(m);
-            if (e >= a.total) continue;
-#pragma unroll 8
-            for (int q = 0; q < a.S; ++q) {
-                const float4 w = *reinterpret_cast<const float4 *>(a.part + q * a.part_stride + e);
-                kv[m].x += w.x;
-                kv[m].y += w.y;
-                kv[m].z += w.z;
-                kv[m].w += w.w;
-            }
-            kv[m].x = fmaf(a.noise, pv[m].x, kv[m].x);
-            kv[m].y = fmaf(a.noise, pv[m].y, kv[m].y);
-            kv[m].z = fmaf(a.noise, pv[m].z, kv[m].z);
-            kv[m].w = fmaf(a.noise, pv[m].w, kv[m].w);
-        }
-    }
+    auto load = [](const float *q) { return *reinterpret_cast<const float4 *>(q); };
     // elements past N t (the last float4 of t = 1, 2) stay out of the sums
     auto add = [&](int m, const float4 &u, const float4 &v) {
         const int e = index(m);
@@ -136,8 +113,59 @@ __global__ void __launch_bounds__(kClThreads, 1) cg_cluster_kernel(const Cluster
         if (e + 2 < a.total) acc_prod2(hi[2], lo[2], u.z, v.z);
         if (e + 3 < a.total) acc_prod2(hi[3], lo[3], u.w, v.w);
     };
+    auto sum_parts = [&](int e, const float4 &p4) {
+        float4 k4 = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
+        for (int q = 0; q < a.S; ++q) {
+            const float4 w = load(a.part + q * a.part_stride + e);
+            k4.x += w.x;
+            k4.y += w.y;
+            k4.z += w.z;
+            k4.w += w.w;
+        }
+        k4.x = fmaf(a.noise, p4.x, k4.x);
+        k4.y = fmaf(a.noise, p4.y, k4.y);
+        k4.z = fmaf(a.noise, p4.z, k4.z);
+        k4.w = fmaf(a.noise, p4.w, k4.w);
+        return k4;
+    };
 #pragma unroll
-    for (int m = 0; m < kClVecs; ++m) add(m, pv[m], kv[m]);
+    for (int m = 0; m < VECS; ++m) {
+        const int e = index(m);
+        pv[m] = rv[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if constexpr (kHold) kv[m] = xv[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (e < a.total) {
+            pv[m] = load(a.p + e);
+            rv[m] = load(a.r + e);
+            if constexpr (kHold) {
+                xv[m] = load(a.x + e);
+                if (!a.part) kv[m] = load(a.Kp + e);
+            }
+        }
+    }
+    if constexpr (kHold) {
+        if (a.part) {
+#pragma unroll
+            for (int m = 0; m < VECS; ++m)
+                if (index(m) < a.total) kv[m] = sum_parts(index(m), pv[m]);
+        }
+#pragma unroll
+        for (int m = 0; m < VECS; ++m) add(m, pv[m], kv[m]);
+    } else {
+#pragma unroll
+        for (int m = 0; m < VECS; ++m) {
+            const int e = index(m);
+            if (e >= a.total) continue;
+            float4 k4;
+            if (a.part) {
+                k4 = sum_parts(e, pv[m]);
+                *reinterpret_cast<float4 *>(a.Kp + e) = k4;
+            } else {
+                k4 = load(a.Kp + e);
+            }
+            add(m, pv[m], k4);
+        }
+    }
     block_pairs_reduce<4>(hi, lo, t, red, sum1);
     const double pkp = cluster_sum<CL>(sum1, t);
     int bad = 0, nonfinite = 0;
@@ -161,14 +189,22 @@ __global__ void __launch_bounds__(kClThreads, 1) cg_cluster_kernel(const Cluster
     }
     auto axpy = [](float s, float u, float v) { return s != 0.0f ? fmaf(s, u, v) : v; };
 #pragma unroll
-    for (int m = 0; m < kClVecs; ++m) {
+    for (int m = 0; m < VECS; ++m) {
         const int e = index(m);
         if (e >= a.total) continue;
-        xv[m] = make_float4(axpy(al[0], pv[m].x, xv[m].x), axpy(al[1], pv[m].y, xv[m].y), axpy(al[2], pv[m].z, xv[m].z),
-                            axpy(al[3], pv[m].w, xv[m].w));
-        rv[m] = make_float4(axpy(-al[0], kv[m].x, rv[m].x), axpy(-al[1], kv[m].y, rv[m].y), axpy(-al[2], kv[m].z, rv[m].z),
-                            axpy(-al[3], kv[m].w, rv[m].w));
-        *reinterpret_cast<float4 *>(a.x + e) = xv[m];
+        float4 x4, k4;
+        if constexpr (kHold) {
+            x4 = xv[m];
+            k4 = kv[m];
+        } else {
+            x4 = load(a.x + e);
+            k4 = load(a.Kp + e);
+        }
+        x4 = make_float4(axpy(al[0], pv[m].x, x4.x), axpy(al[1], pv[m].y, x4.y), axpy(al[2], pv[m].z, x4.z),
+                         axpy(al[3], pv[m].w, x4.w));
+        rv[m] = make_float4(axpy(-al[0], k4.x, rv[m].x), axpy(-al[1], k4.y, rv[m].y), axpy(-al[2], k4.z, rv[m].z),
+                            axpy(-al[3], k4.w, rv[m].w));
+        *reinterpret_cast<float4 *>(a.x + e) = x4;
         *reinterpret_cast<float4 *>(a.r + e) = rv[m];
         add(m, rv[m], rv[m]);
         m4[0] = fmaxf(m4[0], fabsf(rv[m].x));
@@ -217,7 +253,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cg_cluster_kernel(const Cluster
         m4[k] = 0.0f;
     }
 #pragma unroll
-    for (int m = 0; m < kClVecs; ++m) {
+    for (int m = 0; m < VECS; ++m) {
         const int e = index(m);
         if (e < a.total) {
             if (ac[0]) pv[m].x = fmaf(be[0], pv[m].x, rv[m].x);
@@ -305,13 +341,12 @@ __global__ void __launch_bounds__(kClThreads, 1) cg_cluster_kernel(const Cluster
     if constexpr (CL > 1) cg::this_cluster().sync();  // rank 0 has read the others' maxima
 }
 
-template <int CL>
-cudaError_t launch_cluster(const ClusterArgs &a, cudaStream_t st) {
+template <int CL, int VECS>
+cudaLaunchConfig_t cluster_config(cudaLaunchAttribute (&at)[2], cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(CL, 1, 1);
     cfg.blockDim = dim3(kClThreads, 1, 1);
     cfg.stream = st;
-    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[0].val.programmaticStreamSerializationAllowed = 1;
     at[1].id = cudaLaunchAttributeClusterDimension;
@@ -320,13 +355,38 @@ cudaError_t launch_cluster(const ClusterArgs &a, cudaStream_t st) {
     at[1].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = CL > 1 ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, cg_cluster_kernel<CL>, a);
+    return cfg;
 }
+
+template <int CL, int VECS> cudaError_t launch_cluster(const ClusterArgs &a, cudaStream_t st) {
+    cudaLaunchAttribute at[2];
+    const cudaLaunchConfig_t cfg = cluster_config<CL, VECS>(at, st);
+    return cudaLaunchKernelEx(&cfg, cg_cluster_kernel<CL, VECS>, a);
+}
+
+// Whether the device takes clusters of 16 CTAs of the step (above the portable size of 8), asked once.
+bool wide_cluster_ok() {
+    static const bool ok = [] {
+        auto kernel = cg_cluster_kernel<kClWide, kClWideVecs>;
+        cudaLaunchAttribute at[2];
+        const cudaLaunchConfig_t cfg = cluster_config<kClWide, kClWideVecs>(at, nullptr);
+        int n = 0;
+        const bool fits = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                          cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0;
+        if (!fits) (void)cudaGetLastError();
+        return fits;
+    }();
+    return ok;
+}
+
+constexpr int64_t floats_of(int cl, int vecs) { return (int64_t)cl * kClThreads * 4 * vecs; }
 
 }  // namespace
 
-bool cg_cluster_ok(int64_t N, int t, const CgBuffers &b) {
-    return b.pc.k == 0 && t <= 64 && (t & (t - 1)) == 0 && N * t <= 8ll * kClThreads * 4 * kClVecs;
+bool cg_cluster_ok(int64_t N, int t, const CgBuffers &b, int S) {
+    if (b.pc.k > 0 || t > 64 || (t & (t - 1)) != 0) return false;
+    if (N * t <= floats_of(8, kClVecs)) return true;
+    return N * t <= floats_of(kClWide, kClWideVecs) && N * t * S <= kClWideParts && wide_cluster_ok();
 }
 
 cudaError_t launch_cg_cluster(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,
@@ -349,7 +409,8 @@ cudaError_t launch_cg_cluster(int64_t N, int t, const CgBuffers &b, const Produc
     if (split) a.sp = *split;
     a.N = N;
     const bool one = N * t <= kClThreads * 4 * kClVecs && N * t * std::max(1, tail.S) <= kClusterOneFloats;
-    return one ? launch_cluster<1>(a, st) : launch_cluster<8>(a, st);
+    if (one) return launch_cluster<1, kClVecs>(a, st);
+    return N * t <= floats_of(8, kClVecs) ? launch_cluster<8, kClVecs>(a, st) : launch_cluster<kClWide, kClWideVecs>(a, st);
 }
 
 }  // namespace lgp

@@ -606,7 +606,9 @@ lgp_status build_precond(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X, con
 // form), the split of p where it is not part of the step, and the step.
 int cg_iteration_launches(const lgp_ctx *ctx, const Prepared &pp, int t, int prec, const CgBuffers &b, int dist_form = -1) {
     const bool precond = b.pc.k > 0;
-    int n = 1 + (cg_cluster_ok(pp.N, t, b) ? 1 : 3);
+    const int64_t parts = is_tc(prec) ? mv_tc_partial_floats(pp.Np, t, ctx->num_sms, tc_splits_for(ctx, pp, t, prec))
+                                      : mv_simt_partial_floats(pp.N, pp.Np, t, ctx->num_sms);
+    int n = 1 + (cg_cluster_ok(pp.N, t, b, (int)(parts / (pp.Np * t))) ? 1 : 3);
     if (is_tc(prec)) {
         if (needs_dot(ctx, pp, t, prec) && dist_form < 0) ++n;
         if (precond) n += tc_fmt(prec) == 1 ? 2 : 1;

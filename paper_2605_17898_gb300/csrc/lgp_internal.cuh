@@ -396,7 +396,7 @@ struct CgBuffers {
 void launch_cg_init(const float *B, int64_t ldb, int64_t N, int64_t Np, int t, const CgBuffers &b, double tol,
                     int max_iter, int hist_len, cudaStream_t st, const float *X0 = nullptr, int64_t ldx0 = 0);
 // cg_cluster.cu: the whole step after the product as one launch, where the vectors are small enough for one cluster.
-bool cg_cluster_ok(int64_t N, int t, const CgBuffers &b);
+bool cg_cluster_ok(int64_t N, int t, const CgBuffers &b, int S);
 cudaError_t launch_cg_cluster(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,
                               cudaStream_t st);
 // One CG iteration after its product (b.Kp, or its partial sums in tail); split: p's halves for the next product.

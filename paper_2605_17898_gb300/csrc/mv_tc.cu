@@ -403,9 +403,9 @@ int64_t tc_vsplit_bytes(int64_t Np, int t) {
 
 // LGP_TC_BANDS=1 lets the dot-form symmetric product walk its tiles in column bands (tile_walk.cuh).
 // Measured at N = 500000, t = 32: the one-band order (every CTA on its own rows across all columns)
-// read 80.6 GB and wrote 34.0 GB of DRAM per product, against about 0.26 GB of operands, and took
-// 65.6 ms; the banded order moved 0.96 GB and took 68.2 ms (its walk costs registers in a kernel at
-// its register limit). So the default keeps the single band.
+// read 80.6 GB and wrote 34.0 GB of DRAM per product, against about 0.26 GB of operands; the banded order
+// moved 0.96 GB. They take 70.5 and 75.4 ms (D = 8, Matern-5/2; RBF, D = 2: 56.7 and 67.3), because the banded walk
+// costs registers in a kernel at its register limit. So the default keeps the single band.
 bool tcs_bands_enabled() {
     const char *env = std::getenv("LGP_TC_BANDS");
     return env && std::strcmp(env, "1") == 0;
