@@ -208,8 +208,9 @@ int32_t lgp_tc_kernel_choice(const lgp_ctx *ctx, int64_t N, int32_t D, int32_t k
  * inner products on the tensor cores (split float16 operands, float32 accumulation; Sec. 3 names
  * this rewriting of the distance as the reason its product time barely depends on D). The dot
  * form is used for RBF, Matern-3/2 and Matern-5/2 at D >= 2 when max_j |u_j|^2 stays below a
- * per-kernel limit that bounds its rounding error; otherwise, for Matern-1/2, D = 1, or with
- * LGP_DISTANCE=diff in the environment, the difference form runs.
+ * per-kernel limit that bounds its rounding error; otherwise, for Matern-1/2, D = 1, problems that
+ * the autotuner timed below 6144 rows (8192 at D <= 4), or with LGP_DISTANCE=diff in the environment, the
+ * difference form runs.
  * *form receives LGP_DIST_NONE (no symmetric product yet), LGP_DIST_DIFF or LGP_DIST_DOT;
  * *norm_max (may be NULL) the measured max_j |u_j|^2 when the dot form was considered, else -1.
  * Waits for the context's work and the given stream to finish. */
@@ -321,7 +322,7 @@ lgp_status lgp_rademacher_probes(lgp_ctx *ctx, uint64_t seed, int64_t N, int32_t
  * problem costs on each route on the caller's own data (the Sec. 5 gap: no batched solves):
  *   - the persistent batch: all such problems advance together, each CG iteration one
  *     float32 product launch over a work list of (problem, row block, column range)
- *     items plus one launch per vector update, the loop one CUDA graph with a
+ *     items plus one launch for every problem's CG step, the loop one CUDA graph with a
  *     device-side while node. A problem's cost there is its float32 product less that
  *     product's launch floor (timed on its first 256 rows), which the batch pays once;
  *   - the tensor-core route (problems of at least 2048 rows whose standalone CG iteration

@@ -410,10 +410,10 @@ bool kernel_timing_on(const lgp_ctx *ctx, cudaStream_t st) {
     return cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone;
 }
 
-// v_ready, tail: see launch_mv_tc (v_ready for the tensor-core products only).
+// v_ready, tail: see launch_mv_tc (v_ready for the tensor-core products only). rows: the float32 row kernel at any t.
 lgp_status matvec_prepared(lgp_ctx *ctx, const Prepared &pp, const float *V, int64_t ldv, float *out, int64_t ldo,
                            int t, int prec, const int *skip, cudaStream_t st, int dist_form = -1, bool v_ready = false,
-                           ProductTail *tail = nullptr, bool zeroed = false) {
+                           ProductTail *tail = nullptr, bool zeroed = false, bool rows = false) {
     if (is_tc(prec)) {
         lgp_status s = ensure(ctx, ctx->vsplit, (size_t)tc_vsplit_bytes(pp.Np, t));
         if (s != LGP_OK) return s;
@@ -441,10 +441,12 @@ lgp_status matvec_prepared(lgp_ctx *ctx, const Prepared &pp, const float *V, int
         }
         return LGP_OK;
     }
-    const int64_t pf = mv_simt_partial_floats(pp.N, pp.Np, t, ctx->num_sms);
+    const int64_t pf = rows ? mv_simt_cross_partial_floats(pp.N, pp.Np, pp.N, t, ctx->num_sms)
+                            : mv_simt_partial_floats(pp.N, pp.Np, t, ctx->num_sms);
     lgp_status s = ensure(ctx, ctx->mv_partial, (size_t)std::max<int64_t>(pf, 1) * sizeof(float));
     if (s != LGP_OK) return s;
     MvLaunch m;
+    m.rows = rows;
     m.kp = &pp.kp;
     m.Xs = pp.xs;
     m.N = pp.N;
@@ -931,10 +933,14 @@ lgp_status batch_route(lgp_ctx *ctx, const lgp_hyper *h, const float *X, int64_t
     };
     float ms_floor = 0.0f, ms_fp32 = 0.0f, ms_tc = 0.0f;
     Prepared pp;
+    // the product the persistent launch runs (at t <= 4 lgp_kernel_matvec has a faster one)
+    auto row_product = [&] {
+        return matvec_prepared(ctx, pp, B, t, out, t, t, LGP_PREC_FP32, nullptr, st, -1, false, nullptr, false, true);
+    };
     // the launch floor: the float32 product of the first rows only (B is row-major, so its first rows
     // are that problem's right-hand sides)
     if ((s = prepare_x(ctx, h, X, kFloorRows, st, &pp)) == LGP_OK)
-        s = timed([&] { return matvec_prepared(ctx, pp, B, t, out, t, t, LGP_PREC_FP32, nullptr, st); }, 2, &ms_floor);
+        s = timed(row_product, 2, &ms_floor);
     if (s == LGP_OK) s = prepare_x(ctx, h, X, N, st, &pp);
     if (s == LGP_OK) {
         LGP_CUDA(cudaMemsetAsync(vpad, 0, (size_t)pp.Np * tp * sizeof(float), st));
@@ -943,7 +949,7 @@ lgp_status batch_route(lgp_ctx *ctx, const lgp_hyper *h, const float *X, int64_t
         s = autotune_tc(ctx, pp, vpad, tp, out, tp, tp, LGP_PREC_SPLIT_F16, st);
     }
     if (s == LGP_OK)
-        s = timed([&] { return matvec_prepared(ctx, pp, B, t, out, t, t, LGP_PREC_FP32, nullptr, st); }, 2, &ms_fp32);
+        s = timed(row_product, 2, &ms_fp32);
     if (s == LGP_OK)
         s = timed([&] { return matvec_prepared(ctx, pp, vpad, tp, out, tp, tp, LGP_PREC_SPLIT_F16, nullptr, st); }, 2,
                   &ms_tc);

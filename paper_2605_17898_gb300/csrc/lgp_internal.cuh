@@ -271,6 +271,7 @@ struct MvLaunch {
     int num_sms;
     // With tail set, column-split partial sums are left to the caller (see ProductTail).
     struct ProductTail *tail = nullptr;
+    bool rows = false;    // the row-by-row kernel also where the symmetric one would run
     // Cross product out = K(Xr, Xs) V (no noise term): prescaled row points [Npr, dpad] and their
     // count; Xr == nullptr gives the square product K_y V.
     const float *Xr = nullptr;

@@ -199,7 +199,7 @@ cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st) {
     const bool cross = m.Xr != nullptr;
     const int64_t Nr = cross ? m.Nr : m.N, Npr = cross ? m.Npr : m.Np;
     if (m.tail) *m.tail = ProductTail();
-    const SymGrid sg = cross ? SymGrid() : sym_grid(m.N, m.Np, m.t, m.num_sms);
+    const SymGrid sg = cross || m.rows ? SymGrid() : sym_grid(m.N, m.Np, m.t, m.num_sms);
     if (sg.E && m.partial != nullptr && (int64_t)sg.G * m.Np * m.t <= m.partial_cap) {
         SymArgs a;
         a.Xs = m.Xs;
