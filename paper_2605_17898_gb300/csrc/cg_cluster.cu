@@ -14,6 +14,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "cg_reduce.cuh"
 #include "split.cuh"
@@ -364,9 +365,13 @@ template <int CL, int VECS> cudaError_t launch_cluster(const ClusterArgs &a, cud
     return cudaLaunchKernelEx(&cfg, cg_cluster_kernel<CL, VECS>, a);
 }
 
-// Whether the device takes clusters of 16 CTAs of the step (above the portable size of 8), asked once.
+// Whether the current device takes clusters of 16 CTAs of the step (above the portable size of 8); asked once per device.
 bool wide_cluster_ok() {
-    static const bool ok = [] {
+    static std::atomic<signed char> known[64];  // 0 not asked, 1 yes, -1 no
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return false;
+    signed char k = known[dev].load();
+    if (k == 0) {
         auto kernel = cg_cluster_kernel<kClWide, kClWideVecs>;
         cudaLaunchAttribute at[2];
         const cudaLaunchConfig_t cfg = cluster_config<kClWide, kClWideVecs>(at, nullptr);
@@ -374,9 +379,9 @@ bool wide_cluster_ok() {
         const bool fits = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
                           cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n > 0;
         if (!fits) (void)cudaGetLastError();
-        return fits;
-    }();
-    return ok;
+        known[dev].store(k = fits ? 1 : -1);
+    }
+    return k > 0;
 }
 
 constexpr int64_t floats_of(int cl, int vecs) { return (int64_t)cl * kClThreads * 4 * vecs; }

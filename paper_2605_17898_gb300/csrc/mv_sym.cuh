@@ -268,14 +268,10 @@ cudaError_t mv_sym_dispatch_m32(int D, int TT, const SymArgs &a, cudaStream_t st
 template <int KIND, int D, int TT>
 cudaError_t launch_mv_sym_inst(const SymArgs &a, cudaStream_t st) {
     const int bytes = sym_smem_bytes<D, TT>(a.E);
-    if (bytes > 48 * 1024) {
-        static bool configured = false;
-        if (!configured) {
-            const cudaError_t e = cudaFuncSetAttribute(mv_sym_kernel<KIND, D, TT>,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-            if (e != cudaSuccess) return e;
-            configured = true;
-        }
+    if (bytes > 48 * 1024) {  // set at every such launch: the attribute belongs to the current device
+        const cudaError_t e = cudaFuncSetAttribute(mv_sym_kernel<KIND, D, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   200 * 1024);
+        if (e != cudaSuccess) return e;
     }
     return launch_chained(mv_sym_kernel<KIND, D, TT>, dim3((unsigned)(a.G * (a.G + 1) / 2)), kSymThreads, bytes, st, a);
 }
