@@ -13,6 +13,7 @@ struct BatchGp {
     int64_t vec_off;   // row offset of this problem's vectors in the shared [rows, t] buffers
     int kind, dpad, D;
     float log2s2, noise;
+    EntryScale scale;
     int blk0, blk1;    // this problem's vector blocks [blk0, blk1)
     int splits;        // column splits of the product (1: items write K_y p directly)
     int64_t cols_per_split;

@@ -126,17 +126,17 @@ template <> struct Entry<LGP_MATERN32> {
     }
 };
 
-// Two entries at once from squared distances accumulated on packed float32x2 operations. The accumulation starts at
-// acc0: RBF folds the outputscale exponent into it (acc = rh2 - log2 s^2, k = 2^-acc), Matern-5/2 uses k = e + e (rh +
-// rh2 / 3). A packed operation on three different register pairs runs at half rate (mv_sym.cuh), so the
-// multiply-adds by constants are scalar.
+// Two entries at once from squared distances accumulated on packed float32x2 operations. The Matern entries take s^2 in
+// their exponent's one multiply-add; RBF entries are k / s^2 = 2^-rh2, and s^2 goes into V or the finished sums
+// (EntryScale): an accumulation that started at -log2 s^2 would save the same instruction, but each of its D additions
+// rounds at the size of log2 s^2 (D = 8, s^2 = 100, entry error 2.6e-7 against 9e-8; more where the distances are
+// small). Matern-5/2 uses k = e + e (rh + rh2 / 3). A packed operation on three different register pairs runs at half
+// rate (mv_sym.cuh), so the multiply-adds by constants are scalar.
 template <int KIND> struct PackedEntry;
 template <> struct PackedEntry<LGP_RBF> {
-    static __device__ __forceinline__ float2 acc0(float ls2) { return make_float2(-ls2, -ls2); }
-    static __device__ __forceinline__ float2 k(float2 acc, float) { return make_float2(ex2_approx(-acc.x), ex2_approx(-acc.y)); }
+    static __device__ __forceinline__ float2 k(float2 r2, float) { return make_float2(ex2_approx(-r2.x), ex2_approx(-r2.y)); }
 };
 template <> struct PackedEntry<LGP_MATERN52> {
-    static __device__ __forceinline__ float2 acc0(float) { return make_float2(0.0f, 0.0f); }
     static __device__ __forceinline__ float2 k(float2 r2, float ls2) {
         const float2 r = make_float2(sqrt_approx(r2.x), sqrt_approx(r2.y));
         const float2 e = make_float2(ex2_approx(fmaf(r.x, -kLog2e, ls2)), ex2_approx(fmaf(r.y, -kLog2e, ls2)));
@@ -145,19 +145,28 @@ template <> struct PackedEntry<LGP_MATERN52> {
     }
 };
 template <> struct PackedEntry<LGP_MATERN12> {
-    static __device__ __forceinline__ float2 acc0(float) { return make_float2(0.0f, 0.0f); }
     static __device__ __forceinline__ float2 k(float2 r2, float ls2) {
         return make_float2(ex2_approx(ls2 - sqrt_approx(r2.x)), ex2_approx(ls2 - sqrt_approx(r2.y)));
     }
 };
 template <> struct PackedEntry<LGP_MATERN32> {
-    static __device__ __forceinline__ float2 acc0(float) { return make_float2(0.0f, 0.0f); }
     static __device__ __forceinline__ float2 k(float2 r2, float ls2) {
         const float2 r = make_float2(sqrt_approx(r2.x), sqrt_approx(r2.y));
         const float2 e = make_float2(ex2_approx(fmaf(r.x, -kLog2e, ls2)), ex2_approx(fmaf(r.y, -kLog2e, ls2)));
         return __ffma2_rn(e, r, e);
     }
 };
+
+// What the kernels on PackedEntry multiply V and their finished sums by: s^2 for RBF, on the side where neither the
+// products nor the sums can leave the float32 range that the full entries had.
+struct EntryScale {
+    float v = 1.0f, out = 1.0f;
+};
+inline EntryScale entry_scale(int kind, float s2) {
+    EntryScale s;
+    if (kind == LGP_RBF) (s2 < 1.0f ? s.v : s.out) = s2;
+    return s;
+}
 
 // Host: the kind is one the library implements.
 inline bool kind_supported(int kind) {

@@ -34,6 +34,7 @@ struct SimtArgs {
     int64_t cols_per_split;
     int t;
     float log2s2;
+    EntryScale scale;
     float noise;
 };
 
@@ -99,14 +100,14 @@ template <int TT_, int R_, int THREADS> struct RowTile {
 template <int TT> using RowShape = RowTile<TT, TT == 32 ? 2 : 4, 64>;
 
 // sum_j k(x_i, x_j) V[j, c0..c0+TT) over jb <= j < je for this thread's rows i = row0 + r kThreads + tid, added up per
-// tile of kSimtBN columns. Distances run on packed operations over pairs of columns (x_j - x_i as x_j + (-x_i), the
+// tile of kSimtBN columns (scale: EntryScale). Distances run on packed operations over pairs of columns (x_j - x_i as x_j + (-x_i), the
 // row's coordinates kept twice), the V multiply-adds are scalar (three different register pairs would run at half
 // rate). xs [D][kSimtBN], vs [kSimtBN][TT], tot [kTotFloats]: shared memory.
 template <int KIND, int D, class S>
 __device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t row0, int64_t Npr,
                                           const float *__restrict__ Xs, int64_t Np, const float *__restrict__ V, int64_t ldv,
-                                          int c0, int t, int64_t jb, int64_t je, float log2s2, float *xs, float *vs, float *tot,
-                                          float (&sum)[S::R][S::TT]) {
+                                          int c0, int t, int64_t jb, int64_t je, float log2s2, EntryScale scale, float *xs, float *vs,
+                                          float *tot, float (&sum)[S::R][S::TT]) {
     constexpr int DP = DPad<D>::value, TT = S::TT, R = S::R, NT = S::kThreads;
     const int tid = threadIdx.x;
     float2 xi[R][D];
@@ -124,7 +125,6 @@ __device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t 
             if constexpr (S::kTotShared) tot[(r * TT + c) * NT + tid] = 0.0f;
         }
     }
-    const float2 acc0 = PackedEntry<KIND>::acc0(log2s2);
     for (int64_t j0 = jb; j0 < je; j0 += kSimtBN) {
         __syncthreads();
         for (int e = tid; e < kSimtBN * (DP / 4); e += NT) {
@@ -138,7 +138,7 @@ __device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t 
         }
         for (int e = tid; e < kSimtBN * TT; e += NT) {
             const int jj = e / TT, c = e - jj * TT;
-            vs[e] = (j0 + jj < je && c0 + c < t) ? V[(j0 + jj) * ldv + c0 + c] : 0.0f;
+            vs[e] = (j0 + jj < je && c0 + c < t) ? V[(j0 + jj) * ldv + c0 + c] * scale.v : 0.0f;
         }
         __syncthreads();
         float acc[R][TT];
@@ -154,7 +154,7 @@ __device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t 
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 float2 dd = __fadd2_rn(xj[0], xi[r][0]);
-                float2 r2 = __ffma2_rn(dd, dd, acc0);
+                float2 r2 = __fmul2_rn(dd, dd);
 #pragma unroll
                 for (int d = 1; d < D; ++d) {
                     dd = __fadd2_rn(xj[d], xi[r][d]);
@@ -192,12 +192,13 @@ __device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t 
                 else sum[r][c] += acc[r][c];
             }
     }
-    if constexpr (S::kTotShared) {
 #pragma unroll
-        for (int r = 0; r < R; ++r)
+    for (int r = 0; r < R; ++r)
 #pragma unroll
-            for (int c = 0; c < TT; ++c) sum[r][c] = tot[(r * TT + c) * NT + tid];
-    }
+        for (int c = 0; c < TT; ++c) {
+            if constexpr (S::kTotShared) sum[r][c] = tot[(r * TT + c) * NT + tid];
+            sum[r][c] *= scale.out;
+        }
 }
 
 template <int KIND, int D, int TT>
@@ -214,7 +215,7 @@ __global__ void __launch_bounds__(RowShape<TT>::kThreads) mv_simt_kernel(SimtArg
     const int64_t jb = (int64_t)blockIdx.y * a.cols_per_split;
     const int64_t je = min(a.N, jb + a.cols_per_split);
     float sum[S::R][TT];
-    simt_rows<KIND, D, S>(a.Xr, row0, a.Npr, a.Xs, a.Np, a.V, a.ldv, c0, a.t, jb, je, a.log2s2, xs, vs, tot, sum);
+    simt_rows<KIND, D, S>(a.Xr, row0, a.Npr, a.Xs, a.Np, a.V, a.ldv, c0, a.t, jb, je, a.log2s2, a.scale, xs, vs, tot, sum);
 #pragma unroll
     for (int r = 0; r < S::R; ++r) {
         const int64_t i = row0 + r * S::kThreads + threadIdx.x;

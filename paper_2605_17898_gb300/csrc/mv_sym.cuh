@@ -41,6 +41,7 @@ struct SymArgs {
     int64_t N, Np, ldv;
     int E, G, t;
     float log2s2;
+    EntryScale scale;
 };
 
 constexpr int kSymThreads = 128;  // 4 warps, a quarter of the tile's columns each
@@ -131,13 +132,12 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
     }
     for (int e = tid; e < E * TT; e += kSymThreads) {
         const int j = e / TT, c = e - j * TT;
-        vs[e] = (j0 + j < a.N && c < a.t) ? a.V[(j0 + j) * a.ldv + c] : 0.0f;
+        vs[e] = (j0 + j < a.N && c < a.t) ? a.V[(j0 + j) * a.ldv + c] * a.scale.v : 0.0f;
     }
     for (int e = tid; e < WR * E * TT; e += kSymThreads) col[e] = 0.0f;
     __syncthreads();
 
     const float ls2 = a.log2s2;
-    const float2 acc_init = PackedEntry<KIND>::acc0(ls2);
     const int wr = warp / WC, wc = warp % WC;
     const int cw = E / WC, c_lo = wc * cw;  // columns of this warp
     float *mycol = col + wr * E * TT + sym_fold_index<NV>(lane);
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
             for (int d = 0; d < D; ++d) xi[r][d] = make_float2(x[d], x[d]);
 #pragma unroll
             for (int c = 0; c < TT; ++c) {
-                vi[r][c] = i < a.N && c < a.t ? a.V[i * a.ldv + c] : 0.0f;
+                vi[r][c] = i < a.N && c < a.t ? a.V[i * a.ldv + c] * a.scale.v : 0.0f;
                 acc[r][c] = 0.0f;
             }
         }
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     float2 dd = __fadd2_rn(xj[h][0], xi[r][0]);
-                    float2 r2 = __ffma2_rn(dd, dd, acc_init);
+                    float2 r2 = __fmul2_rn(dd, dd);
 #pragma unroll
                     for (int d = 1; d < D; ++d) {
                         dd = __fadd2_rn(xj[h][d], xi[r][d]);
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
                 const int64_t i = i0 + rb + rl * R + r;
                 if (cl == (r & 3)) {
                     if (WC > 1) rowbuf[(warp * RB + rl * R + r) * TT + q] = v;
-                    else if (i < a.N && q < a.t) a.part[((int64_t)J * a.Np + i) * a.t + q] = v;
+                    else if (i < a.N && q < a.t) a.part[((int64_t)J * a.Np + i) * a.t + q] = v * a.scale.out;
                 }
             }
         if (WC > 1) {
@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
                 const int64_t i = i0 + rb0 + e / TT;
                 float v = 0.0f;
                 for (int k = 0; k < WC; ++k) v += rowbuf[(w0 * WC + k) * RB * TT + e - w0 * RB * TT];
-                if (i < a.N && c < a.t) a.part[((int64_t)J * a.Np + i) * a.t + c] = v;
+                if (i < a.N && c < a.t) a.part[((int64_t)J * a.Np + i) * a.t + c] = v * a.scale.out;
             }
             __syncthreads();
         }
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
         const int j = e / TT, c = e - j * TT;
         float v = 0.0f;
         for (int w = 0; w < WR; ++w) v += col[w * E * TT + e];
-        if (j0 + j < a.N && c < a.t) a.part[((int64_t)I * a.Np + j0 + j) * a.t + c] = v;
+        if (j0 + j < a.N && c < a.t) a.part[((int64_t)I * a.Np + j0 + j) * a.t + c] = v * a.scale.out;
     }
 }
 
