@@ -442,7 +442,7 @@ lgp_status matvec_prepared(lgp_ctx *ctx, const Prepared &pp, const float *V, int
         return LGP_OK;
     }
     const int64_t pf = rows ? mv_simt_cross_partial_floats(pp.N, pp.Np, pp.N, t, ctx->num_sms)
-                            : mv_simt_partial_floats(pp.N, pp.Np, t, ctx->num_sms);
+                            : mv_simt_partial_floats(pp.N, pp.Np, t, pp.kp.D, ctx->num_sms);
     lgp_status s = ensure(ctx, ctx->mv_partial, (size_t)std::max<int64_t>(pf, 1) * sizeof(float));
     if (s != LGP_OK) return s;
     MvLaunch m;
@@ -609,7 +609,7 @@ lgp_status build_precond(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X, con
 int cg_iteration_launches(const lgp_ctx *ctx, const Prepared &pp, int t, int prec, const CgBuffers &b, int dist_form = -1) {
     const bool precond = b.pc.k > 0;
     const int64_t parts = is_tc(prec) ? mv_tc_partial_floats(pp.Np, t, ctx->num_sms, tc_splits_for(ctx, pp, t, prec))
-                                      : mv_simt_partial_floats(pp.N, pp.Np, t, ctx->num_sms);
+                                      : mv_simt_partial_floats(pp.N, pp.Np, t, pp.kp.D, ctx->num_sms);
     int n = 1 + (cg_cluster_ok(pp.N, t, b, (int)(parts / (pp.Np * t))) ? 1 : 3);
     if (is_tc(prec)) {
         if (needs_dot(ctx, pp, t, prec) && dist_form < 0) ++n;
@@ -635,7 +635,7 @@ lgp_status run_cg(lgp_ctx *ctx, const Prepared &pp, const float *B, int64_t ldb,
         const int64_t pf = mv_tc_partial_floats(pp.Np, t, ctx->num_sms, tc_splits_for(ctx, pp, t, prec));
         if ((s = ensure(ctx, ctx->mv_partial, (size_t)std::max<int64_t>(pf, 1) * sizeof(float))) != LGP_OK) return s;
     } else {
-        const int64_t pf = mv_simt_partial_floats(pp.N, pp.Np, t, ctx->num_sms);
+        const int64_t pf = mv_simt_partial_floats(pp.N, pp.Np, t, pp.kp.D, ctx->num_sms);
         if ((s = ensure(ctx, ctx->mv_partial, (size_t)std::max<int64_t>(pf, 1) * sizeof(float))) != LGP_OK) return s;
     }
     // the X-only operands of the products, once for the whole solve (outside the captured loop)

@@ -287,7 +287,7 @@ struct MvLaunch {
     int64_t Nr = 0, Npr = 0;
 };
 cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st);
-int64_t mv_simt_partial_floats(int64_t N, int64_t Np, int t, int num_sms);
+int64_t mv_simt_partial_floats(int64_t N, int64_t Np, int t, int D, int num_sms);
 // Split partial floats of the cross product with Nr output rows (Npr padded) and N columns.
 int64_t mv_simt_cross_partial_floats(int64_t Nr, int64_t Npr, int64_t N, int t, int num_sms);
 

@@ -44,15 +44,18 @@ int64_t choose_split(int64_t N, int64_t row_blocks, int64_t col_groups, int num_
 }
 
 // Symmetric product (mv_sym.cuh): block edge E, blocks G and padded column count TT for a square product of N rows
-// and t columns, or E = 0 where the row-by-row kernel runs (t > 4; or N so large that the partial sums, G per row,
-// would take more than 256 MiB even with the largest blocks).
+// and t columns, or E = 0 where the row-by-row kernel runs: t > 4; or N so large that the partial sums, G per row,
+// would take more than 256 MiB with E = 512 and E = 1024 does not help. Blocks of 1024 need two CTAs of 4 warps on an SM:
+// with one (114 KB of shared memory at D = 8, 4 padded columns) N = 100000, D = 8, t = 4, Matern-5/2 took 10.3 ms, the row
+// kernel takes 7.2; at D = 7 they take 6.8 against 8.1 (N = 110000), at t = 1, N = 200000, D = 4 10.0 against 17.2.
 struct SymGrid {
     int E = 0, G = 0, TT = 0;
 };
 
 constexpr int64_t kSymMaxPartial = 256ll << 20;
+constexpr int kSmShared = 228 * 1024, kCtaReserved = 1024;  // bytes of shared memory of an SM, and the system's share per CTA
 
-SymGrid sym_grid(int64_t N, int64_t Np, int t, int num_sms) {
+SymGrid sym_grid(int64_t N, int64_t Np, int t, int D, int num_sms) {
     SymGrid g;
     if (t > 4) return g;
     // The largest blocks that still give every SM enough tiles to even out the last ones (a tile's set-up and its
@@ -68,7 +71,7 @@ SymGrid sym_grid(int64_t N, int64_t Np, int t, int num_sms) {
     else if (tiles_per_sm(256) >= 8) E = 256;
     else if (tiles_per_sm(128) >= 5) E = 128;
     auto bytes = [&](int64_t e) { return (N + e - 1) / e * Np * t * (int64_t)sizeof(float); };
-    if (E == 512 && bytes(E) > kSymMaxPartial) E = 1024;
+    if (E == 512 && bytes(E) > kSymMaxPartial && 2 * (sym_smem_bytes(D, TT, 1024) + kCtaReserved) <= kSmShared) E = 1024;
     if (bytes(E) > kSymMaxPartial) return g;
     g.E = (int)E;
     g.G = (int)((N + E - 1) / E);
@@ -157,8 +160,8 @@ inline int grid_for(int64_t n) {
 
 }  // namespace
 
-int64_t mv_simt_partial_floats(int64_t N, int64_t Np, int t, int num_sms) {
-    const SymGrid sg = sym_grid(N, Np, t, num_sms);
+int64_t mv_simt_partial_floats(int64_t N, int64_t Np, int t, int D, int num_sms) {
+    const SymGrid sg = sym_grid(N, Np, t, D, num_sms);
     if (sg.E) return (int64_t)sg.G * Np * t;
     const SimtShape sh = simt_shape(t);
     const int64_t BM = sh.BM;
@@ -199,7 +202,7 @@ cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st) {
     const bool cross = m.Xr != nullptr;
     const int64_t Nr = cross ? m.Nr : m.N, Npr = cross ? m.Npr : m.Np;
     if (m.tail) *m.tail = ProductTail();
-    const SymGrid sg = cross || m.rows ? SymGrid() : sym_grid(m.N, m.Np, m.t, m.num_sms);
+    const SymGrid sg = cross || m.rows ? SymGrid() : sym_grid(m.N, m.Np, m.t, m.kp->D, m.num_sms);
     if (sg.E && m.partial != nullptr && (int64_t)sg.G * m.Np * m.t <= m.partial_cap) {
         SymArgs a;
         a.Xs = m.Xs;

@@ -57,9 +57,10 @@ template <int D, int TT> struct SymShape {
 template <int D, int TT> __host__ __device__ constexpr int sym_row_sets(int E) {
     return E >= 4 * SymShape<D, TT>::RB ? 4 : E / SymShape<D, TT>::RB;
 }
-template <int D, int TT>
-constexpr int sym_smem_bytes(int E) {
-    return (E * (D + TT + TT * sym_row_sets<D, TT>(E)) + 4 * SymShape<D, TT>::RB * TT) * 4;
+// Shared memory of a CTA: column side, column sums of the row sets, row sums.
+constexpr int sym_smem_bytes(int D, int TT, int E) {
+    const int RB = D <= 4 && TT <= 2 ? 64 : 32, sets = E >= 4 * RB ? 4 : E / RB;
+    return (E * (D + TT + TT * sets) + 4 * RB * TT) * 4;
 }
 
 // v[0..NV) summed over the 8 lanes that differ in bits 0..2: the lane keeps values sym_fold_index(lane) + 0 ..
@@ -267,7 +268,8 @@ cudaError_t mv_sym_dispatch_m32(int D, int TT, const SymArgs &a, cudaStream_t st
 
 template <int KIND, int D, int TT>
 cudaError_t launch_mv_sym_inst(const SymArgs &a, cudaStream_t st) {
-    const int bytes = sym_smem_bytes<D, TT>(a.E);
+    static_assert(SymShape<D, TT>::RB == (D <= 4 && TT <= 2 ? 64 : 32), "sym_smem_bytes and SymShape agree");
+    const int bytes = sym_smem_bytes(D, TT, a.E);
     if (bytes > 48 * 1024) {  // set at every such launch: the attribute belongs to the current device
         const cudaError_t e = cudaFuncSetAttribute(mv_sym_kernel<KIND, D, TT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    200 * 1024);
