@@ -355,6 +355,11 @@ int32_t lgp_batch_split_choice(const lgp_ctx *ctx, int64_t N, int32_t D, int32_t
  * persistent launch, at least four 64-column tiles per split (diagnostic). */
 int32_t lgp_batch_split_rule(const lgp_ctx *ctx, int64_t N);
 
+/* How the last CG solve of this context ran the vector updates of an iteration (diagnostic): the CTAs of the one
+ * thread-block cluster that ran them (1, 8 or 16), 0 for three launches, -1 before the first solve (the
+ * persistent part of a batched solve does not count). */
+int32_t lgp_cg_step_ctas(const lgp_ctx *ctx);
+
 /*
  * Measurement support (no counterpart in the paper): throughput of one GPU pipe on the
  * current device, timed with CUDA events on `stream` at the clock the GPU runs.

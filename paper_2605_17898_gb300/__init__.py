@@ -56,7 +56,7 @@ EXPORTED = [
     "lgp_kernel_matvec", "lgp_kernel_matvec_grad", "lgp_cg_solve", "lgp_lml_and_grad",
     "lgp_rademacher_probes", "lgp_batch_cg_solve", "lgp_kernel_matvec_noalloc",
     "lgp_measure_pipe_peak", "lgp_tc_kernel_choice", "lgp_predict", "lgp_tc_distance_form",
-    "lgp_kernel_matvec_noalloc_status", "lgp_batch_route_choice", "lgp_batch_split_choice", "lgp_batch_split_rule",
+    "lgp_kernel_matvec_noalloc_status", "lgp_batch_route_choice", "lgp_batch_split_choice", "lgp_cg_step_ctas", "lgp_batch_split_rule",
     "lgp_set_kernel_timing", "lgp_last_kernel_ms",
 ]
 
@@ -134,6 +134,7 @@ def load(path: str | None = None) -> ctypes.CDLL:
         "lgp_batch_route_choice": (c.c_int32, [vp, c.c_int64, c.c_int32, c.c_int32, c.c_int32]),
         "lgp_batch_split_choice": (c.c_int32, [vp, c.c_int64, c.c_int32, c.c_int32, c.c_int32]),
         "lgp_batch_split_rule": (c.c_int32, [vp, c.c_int64]),
+        "lgp_cg_step_ctas": (c.c_int32, [vp]),
         "lgp_set_kernel_timing": (c.c_int32, [vp, c.c_int32]),
         "lgp_last_kernel_ms": (c.c_int32, [vp, c.POINTER(c.c_float)]),
     }
@@ -274,6 +275,10 @@ class Context:
     def batch_split_rule(self, N: int) -> int:
         """The fixed rule's column-split count for a problem of N rows alone."""
         return int(self.lib.lgp_batch_split_rule(self.h, int(N)))
+
+    def cg_step_ctas(self) -> int:
+        """CTAs of the cluster that ran the last CG solve's vector updates, 0 for three launches, -1 before the first."""
+        return int(self.lib.lgp_cg_step_ctas(self.h))
 
     def tc_distance_form(self, stream=None) -> tuple[int, float]:
         """(LGP_DIST_NONE / LGP_DIST_DIFF / LGP_DIST_DOT, max |u|^2 or -1) of the last symmetric product."""

@@ -5,8 +5,13 @@
 // What bounds it: latency. The three launches of solver.cu cost about 2 us each beyond their work, and between them
 // every vector goes to L2 and back; here up to 65536 elements of x, r, p and Kp are read once into the registers of 8
 // CTAs (the portable cluster size; one CTA, without a barrier, where a single SM can take the product's partial sums in
-// about a microsecond). Up to 262144 elements 16 CTAs keep p and r and read x and Kp once more; that holds while their SMs
-// can also take the product's partial sums in a few microseconds.
+// about a microsecond). Up to 262144 elements 16 CTAs keep p and r and read x and Kp once more.
+//
+// The product's partial sums (S per element) are read by the cluster's SMs alone, so they bound each size (cg_step_rule): 8
+// CTAs take 2^20 of them, 16 CTAs 2^22, beyond that the three launches' 76 blocks are faster. Time of an iteration with its
+// product (us), 8 CTAs / 16 CTAs / three launches: N = 8000, t = 2, 1.0M 47.9 / 49.8 / 54.8; N = 4500, t = 4, 1.3M 52.0 / 47.9 /
+// 52.8; N = 4000, t = 8, 2.0M 39.8 / 36.2 / 41.9; N = 12000, t = 2, 2.3M 93.1 / 84.9 / 90.7; N = 16000, t = 4, 4.0M 165.8 / 155.7 /
+// 158.0; N = 8000, t = 8, 8M 108 / - / 82.8; N = 9000, t = 8, 5.1M - / 98.8 / 93.6.
 //
 // Measured against the three launches: solve of N = 1024, t = 1, ~90 iterations 1.62 -> 0.95 ms; training step of N = 2000,
 // D = 8, t = 16 4.65 -> 3.73 ms; with 16 CTAs, solves at t = 32 of N = 3000 4.54 -> 4.18 ms, N = 8000 8.02 -> 7.53; at
@@ -28,8 +33,8 @@ namespace cg = cooperative_groups;
 constexpr int kClThreads = 512;
 constexpr int kClVecs = 4;  // float4s per thread and vector that are all held in registers
 constexpr int kClWide = 16, kClWideVecs = 8;  // larger vectors
-constexpr int64_t kClWideParts = 1 << 21;     // partial sums that a cluster of 16 takes (about 4 us of its SMs' loads)
-constexpr int64_t kClusterOneFloats = 1 << 15;  // partial sums that one CTA takes alone (about 1.3 us of its SM's loads)
+// partial sums that a cluster of 1, 8 and 16 CTAs takes (about 1.3, 4 and 8 us of its SMs' loads)
+constexpr int64_t kClusterOneParts = 1 << 15, kClParts = 1 << 20, kClWideParts = 1 << 22;
 
 struct ClusterArgs {
     float *x, *r, *p, *Kp;
@@ -388,13 +393,19 @@ constexpr int64_t floats_of(int cl, int vecs) { return (int64_t)cl * kClThreads 
 
 }  // namespace
 
-bool cg_cluster_ok(int64_t N, int t, const CgBuffers &b, int S) {
-    if (b.pc.k > 0 || t > 64 || (t & (t - 1)) != 0) return false;
-    if (N * t <= floats_of(8, kClVecs)) return true;
-    return N * t <= floats_of(kClWide, kClWideVecs) && N * t * S <= kClWideParts && wide_cluster_ok();
+int cg_step_rule(int64_t N, int t, int S, bool wide) {
+    if (t > 64 || (t & (t - 1)) != 0) return 0;
+    const int64_t elems = N * t, parts = elems * S;
+    if (elems <= floats_of(1, kClVecs) && std::max(elems, parts) <= kClusterOneParts) return 1;
+    if (elems <= floats_of(8, kClVecs) && parts <= kClParts) return 8;
+    return wide && elems <= floats_of(kClWide, kClWideVecs) && parts <= kClWideParts ? kClWide : 0;
 }
 
-cudaError_t launch_cg_cluster(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,
+int cg_step_ctas(int64_t N, int t, const CgBuffers &b, int S) {
+    return b.pc.k > 0 ? 0 : cg_step_rule(N, t, S, wide_cluster_ok());
+}
+
+cudaError_t launch_cg_cluster(int ctas, int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,
                               cudaStream_t st) {
     ClusterArgs a = {};
     a.x = b.x;
@@ -413,9 +424,9 @@ cudaError_t launch_cg_cluster(int64_t N, int t, const CgBuffers &b, const Produc
     a.split = split ? 1 : 0;
     if (split) a.sp = *split;
     a.N = N;
-    const bool one = N * t <= kClThreads * 4 * kClVecs && N * t * std::max(1, tail.S) <= kClusterOneFloats;
-    if (one) return launch_cluster<1, kClVecs>(a, st);
-    return N * t <= floats_of(8, kClVecs) ? launch_cluster<8, kClVecs>(a, st) : launch_cluster<kClWide, kClWideVecs>(a, st);
+    return ctas == 1 ? launch_cluster<1, kClVecs>(a, st)
+         : ctas == 8 ? launch_cluster<8, kClVecs>(a, st)
+                     : launch_cluster<kClWide, kClWideVecs>(a, st);
 }
 
 }  // namespace lgp

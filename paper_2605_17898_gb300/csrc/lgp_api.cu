@@ -65,6 +65,7 @@ struct lgp_ctx {
     int sym_kind = -1, sym_D = 0, sym_t = 0;
     int64_t sym_Np = 0;
     bool sym_dot = false;  // whether it considered the dot form
+    int cg_step = -1;      // the last CG solve's vector step (lgp_cg_step_ctas)
     // prepare_x calls so far; the X-only operands of the tensor-core products in vsplit (transposed X,
     // with opnd_dot also the dot-form distance operands) belong to prepared X number opnd_version (built for
     // opnd_t columns at workspace address opnd_buf), 0 = none
@@ -604,13 +605,18 @@ lgp_status build_precond(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X, con
     return LGP_OK;
 }
 
+// CTAs of the cluster that runs the vector step of a CG solve (cg_step_ctas).
+int cg_solve_step(const lgp_ctx *ctx, const Prepared &pp, int t, int prec, const CgBuffers &b) {
+    const int64_t parts = is_tc(prec) ? mv_tc_partial_floats(pp.Np, t, ctx->num_sms, tc_splits_for(ctx, pp, t, prec))
+                                      : mv_simt_partial_floats(pp.N, pp.Np, t, pp.kp.D, ctx->num_sms);
+    return cg_step_ctas(pp.N, t, b, (int)(parts / (pp.Np * t)));
+}
+
 // Kernel launches of one CG iteration: the product kernel (both distance instances where the host does not know the
 // form), the split of p where it is not part of the step, and the step.
 int cg_iteration_launches(const lgp_ctx *ctx, const Prepared &pp, int t, int prec, const CgBuffers &b, int dist_form = -1) {
     const bool precond = b.pc.k > 0;
-    const int64_t parts = is_tc(prec) ? mv_tc_partial_floats(pp.Np, t, ctx->num_sms, tc_splits_for(ctx, pp, t, prec))
-                                      : mv_simt_partial_floats(pp.N, pp.Np, t, pp.kp.D, ctx->num_sms);
-    int n = 1 + (cg_cluster_ok(pp.N, t, b, (int)(parts / (pp.Np * t))) ? 1 : 3);
+    int n = 1 + (cg_solve_step(ctx, pp, t, prec, b) > 0 ? 1 : 3);
     if (is_tc(prec)) {
         if (needs_dot(ctx, pp, t, prec) && dist_form < 0) ++n;
         if (precond) n += tc_fmt(prec) == 1 ? 2 : 1;
@@ -657,6 +663,7 @@ lgp_status run_cg(lgp_ctx *ctx, const Prepared &pp, const float *B, int64_t ldb,
     s = cg_buffers(ctx, pp.N, pp.Np, t, hist_len, &b);
     if (s != LGP_OK) return s;
     if (pc) b.pc = *pc;
+    ctx->cg_step = cg_solve_step(ctx, pp, t, prec, b);
 
     if (X0) {
         // warm start: r0 = b - K_y x0 needs one product first (into Kp)
@@ -1380,6 +1387,8 @@ int32_t lgp_batch_split_rule(const lgp_ctx *ctx, int64_t N) {
     if (!ctx || N < 1) return LGP_ERR_INVALID_ARG;
     return (int32_t)batch_split_rule(ctx, N);
 }
+
+int32_t lgp_cg_step_ctas(const lgp_ctx *ctx) { return ctx ? ctx->cg_step : LGP_ERR_INVALID_ARG; }
 
 lgp_status lgp_tc_distance_form(lgp_ctx *ctx, lgp_stream stream, int32_t *form, float *norm_max) {
     if (!ctx || !form) return LGP_ERR_INVALID_ARG;

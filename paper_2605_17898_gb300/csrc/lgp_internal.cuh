@@ -405,9 +405,11 @@ struct CgBuffers {
 // X0 (may be null): warm start x0 [N, ldx0], with K_y x0 already in b.Kp.
 void launch_cg_init(const float *B, int64_t ldb, int64_t N, int64_t Np, int t, const CgBuffers &b, double tol,
                     int max_iter, int hist_len, cudaStream_t st, const float *X0 = nullptr, int64_t ldx0 = 0);
-// cg_cluster.cu: the whole step after the product as one launch, where the vectors are small enough for one cluster.
-bool cg_cluster_ok(int64_t N, int t, const CgBuffers &b, int S);
-cudaError_t launch_cg_cluster(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,
+// cg_cluster.cu: the whole step after the product as one launch of a cluster, where the vectors and the S partial sums per
+// element that the product left are few enough: its CTAs (1, 8 or 16), or 0 for three launches. wide: 16 are possible.
+int cg_step_rule(int64_t N, int t, int S, bool wide);
+int cg_step_ctas(int64_t N, int t, const CgBuffers &b, int S);
+cudaError_t launch_cg_cluster(int ctas, int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,
                               cudaStream_t st);
 // One CG iteration after its product (b.Kp, or its partial sums in tail); split: p's halves for the next product.
 void launch_cg_after_matvec(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,

@@ -791,7 +791,8 @@ void launch_step(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, 
 
 void launch_cg_after_matvec(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,
                             cudaStream_t st) {
-    if (cg_cluster_ok(N, t, b, tail.part ? tail.S : 0)) launch_cg_cluster(N, t, b, tail, split, st);
+    const int ctas = cg_step_ctas(N, t, b, tail.part ? tail.S : 0);
+    if (ctas > 0) launch_cg_cluster(ctas, N, t, b, tail, split, st);
     else if (t <= 64 && (t & (t - 1)) == 0) launch_step<4>(N, t, b, tail, split, st);
     else launch_step<1>(N, t, b, tail, split, st);
 }

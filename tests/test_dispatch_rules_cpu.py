@@ -35,3 +35,26 @@ def test_blocks_of_1024_rows_need_two_ctas_on_an_sm(slots, N, t, D):
     else:
         assert slots(N, t, D) not in (blocks, -(-N // 512))
     assert slots(N, t, D) * N * t * 4 <= 256 << 20
+
+
+@pytest.fixture(scope="module")
+def step():
+    from paper_2605_17898_gb300 import build as b
+    fn = getattr(ctypes.CDLL(b.build()), "_ZN3lgp12cg_step_ruleEliib")  # lgp::cg_step_rule
+    fn.restype = ctypes.c_int
+    fn.argtypes = [ctypes.c_int64, ctypes.c_int, ctypes.c_int, ctypes.c_bool]
+    return fn
+
+
+@pytest.mark.parametrize("N,t,S,ctas", [
+    (1024, 1, 16, 1), (500, 8, 8, 1), (8192, 1, 5, 8), (1, 1, 0, 1), (8192, 1, 0, 1), (8193, 1, 0, 8),
+    (8000, 2, 63, 8), (4500, 4, 71, 16), (8000, 8, 125, 0),   # 1.0, 1.3 and 8 million partial sums
+    (65000, 1, 127, 0), (16000, 4, 63, 16), (9000, 8, 71, 0),
+    (65536, 1, 16, 8), (65536, 1, 17, 16), (262144, 1, 16, 16), (262144, 1, 17, 0), (8193, 32, 0, 0),
+    (1000, 3, 1, 0), (100, 128, 0, 0),
+])
+def test_cluster_of_the_cg_step(step, N, t, S, ctas):
+    """One cluster runs a CG step only where its SMs can also take the product's S partial sums per element: beyond 2^20 (8 CTAs) and
+    2^22 (16) the step had become slower than the launches it replaced."""
+    assert step(N, t, S, True) == ctas
+    assert step(N, t, S, False) == (0 if ctas == 16 else ctas)
