@@ -12,7 +12,7 @@ struct BatchGp {
     int64_t xs_off;    // float offset of this problem's prescaled X in the shared buffer
     int64_t vec_off;   // row offset of this problem's vectors in the shared [rows, t] buffers
     int kind, dpad, D;
-    float log2s2, noise;
+    float noise;
     EntryScale scale;
     int blk0, blk1;    // this problem's vector blocks [blk0, blk1)
     int splits;        // column splits of the product (1: items write K_y p directly)

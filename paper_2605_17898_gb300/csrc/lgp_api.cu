@@ -1051,8 +1051,7 @@ void plan_add_problem(BatchPlan &P, int64_t N, const KernelParams &kp, const flo
     G.kind = kp.kind;
     G.dpad = kp.dpad;
     G.D = kp.D;
-    G.log2s2 = kp.log2_s2;
-    G.scale = entry_scale(kp.kind, kp.s2);
+    G.scale = entry_scale(kp);
     G.noise = kp.noise;
     G.B = B;
     G.Xsol = Xsol;

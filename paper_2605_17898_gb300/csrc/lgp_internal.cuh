@@ -126,17 +126,20 @@ template <> struct Entry<LGP_MATERN32> {
     }
 };
 
-// Two entries at once from squared distances accumulated on packed float32x2 operations. The Matern entries take s^2 in
-// their exponent's one multiply-add; RBF entries are k / s^2 = 2^-rh2, and s^2 goes into V or the finished sums
-// (EntryScale): an accumulation that started at -log2 s^2 would save the same instruction, but each of its D additions
-// rounds at the size of log2 s^2 (D = 8, s^2 = 100, entry error 2.6e-7 against 9e-8; more where the distances are
-// small). Matern-5/2 uses k = e + e (rh + rh2 / 3). A packed operation on three different register pairs runs at half
-// rate (mv_sym.cuh), so the multiply-adds by constants are scalar.
+// Two entries at once from squared distances accumulated on packed float32x2 operations from acc0. The Matern entries take
+// s^2 in their exponent's one multiply-add; RBF entries are k = 2^-(rh2 + acc0) with an ls2 of 0 (EntryScale), and s^2 goes
+// into V or the finished sums: accumulated from -log2 s^2, each of the D additions rounds at that size (D = 8, s^2 = 100,
+// entry error 2.6e-7 against 9e-8; more where the distances are small). (The start stays an operand: with a plain product for the
+// first square the row kernel's schedule comes out 4% slower, N = 20000, D = 2, t = 48 1310 -> 1364 us.) Matern-5/2 uses
+// k = e + e (rh + rh2 / 3). A packed operation on three different register pairs runs at half rate (mv_sym.cuh), so the
+// multiply-adds by constants are scalar.
 template <int KIND> struct PackedEntry;
 template <> struct PackedEntry<LGP_RBF> {
-    static __device__ __forceinline__ float2 k(float2 r2, float) { return make_float2(ex2_approx(-r2.x), ex2_approx(-r2.y)); }
+    static __device__ __forceinline__ float2 acc0(float ls2) { return make_float2(-ls2, -ls2); }
+    static __device__ __forceinline__ float2 k(float2 acc, float) { return make_float2(ex2_approx(-acc.x), ex2_approx(-acc.y)); }
 };
 template <> struct PackedEntry<LGP_MATERN52> {
+    static __device__ __forceinline__ float2 acc0(float) { return make_float2(0.0f, 0.0f); }
     static __device__ __forceinline__ float2 k(float2 r2, float ls2) {
         const float2 r = make_float2(sqrt_approx(r2.x), sqrt_approx(r2.y));
         const float2 e = make_float2(ex2_approx(fmaf(r.x, -kLog2e, ls2)), ex2_approx(fmaf(r.y, -kLog2e, ls2)));
@@ -145,11 +148,13 @@ template <> struct PackedEntry<LGP_MATERN52> {
     }
 };
 template <> struct PackedEntry<LGP_MATERN12> {
+    static __device__ __forceinline__ float2 acc0(float) { return make_float2(0.0f, 0.0f); }
     static __device__ __forceinline__ float2 k(float2 r2, float ls2) {
         return make_float2(ex2_approx(ls2 - sqrt_approx(r2.x)), ex2_approx(ls2 - sqrt_approx(r2.y)));
     }
 };
 template <> struct PackedEntry<LGP_MATERN32> {
+    static __device__ __forceinline__ float2 acc0(float) { return make_float2(0.0f, 0.0f); }
     static __device__ __forceinline__ float2 k(float2 r2, float ls2) {
         const float2 r = make_float2(sqrt_approx(r2.x), sqrt_approx(r2.y));
         const float2 e = make_float2(ex2_approx(fmaf(r.x, -kLog2e, ls2)), ex2_approx(fmaf(r.y, -kLog2e, ls2)));
@@ -157,14 +162,16 @@ template <> struct PackedEntry<LGP_MATERN32> {
     }
 };
 
-// What the kernels on PackedEntry multiply V and their finished sums by: s^2 for RBF, on the side where neither the
-// products nor the sums can leave the float32 range that the full entries had.
+// The outputscale of the kernels on PackedEntry: log2 s^2 in the exponent (Matern), or for RBF s^2 as the factor of V or
+// of the finished sums, on the side where neither the products nor the sums can leave the float32 range that the full
+// entries had.
 struct EntryScale {
-    float v = 1.0f, out = 1.0f;
+    float log2s2 = 0.0f, v = 1.0f, out = 1.0f;
 };
-inline EntryScale entry_scale(int kind, float s2) {
+inline EntryScale entry_scale(const KernelParams &kp) {
     EntryScale s;
-    if (kind == LGP_RBF) (s2 < 1.0f ? s.v : s.out) = s2;
+    if (kp.kind != LGP_RBF) s.log2s2 = kp.log2_s2;
+    else (kp.s2 < 1.0f ? s.v : s.out) = kp.s2;
     return s;
 }
 

@@ -217,8 +217,7 @@ cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st) {
         a.E = sg.E;
         a.G = sg.G;
         a.t = m.t;
-        a.log2s2 = m.kp->log2_s2;
-        a.scale = entry_scale(m.kp->kind, m.kp->s2);
+        a.scale = entry_scale(*m.kp);
         cudaError_t e;
         switch (m.kp->kind) {
             case LGP_RBF: e = mv_sym_dispatch_rbf(m.kp->D, sg.TT, a, st); break;
@@ -255,8 +254,7 @@ cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st) {
     a.ldo = m.ldo;
     a.cols_per_split = cps;
     a.t = m.t;
-    a.log2s2 = m.kp->log2_s2;
-    a.scale = entry_scale(m.kp->kind, m.kp->s2);
+    a.scale = entry_scale(*m.kp);
     a.noise = m.kp->noise;
     const dim3 grid((unsigned)rb, (unsigned)S, (unsigned)cg);
     cudaError_t e;

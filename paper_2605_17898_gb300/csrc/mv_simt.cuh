@@ -33,7 +33,6 @@ struct SimtArgs {
     int cross;         // 1: out = K(Xr, Xs) V with no noise term
     int64_t cols_per_split;
     int t;
-    float log2s2;
     EntryScale scale;
     float noise;
 };
@@ -106,7 +105,7 @@ template <int TT> using RowShape = RowTile<TT, TT == 32 ? 2 : 4, 64>;
 template <int KIND, int D, class S>
 __device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t row0, int64_t Npr,
                                           const float *__restrict__ Xs, int64_t Np, const float *__restrict__ V, int64_t ldv,
-                                          int c0, int t, int64_t jb, int64_t je, float log2s2, EntryScale scale, float *xs, float *vs,
+                                          int c0, int t, int64_t jb, int64_t je, EntryScale scale, float *xs, float *vs,
                                           float *tot, float (&sum)[S::R][S::TT]) {
     constexpr int DP = DPad<D>::value, TT = S::TT, R = S::R, NT = S::kThreads;
     const int tid = threadIdx.x;
@@ -125,6 +124,7 @@ __device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t 
             if constexpr (S::kTotShared) tot[(r * TT + c) * NT + tid] = 0.0f;
         }
     }
+    const float2 acc0 = PackedEntry<KIND>::acc0(scale.log2s2);
     for (int64_t j0 = jb; j0 < je; j0 += kSimtBN) {
         __syncthreads();
         for (int e = tid; e < kSimtBN * (DP / 4); e += NT) {
@@ -154,13 +154,13 @@ __device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t 
 #pragma unroll
             for (int r = 0; r < R; ++r) {
                 float2 dd = __fadd2_rn(xj[0], xi[r][0]);
-                float2 r2 = __fmul2_rn(dd, dd);
+                float2 r2 = __ffma2_rn(dd, dd, acc0);
 #pragma unroll
                 for (int d = 1; d < D; ++d) {
                     dd = __fadd2_rn(xj[d], xi[r][d]);
                     r2 = __ffma2_rn(dd, dd, r2);
                 }
-                k[r] = PackedEntry<KIND>::k(r2, log2s2);
+                k[r] = PackedEntry<KIND>::k(r2, scale.log2s2);
             }
             constexpr int CV = TT < 4 ? TT : 4;  // V columns per load
 #pragma unroll
@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(RowShape<TT>::kThreads) mv_simt_kernel(SimtArg
     const int64_t jb = (int64_t)blockIdx.y * a.cols_per_split;
     const int64_t je = min(a.N, jb + a.cols_per_split);
     float sum[S::R][TT];
-    simt_rows<KIND, D, S>(a.Xr, row0, a.Npr, a.Xs, a.Np, a.V, a.ldv, c0, a.t, jb, je, a.log2s2, a.scale, xs, vs, tot, sum);
+    simt_rows<KIND, D, S>(a.Xr, row0, a.Npr, a.Xs, a.Np, a.V, a.ldv, c0, a.t, jb, je, a.scale, xs, vs, tot, sum);
 #pragma unroll
     for (int r = 0; r < S::R; ++r) {
         const int64_t i = row0 + r * S::kThreads + threadIdx.x;

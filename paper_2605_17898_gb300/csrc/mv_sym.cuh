@@ -40,7 +40,6 @@ struct SymArgs {
     const int *skip;
     int64_t N, Np, ldv;
     int E, G, t;
-    float log2s2;
     EntryScale scale;
 };
 
@@ -138,7 +137,8 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
     for (int e = tid; e < WR * E * TT; e += kSymThreads) col[e] = 0.0f;
     __syncthreads();
 
-    const float ls2 = a.log2s2;
+    const float ls2 = a.scale.log2s2;
+    const float2 acc_init = PackedEntry<KIND>::acc0(ls2);
     const int wr = warp / WC, wc = warp % WC;
     const int cw = E / WC, c_lo = wc * cw;  // columns of this warp
     float *mycol = col + wr * E * TT + sym_fold_index<NV>(lane);
@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
 #pragma unroll
                 for (int r = 0; r < R; ++r) {
                     float2 dd = __fadd2_rn(xj[h][0], xi[r][0]);
-                    float2 r2 = __fmul2_rn(dd, dd);
+                    float2 r2 = __ffma2_rn(dd, dd, acc_init);
 #pragma unroll
                     for (int d = 1; d < D; ++d) {
                         dd = __fadd2_rn(xj[h][d], xi[r][d]);
