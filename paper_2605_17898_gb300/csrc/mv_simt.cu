@@ -11,8 +11,16 @@ namespace {
 // CTAs per SM that the row kernel's splits aim at (64 threads each), down to one column tile per split: at small N the
 // tiles of a split are a serial chain of loads and barriers. Against at least 4 tiles per split: N = 1200, D = 6, t = 8
 // 35 -> 15 us, N = 4099, D = 5, t = 5 39 -> 25 us; 16 -> 32 CTAs: N = 20000, D = 8, t = 8 410 -> 388 us. (The partial
-// sums stay at kRowCtas x SMs x rows of a CTA x t floats.)
-constexpr int kRowCtas = 32;
+// sums stay at that many CTAs x SMs x rows of a CTA x t floats.)
+// From 16 columns on a split's partial sums cost more than its share of the entries, so there it is 8 CTAs (6 from 32
+// columns on), 16 where the row blocks and column groups alone give every second SM a CTA and 32 where they give every SM one
+// (the last wave is long): N = 6000, D = 8, t = 32 6 CTAs 111 us, 8 122, 16 134, 32 163; t = 16 8 77, 16 and 32 87; N = 16000, t = 32
+// 8 711, 16 618, 32 638; N = 20000, D = 2, t = 32 16 734, 32 707. At t = 12 (N = 10000, D = 8) 8 169, 16 149, 32 160.
+int row_ctas(int t, int64_t ctas, int num_sms) {
+    if (t < 16 || ctas >= num_sms) return 32;
+    if (2 * ctas >= num_sms) return 16;
+    return t < 32 ? 8 : 6;
+}
 
 // Padded columns of a launch and its CTA's rows.
 struct SimtShape {
@@ -170,7 +178,7 @@ int64_t mv_simt_partial_floats(int64_t N, int64_t Np, int t, int D, int num_sms)
     const int64_t rb = (N + BM - 1) / BM;
     const int64_t cg = (t + sh.TT - 1) / sh.TT;
     int64_t cps;
-    const int64_t S = choose_split(N, rb, cg, num_sms, &cps, kRowCtas, 1);
+    const int64_t S = choose_split(N, rb, cg, num_sms, &cps, row_ctas(t, rb * cg, num_sms), 1);
     return S > 1 ? S * Np * t : 0;
 }
 
@@ -180,7 +188,7 @@ int64_t mv_simt_cross_partial_floats(int64_t Nr, int64_t Npr, int64_t N, int t, 
     const int64_t rb = (Nr + BM - 1) / BM;
     const int64_t cg = (t + sh.TT - 1) / sh.TT;
     int64_t cps;
-    const int64_t S = choose_split(N, rb, cg, num_sms, &cps, kRowCtas, 1);
+    const int64_t S = choose_split(N, rb, cg, num_sms, &cps, row_ctas(t, rb * cg, num_sms), 1);
     return S > 1 ? S * Npr * t : 0;
 }
 
@@ -233,7 +241,7 @@ cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st) {
     const int64_t rb = (Nr + BM - 1) / BM;
     const int64_t cg = (m.t + sh.TT - 1) / sh.TT;
     int64_t cps;
-    int64_t S = choose_split(m.N, rb, cg, m.num_sms, &cps, kRowCtas, 1);
+    int64_t S = choose_split(m.N, rb, cg, m.num_sms, &cps, row_ctas(m.t, rb * cg, m.num_sms), 1);
     if (S > 1 && (m.partial == nullptr || S * Npr * m.t > m.partial_cap)) {
         S = 1;
         cps = m.N;

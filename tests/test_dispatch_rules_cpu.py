@@ -58,3 +58,13 @@ def test_cluster_of_the_cg_step(step, N, t, S, ctas):
     2^22 (16) the step had become slower than the launches it replaced."""
     assert step(N, t, S, True) == ctas
     assert step(N, t, S, False) == (0 if ctas == 16 else ctas)
+
+
+@pytest.mark.parametrize("t,rows", [(16, 256), (32, 128), (64, 64)])
+@pytest.mark.parametrize("N", [3000, 4500, 6000, 8000])
+def test_row_kernel_splits_of_many_columns(slots, N, t, rows):
+    """From 16 columns on the row kernel aims at 8 CTAs per SM while its row blocks (64 columns: two groups of 32 over 128 rows) are fewer
+    than half the SMs, and at 16 up to their number: with 32, splits of one column tile, N = 6000 had become 11% to 18% slower."""
+    blocks = -(-N // rows)
+    assert blocks < SMS
+    assert 1 < slots(N, t, 8) and (slots(N, t, 8) - 1) * blocks < (8 if 2 * blocks < SMS else 16) * SMS
