@@ -110,9 +110,11 @@ lgp_status fail(lgp_ctx *c, lgp_status s, const char *fmt, ...) {
 #define LGP_CUDA(call)                                                                                 \
     do {                                                                                               \
         cudaError_t e_ = (call);                                                                       \
-        if (e_ != cudaSuccess)                                                                         \
+        if (e_ != cudaSuccess) {                                                                       \
+            (void)cudaGetLastError(); /* reported here, not by a later call too */                     \
             return fail(ctx, LGP_ERR_CUDA, "%s failed: %s (%s:%d)", #call, cudaGetErrorString(e_),     \
                         __FILE__, __LINE__);                                                           \
+        }                                                                                              \
     } while (0)
 
 lgp_status ensure(lgp_ctx *ctx, DevBuf &b, size_t bytes) {
@@ -687,8 +689,9 @@ lgp_status run_cg(lgp_ctx *ctx, const Prepared &pp, const float *B, int64_t ldb,
         ProductTail tail;
         const lgp_status r =
             matvec_prepared(ctx, pp, b.p, t, b.Kp, t, t, prec, &b.state->done, st, dist_form, fused_split, &tail);
-        if (r == LGP_OK) launch_cg_after_matvec(pp.N, t, b, tail, fused_split ? &split : nullptr, st);
-        return r;
+        if (r != LGP_OK) return r;
+        LGP_CUDA(launch_cg_after_matvec(pp.N, t, b, tail, fused_split ? &split : nullptr, st));
+        return LGP_OK;
     };
 
     const char *graph_env = std::getenv("LGP_CG_GRAPH");
@@ -699,7 +702,7 @@ lgp_status run_cg(lgp_ctx *ctx, const Prepared &pp, const float *B, int64_t ldb,
         while (true) {
             for (int k = 0; k < kChunk; ++k)
                 if ((s = iteration()) != LGP_OK) return s;
-            launch_cg_chunk_tally(b.state, st);
+            LGP_CUDA(launch_cg_chunk_tally(b.state, st));
             ++launched;
             LGP_CUDA(cudaMemcpyAsync(ctx->h_state, b.state, sizeof(CgState), cudaMemcpyDeviceToHost, st));
             LGP_CUDA(cudaStreamSynchronize(st));
@@ -767,9 +770,11 @@ lgp_status run_cg(lgp_ctx *ctx, const Prepared &pp, const float *B, int64_t ldb,
         }
         lgp_status cs = LGP_OK;
         for (int k = 0; k < kChunk && cs == LGP_OK; ++k) cs = iteration();
-        if (cs == LGP_OK) launch_cg_loop_condition(h, b.state, st);
+        const cudaError_t le = cs == LGP_OK ? launch_cg_loop_condition(h, b.state, st) : cudaSuccess;
         cudaGraph_t captured = nullptr;
         ce = cudaStreamEndCapture(st, &captured);
+        if (le != cudaSuccess) ce = le;
+        if (cs != LGP_OK || ce != cudaSuccess) (void)cudaGetLastError();
         if (cs != LGP_OK) {
             cudaGraphDestroy(g);
             return cs;
@@ -1962,6 +1967,7 @@ lgp_status lgp_batch_cg_solve(lgp_ctx *ctx, int32_t n_gp, const lgp_hyper *hyp, 
     cudaGraph_t captured = nullptr;
     cudaError_t ce2 = cudaStreamEndCapture(st, &captured);
     if (ce != cudaSuccess || ce2 != cudaSuccess) {
+        (void)cudaGetLastError();
         cudaGraphDestroy(graph);
         return fail(ctx, LGP_ERR_CUDA, "batch graph capture failed: %s",
                     cudaGetErrorString(ce != cudaSuccess ? ce : ce2));

@@ -349,7 +349,7 @@ CgSplit tc_cg_split(const KernelParams &kp, int64_t Np, int t, int fmt, void *vs
 cudaError_t launch_v_split(const KernelParams &kp, int64_t N, int64_t Np, const float *V, int64_t ldv, int t, int fmt,
                            void *vsplit, float *out_init, int64_t ldo, const int *skip, int num_sms, cudaStream_t st);
 // p = r + beta p for the active columns and p's split operands, in one pass (the CG step's last launch).
-void launch_p_split(const CgSplit &sp, float *p, const float *r, int64_t N, int t, CgState *state, cudaStream_t st);
+cudaError_t launch_p_split(const CgSplit &sp, float *p, const float *r, int64_t N, int t, CgState *state, cudaStream_t st);
 // The operands of the tensor-core products that depend on X alone, into the t-column V-split workspace:
 // the transposed prescaled X, and with dot = true the dot-form distance data of the symmetric product
 // (box, centred split operands, squared norms, the gate word).
@@ -392,7 +392,7 @@ void launch_gram(const double *L64, int64_t Np, int64_t N, int k, double *partia
 void launch_to_f32(const double *src, float *dst, int64_t n, cudaStream_t st);
 // Z = P^{-1} R for rows < N (t <= 32, k t <= 1024); Pcopy (may be null) receives Z too; rz_partial (may be
 // null) gets [G_vec][t] block partials of r^T z; state (may be null) skips the work once the CG is done.
-void launch_precond_apply(const Precond &pc, const float *R, int64_t ldr, float *Z, int64_t ldz, float *Pcopy,
+cudaError_t launch_precond_apply(const Precond &pc, const float *R, int64_t ldr, float *Z, int64_t ldz, float *Pcopy,
                           int64_t N, int t, double *rz_partial, int G_vec, const CgState *state, cudaStream_t st);
 // rhs[:, col0 + c] = L E[N:, c] + sigma E[:N, c] for the [N + k, m] Rademacher block E
 void launch_precond_probes(const double *L64, int64_t Np, int k, const float *E, int64_t N, int m, double sigma,
@@ -419,17 +419,17 @@ int cg_step_ctas(int64_t N, int t, const CgBuffers &b, int S);
 cudaError_t launch_cg_cluster(int ctas, int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,
                               cudaStream_t st);
 // One CG iteration after its product (b.Kp, or its partial sums in tail); split: p's halves for the next product.
-void launch_cg_after_matvec(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,
-                            cudaStream_t st);
+cudaError_t launch_cg_after_matvec(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,
+                                   cudaStream_t st);
 void launch_cg_copy_out(const CgBuffers &b, int64_t N, int t, float *Xsol, int64_t ldx, cudaStream_t st);
 // Column 0 of the single-column run b1 (state, first hist_len Lanczos coefficients) into column c of a
 // t-column state and history; dst->loop_chunks accumulates.
 void launch_cg_gather_column(const CgBuffers &b1, int hist_len, CgState *dst, double *dst_alpha, double *dst_beta,
                              int t, int c, cudaStream_t st);
 // Body tail of the device-side CG loop: sets the while-node condition to "not done and under the chunk cap".
-void launch_cg_loop_condition(cudaGraphConditionalHandle h, CgState *state, cudaStream_t st);
+cudaError_t launch_cg_loop_condition(cudaGraphConditionalHandle h, CgState *state, cudaStream_t st);
 // Host-driven loop (LGP_CG_GRAPH=0): counts one chunk in state->loop_chunks.
-void launch_cg_chunk_tally(CgState *state, cudaStream_t st);
+cudaError_t launch_cg_chunk_tally(CgState *state, cudaStream_t st);
 int cg_num_blocks(int64_t N, int t, int num_sms);
 int64_t cg_partial_doubles(int G, int t);
 

@@ -555,11 +555,11 @@ void tc_max_words(int64_t Np, int t, void *vsplit, unsigned int **vmax, unsigned
     *words = *vmax + 128 + 8 * Np;
 }
 
-void launch_p_split(const CgSplit &sp, float *p, const float *r, int64_t N, int t, CgState *state, cudaStream_t st) {
+cudaError_t launch_p_split(const CgSplit &sp, float *p, const float *r, int64_t N, int t, CgState *state, cudaStream_t st) {
     const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(((N + 7) / 8 * t + 255) / 256, 8192));
     auto k = t == 16 ? (sp.fmt == kFmtF16 ? p_split_kernel<16, kFmtF16> : p_split_kernel<16, kFmtBF16>)
                      : (sp.fmt == kFmtF16 ? p_split_kernel<32, kFmtF16> : p_split_kernel<32, kFmtBF16>);
-    launch_chained(k, blocks, 256, 0, st, p, r, N, state, sp);
+    return launch_chained(k, blocks, 256, 0, st, p, r, N, state, sp);
 }
 
 cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, const float *V, int64_t ldv,
@@ -691,8 +691,7 @@ cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int
         return cudaSuccess;
     }
     const int rblocks = (int)std::min<int64_t>((N * t + 255) / 256, 4096);
-    launch_chained(tc_reduce_kernel, rblocks, 256, 0, st, partial, g.S, Np, N, t, V, ldv, out, ldo, kp.noise, skip);
-    return cudaGetLastError();
+    return launch_chained(tc_reduce_kernel, rblocks, 256, 0, st, partial, g.S, Np, N, t, V, ldv, out, ldo, kp.noise, skip);
 }
 
 }  // namespace lgp

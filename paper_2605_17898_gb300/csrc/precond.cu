@@ -253,12 +253,13 @@ void launch_to_f32(const double *src, float *dst, int64_t n, cudaStream_t st) {
     to_f32_kernel<<<grid_for(n), 256, 0, st>>>(src, dst, n);
 }
 
-void launch_precond_apply(const Precond &pc, const float *R, int64_t ldr, float *Z, int64_t ldz, float *Pcopy,
-                          int64_t N, int t, double *rz_partial, int G_vec, const CgState *state, cudaStream_t st) {
+cudaError_t launch_precond_apply(const Precond &pc, const float *R, int64_t ldr, float *Z, int64_t ldz, float *Pcopy,
+                                 int64_t N, int t, double *rz_partial, int G_vec, const CgState *state, cudaStream_t st) {
     pc_ltr_kernel<<<pc.G, 256, 0, st>>>(pc.L32, pc.Np, pc.k, R, ldr, N, t, pc.part, state);
     pc_small_kernel<<<1, pc.k * t, 0, st>>>(pc.part, pc.G, pc.k, t, pc.Cinv, pc.U, state);
     pc_apply_kernel<<<G_vec, (256 / t) * t, 0, st>>>(pc.L32, pc.Np, pc.k, pc.U, R, ldr, Z, ldz, Pcopy, N, t,
                                                      1.0 / pc.noise, rz_partial, state);
+    return cudaPeekAtLastError();
 }
 
 void launch_precond_probes(const double *L64, int64_t Np, int k, const float *E, int64_t N, int m, double sigma,

@@ -755,53 +755,58 @@ int step_blocks(int64_t N, int t) {
 }
 
 template <int VEC>
-void launch_step(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split, cudaStream_t st) {
+cudaError_t launch_step(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split, cudaStream_t st) {
     const int bd = VEC == 4 ? kStepThreads : (kStepThreads / t) * t;
     const int G = step_blocks(N, t);
     unsigned int *vbound = split ? split->vmax : nullptr;
+    cudaError_t e;
     if (tail.part && tail.S >= 16 && VEC == 4) {
         const int64_t per = kStepThreads / 8 * VEC;  // elements of a block's round
         const int G8 = (int)std::min<int64_t>(kStepBlocks, (N * t + per - 1) / per);
-        launch_chained(cg_pkp_alpha_kernel<VEC, VEC == 4 ? 8 : 1>, G8, bd, 0, st, b.p, b.Kp, tail.part, tail.S, tail.stride,
-                       tail.noise, N, t, b.state, b.partial, b.hist_alpha);
+        e = launch_chained(cg_pkp_alpha_kernel<VEC, VEC == 4 ? 8 : 1>, G8, bd, 0, st, b.p, b.Kp, tail.part, tail.S,
+                           tail.stride, tail.noise, N, t, b.state, b.partial, b.hist_alpha);
     } else if (tail.part) {
-        launch_chained(cg_pkp_alpha_kernel<VEC, 1>, G, bd, 0, st, b.p, b.Kp, tail.part, tail.S, tail.stride, tail.noise, N, t,
-                       b.state, b.partial, b.hist_alpha);
+        e = launch_chained(cg_pkp_alpha_kernel<VEC, 1>, G, bd, 0, st, b.p, b.Kp, tail.part, tail.S, tail.stride, tail.noise, N,
+                           t, b.state, b.partial, b.hist_alpha);
     } else {
-        launch_chained(cg_pkp_alpha_kernel<VEC, 0>, G, bd, 0, st, b.p, b.Kp, nullptr, 0, 0, 0.0f, N, t, b.state, b.partial,
-                       b.hist_alpha);
+        e = launch_chained(cg_pkp_alpha_kernel<VEC, 0>, G, bd, 0, st, b.p, b.Kp, nullptr, 0, 0, 0.0f, N, t, b.state, b.partial,
+                           b.hist_alpha);
     }
+    if (e != cudaSuccess) return e;
     if (b.pc.k > 0) {
         double *rz_partial = b.partial + (int64_t)b.G * t;
-        launch_chained(cg_xr_beta_kernel<VEC, false>, G, bd, 0, st, b.x, b.r, b.p, b.Kp, N, t, b.state, b.partial, b.hist_beta,
-                       nullptr);
-        launch_precond_apply(b.pc, b.r, t, b.z, t, nullptr, N, t, rz_partial, b.G, b.state, st);
-        launch_chained(cg_beta_kernel, 1, 1024, 0, st, b.state, b.partial, G, rz_partial, b.G, t, b.hist_beta);
+        if ((e = launch_chained(cg_xr_beta_kernel<VEC, false>, G, bd, 0, st, b.x, b.r, b.p, b.Kp, N, t, b.state, b.partial,
+                                b.hist_beta, nullptr)) != cudaSuccess ||
+            (e = launch_precond_apply(b.pc, b.r, t, b.z, t, nullptr, N, t, rz_partial, b.G, b.state, st)) != cudaSuccess)
+            return e;
+        e = launch_chained(cg_beta_kernel, 1, 1024, 0, st, b.state, b.partial, G, rz_partial, b.G, t, b.hist_beta);
     } else {
-        launch_chained(cg_xr_beta_kernel<VEC, true>, G, bd, 0, st, b.x, b.r, b.p, b.Kp, N, t, b.state, b.partial, b.hist_beta,
-                       vbound);
+        e = launch_chained(cg_xr_beta_kernel<VEC, true>, G, bd, 0, st, b.x, b.r, b.p, b.Kp, N, t, b.state, b.partial,
+                           b.hist_beta, vbound);
     }
-    if (split)
-        launch_p_split(*split, b.p, b.r, N, t, b.state, st);
-    else
-        launch_chained(cg_p_kernel<VEC>, G, bd, 0, st, b.p, b.pc.k > 0 ? b.z : b.r, N, t, b.state);
+    if (e != cudaSuccess) return e;
+    return split ? launch_p_split(*split, b.p, b.r, N, t, b.state, st)
+                 : launch_chained(cg_p_kernel<VEC>, G, bd, 0, st, b.p, b.pc.k > 0 ? b.z : b.r, N, t, b.state);
 }
 
 }  // namespace
 
-void launch_cg_after_matvec(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,
-                            cudaStream_t st) {
+cudaError_t launch_cg_after_matvec(int64_t N, int t, const CgBuffers &b, const ProductTail &tail, const CgSplit *split,
+                                   cudaStream_t st) {
     const int ctas = cg_step_ctas(N, t, b, tail.part ? tail.S : 0);
-    if (ctas > 0) launch_cg_cluster(ctas, N, t, b, tail, split, st);
-    else if (t <= 64 && (t & (t - 1)) == 0) launch_step<4>(N, t, b, tail, split, st);
-    else launch_step<1>(N, t, b, tail, split, st);
+    if (ctas > 0) return launch_cg_cluster(ctas, N, t, b, tail, split, st);
+    return t <= 64 && (t & (t - 1)) == 0 ? launch_step<4>(N, t, b, tail, split, st) : launch_step<1>(N, t, b, tail, split, st);
 }
 
-void launch_cg_loop_condition(cudaGraphConditionalHandle h, CgState *state, cudaStream_t st) {
+cudaError_t launch_cg_loop_condition(cudaGraphConditionalHandle h, CgState *state, cudaStream_t st) {
     cg_loop_condition_kernel<<<1, 1, 0, st>>>(h, state);
+    return cudaPeekAtLastError();
 }
 
-void launch_cg_chunk_tally(CgState *state, cudaStream_t st) { cg_chunk_tally_kernel<<<1, 1, 0, st>>>(state); }
+cudaError_t launch_cg_chunk_tally(CgState *state, cudaStream_t st) {
+    cg_chunk_tally_kernel<<<1, 1, 0, st>>>(state);
+    return cudaPeekAtLastError();
+}
 
 void launch_cg_gather_column(const CgBuffers &b1, int hist_len, CgState *dst, double *dst_alpha, double *dst_beta,
                              int t, int c, cudaStream_t st) {
