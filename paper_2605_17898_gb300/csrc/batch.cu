@@ -215,7 +215,7 @@ template <int VEC> __device__ __forceinline__ void store_vec(float *p, const flo
 // values from a multiple of 16 bytes, so a last float4 that crosses N t stays inside them.)
 template <int VEC, int CL>
 __global__ void __launch_bounds__(kVec) batch_step_kernel(BatchArgs a) {
-    __shared__ float2 red[kMaxBatchT * 32 > kVec ? kMaxBatchT * 32 : kVec];
+    __shared__ ColSums acc1, acc2;
     __shared__ double sum1[kMaxBatchT], sum2[kMaxBatchT];
     __shared__ float s_alpha[kMaxBatchT], s_beta[kMaxBatchT];
     __shared__ int s_act[kMaxBatchT];
@@ -224,6 +224,9 @@ __global__ void __launch_bounds__(kVec) batch_step_kernel(BatchArgs a) {
     const int gi = blockIdx.x / CL, rank = blockIdx.x % CL;
     if (blockIdx.x == 0 && threadIdx.x == 0) *a.item_counter = 0;
     if (*a.done || a.gp_done[gi]) return;  // the same for the whole cluster: its rank 0 sets gp_done after the last barrier
+    clear_sums(acc1);
+    clear_sums(acc2);
+    __syncthreads();
     const BatchGp g = a.gps[gi];
     const int tid = threadIdx.x, t = a.t, k = gi * t + (tid < t ? tid : 0);
     const int active = a.active[k], iters = a.iters[k];
@@ -263,7 +266,7 @@ __global__ void __launch_bounds__(kVec) batch_step_kernel(BatchArgs a) {
         for (int q = 0; q < VEC; ++q)
             if (VEC == 1 || e + q < total) acc_prod2(hi[q], lo[q], pv[q], kv[q]);
     }
-    block_pairs_reduce<VEC>(hi, lo, t, red, sum1);
+    block_col_sums<VEC>(hi, lo, t, acc1, sum1);
     const double pkp = batch_cluster_sum<CL>(sum1, t);
     int failed = 0;
     if (tid < t) {
@@ -298,7 +301,7 @@ __global__ void __launch_bounds__(kVec) batch_step_kernel(BatchArgs a) {
         store_vec<VEC>(x + e, xv);
         store_vec<VEC>(r + e, rv);
     }
-    block_pairs_reduce<VEC>(hi, lo, t, red, sum2);
+    block_col_sums<VEC>(hi, lo, t, acc2, sum2);
     const double rr = batch_cluster_sum<CL>(sum2, t);
     int act = 0;
     if (tid < t) {

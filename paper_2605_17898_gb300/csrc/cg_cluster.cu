@@ -83,7 +83,7 @@ __device__ void split_tile(const ClusterArgs &a, const float *tile, int row0, in
 // VECS float4s per thread and vector; above kClVecs only p and r stay in registers, Kp and x come from the L2 cache again.
 template <int CL, int VECS>
 __global__ void __launch_bounds__(kClThreads, 1) cg_cluster_kernel(const ClusterArgs a) {
-    __shared__ float2 red[64 * 32];
+    __shared__ ColSums acc1, acc2;
     __shared__ double sum1[kMaxT], sum2[kMaxT];
     __shared__ unsigned int rmax[kMaxT], pmax[kMaxT];
     __shared__ float s_alpha[kMaxT], s_beta[kMaxT];
@@ -103,6 +103,9 @@ __global__ void __launch_bounds__(kClThreads, 1) cg_cluster_kernel(const Cluster
     const int iter = st->iter, hist_len = st->hist_len, max_iter = st->max_iter;
     const float vbound0 = a.split && a.sp.fmt == 1 ? __uint_as_float(a.sp.vmax[c]) : 0.0f;
     if (tid < kMaxT) rmax[tid] = pmax[tid] = 0u;
+    clear_sums(acc1);
+    clear_sums(acc2);
+    __syncthreads();
 
     // ---- p, Kp (with the product's partial sums), r, x into registers; p^T Kp
     constexpr bool kHold = VECS <= kClVecs;
@@ -172,7 +175,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cg_cluster_kernel(const Cluster
             add(m, pv[m], k4);
         }
     }
-    block_pairs_reduce<4>(hi, lo, t, red, sum1);
+    block_col_sums<4>(hi, lo, t, acc1, sum1);
     const double pkp = cluster_sum<CL>(sum1, t);
     int bad = 0, nonfinite = 0;
     double alpha = 0.0;
@@ -222,7 +225,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cg_cluster_kernel(const Cluster
 #pragma unroll
         for (int k = 0; k < 4; ++k) atomicMax(&rmax[col_of<4>(tid, k, t)], __float_as_uint(m4[k]));
     }
-    block_pairs_reduce<4>(hi, lo, t, red, sum2);
+    block_col_sums<4>(hi, lo, t, acc2, sum2);
     const double rr = cluster_sum<CL>(sum2, t);
     double beta = 0.0;
     int act = 0;

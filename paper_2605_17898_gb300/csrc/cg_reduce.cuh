@@ -1,7 +1,8 @@
-// Column sums of the CG kernels: compensated float pairs within a block.
+// Column sums of the CG kernels within a block: compensated float pairs per thread, fixed point across threads.
 #pragma once
 
 #include "lgp_internal.cuh"
+#include "limb_sum.cuh"
 
 namespace lgp {
 
@@ -18,30 +19,53 @@ __device__ __forceinline__ void pair_add(float &h, float &l, float h2, float l2)
 // the block has a multiple of t threads and thread x owns column x mod t.
 template <int VEC> __device__ __forceinline__ int col_of(int tid, int k, int t) { return (VEC * tid + k) % t; }
 
-// Sums the float pairs of every column over the block: out_row[c] = their float64 value, c < t (valid after the next
-// barrier). red: 64 x 32 pairs.
+// Working memory of one block_col_sums call; cleared, and a barrier passed, before it.
+struct ColSums {
+    unsigned int mx[kMaxT];  // largest magnitude per column
+    int limb[3][kMaxT];
+};
+__device__ __forceinline__ void clear_sums(ColSums &s) {
+    if (threadIdx.x < kMaxT) {
+        s.mx[threadIdx.x] = 0u;
+        s.limb[0][threadIdx.x] = s.limb[1][threadIdx.x] = s.limb[2][threadIdx.x] = 0;
+    }
+}
+
+// v[k] of the lanes that hold the same columns (those that agree mod group, group = 2 .. 16) combined by op, each step
+// halving what a lane carries: for group <= 8 the result in r[0] is that of k = 2 bit4 + bit3 of the lane (the same in lanes
+// that differ only in the bits from group to 4), for group = 16 r[0] and r[1] are those of k = 2 bit4 and the next.
+template <class T, class Op> __device__ __forceinline__ void fold_columns(const T (&v)[4], int group, int lane, Op op, T (&r)[2]) {
+    const bool up = lane & 16, second = lane & 8;
+    const T s0 = up ? v[0] : v[2], s1 = up ? v[1] : v[3];
+    r[0] = op(up ? v[2] : v[0], __shfl_xor_sync(0xffffffffu, s0, 16));
+    r[1] = op(up ? v[3] : v[1], __shfl_xor_sync(0xffffffffu, s1, 16));
+    if (group > 8) return;
+    const T s = second ? r[0] : r[1];
+    r[0] = op(second ? r[1] : r[0], __shfl_xor_sync(0xffffffffu, s, 8));
+    for (int off = group; off < 8; off <<= 1) r[0] = op(r[0], __shfl_xor_sync(0xffffffffu, r[0], off));
+}
+
+// Sums the float pairs of every column over the block: out_row[c] = their float64 value, c < t, written by thread c.
+// The sum across threads is the block's largest magnitude per column, then integer sums (limb_sum.cuh): float64 additions
+// would take 64 cycles of a sub-partition per warp (a tree over 512 threads 1650 cycles), float pairs lose bits and
+// overflow where float64 does not. Up to 4 columns a warp's maximum and sums are one reduction instruction each. An
+// iteration with its product, pairs by shuffles -> this: N = 2000, D = 6, t = 1 18.2 -> 16.6 us, t = 8 20.3 -> 20.1, t = 4 20.1 ->
+// 20.3; N = 4000, t = 32 40.5 -> 39.0; N = 20000, D = 8, t = 32 156.3 -> 153.8.
 template <int VEC>
-__device__ void block_pairs_reduce(float (&hi)[VEC], float (&lo)[VEC], int t, float2 *red, double *out_row) {
+__device__ void block_col_sums(float (&hi)[VEC], float (&lo)[VEC], int t, ColSums &s, double *out_row) {
     const int tid = threadIdx.x;
     if constexpr (VEC == 1) {
-        const int nr = blockDim.x / t;
-        red[tid] = make_float2(hi[0], lo[0]);
+        const int c = tid % t;
+        atomicMax(&s.mx[c], max(magnitude_bits(hi[0]), magnitude_bits(lo[0])));
         __syncthreads();
-        int s = 1;
-        while (s < nr) s <<= 1;
-        for (s >>= 1; s >= 1; s >>= 1) {
-            const int slot = tid / t;
-            if (slot < s && slot + s < nr) {
-                float2 a = red[tid];
-                const float2 b = red[tid + s * t];
-                pair_add(a.x, a.y, b.x, b.y);
-                red[tid] = a;
-            }
-            __syncthreads();
-        }
-        if (tid < t) out_row[tid] = (double)red[tid].x + (double)red[tid].y;
+        const float scale = limb_scale(s.mx[c]);
+        int l[3] = {0, 0, 0};
+        add_limbs(hi[0], scale, l);
+        add_limbs(lo[0], scale, l);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) atomicAdd(&s.limb[j][c], l[j]);
     } else {
-        const int lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+        const int lane = tid & 31;
         if (t == 1) {
             pair_add(hi[0], lo[0], hi[1], lo[1]);
             pair_add(hi[2], lo[2], hi[3], lo[3]);
@@ -51,28 +75,59 @@ __device__ void block_pairs_reduce(float (&hi)[VEC], float (&lo)[VEC], int t, fl
             pair_add(hi[1], lo[1], hi[3], lo[3]);
         }
         const int group = t > 4 ? t / 4 : 1;  // lanes that hold one row of columns
-        for (int off = group; off < 32; off <<= 1) {
+        if (group == 1) {
 #pragma unroll
             for (int k = 0; k < VEC; ++k) {
-                const float h2 = __shfl_xor_sync(0xffffffffu, hi[k], off), l2 = __shfl_xor_sync(0xffffffffu, lo[k], off);
-                pair_add(hi[k], lo[k], h2, l2);
+                if (k >= t) break;
+                const unsigned int m = __reduce_max_sync(0xffffffffu, max(magnitude_bits(hi[k]), magnitude_bits(lo[k])));
+                if (lane == 0) atomicMax(&s.mx[k], m);
             }
-        }
-        if (lane < group) {
+            __syncthreads();
 #pragma unroll
-            for (int k = 0; k < VEC; ++k)
-                if (4 * lane + k < t) red[(4 * lane + k) * 32 + warp] = make_float2(hi[k], lo[k]);
-        }
-        __syncthreads();
-        for (int c = warp; c < t; c += nw) {
-            float2 v = lane < nw ? red[c * 32 + lane] : make_float2(0.0f, 0.0f);
-            for (int off = 16; off > 0; off >>= 1) {
-                const float h2 = __shfl_xor_sync(0xffffffffu, v.x, off), l2 = __shfl_xor_sync(0xffffffffu, v.y, off);
-                pair_add(v.x, v.y, h2, l2);
+            for (int k = 0; k < VEC; ++k) {
+                if (k >= t) break;
+                const float scale = limb_scale(s.mx[k]);
+                int l[3] = {0, 0, 0};
+                add_limbs(hi[k], scale, l);
+                add_limbs(lo[k], scale, l);
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    const int v = __reduce_add_sync(0xffffffffu, l[j]);
+                    if (lane == 0) atomicAdd(&s.limb[j][k], v);
+                }
             }
-            if (lane == 0) out_row[c] = (double)v.x + (double)v.y;
+        } else {
+            // this lane's columns after fold_columns, and whether it is the one that adds them
+            const int col = 4 * (lane & (group - 1)) + 2 * (lane >> 4) + (group > 8 ? 0 : (lane >> 3) & 1);
+            const bool adds = group > 8 || (lane & 7) < group;
+            unsigned int m[4], mr[2];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) m[k] = max(magnitude_bits(hi[k]), magnitude_bits(lo[k]));
+            fold_columns(m, group, lane, [](unsigned int a, unsigned int b) { return max(a, b); }, mr);
+            if (adds) atomicMax(&s.mx[col], mr[0]);
+            if (group > 8) atomicMax(&s.mx[col + 1], mr[1]);
+            __syncthreads();
+            int l[3][4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float scale = limb_scale(s.mx[(4 * lane + k) & (t - 1)]);
+                int p[3] = {0, 0, 0};
+                add_limbs(hi[k], scale, p);
+                add_limbs(lo[k], scale, p);
+#pragma unroll
+                for (int j = 0; j < 3; ++j) l[j][k] = p[j];
+            }
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                int r[2];
+                fold_columns(l[j], group, lane, [](int a, int b) { return a + b; }, r);
+                if (adds) atomicAdd(&s.limb[j][col], r[0]);
+                if (group > 8) atomicAdd(&s.limb[j][col + 1], r[1]);
+            }
         }
     }
+    __syncthreads();
+    if (tid < t) out_row[tid] = limb_total(s.limb[0][tid], s.limb[1][tid], s.limb[2][tid], s.mx[tid]);
 }
 
 }  // namespace lgp

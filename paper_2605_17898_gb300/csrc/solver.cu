@@ -7,9 +7,9 @@
 //   alpha_c = r_c^T z_c / p_c^T Kp_c,  x_c += alpha_c p_c,  r_c -= alpha_c Kp_c,
 //   z_c' = P^{-1} r_c',  beta_c = r_c'^T z_c' / r_c^T z_c,  p_c = z_c' + beta_c p_c,
 // column c stops once ||r_c|| <= tol ||b_c||. The optional preconditioner is the pivoted-Cholesky
-// P of precond.cu (the gap Sec. 5 names; plain CG is the paper's loop). Vectors are float32; the dot products
-// are accumulated in float64 with a fixed reduction order (block partials, then one
-// block sums them in index order), so results are reproducible run to run.
+// P of precond.cu (the gap Sec. 5 names; plain CG is the paper's loop). Vectors are float32; a dot product's sum is
+// carried as a float pair within a thread, without rounding across a block's threads (limb_sum.cuh) and in float64 across
+// blocks, in index order, so results are reproducible run to run.
 #include <math.h>
 
 #include <algorithm>
@@ -151,9 +151,9 @@ __global__ void cg_init_scalars_kernel(CgState *st, const double *__restrict__ p
 // block to finish alpha), xr_beta (x, r, r^T r, the columns' max |r|; last block: beta, convergence, the loop's done
 // flag) and p (p, and for the tensor-core products its split halves and the sigma^2 p that their out starts from).
 // What bounds them: up to a few MB per vector the launches and the chain of loads, block reduction and float64
-// reduction, not bandwidth. Hence few launches, 16-byte loads in blocks of 1024 threads, float pairs up to one value per
-// block and column, and at most kStepBlocks float64 values per column: one float64 warp instruction takes 64 cycles
-// of a sub-partition here, so a square root per column would cost more than all the loads (the test of convergence
+// reduction, not bandwidth. Hence few launches, 16-byte loads in blocks of 1024 threads, integer sums up to one value per
+// block and column (cg_reduce.cuh), and at most kStepBlocks float64 values per column: one float64 warp instruction takes 64
+// cycles of a sub-partition here, so a square root per column would cost more than all the loads (the test of convergence
 // compares squares).
 // Measured a solve / training step: N = 1024, t = 1, ~90 iterations 2.33 -> 1.83 ms; N = 2000, D = 8, t = 16 6.5 -> 4.7 ms;
 // prediction at N = 8000, t = 32 (with the product's own gain) 16.7 -> 13.2 ms.
@@ -227,10 +227,13 @@ __global__ void __launch_bounds__(kStepThreads) cg_pkp_alpha_kernel(const float 
                                                                     int64_t part_stride, float noise, int64_t N, int t,
                                                                     CgState *st, double *__restrict__ partial,
                                                                     double *__restrict__ hist_alpha) {
-    __shared__ float2 red[64 * 32];
+    __shared__ float2 red[kStepThreads / 8 * 4];  // LANES = 8: element threads' sums; the grid sum's 128 doubles
+    __shared__ ColSums acc;
     chain_wait();
     chain_next();
     if (st->done) return;
+    clear_sums(acc);
+    __syncthreads();
     const int64_t total = N * t;
     // LANES = 8: element thread u of the block's blockDim / 8 is lanes with (lane & 3) = u mod 4 of warp u / 4
     constexpr int L = LANES > 1 ? LANES : 1;
@@ -292,7 +295,7 @@ __global__ void __launch_bounds__(kStepThreads) cg_pkp_alpha_kernel(const float 
         }
         __syncthreads();
     }
-    block_pairs_reduce<VEC>(hi, lo, t, red, partial + (int64_t)blockIdx.x * t);
+    block_col_sums<VEC>(hi, lo, t, acc, partial + (int64_t)blockIdx.x * t);
     if (!last_block(&st->ticket)) return;
     const double pkp = grid_col_sum(partial, t, reinterpret_cast<double *>(red));
     const int c = threadIdx.x;
@@ -357,7 +360,8 @@ __global__ void __launch_bounds__(kStepThreads) cg_xr_beta_kernel(float *__restr
                                                                   const float *__restrict__ Kp, int64_t N, int t,
                                                                   CgState *st, double *__restrict__ partial,
                                                                   double *__restrict__ hist_beta, unsigned int *vbound) {
-    __shared__ float2 red[64 * 32];
+    __shared__ double red[128];
+    __shared__ ColSums acc;
     __shared__ unsigned int rmax[kMaxT];
     chain_wait();
     chain_next();
@@ -372,6 +376,8 @@ __global__ void __launch_bounds__(kStepThreads) cg_xr_beta_kernel(float *__restr
         hi[k] = lo[k] = m[k] = 0.0f;
     }
     if (threadIdx.x < kMaxT) rmax[threadIdx.x] = 0u;
+    clear_sums(acc);
+    __syncthreads();
     LGP_STEP_LOOP(e) {
         float rv[VEC];
         load_vec<VEC>(r + e, rv);
@@ -398,15 +404,14 @@ __global__ void __launch_bounds__(kStepThreads) cg_xr_beta_kernel(float *__restr
             }
     }
     if (vbound) {
-        __syncthreads();
 #pragma unroll
         for (int k = 0; k < VEC; ++k) atomicMax(&rmax[col_of<VEC>(threadIdx.x, k, t)], __float_as_uint(m[k]));
     }
-    block_pairs_reduce<VEC>(hi, lo, t, red, partial + (int64_t)blockIdx.x * t);
+    block_col_sums<VEC>(hi, lo, t, acc, partial + (int64_t)blockIdx.x * t);
     if (vbound && (int)threadIdx.x < t) atomicMax(&st->rmax[threadIdx.x], rmax[threadIdx.x]);
     if constexpr (FINISH) {
         if (!last_block(&st->ticket)) return;
-        const double rr = grid_col_sum(partial, t, reinterpret_cast<double *>(red));
+        const double rr = grid_col_sum(partial, t, red);
         finish_beta(st, rr, rr, t, hist_beta, vbound);
     }
 }
