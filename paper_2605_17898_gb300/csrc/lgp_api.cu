@@ -224,11 +224,15 @@ struct Prepared {
     int64_t N, Np;
     float *xs;
     uint64_t version;  // distinguishes successive preparations of the context's xs buffer
+    TcZeroed zeroed;   // words cleared for the tensor-core product that follows
 };
 
-// tc_t > 0: a tensor-core product of that many columns follows, whose maxima words are cleared on the way.
+bool needs_dot(const lgp_ctx *ctx, const Prepared &pp, int t, int prec);
+
+// tc_t > 0: a tensor-core product of that many columns follows, whose maxima words are cleared on the way: those of V always,
+// those of X only if it builds the dot form's operands (they answer lgp_tc_distance_form for the last product that did).
 lgp_status prepare_x(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X, int64_t N, cudaStream_t st, Prepared *pp,
-                     int tc_t = 0) {
+                     int tc_t = 0, int prec = LGP_PREC_FP32) {
     NvtxRange nvtx_range("lgp.prepare_x");
     lgp_status s = make_params(ctx, hyp, &pp->kp);
     if (s != LGP_OK) return s;
@@ -244,7 +248,10 @@ lgp_status prepare_x(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X, int64_t
     if (tc_t > 0) {
         if ((s = ensure(ctx, ctx->vsplit, (size_t)tc_vsplit_bytes(pp->Np, tc_t))) != LGP_OK) return s;
         tc_max_words(pp->Np, tc_t, ctx->vsplit.p, &vmax, &words);
+        if (!needs_dot(ctx, *pp, tc_t, prec)) words = nullptr;
     }
+    pp->zeroed.v = vmax != nullptr;
+    pp->zeroed.x = words != nullptr;
     launch_prep_x(X, N, pp->kp.D, pp->kp.dpad, pp->kp.scale, pp->xs, pp->Np, (int *)ctx->flags.p, st, vmax, words);
     LGP_CUDA(cudaGetLastError());
     return LGP_OK;
@@ -416,7 +423,7 @@ bool kernel_timing_on(const lgp_ctx *ctx, cudaStream_t st) {
 // v_ready, tail: see launch_mv_tc (v_ready for the tensor-core products only). rows: the float32 row kernel at any t.
 lgp_status matvec_prepared(lgp_ctx *ctx, const Prepared &pp, const float *V, int64_t ldv, float *out, int64_t ldo,
                            int t, int prec, const int *skip, cudaStream_t st, int dist_form = -1, bool v_ready = false,
-                           ProductTail *tail = nullptr, bool zeroed = false, bool rows = false) {
+                           ProductTail *tail = nullptr, TcZeroed zeroed = {}, bool rows = false) {
     if (is_tc(prec)) {
         lgp_status s = ensure(ctx, ctx->vsplit, (size_t)tc_vsplit_bytes(pp.Np, t));
         if (s != LGP_OK) return s;
@@ -947,7 +954,7 @@ lgp_status batch_route(lgp_ctx *ctx, const lgp_hyper *h, const float *X, int64_t
     Prepared pp;
     // the product the persistent launch runs (at t <= 4 lgp_kernel_matvec has a faster one)
     auto row_product = [&] {
-        return matvec_prepared(ctx, pp, B, t, out, t, t, LGP_PREC_FP32, nullptr, st, -1, false, nullptr, false, true);
+        return matvec_prepared(ctx, pp, B, t, out, t, t, LGP_PREC_FP32, nullptr, st, -1, false, nullptr, {}, true);
     };
     // the launch floor: the float32 product of the first rows only (B is row-major, so its first rows
     // are that problem's right-hand sides)
@@ -1450,7 +1457,7 @@ lgp_status lgp_kernel_matvec(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X,
     if (p < 0) return fail(ctx, (lgp_status)p, "precision %d unsupported for t=%d", prec, t);
     cudaStream_t st = (cudaStream_t)stream;
     Prepared pp;
-    if ((s = prepare_x(ctx, hyp, X, N, st, &pp, is_tc(p) ? tp : 0)) != LGP_OK) return s;
+    if ((s = prepare_x(ctx, hyp, X, N, st, &pp, is_tc(p) ? tp : 0, p)) != LGP_OK) return s;
     // an explicit split precision at other t: the product runs on tp zero-padded columns
     const float *Vu = V;
     float *Ou = out;
@@ -1471,7 +1478,7 @@ lgp_status lgp_kernel_matvec(lgp_ctx *ctx, const lgp_hyper *hyp, const float *X,
         if (cap == cudaStreamCaptureStatusNone && (s = autotune_tc(ctx, pp, Vu, tp, Ou, tp, tp, p, st)) != LGP_OK)
             return s;
     }
-    if ((s = matvec_prepared(ctx, pp, Vu, tp, Ou, tp, tp, p, nullptr, st, -1, false, nullptr, true)) != LGP_OK) return s;
+    if ((s = matvec_prepared(ctx, pp, Vu, tp, Ou, tp, tp, p, nullptr, st, -1, false, nullptr, pp.zeroed)) != LGP_OK) return s;
     if (tp != t) {
         launch_copy_cols(Ou, tp, out, t, N, t, 0, st);
         LGP_CUDA(cudaGetLastError());

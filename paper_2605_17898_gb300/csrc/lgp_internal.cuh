@@ -317,6 +317,10 @@ int64_t tc_vsplit_bytes(int64_t Np, int t);
 // kTcSymmetricDiff = the same, always in the difference form.
 constexpr int kTcSymmetric = -1;
 constexpr int kTcSymmetricDiff = -2;
+// Words of tc_max_words in which nothing has been collected since launch_prep_x cleared them, but for this V and X.
+struct TcZeroed {
+    bool v = false, x = false;
+};
 // operands_ready: the operands that depend on X alone are already in vsplit (launch_tc_operands, once
 // per prepared X): the transposed X and, where the symmetric product may take the dot form, its
 // distance operands; otherwise the product builds them first.
@@ -324,8 +328,7 @@ constexpr int kTcSymmetricDiff = -2;
 // instances launch and the device gate word lets one of them work; 0 / 1 = only the difference / dot
 // instance launches (the caller read the gate word, which must then give the same answer).
 // v_ready: V is already split in the workspace, and out of a symmetric product already holds sigma^2 V
-// (launch_v_split, launch_p_split). tail (optional): see ProductTail. zeroed: nothing has been collected in the words of
-// tc_max_words since launch_prep_x cleared them, but for this X and V.
+// (launch_v_split, launch_p_split). tail (optional): see ProductTail. zeroed: see TcZeroed.
 // ev_begin / ev_end (optional): recorded on st immediately before and after the product kernel's
 // launch(es), after the V split and operand kernels (the kernel timing of lgp_last_kernel_ms).
 cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, const float *V, int64_t ldv,
@@ -333,7 +336,7 @@ cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int
                          const int *skip, int *err_flag, long long wait_budget, int num_sms, cudaStream_t st,
                          int forced_splits = 0, bool operands_ready = false, int dist_form = -1,
                          cudaEvent_t ev_begin = nullptr, cudaEvent_t ev_end = nullptr, bool v_ready = false,
-                         ProductTail *tail = nullptr, bool zeroed = false);
+                         ProductTail *tail = nullptr, TcZeroed zeroed = {});
 // A CG solve's vector p as the split operand of its products (p row stride t, the workspace of one vsplit).
 struct CgSplit {
     int fmt;

@@ -506,7 +506,7 @@ namespace {
 // The passes over a product's inputs that its kernel needs done: with x the transposed X (and with dot the distance
 // operands), with V the split of V. zeroed: the words they collect maxima in are zero already (launch_prep_x).
 cudaError_t launch_tc_inputs(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, bool x, bool dot, const float *V,
-                             int64_t ldv, int t, int fmt, void *vsplit, float *out_init, int64_t ldo, bool zeroed,
+                             int64_t ldv, int t, int fmt, void *vsplit, float *out_init, int64_t ldo, TcZeroed zeroed,
                              const int *skip, int num_sms, cudaStream_t st) {
     const CgSplit sp = tc_cg_split(kp, Np, t, fmt, vsplit, out_init);
     float *XsT = sp.col_scale + 64;
@@ -516,10 +516,8 @@ cudaError_t launch_tc_inputs(const KernelParams &kp, const float *Xs, int64_t N,
     uint8_t *ub = ua + Np * 64;
     const bool absmax = V && fmt == kFmtF16;
     cudaError_t e;
-    if (!zeroed) {
-        if (absmax && (e = cudaMemsetAsync(sp.vmax, 0, 64 * sizeof(unsigned int), st)) != cudaSuccess) return e;
-        if (dot && (e = cudaMemsetAsync(words, 0, 32 * sizeof(unsigned int), st)) != cudaSuccess) return e;
-    }
+    if (absmax && !zeroed.v && (e = cudaMemsetAsync(sp.vmax, 0, 64 * sizeof(unsigned int), st)) != cudaSuccess) return e;
+    if (dot && !zeroed.x && (e = cudaMemsetAsync(words, 0, 32 * sizeof(unsigned int), st)) != cudaSuccess) return e;
     const int xb = x ? (int)std::min<int64_t>((Np + 255) / 256, 2 * num_sms) : 0;
     const int mb = absmax ? (int)std::max<int64_t>(1, std::min<int64_t>((N * t + 255) / 256, 4 * num_sms)) : 0;
     if (xb + mb > 0 && (e = launch_chained(tc_scan_kernel, xb + mb, 256, 0, st, Xs, N, Np, kp.dpad, XsT,
@@ -542,12 +540,12 @@ cudaError_t launch_tc_inputs(const KernelParams &kp, const float *Xs, int64_t N,
 
 cudaError_t launch_tc_operands(const KernelParams &kp, const float *Xs, int64_t N, int64_t Np, int t, void *vsplit, bool dot,
                                int num_sms, cudaStream_t st) {
-    return launch_tc_inputs(kp, Xs, N, Np, true, dot, nullptr, 0, t, kFmtF16, vsplit, nullptr, 0, false, nullptr, num_sms, st);
+    return launch_tc_inputs(kp, Xs, N, Np, true, dot, nullptr, 0, t, kFmtF16, vsplit, nullptr, 0, {}, nullptr, num_sms, st);
 }
 
 cudaError_t launch_v_split(const KernelParams &kp, int64_t N, int64_t Np, const float *V, int64_t ldv, int t, int fmt,
                            void *vsplit, float *out_init, int64_t ldo, const int *skip, int num_sms, cudaStream_t st) {
-    return launch_tc_inputs(kp, nullptr, N, Np, false, false, V, ldv, t, fmt, vsplit, out_init, ldo, false, skip, num_sms, st);
+    return launch_tc_inputs(kp, nullptr, N, Np, false, false, V, ldv, t, fmt, vsplit, out_init, ldo, {}, skip, num_sms, st);
 }
 
 void tc_max_words(int64_t Np, int t, void *vsplit, unsigned int **vmax, unsigned int **words) {
@@ -566,7 +564,7 @@ cudaError_t launch_mv_tc(const KernelParams &kp, const float *Xs, int64_t N, int
                          float *out, int64_t ldo, int t, int fmt, void *vsplit, float *partial, int64_t partial_cap,
                          const int *skip, int *err_flag, long long wait_budget, int num_sms, cudaStream_t st,
                          int forced_splits, bool operands_ready, int dist_form, cudaEvent_t ev_begin,
-                         cudaEvent_t ev_end, bool v_ready, ProductTail *tail, bool zeroed) {
+                         cudaEvent_t ev_end, bool v_ready, ProductTail *tail, TcZeroed zeroed) {
     auto mark = [&](cudaEvent_t ev) {
         if (ev) cudaEventRecord(ev, st);
     };

@@ -9,16 +9,16 @@ struct ScaleArg {
     float s[kMaxD];
 };
 
-// Xs[i, d] = X[i, d] * scale[d] for i < N, d < D; zero in the padded rows and columns. Clears 64 and 32 words for the
-// kernels that follow (a memset node would end the chain of launches).
+// Xs[i, d] = X[i, d] * scale[d] for i < N, d < D; zero in the padded rows and columns. Clears 64 and 32 words (where given)
+// for the kernels that follow (a memset node would end the chain of launches).
 __global__ void prep_x_kernel(const float *__restrict__ X, int64_t N, int D, int dpad, ScaleArg sc,
                               float *__restrict__ Xs, int64_t Np, int *err_flag, unsigned int *zero64,
                               unsigned int *zero32) {
     chain_wait();
     chain_next();
-    if (blockIdx.x == 0 && zero64 && threadIdx.x < 64) {
-        zero64[threadIdx.x] = 0u;
-        if (threadIdx.x < 32) zero32[threadIdx.x] = 0u;
+    if (blockIdx.x == 0 && threadIdx.x < 64) {
+        if (zero64) zero64[threadIdx.x] = 0u;
+        if (zero32 && threadIdx.x < 32) zero32[threadIdx.x] = 0u;
     }
     const int64_t total = Np * dpad;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
