@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "device_once.cuh"
 #include "lgp.h"
 
 namespace lgp {
@@ -216,6 +217,15 @@ cudaError_t launch_chained(void (*kernel)(Params...), dim3 grid, int threads, si
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
+// Lets a kernel be launched with `bytes` of dynamic shared memory on the current device (set once per device).
+template <class Kernel> cudaError_t allow_shared(DeviceOnce &once, Kernel kernel, int bytes) {
+    int dev = -1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess || once.has(dev)) return e;
+    if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)) == cudaSuccess) once.add(dev);
+    return e;
 }
 
 // ---------------------------------------------------------------- CG state on the device

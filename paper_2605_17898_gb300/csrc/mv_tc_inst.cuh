@@ -11,13 +11,9 @@ cudaError_t launch_tc_inst(dim3 grid, const CUtensorMap &mx, const CUtensorMap &
                            const TcArgs &a, cudaStream_t st) {
     constexpr int DP = D <= 4 ? 4 : 8;
     constexpr int bytes = TcLayout<T, DP, (D <= 4)>::kBytes;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(mv_tc_kernel<KIND, D, T, FMT>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static DeviceOnce configured;
+    const cudaError_t e = allow_shared(configured, mv_tc_kernel<KIND, D, T, FMT>, bytes);
+    if (e != cudaSuccess) return e;
     return launch_chained(mv_tc_kernel<KIND, D, T, FMT>, grid, kThreads, bytes, st, mx, mv, a);
 }
 

@@ -13,13 +13,9 @@ cudaError_t launch_tcs_inst(dim3 grid, const CUtensorMap &mx, const CUtensorMap 
                             cudaStream_t st) {
     constexpr int DP = D <= 4 ? 4 : 8;
     constexpr int bytes = TcsLayout<T, DP, DOT>::kBytes;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(mv_tcs_kernel<KIND, D, T, FMT, DOT, BANDED>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static DeviceOnce configured;
+    const cudaError_t e = allow_shared(configured, mv_tcs_kernel<KIND, D, T, FMT, DOT, BANDED>, bytes);
+    if (e != cudaSuccess) return e;
     return launch_chained(mv_tcs_kernel<KIND, D, T, FMT, DOT, BANDED>, grid, kTcsThreads, bytes, st, mx, mv, mo, a);
 }
 
