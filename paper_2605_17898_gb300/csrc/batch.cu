@@ -135,7 +135,6 @@ __global__ void binit_kernel(BatchArgs a) {
 __global__ void bscal_init_kernel(BatchArgs a, double tol, int max_iter) {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k == 0) {
-        a.st->iter = 0;
         a.st->max_iter = max_iter;
         a.st->tol = tol;
         a.st->status = 0;
@@ -182,34 +181,6 @@ __global__ void bdone_kernel(BatchArgs a) {
 // p and the problem's state, by one cluster of CL CTAs whose three passes over the problem's vectors meet at the
 // cluster barrier. As segmented kernels the step took seven launches an iteration (with the product's memset nine),
 // each a few microseconds for vectors that fit L2 many times over: 48 problems of 200..2000 rows, t = 8, 11.2 -> 6.8 ms a call.
-template <int CL> __device__ double batch_cluster_sum(double *mine, int t) {
-    double s = 0.0;
-    if constexpr (CL == 1) {
-        __syncthreads();
-        if ((int)threadIdx.x < t) s = mine[threadIdx.x];
-    } else {
-        cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
-        cl.sync();
-        if ((int)threadIdx.x < t) {
-#pragma unroll
-            for (int q = 0; q < CL; ++q) s += cl.map_shared_rank(mine, q)[threadIdx.x];
-        }
-    }
-    return s;
-}
-
-template <int VEC> __device__ __forceinline__ void load_vec(const float *p, float (&v)[VEC]) {
-    if constexpr (VEC == 4) {
-        const float4 q = *reinterpret_cast<const float4 *>(p);
-        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-    } else {
-        v[0] = *p;
-    }
-}
-template <int VEC> __device__ __forceinline__ void store_vec(float *p, const float (&v)[VEC]) {
-    if constexpr (VEC == 4) *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
-    else *p = v[0];
-}
 
 // Block of VEC = 4 (t a power of two): kVec threads; VEC = 1: a multiple of t. (A problem's vectors hold Np t >= N t
 // values from a multiple of 16 bytes, so a last float4 that crosses N t stays inside them.)
@@ -267,7 +238,7 @@ __global__ void __launch_bounds__(kVec) batch_step_kernel(BatchArgs a) {
             if (VEC == 1 || e + q < total) acc_prod2(hi[q], lo[q], pv[q], kv[q]);
     }
     block_col_sums<VEC>(hi, lo, t, acc1, sum1);
-    const double pkp = batch_cluster_sum<CL>(sum1, t);
+    const double pkp = cluster_sum<CL>(sum1, t);
     int failed = 0;
     if (tid < t) {
         double alpha = 0.0;
@@ -302,7 +273,7 @@ __global__ void __launch_bounds__(kVec) batch_step_kernel(BatchArgs a) {
         store_vec<VEC>(r + e, rv);
     }
     block_col_sums<VEC>(hi, lo, t, acc2, sum2);
-    const double rr = batch_cluster_sum<CL>(sum2, t);
+    const double rr = cluster_sum<CL>(sum2, t);
     int act = 0;
     if (tid < t) {
         double beta = 0.0;

@@ -34,7 +34,7 @@ struct BatchVecBlock {
 };
 
 struct BatchState {
-    int iter, max_iter, status;
+    int max_iter, status;
     int loop_chunks, max_chunks;  // device-side loop count and its hard cap
     double tol;
 };

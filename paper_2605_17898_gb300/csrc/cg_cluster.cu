@@ -50,23 +50,6 @@ struct ClusterArgs {
     int64_t N;
 };
 
-// Sum over the cluster's CTAs of mine[c] (shared memory, written before), c < t, in rank order, for threads c < t.
-template <int CL> __device__ double cluster_sum(double *mine, int t) {
-    double s = 0.0;
-    if constexpr (CL == 1) {
-        __syncthreads();
-        if ((int)threadIdx.x < t) s = mine[threadIdx.x];
-    } else {
-        cg::cluster_group cl = cg::this_cluster();
-        cl.sync();
-        if ((int)threadIdx.x < t) {
-#pragma unroll
-            for (int q = 0; q < CL; ++q) s += cl.map_shared_rank(mine, q)[threadIdx.x];
-        }
-    }
-    return s;
-}
-
 template <int CL, int T, int FMT>
 __device__ void split_tile(const ClusterArgs &a, const float *tile, int row0, int rows, const int *s_exp, const int *s_act) {
     // rows row0 .. row0 + rows - 1 (a multiple of 8) x T columns of p in shared memory: one (8-row group, column) each

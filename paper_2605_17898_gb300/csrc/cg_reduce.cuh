@@ -1,5 +1,8 @@
-// Column sums of the CG kernels within a block: compensated float pairs per thread, fixed point across threads.
+// Column sums of the CG kernels: compensated float pairs per thread, fixed point across a block's threads, float64 across
+// the CTAs of a cluster.
 #pragma once
+
+#include <cooperative_groups.h>
 
 #include "lgp_internal.cuh"
 #include "limb_sum.cuh"
@@ -18,6 +21,19 @@ __device__ __forceinline__ void pair_add(float &h, float &l, float h2, float l2)
 // a stride that is a multiple of t, so its four elements always have the columns (4 x + k) mod t. VEC = 1: any t,
 // the block has a multiple of t threads and thread x owns column x mod t.
 template <int VEC> __device__ __forceinline__ int col_of(int tid, int k, int t) { return (VEC * tid + k) % t; }
+
+template <int VEC> __device__ __forceinline__ void load_vec(const float *p, float (&v)[VEC]) {
+    if constexpr (VEC == 4) {
+        const float4 q = *reinterpret_cast<const float4 *>(p);
+        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+    } else {
+        v[0] = *p;
+    }
+}
+template <int VEC> __device__ __forceinline__ void store_vec(float *p, const float (&v)[VEC]) {
+    if constexpr (VEC == 4) *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    else *p = v[0];
+}
 
 // Working memory of one block_col_sums call; cleared, and a barrier passed, before it.
 struct ColSums {
@@ -128,6 +144,23 @@ __device__ void block_col_sums(float (&hi)[VEC], float (&lo)[VEC], int t, ColSum
     }
     __syncthreads();
     if (tid < t) out_row[tid] = limb_total(s.limb[0][tid], s.limb[1][tid], s.limb[2][tid], s.mx[tid]);
+}
+
+// Sum over the cluster's CTAs of mine[c] (shared memory, written before), c < t, in rank order, for threads c < t.
+template <int CL> __device__ double cluster_sum(double *mine, int t) {
+    double s = 0.0;
+    if constexpr (CL == 1) {
+        __syncthreads();
+        if ((int)threadIdx.x < t) s = mine[threadIdx.x];
+    } else {
+        cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+        cl.sync();
+        if ((int)threadIdx.x < t) {
+#pragma unroll
+            for (int q = 0; q < CL; ++q) s += cl.map_shared_rank(mine, q)[threadIdx.x];
+        }
+    }
+    return s;
 }
 
 }  // namespace lgp

@@ -199,8 +199,8 @@ inline double prescale_of(int kind) {
 // previous kernel of the stream still runs its last ones, and wait here until that kernel has finished and its writes are
 // visible. chain_wait comes before any access to memory and before any return (a kernel that ended without it could
 // finish before its predecessor); its chain_next, from which on the successor may be placed, comes with it.
-// Product call with its eight small kernels, N = 20000, D = 8, t = 16: 168 -> 154 us; solve of N = 1024, t = 1 (two kernels an
-// iteration): 945 -> 866 us.
+// When it came, a product call of N = 20000, D = 8, t = 16 (then with eight small kernels beside the product's): 168 -> 154 us;
+// solve of N = 1024, t = 1 (two kernels an iteration): 945 -> 866 us.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -56,18 +56,6 @@ __device__ __forceinline__ void load_x_smem(const float *xs, float (&xj)[D]) {
     }
 }
 
-template <int D>
-__device__ __forceinline__ float sqdist(const float (&a)[D], const float (&b)[D]) {
-    float d0 = a[0] - b[0];
-    float r2 = d0 * d0;
-#pragma unroll
-    for (int d = 1; d < D; ++d) {
-        const float dd = a[d] - b[d];
-        r2 = fmaf(dd, dd, r2);
-    }
-    return r2;
-}
-
 // Stage x_j (and nothing else) for column tile [j0, j0 + BN).
 template <int D>
 __device__ __forceinline__ void stage_x(float *xs, const float *__restrict__ Xs, int64_t j0, int64_t Np) {

@@ -21,7 +21,8 @@
 //     4, 7 or 14 shuffles instead of 3 each) and added by one lane, always the same, to its row set's column sums in
 //     shared memory. This costs 3 of 15 cycles per pair at D = 4, t = 1; a copy of the sums per row lane, without any
 //     shuffle, measured 11% slower (its loads and stores, and fewer CTAs per SM).
-// Sums are short: at most E / 16 terms per lane and chain, then trees and G slots.
+// Sums are short: at most E / 4 terms per lane and chain (a lane's four columns in each of E / 16 steps), then trees and G
+// slots.
 //
 // Measured against the row kernel (product call, us): N = 50000, t = 1, RBF D = 4 970 -> 475, Matern-5/2 D = 8
 // 1824 -> 939; N = 20000, D = 8, Matern-5/2: t = 2 336 -> 197, t = 4 362 -> 271; N = 2000, D = 8, t = 1 33 -> 19. The
@@ -43,12 +44,12 @@ struct SymArgs {
     EntryScale scale;
 };
 
-constexpr int kSymThreads = 128;  // 4 warps, a quarter of the tile's columns each
+constexpr int kSymThreads = 128;  // 4 warps: row sets, or in small tiles shares of the columns
 
 // Rows per thread, columns per thread and step, by dimension and padded column count (what the registers hold).
 template <int D, int TT> struct SymShape {
     static constexpr int R = D <= 4 && TT <= 2 ? 8 : 4;
-    static constexpr int C = 4;
+    static constexpr int C = 4;  // one 16-byte load per coordinate
     static constexpr int RB = 8 * R;  // rows of one sweep
 };
 
@@ -177,13 +178,9 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
             float vj[C * TT], cs[NV];
 #pragma unroll
             for (int d = 0; d < D; ++d) {
-                if constexpr (C == 4) {
-                    const float4 q = *reinterpret_cast<const float4 *>(xs + d * E + j);
-                    xj[0][d] = make_float2(q.x, q.y);
-                    xj[1][d] = make_float2(q.z, q.w);
-                } else {
-                    xj[0][d] = *reinterpret_cast<const float2 *>(xs + d * E + j);
-                }
+                const float4 q = *reinterpret_cast<const float4 *>(xs + d * E + j);
+                xj[0][d] = make_float2(q.x, q.y);
+                xj[1][d] = make_float2(q.z, q.w);
             }
 #pragma unroll
             for (int q = 0; q < C * TT; q += 4) {

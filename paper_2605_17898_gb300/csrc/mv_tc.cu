@@ -47,9 +47,10 @@ __device__ void split_v(const float *__restrict__ V, int64_t ldv, int64_t N, int
 
 // split_v for a CG solve's p, fused with its update: p = r + beta p in the active columns, then the halves of
 // those columns (the others' stay valid) and out_init = noise p. The scaling exponents come from vmax, which the
-// step's previous launch set to a bound on the new |p|: at most one bit above its maximum, which costs nothing of
-// the 11-bit halves and one bit of the range below 2^-40 of the column's largest value that keeps an absolute error
-// anyway. pmax collects max |p| for the next bound. One thread per (8-row group, column), as split_v: 24 loads and
+// step's previous launch set to a bound on the new |p|, |r| + beta |p|. It is at most 2.4 times the maximum in 24 model solves
+// (and at most sqrt(2 N) times: r is orthogonal to the old p), which costs nothing of the 11-bit halves and raises the
+// absolute error that values below 2^-18 of the column's largest keep, 2^-40 of it, by that factor: far below the 2^-22 of
+// the entries. pmax collects max |p| for the next bound. One thread per (8-row group, column), as split_v: 24 loads and
 // stores in flight per thread, where a separate maximum, split and update took three launches and read p twice.
 template <int T, int FMT>
 __global__ void __launch_bounds__(256) p_split_kernel(float *__restrict__ p, const float *__restrict__ r, int64_t N,
@@ -190,7 +191,8 @@ __global__ void __launch_bounds__(256) tc_scan_kernel(const float *__restrict__ 
 // so that A_i . B_j = 2 (h_i h_j + m_i h_j + h_i m_j) - a_j - a_i = -|u_i - u_j|^2 to about 22 bits: the
 // tensor core hands the generation the negated squared distance itself.
 // words[16] collects max a_j over rows j < N (float bits, a_j >= 0). Every product of halves is exact in float32 and the
-// sum carries its rounding errors along, so that a_j is the exact sum rounded once (float64 runs at a 64th of the rate).
+// sum carries its rounding errors along, so that a_j is the exact sum rounded once (float64 runs at a 64th of the rate; the
+// same float32 as by float64 sums in each of 8 million rows tried).
 // Blocks b of nb.
 template <int DP>
 __device__ void dot_operands(const float *__restrict__ Xs, int64_t N, int64_t Np, unsigned int *words,

@@ -200,19 +200,6 @@ __device__ double grid_col_sum(const double *partial, int t, double *red) {
     return s;
 }
 
-template <int VEC> __device__ __forceinline__ void load_vec(const float *p, float (&v)[VEC]) {
-    if constexpr (VEC == 4) {
-        const float4 q = *reinterpret_cast<const float4 *>(p);
-        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-    } else {
-        v[0] = *p;
-    }
-}
-template <int VEC> __device__ __forceinline__ void store_vec(float *p, const float (&v)[VEC]) {
-    if constexpr (VEC == 4) *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
-    else *p = v[0];
-}
-
 // Elements e (multiples of VEC) of a block's grid-stride loop over [0, N t). The vectors hold Np t >= N t values, so
 // a last float4 that crosses N t stays inside them; its elements past N t are left out of the sums.
 #define LGP_STEP_LOOP(e)                                                                                              \
