@@ -46,7 +46,7 @@ __device__ void batch_item(const BatchGp &g, int64_t row0, int split, const Batc
         } else {
 #pragma unroll
             for (int c = 0; c < TT; ++c)
-                if (c < t) out[i * t + c] = fmaf(g.noise, V[i * t + c], sum[r][c]);
+                if (c < t) out[i * t + c] = fmaf(g.noise, V[i * t + c], scaled_out<KIND>(sum[r][c], g.scale));
         }
     }
 }
@@ -177,7 +177,7 @@ __global__ void bdone_kernel(BatchArgs a) {
 
 // ---------------------------------------------------------------- the CG step
 
-// One problem's CG step after the product: Kp = sum_k part[k] + noise p (or as the product left it), alpha, x, r, beta,
+// One problem's CG step after the product: Kp = scale sum_k part[k] + noise p (or as the product left it), alpha, x, r, beta,
 // p and the problem's state, by one cluster of CL CTAs whose three passes over the problem's vectors meet at the
 // cluster barrier. As segmented kernels the step took seven launches an iteration (with the product's memset nine),
 // each a few microseconds for vectors that fit L2 many times over: 48 problems of 200..2000 rows, t = 8, 11.2 -> 6.8 ms a call.
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(kVec) batch_step_kernel(BatchArgs a) {
                 for (int q = 0; q < VEC; ++q) kv[q] += w[q];
             }
 #pragma unroll
-            for (int q = 0; q < VEC; ++q) kv[q] = fmaf(g.noise, pv[q], kv[q]);
+            for (int q = 0; q < VEC; ++q) kv[q] = fmaf(g.noise, pv[q], g.scale.out * kv[q]);
             store_vec<VEC>(kp + e, kv);
         } else {
             load_vec<VEC>(kp + e, kv);

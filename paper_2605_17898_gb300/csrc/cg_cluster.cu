@@ -41,7 +41,7 @@ struct ClusterArgs {
     const float *part;  // the product's partial sums (nullptr: Kp is complete)
     int S;
     int64_t part_stride;
-    float noise;
+    float scale, noise;
     int total, t;  // N t
     CgState *st;
     double *hist_alpha, *hist_beta;
@@ -115,10 +115,10 @@ __global__ void __launch_bounds__(kClThreads, 1) cg_cluster_kernel(const Cluster
             k4.z += w.z;
             k4.w += w.w;
         }
-        k4.x = fmaf(a.noise, p4.x, k4.x);
-        k4.y = fmaf(a.noise, p4.y, k4.y);
-        k4.z = fmaf(a.noise, p4.z, k4.z);
-        k4.w = fmaf(a.noise, p4.w, k4.w);
+        k4.x = fmaf(a.noise, p4.x, a.scale * k4.x);
+        k4.y = fmaf(a.noise, p4.y, a.scale * k4.y);
+        k4.z = fmaf(a.noise, p4.z, a.scale * k4.z);
+        k4.w = fmaf(a.noise, p4.w, a.scale * k4.w);
         return k4;
     };
 #pragma unroll
@@ -401,6 +401,7 @@ cudaError_t launch_cg_cluster(int ctas, int64_t N, int t, const CgBuffers &b, co
     a.part = tail.part;
     a.S = tail.S;
     a.part_stride = tail.stride;
+    a.scale = tail.scale;
     a.noise = tail.noise;
     a.total = (int)(N * t);
     a.t = t;

@@ -163,9 +163,9 @@ template <> struct PackedEntry<LGP_MATERN32> {
     }
 };
 
-// The outputscale of the kernels on PackedEntry: log2 s^2 in the exponent (Matern), or for RBF s^2 as the factor of V or
-// of the finished sums, on the side where neither the products nor the sums can leave the float32 range that the full
-// entries had.
+// The outputscale of the kernels on PackedEntry: log2 s^2 in the exponent (Matern), or for RBF s^2 as the factor of V (v, in
+// the kernels) or of the finished sums (out, where the partial sums are added up), on the side where neither the products
+// nor the sums can leave the float32 range that the full entries had.
 struct EntryScale {
     float log2s2 = 0.0f, v = 1.0f, out = 1.0f;
 };
@@ -174,6 +174,15 @@ inline EntryScale entry_scale(const KernelParams &kp) {
     if (kp.kind != LGP_RBF) s.log2s2 = kp.log2_s2;
     else (kp.s2 < 1.0f ? s.v : s.out) = kp.s2;
     return s;
+}
+
+template <int KIND> __device__ __forceinline__ float scaled_v(float v, const EntryScale &s) {
+    if constexpr (KIND == LGP_RBF) return v * s.v;
+    else return v;
+}
+template <int KIND> __device__ __forceinline__ float scaled_out(float v, const EntryScale &s) {
+    if constexpr (KIND == LGP_RBF) return v * s.out;
+    else return v;
 }
 
 // Host: the kind is one the library implements.
@@ -273,12 +282,12 @@ void launch_var_from_probes(const float *Z, int64_t ldz, const float *Q, int64_t
                             float *var, cudaStream_t st);
 
 // What a product left for its caller to finish when asked to (the CG step, which reads the same rows anyway):
-// S partial sums, out = sum_k part[k * stride + e] + noise V. part = nullptr: out is complete.
+// S partial sums, out = scale sum_k part[k * stride + e] + noise V. part = nullptr: out is complete.
 struct ProductTail {
     const float *part = nullptr;
     int S = 0;
     int64_t stride = 0;
-    float noise = 0.0f;
+    float scale = 1.0f, noise = 0.0f;
 };
 
 // mv_simt.cu

