@@ -33,7 +33,7 @@ __device__ void batch_item(const BatchGp &g, int64_t row0, int split, const Batc
     const int64_t jb = (int64_t)split * g.cols_per_split;
     const int64_t je = min(g.N, jb + g.cols_per_split);
     float sum[S::R][TT];
-    simt_rows<KIND, D, S>(Xs, row0, g.Np, Xs, g.Np, V, t, 0, t, jb, je, g.scale, xs, vs, tot, sum);
+    simt_rows<KIND, D, S>(Xs, row0, g.Np, Xs, g.Np, V, t, 0, t, jb, je, g.scale.log2s2, g.scale.v, xs, vs, tot, sum);
 #pragma unroll
     for (int r = 0; r < S::R; ++r) {
         const int64_t i = row0 + r * S::kThreads + threadIdx.x;
@@ -46,7 +46,7 @@ __device__ void batch_item(const BatchGp &g, int64_t row0, int split, const Batc
         } else {
 #pragma unroll
             for (int c = 0; c < TT; ++c)
-                if (c < t) out[i * t + c] = fmaf(g.noise, V[i * t + c], scaled_out<KIND>(sum[r][c], g.scale));
+                if (c < t) out[i * t + c] = fmaf(g.noise, V[i * t + c], rbf_scaled<KIND>(sum[r][c], g.scale.out));
         }
     }
 }

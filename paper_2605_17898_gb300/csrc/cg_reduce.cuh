@@ -47,7 +47,7 @@ __device__ __forceinline__ void clear_sums(ColSums &s) {
     }
 }
 
-// v[k] of the lanes that hold the same columns (those that agree mod group, group = 2 .. 16) combined by op, each step
+// v[k] of the lanes that hold the same columns (those that agree mod group, group = 1 .. 16) combined by op, each step
 // halving what a lane carries: for group <= 8 the result in r[0] is that of k = 2 bit4 + bit3 of the lane (the same in lanes
 // that differ only in the bits from group to 4), for group = 16 r[0] and r[1] are those of k = 2 bit4 and the next.
 template <class T, class Op> __device__ __forceinline__ void fold_columns(const T (&v)[4], int group, int lane, Op op, T (&r)[2]) {
@@ -64,9 +64,10 @@ template <class T, class Op> __device__ __forceinline__ void fold_columns(const 
 // Sums the float pairs of every column over the block: out_row[c] = their float64 value, c < t, written by thread c.
 // The sum across threads is the block's largest magnitude per column, then integer sums (limb_sum.cuh): float64 additions
 // would take 64 cycles of a sub-partition per warp (a tree over 512 threads 1650 cycles), float pairs lose bits and
-// overflow where float64 does not. Up to 4 columns a warp's maximum and sums are one reduction instruction each. An
-// iteration with its product, pairs by shuffles -> this: N = 2000, D = 6, t = 1 18.2 -> 16.6 us, t = 8 20.3 -> 20.1, t = 4 20.1 ->
-// 20.3; N = 4000, t = 32 40.5 -> 39.0; N = 20000, D = 8, t = 32 156.3 -> 153.8.
+// overflow where float64 does not. At 1 and 2 columns a warp's maximum and sums are one reduction instruction each (at 4
+// their 16 are slower than folding: N = 500, t = 4 15.3 and 14.7 us an iteration). An iteration with its product, pairs by
+// shuffles -> this: N = 2000, D = 6, t = 1 18.2 -> 16.6 us, t = 8 20.3 -> 20.1; N = 500, t = 4 14.2 -> 14.7; N = 4000, t = 32 40.5 ->
+// 39.0; N = 20000, D = 8, t = 32 156.3 -> 153.8.
 template <int VEC>
 __device__ void block_col_sums(float (&hi)[VEC], float (&lo)[VEC], int t, ColSums &s, double *out_row) {
     const int tid = threadIdx.x;
@@ -91,7 +92,7 @@ __device__ void block_col_sums(float (&hi)[VEC], float (&lo)[VEC], int t, ColSum
             pair_add(hi[1], lo[1], hi[3], lo[3]);
         }
         const int group = t > 4 ? t / 4 : 1;  // lanes that hold one row of columns
-        if (group == 1) {
+        if (t < 4) {
 #pragma unroll
             for (int k = 0; k < VEC; ++k) {
                 if (k >= t) break;

@@ -176,12 +176,8 @@ inline EntryScale entry_scale(const KernelParams &kp) {
     return s;
 }
 
-template <int KIND> __device__ __forceinline__ float scaled_v(float v, const EntryScale &s) {
-    if constexpr (KIND == LGP_RBF) return v * s.v;
-    else return v;
-}
-template <int KIND> __device__ __forceinline__ float scaled_out(float v, const EntryScale &s) {
-    if constexpr (KIND == LGP_RBF) return v * s.out;
+template <int KIND> __device__ __forceinline__ float rbf_scaled(float v, float scale) {
+    if constexpr (KIND == LGP_RBF) return v * scale;
     else return v;
 }
 

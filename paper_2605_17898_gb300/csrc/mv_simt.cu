@@ -265,7 +265,10 @@ cudaError_t launch_mv_simt(const MvLaunch &m, cudaStream_t st) {
     a.ldo = m.ldo;
     a.cols_per_split = cps;
     a.t = m.t;
-    a.scale = entry_scale(*m.kp);
+    const EntryScale es = entry_scale(*m.kp);
+    a.log2s2 = es.log2s2;
+    a.v_scale = es.v;
+    a.out_scale = es.out;
     a.noise = m.kp->noise;
     const dim3 grid((unsigned)rb, (unsigned)S, (unsigned)cg);
     cudaError_t e;

@@ -31,11 +31,14 @@ struct SimtArgs {
     int64_t N, Np, ldv, ldo;
     int64_t Nr, Npr;   // rows of the output, and of Xr
     int cross;         // 1: out = K(Xr, Xs) V with no noise term
-    int64_t cols_per_split;
+    float v_scale;     // EntryScale, between the others: with more than 128 bytes of arguments the compiler allots registers
+    int64_t cols_per_split;  // differently, up to 9% slower (Matern-5/2, D = 5, t = 12, N = 25000 726 -> 793 us)
     int t;
-    EntryScale scale;
+    float log2s2;
     float noise;
+    float out_scale;
 };
+static_assert(sizeof(SimtArgs) == 128, "see v_scale");
 
 template <int D> struct DPad { static constexpr int value = D <= 4 ? 4 : 8; };
 
@@ -87,13 +90,13 @@ template <int TT_, int R_, int THREADS> struct RowTile {
 template <int TT> using RowShape = RowTile<TT, TT == 32 ? 2 : 4, 64>;
 
 // sum_j k(x_i, x_j) V[j, c0..c0+TT) over jb <= j < je for this thread's rows i = row0 + r kThreads + tid, added up per
-// tile of kSimtBN columns (without the factor scale.out). Distances run on packed operations over pairs of columns (x_j - x_i as x_j + (-x_i), the
-// row's coordinates kept twice), the V multiply-adds are scalar (three different register pairs would run at half
+// tile of kSimtBN columns (RBF: without EntryScale's out). Distances run on packed operations over pairs of columns (x_j -
+// x_i as x_j + (-x_i), the row's coordinates kept twice), the V multiply-adds are scalar (three different register pairs would run at half
 // rate). xs [D][kSimtBN], vs [kSimtBN][TT], tot [kTotFloats]: shared memory.
 template <int KIND, int D, class S>
 __device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t row0, int64_t Npr,
                                           const float *__restrict__ Xs, int64_t Np, const float *__restrict__ V, int64_t ldv,
-                                          int c0, int t, int64_t jb, int64_t je, EntryScale scale, float *xs, float *vs,
+                                          int c0, int t, int64_t jb, int64_t je, float log2s2, float v_scale, float *xs, float *vs,
                                           float *tot, float (&sum)[S::R][S::TT]) {
     constexpr int DP = DPad<D>::value, TT = S::TT, R = S::R, NT = S::kThreads;
     const int tid = threadIdx.x;
@@ -112,7 +115,7 @@ __device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t 
             if constexpr (S::kTotShared) tot[(r * TT + c) * NT + tid] = 0.0f;
         }
     }
-    const float2 acc0 = PackedEntry<KIND>::acc0(scale.log2s2);
+    const float2 acc0 = PackedEntry<KIND>::acc0(log2s2);
     for (int64_t j0 = jb; j0 < je; j0 += kSimtBN) {
         __syncthreads();
         for (int e = tid; e < kSimtBN * (DP / 4); e += NT) {
@@ -126,7 +129,7 @@ __device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t 
         }
         for (int e = tid; e < kSimtBN * TT; e += NT) {
             const int jj = e / TT, c = e - jj * TT;
-            vs[e] = (j0 + jj < je && c0 + c < t) ? scaled_v<KIND>(V[(j0 + jj) * ldv + c0 + c], scale) : 0.0f;
+            vs[e] = (j0 + jj < je && c0 + c < t) ? rbf_scaled<KIND>(V[(j0 + jj) * ldv + c0 + c], v_scale) : 0.0f;
         }
         __syncthreads();
         float acc[R][TT];
@@ -148,7 +151,7 @@ __device__ __forceinline__ void simt_rows(const float *__restrict__ Xr, int64_t 
                     dd = __fadd2_rn(xj[d], xi[r][d]);
                     r2 = __ffma2_rn(dd, dd, r2);
                 }
-                k[r] = PackedEntry<KIND>::k(r2, scale.log2s2);
+                k[r] = PackedEntry<KIND>::k(r2, log2s2);
             }
             constexpr int CV = TT < 4 ? TT : 4;  // V columns per load
 #pragma unroll
@@ -202,7 +205,7 @@ __global__ void __launch_bounds__(RowShape<TT>::kThreads) mv_simt_kernel(SimtArg
     const int64_t jb = (int64_t)blockIdx.y * a.cols_per_split;
     const int64_t je = min(a.N, jb + a.cols_per_split);
     float sum[S::R][TT];
-    simt_rows<KIND, D, S>(a.Xr, row0, a.Npr, a.Xs, a.Np, a.V, a.ldv, c0, a.t, jb, je, a.scale, xs, vs, tot, sum);
+    simt_rows<KIND, D, S>(a.Xr, row0, a.Npr, a.Xs, a.Np, a.V, a.ldv, c0, a.t, jb, je, a.log2s2, a.v_scale, xs, vs, tot, sum);
 #pragma unroll
     for (int r = 0; r < S::R; ++r) {
         const int64_t i = row0 + r * S::kThreads + threadIdx.x;
@@ -215,9 +218,8 @@ __global__ void __launch_bounds__(RowShape<TT>::kThreads) mv_simt_kernel(SimtArg
         } else {
 #pragma unroll
             for (int c = 0; c < TT; ++c)
-                if (c0 + c < a.t)
-                    {
-                    const float v = scaled_out<KIND>(sum[r][c], a.scale);
+                if (c0 + c < a.t) {
+                    const float v = rbf_scaled<KIND>(sum[r][c], a.out_scale);
                     a.out[i * a.ldo + c0 + c] = a.cross ? v : fmaf(a.noise, a.V[i * a.ldv + c0 + c], v);
                 }
         }

@@ -133,7 +133,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
     }
     for (int e = tid; e < E * TT; e += kSymThreads) {
         const int j = e / TT, c = e - j * TT;
-        vs[e] = (j0 + j < a.N && c < a.t) ? scaled_v<KIND>(a.V[(j0 + j) * a.ldv + c], a.scale) : 0.0f;
+        vs[e] = (j0 + j < a.N && c < a.t) ? rbf_scaled<KIND>(a.V[(j0 + j) * a.ldv + c], a.scale.v) : 0.0f;
     }
     for (int e = tid; e < WR * E * TT; e += kSymThreads) col[e] = 0.0f;
     __syncthreads();
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kSymThreads) mv_sym_kernel(SymArgs a) {
             for (int d = 0; d < D; ++d) xi[r][d] = make_float2(x[d], x[d]);
 #pragma unroll
             for (int c = 0; c < TT; ++c) {
-                vi[r][c] = i < a.N && c < a.t ? scaled_v<KIND>(a.V[i * a.ldv + c], a.scale) : 0.0f;
+                vi[r][c] = i < a.N && c < a.t ? rbf_scaled<KIND>(a.V[i * a.ldv + c], a.scale.v) : 0.0f;
                 acc[r][c] = 0.0f;
             }
         }
