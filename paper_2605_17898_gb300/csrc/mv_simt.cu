@@ -68,9 +68,9 @@ SymGrid sym_grid(int64_t N, int64_t Np, int t, int D, int num_sms) {
     if (t > 4) return g;
     // The largest blocks that still give every SM enough tiles to even out the last ones (a tile's set-up and its
     // sums are paid per tile, and each block is one more partial sum per row: N = 50000, D = 4, t = 1 with
-    // E = 256 535 us, 512 476); larger ones only to keep the partial sums in bounds. Blocks of 128 from one tile per SM
-    // on, because a solve's vector step reads every partial sum: an iteration at N = 4500, t = 4, D = 6 with
-    // E = 64 52 us, 128 36; N = 2500, t = 1 21.8 and 18.2; N = 1200, D = 8, t = 4 (55 tiles) 19.2 and 21.6.
+    // E = 256 535 us, 512 476); larger ones only to keep the partial sums in bounds. (A solve's vector step reads every
+    // partial sum, so that blocks of 128 from one tile per SM on would make its iterations faster, N = 2500, t = 1 21.8 ->
+    // 18.2 us; but their sums' chains are twice as long, and the products' errors 10% larger there.)
     auto tiles_per_sm = [&](int64_t E) {
         const int64_t G = (N + E - 1) / E;
         return G * (G + 1) / 2 / num_sms;
@@ -79,7 +79,7 @@ SymGrid sym_grid(int64_t N, int64_t Np, int t, int D, int num_sms) {
     int64_t E = 64;
     if (tiles_per_sm(512) >= 16) E = 512;
     else if (tiles_per_sm(256) >= 8) E = 256;
-    else if (tiles_per_sm(128) >= 1) E = 128;
+    else if (tiles_per_sm(128) >= 5) E = 128;
     auto bytes = [&](int64_t e) { return (N + e - 1) / e * Np * t * (int64_t)sizeof(float); };
     if (E == 512 && bytes(E) > kSymMaxPartial && 2 * (sym_smem_bytes(D, TT, 1024) + kCtaReserved) <= kSmShared) E = 1024;
     if (bytes(E) > kSymMaxPartial) return g;
